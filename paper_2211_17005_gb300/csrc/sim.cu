@@ -1,18 +1,16 @@
 // Inner-default kernel of the hierarchical CVA simulation, and the dispatch
 // of the outer-path kernel instantiations (outer_*.cu).
 //
-// Inner defaults (Sec. 3.2 / eq. (e:tau)), two kernels:
-//   inner_count_kernel   one warp per outer path: N default clocks per
-//     counterparty; tau^{k,l} falls in (t_{j-1}, t_j] when the uniform w
-//     (epsilon = -log(1 - w)) satisfies T(j-1) < w <= T(j), T = 1 - e^{-Lambda};
-//     the default step is the lower bound of w in the monotone thresholds, and
-//     the integer count of defaults per (counterparty, step) goes to global memory;
-//   inner_target_kernel  one thread per outer path: the averaged target of eq.
-//     (eq:CVA_portfolio) of every portfolio from the counts,
-//       xi_bar_i = beta_i^{-1} (1/N) sum_{j>i} sum_c V_c(j) count_c(j),
-//     as a running sum over the dates from the last, every load and store
-//     coalesced over consecutive paths.
-// The counts are integers, so the targets do not depend on the order of the draws.
+// Inner defaults (Sec. 3.2 / eq. (e:tau)): N default clocks per counterparty and
+// path; tau^{k,l} falls in (t_{j-1}, t_j] when the uniform w (epsilon = -log(1 - w))
+// satisfies T(j-1) < w <= T(j), T = 1 - e^{-Lambda}: the default step is the lower
+// bound of w in the monotone thresholds. The averaged target of eq.
+// (eq:CVA_portfolio) of every portfolio follows from the integer counts of defaults
+// per (counterparty, step),
+//   xi_bar_i = beta_i^{-1} (1/N) sum_{j>i} sum_c V_c(j) count_c(j),
+// so the targets do not depend on the order of the draws.
+#include <algorithm>
+#include <atomic>
 #include <mutex>
 
 #include "cva_internal.h"
@@ -25,14 +23,15 @@ namespace {
 struct InnerArgs {
     uint32_t M, k0, seed_lo, seed_hi, N;
     uint32_t branch;                  // third counter word of the clocks (twin copy id, 0 otherwise)
-    int n, NPF, P;
+    int n, NPF;
+    int lg;                           // log2 of the paths per block
+    int rows;                         // rows of the threshold area: n max(C, NPF)
+    int packed;                       // 1: two 16-bit counters a word (N <= 65535)
     const float *__restrict__ thr;    // [n+1][C][M]
     const float *__restrict__ expo;   // [NPF][n+1][C][M]
     const float *__restrict__ disc;   // [n+1][M]
     float *targets;                   // [NPF][n][M]
     uint8_t *idx;                     // [M][N][C] or null
-    uint16_t *cnt16;                  // [n+1][C][M] default counts (N <= 65535) ...
-    uint32_t *cnt32;                  // ... or these (larger N)
 };
 
 // First j in [1, n] with T(j) >= w for nondecreasing thresholds T, else n + 1
@@ -51,33 +50,80 @@ __device__ __forceinline__ int lower_bound_pow2(Thr T, int n, float w)
     return pos + 1;
 }
 
-template <int C>
-__global__ void __launch_bounds__(256) inner_count_kernel(InnerArgs a)
+// Clocks, counts and targets of a tile of PT = 2^lg outer paths in one block.
+//
+// A lane owns one path of the tile (lane mod PT) throughout, so shared memory is laid
+// out with the path innermost: the thresholds, staged by cp.async, as [n C][PT]; the
+// counts as [n C][PT], two 16-bit counters a word when every count fits (N <= 65535).
+// Lanes of different paths then never share a bank, and whole rows move between shared
+// and global memory without a transpose.
+//
+// What bounds it: instruction issue while the clocks are drawn, HBM while thresholds and
+// exposures are read. Most clocks outlive the horizon (w > T(n)): a lane compares each
+// with its path's T(n), as an integer bound on the draw's 23 bits, and only queues the
+// ones that default (two draws' at most, in its own column of the queue), so that the
+// lower bounds run over queues a few entries long. The blocks of a multiprocessor are in
+// different phases, which overlaps the two bounds.
+// IDX: the default steps are kept too (cva_sim's validation output).
+template <int C, bool IDX>
+__global__ void __launch_bounds__(512) inner_kernel(InnerArgs a)
 {
     extern __shared__ __align__(16) unsigned char smem[];
-    const int P = a.P, n = a.n, np1 = n + 1;
-    float *thr_s = reinterpret_cast<float *>(smem);                 // [P][C][n+1]
-    // counters [P][C][n+1]: two 16-bit counters per word when every count fits (N <= 65535)
-    uint32_t *cnt_s = reinterpret_cast<uint32_t *>(thr_s + P * C * np1);
-    const bool packed = a.cnt16 != nullptr;
-    const int n_words = packed ? (P * C * np1 + 1) / 2 : P * C * np1;
-    const uint32_t M = a.M, tile0 = blockIdx.x * (uint32_t)P;
-    const int tid = threadIdx.x, nthr = blockDim.x, warp = tid >> 5, lane = tid & 31;
-    const int nwarps = nthr >> 5;
+    const int n = a.n, lg = a.lg, PT = 1 << lg, NPF = a.NPF;
+    const int ps = a.packed;                                                     // 1: two counters a word
+    const int tid = threadIdx.x, nthr = blockDim.x;
+    float *T = reinterpret_cast<float *>(smem);                                  // [rows][PT]: thresholds, then sums
+    uint32_t *cnt = reinterpret_cast<uint32_t *>(T + ((size_t)a.rows << lg));    // counts
+    const int cnt_words = ((n * C + ps) >> ps) << lg;
+    uint32_t *queue = cnt + cnt_words + tid;                                     // [2 C][nthr], this thread's column
+    const uint32_t M = a.M, tile0 = blockIdx.x << lg;
+    const int p = tid & (PT - 1);
+    const bool live = tile0 + (uint32_t)p < M;
 
-    for (int i = tid; i < n * C * P; i += nthr) {
-        const int pk = i % P, jc = i / P, c = jc % C, j = 1 + jc / C;
-        const uint32_t kl = tile0 + pk;
-        thr_s[(pk * C + c) * np1 + j] = (kl < M) ? __ldg(a.thr + ((size_t)j * C + c) * M + kl) : 2.f;
+    {   // row r = (j - 1) C + c of the thresholds, PT consecutive paths
+        const float *src = a.thr + (size_t)C * M + tile0;
+        const uint32_t dst = (uint32_t)__cvta_generic_to_shared(T);
+        if (lg >= 2 && (M & 3u) == 0) {   // every piece of four paths is aligned and whole
+            const int lq = lg - 2;
+            for (int i = tid; i < (n * C) << lq; i += nthr) {
+                const int q = i & ((1 << lq) - 1), r = i >> lq;
+                if (tile0 + 4u * (uint32_t)q < M)
+                    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + 16u * (uint32_t)i),
+                                 "l"(src + (size_t)r * M + 4 * q)
+                                 : "memory");
+            }
+        } else {
+            for (int i = tid; i < (n * C) << lg; i += nthr)
+                if (live)
+                    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst + 4u * (uint32_t)i),
+                                 "l"(src + (size_t)(i >> lg) * M + p)
+                                 : "memory");
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
     }
-    for (int i = tid; i < n_words; i += nthr) cnt_s[i] = 0u;
+    for (int i = tid; i < cnt_words; i += nthr) cnt[i] = 0u;
+    asm volatile("cp.async.wait_all;" ::: "memory");
     __syncthreads();
 
-    for (int pk = warp; pk < P; pk += nwarps) {
-        const uint32_t kl = tile0 + pk;
-        if (kl >= M) continue;
-        const uint32_t k = a.k0 + kl;
-        for (uint32_t l = lane; l < a.N; l += 32) {
+    if (live) {
+        const uint32_t kl = tile0 + (uint32_t)p, k = a.k0 + kl, stride = (uint32_t)(nthr >> lg);
+        // w = (m + 1/2) 2^-23 <= T(n)  <=>  m < bound = floor(2^23 T(n) - 1/2) + 1, every
+        // operation exact (T <= 1; a NaN takes every clock, as the comparison of w would)
+        uint32_t bound[C];
+#pragma unroll
+        for (int c = 0; c < C; ++c) {
+            const float t = T[(((n - 1) * C + c) << lg) + p] * 8388608.f;
+            bound[c] = t >= 0.5f ? (uint32_t)floorf(fminf(t, 8388608.f) - 0.5f) + 1u : t < 0.5f ? 0u : 8388608u;
+        }
+        const uint32_t Tp = (uint32_t)__cvta_generic_to_shared(T + p);
+        auto lds = [](uint32_t addr) {
+            float v;
+            asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(addr));
+            return v;
+        };
+        int queued = 0;
+        bool even = false;
+        for (uint32_t l = (uint32_t)(tid >> lg); l < a.N; l += stride) {
 #pragma unroll
             for (int cb = 0; cb < (C + 3) / 4; ++cb) {
                 const uint4 x = philox4x32_10(make_uint4(k, l, a.branch, (kStreamInner << 24) | (uint32_t)cb),
@@ -87,64 +133,98 @@ __global__ void __launch_bounds__(256) inner_count_kernel(InnerArgs a)
                 for (int i = 0; i < 4; ++i) {
                     const int c = 4 * cb + i;
                     if (c < C) {
-                        const float w = uniform23(xs[i]);
-                        const float *T = thr_s + (pk * C + c) * np1;
-                        const int lo = lower_bound_pow2([T](int j) { return T[j]; }, n, w);
-                        if (a.idx) a.idx[((size_t)kl * a.N + l) * C + c] = (uint8_t)lo;
-                        if (lo <= n) {
-                            const int ci = (pk * C + c) * np1 + lo;
-                            if (packed) atomicAdd(&cnt_s[ci >> 1], 1u << (16 * (ci & 1)));
-                            else atomicAdd(&cnt_s[ci], 1u);
-                        }
+                        const bool hit = (xs[i] >> 9) < bound[c];
+                        if (hit) queue[queued] = (xs[i] & ~0x1ffu) | (uint32_t)c;
+                        queued += hit ? nthr : 0;
+                        if (IDX && !hit) a.idx[((size_t)kl * a.N + l) * C + c] = (uint8_t)(n + 1);
                     }
                 }
             }
+            even = !even;
+            if (!IDX && even && l + stride < a.N) continue;   // the queue holds two draws' defaults
+            even = false;
+            // four entries at a time: their searches interleave
+            for (int t = 0; t < queued; t += 4 * nthr) {
+                float w[4];
+                uint32_t at[4];      // shared address of the search's lower end
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const uint32_t x = t + u * nthr < queued ? queue[t + u * nthr] : 0u;
+                    w[u] = uniform23(x);
+                    at[u] = Tp + ((x & 0x1ffu) << (lg + 2));
+                }
+                // first j with T(j) >= w among 1..n (T(n) >= w): the halving of a range of
+                // n depends on n only, so its steps are the same for every lane
+                for (int len = n; len > 1;) {
+                    const int half = len >> 1;
+                    const uint32_t span = (uint32_t)(half * C) << (lg + 2), probe = span - ((uint32_t)C << (lg + 2));
+#pragma unroll
+                    for (int u = 0; u < 4; ++u)
+                        if (lds(at[u] + probe) < w[u]) at[u] += span;
+                    len -= half;
+                }
+#pragma unroll
+                for (int u = 0; u < 4; ++u)
+                    if (t + u * nthr < queued) {
+                        const uint32_t ci = (at[u] - Tp) >> (lg + 2);   // step (at 0) x C + counterparty
+                        atomicAdd(&cnt[((ci >> ps) << lg) + p], 1u << (16 * (ci & (uint32_t)ps)));
+                        if (IDX) a.idx[((size_t)kl * a.N + l) * C + ci % C] = (uint8_t)(ci / C + 1);
+                    }
+            }
+            queued = 0;
         }
     }
     __syncthreads();
-    // the counts of steps 1..n, P consecutive paths per (step, counterparty) row
-    for (int i = tid; i < n * C * P; i += nthr) {
-        const int pk = i % P, jc = i / P, c = jc % C, j = 1 + jc / C;
-        const uint32_t kl = tile0 + pk;
-        if (kl < M) {
-            const int ci = (pk * C + c) * np1 + j;
-            const uint32_t v = packed ? (cnt_s[ci >> 1] >> (16 * (ci & 1))) & 0xffffu : cnt_s[ci];
-            const size_t o = ((size_t)j * C + c) * M + kl;
-            if (a.cnt16) a.cnt16[o] = (uint16_t)v;
-            else a.cnt32[o] = v;
-        }
-    }
-}
 
-template <int C>
-__global__ void __launch_bounds__(256) inner_target_kernel(InnerArgs a)
-{
-    const uint32_t kl = blockIdx.x * blockDim.x + threadIdx.x;
-    if (kl >= a.M) return;
-    const size_t M = a.M;
-    const int n = a.n, np1 = n + 1, NPF = a.NPF;
-    const float invN = 1.0f / (float)a.N;
-    float S[kMaxPF];   // sum_{j > i} sum_c V_c(j) count_c(j) of each portfolio
+    // sum_c V_c(j) count_c(j) of every (portfolio, date), over the thresholds' area
+    const uint32_t kl = tile0 + (uint32_t)p;
+    const uint32_t mask = ps ? 0xffffu : 0xffffffffu;
+    if (live)
+        for (int j = 1 + (tid >> lg); j <= n; j += nthr >> lg) {
+            float cn[C];
 #pragma unroll
-    for (int pf = 0; pf < kMaxPF; ++pf) S[pf] = 0.f;
-    for (int j = n; j >= 1; --j) {
-        float cnt[C];
-#pragma unroll
-        for (int c = 0; c < C; ++c) {
-            const size_t o = ((size_t)j * C + c) * M + kl;
-            cnt[c] = a.cnt16 ? (float)__ldg(a.cnt16 + o) : (float)__ldg(a.cnt32 + o);
-        }
-        const float bi = expf(__ldg(a.disc + (size_t)(j - 1) * M + kl)) * invN;   // beta_{j-1}^{-1} / N
-#pragma unroll
-        for (int pf = 0; pf < kMaxPF; ++pf) {
-            if (pf < NPF) {
+            for (int c = 0; c < C; ++c) {
+                const int ci = (j - 1) * C + c;
+                cn[c] = (float)((cnt[((ci >> ps) << lg) + p] >> (16 * (ci & ps))) & mask);
+            }
+            const float *ex = a.expo + (size_t)j * C * M + kl;
+            for (int pf = 0; pf < NPF; ++pf) {
                 float h = 0.f;
 #pragma unroll
-                for (int c = 0; c < C; ++c)
-                    h = fmaf(__ldg(a.expo + ((size_t)(pf * np1 + j) * C + c) * M + kl), cnt[c], h);
-                S[pf] += h;
-                a.targets[((size_t)pf * n + j - 1) * M + kl] = S[pf] * bi;
+                for (int c = 0; c < C; ++c) h = fmaf(__ldg(ex + (size_t)c * M), cn[c], h);
+                T[((pf * n + j - 1) << lg) + p] = h;
+                ex += (size_t)(n + 1) * C * M;
             }
+        }
+    __syncthreads();
+    // running sums over the dates from the last, a thread per (portfolio, path); eight
+    // loads ahead of the adds
+    for (int t = tid; t < NPF << lg; t += nthr) {
+        float *h = T + (((t >> lg) * n) << lg) + (t & (PT - 1));
+        float S = 0.f;
+        int j = n - 1;
+        for (; j >= 7; j -= 8) {
+            float v[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) v[i] = h[(j - i) << lg];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                S += v[i];
+                h[(j - i) << lg] = S;
+            }
+        }
+        for (; j >= 0; --j) {
+            S += h[j << lg];
+            h[j << lg] = S;
+        }
+    }
+    __syncthreads();
+    if (live) {
+        const float invN = 1.0f / (float)a.N;
+        for (int j = tid >> lg; j < n; j += nthr >> lg) {
+            const float bi = expf(__ldg(a.disc + (size_t)j * M + kl)) * invN;   // beta_j^{-1} / N
+            for (int pf = 0; pf < NPF; ++pf)
+                a.targets[((size_t)pf * n + j) * M + kl] = T[((pf * n + j) << lg) + p] * bi;
         }
     }
 }
@@ -328,28 +408,40 @@ cva_status launch_outer(Sim &s, uint64_t seed, uint64_t k0, cudaStream_t st)
     return o->launch(s, seed, k0, st);
 }
 
-// thresholds (FP32) and counters (16-bit pairs when packed) of P paths
-static size_t inner_smem(int P, int C, int n, bool packed)
+// Shared memory of a tile: thresholds (later the portfolio sums), counters, queues.
+static size_t inner_smem(int lg, int threads, int C, int n, int NPF, bool packed)
 {
-    const size_t cells = (size_t)P * C * (n + 1);
-    return 4 * cells + 4 * (packed ? (cells + 1) / 2 : cells);
+    const size_t rows = (size_t)n * std::max(C, NPF), words = packed ? ((size_t)n * C + 1) / 2 : (size_t)n * C;
+    return 4 * (((rows + words) << lg) + (size_t)2 * C * threads);
 }
 
 template <int C>
-static cudaError_t launch_inner_t(const InnerArgs &args, size_t smem, cudaStream_t st)
+static cudaError_t launch_inner_t(InnerArgs &args, int tune, int sms, int dev, cudaStream_t st)
 {
-    static bool attr = false;
-    if (!attr) {
-        cudaError_t e = cudaFuncSetAttribute(inner_count_kernel<C>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             200 * 1024);
+    const bool packed = args.N <= 65535u, keep = args.idx != nullptr;
+    const auto kern = keep ? inner_kernel<C, true> : inner_kernel<C, false>;
+    static std::atomic<bool> attr[2][64];
+    if (!attr[keep][dev].load(std::memory_order_acquire)) {
+        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 216 * 1024);
         if (e != cudaSuccess) return e;
-        attr = true;
+        attr[keep][dev].store(true, std::memory_order_release);
     }
-    const unsigned blocks = (args.M + args.P - 1) / args.P;
-    inner_count_kernel<C><<<blocks, 32 * args.P, smem, st>>>(args);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    inner_target_kernel<C><<<(args.M + 255) / 256, 256, 0, st>>>(args);
+    // 32 paths a tile (whole 128-byte rows, no bank shared) unless two such blocks do not
+    // fit a multiprocessor or the tiles do not fill the chip twice; a tile of fewer than
+    // 8 paths only where 8 do not fit at all. A tile shape set by the caller (2, 4, 8:
+    // tiles of 8, 16, 32 paths) replaces the first rule as far as it fits.
+    auto threads_of = [&](int lg) {
+        const uint64_t want = (uint64_t)args.N << lg;
+        return want >= 512 ? 512 : want >= 256 ? 256 : 128;
+    };
+    auto smem_of = [&](int lg) { return inner_smem(lg, threads_of(lg), C, args.n, args.NPF, packed); };
+    int lg = tune == 2 ? 3 : tune == 4 ? 4 : 5;
+    while (tune == 0 && lg > 3 && (smem_of(lg) > 108 * 1024 || (args.M >> lg) < 2u * (unsigned)sms)) --lg;
+    while (lg > 0 && smem_of(lg) > 216 * 1024) --lg;
+    args.lg = lg;
+    args.packed = packed;
+    args.rows = args.n * std::max(C, args.NPF);
+    kern<<<(unsigned)((args.M + (1ull << lg) - 1) >> lg), threads_of(lg), smem_of(lg), st>>>(args);
     return cudaGetLastError();
 }
 
@@ -364,26 +456,23 @@ cva_status launch_inner(Sim &s, uint64_t seed, uint64_t k0, cudaStream_t st)
     args.branch = s.branch;
     args.n = s.n;
     args.NPF = s.NPF;
-    int P = (s.tune_inner_P >= 1 && s.tune_inner_P <= 8) ? s.tune_inner_P : 8;
-    const bool packed = s.N <= 65535u;
-    while (P > 1 && inner_smem(P, s.C, s.n, packed) > 160 * 1024) P >>= 1;
-    args.P = P;
     args.thr = s.d_thr;
     args.expo = s.d_expo;
     args.disc = s.d_disc;
     args.targets = s.d_targets;
     args.idx = s.d_idx;
-    args.cnt16 = packed ? static_cast<uint16_t *>(s.d_cnt) : nullptr;
-    args.cnt32 = packed ? nullptr : static_cast<uint32_t *>(s.d_cnt);
-    const size_t smem = inner_smem(P, s.C, s.n, packed);
-    static constexpr cudaError_t (*by_c[kMaxC])(const InnerArgs &, size_t, cudaStream_t) = {
+    static constexpr cudaError_t (*by_c[kMaxC])(InnerArgs &, int, int, int, cudaStream_t) = {
         launch_inner_t<1>,  launch_inner_t<2>,  launch_inner_t<3>,  launch_inner_t<4>,
         launch_inner_t<5>,  launch_inner_t<6>,  launch_inner_t<7>,  launch_inner_t<8>,
         launch_inner_t<9>,  launch_inner_t<10>, launch_inner_t<11>, launch_inner_t<12>,
         launch_inner_t<13>, launch_inner_t<14>, launch_inner_t<15>, launch_inner_t<16>};
     if (s.C < 1 || s.C > kMaxC) return fail(CVA_ENOTSUP, "inner kernel: 1 <= C <= 16");
-    const cudaError_t e = by_c[s.C - 1](args, smem, st);
-    if (e != cudaSuccess) return cuda_fail(e, "inner kernels launch");
+    int dev = 0, sms = 0;
+    CVA_CUDA_TRY(cudaGetDevice(&dev));
+    if (dev < 0 || dev >= 64) return fail(CVA_EINVAL, "device index out of range");
+    CVA_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    const cudaError_t e = by_c[s.C - 1](args, s.tune_inner_P, sms, dev, st);
+    if (e != cudaSuccess) return cuda_fail(e, "inner kernel launch");
     return CVA_OK;
 }
 
