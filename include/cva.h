@@ -348,7 +348,8 @@ CVA_API cva_status cva_autotune(cva_sim *sim, uint64_t seed, int basis, char *re
                                 void *stream);
 
 /* Sets the tile shapes of a simulation directly (e.g. a choice cva_autotune made
- * in an earlier process): sim_block in {64, 128}, price_block in {128, 256},
+ * in an earlier process): sim_block in {64, 128} (4 and 8
+ * warps per 32 paths), price_block in {128, 256},
  * inner_paths_per_block in {0 (automatic), 2, 4, 8 (tiles of 8, 16 and 32 paths, as
  * far as they fit shared memory)}, lsq_chunk_target in
  * [152, 2^20], and the pricing form portfolios_per_price_block: 1, 2 or 3 dividing

@@ -226,7 +226,10 @@ cva_status cva_sim_create(const cva_model_desc *model, const cva_portfolio_desc 
     k.ds = (float)ds;
     k.sqds = (float)std::sqrt(ds);
     for (int i = 0; i < F; ++i)
-        for (int j = 0; j <= i; ++j) k.L[i * (i + 1) / 2 + j] = (float)L[i * F + j];
+        for (int j = 0; j <= i; ++j) {
+            k.L[i * (i + 1) / 2 + j] = (float)L[i * F + j];
+            k.Lc[j * ((F + 1) / 2 * 2) + i] = (float)L[i * F + j];
+        }
     std::vector<HW> hw(E);
     for (int e = 0; e < E; ++e) {
         hw[e] = HW{model->hw_a[e], model->hw_sigma[e], model->curve[e]};

@@ -36,6 +36,7 @@ struct SimConsts {
     double ds_d;                           // sub-step length in FP64 (discount integral)
     float ds, sqds;
     float L[kMaxF * (kMaxF + 1) / 2];      // packed lower Cholesky factor, row-major
+    alignas(16) float Lc[kMaxF * (kMaxF + 1)];   // its columns, [F][F rounded up to even], zeros above the diagonal
     float hw_a_ds[kMaxE];                  // a_e * ds
     float hw_sig_sqds[kMaxE];              // sigma^r_e * sqrt(ds)
     float fx_drift_ds[kMaxE];              // -sigma^chi_e^2 / 2 * ds
@@ -86,8 +87,8 @@ struct Sim {
     // device image of consts + weights (constant uploads are device-to-device, so
     // they can be captured in a CUDA graph)
     unsigned char *d_const_img = nullptr;
-    // tile shapes, set by cva_autotune
-    int tune_sim_block = 128, tune_price_block = 256, tune_inner_P = 0, tune_lsq_chunks = 2432;
+    // tile shapes, set by cva_autotune (sim_block 0: by the number of paths)
+    int tune_sim_block = 0, tune_price_block = 256, tune_inner_P = 0, tune_lsq_chunks = 2432;
     int tune_price_pf = 1;         // portfolios per pricing block (1, 2 or 3, dividing n_pf; 0: all, from shared memory)
     // scratch of the portfolio-grouped regression, owned by the simulation
     double *d_lsq = nullptr;

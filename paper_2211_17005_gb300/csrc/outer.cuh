@@ -3,7 +3,7 @@
 // the constant-memory tables and of their ownership state, so instantiations
 // compile in parallel.
 //
-// sim_kernel (one thread per outer path k, Sec. 3.2): the time loop. Per
+// sim_kernel (32 outer paths per block, Sec. 3.2): the time loop. Per
 // Euler-Maruyama sub-step (Remark rem:finecoarse): Philox normals, correlation
 // by the Cholesky factor, Hull-White rates with the quanto drift, lognormal FX,
 // CIR intensities with full truncation (App. B), and the left-point integrals
@@ -20,6 +20,7 @@
 // Outputs are structure-of-arrays with the path index fastest.
 #pragma once
 #include <algorithm>
+#include <climits>
 #include <mutex>
 
 #include "cva_internal.h"
@@ -31,6 +32,33 @@ namespace {
 
 static __constant__ SimConsts c_sim;
 static __constant__ SimWeights c_w;
+
+// two FP32 values in one register pair, operated on together
+using f32x2 = unsigned long long;
+__device__ __forceinline__ f32x2 pack2(float a, float b)
+{
+    f32x2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ float2 unpack2(f32x2 v)
+{
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+    return r;
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c)
+{
+    f32x2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b)
+{
+    f32x2 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
 
 // expm1(x) by its Taylor series to degree 8 for |x| <= 1/4 (relative error below
 // 2e-10 there, so the rounding of the FMAs dominates), library expm1f elsewhere.
@@ -50,7 +78,7 @@ __device__ __forceinline__ float expm1_small(float x)
 
 struct OuterArgs {
     uint32_t M, k0, seed_lo, seed_hi;
-    int branch_date;                   // steps j > branch_date draw with counter word `branch`
+    int branch_step;                   // fine steps q >= branch_step draw with counter word `branch`
     uint32_t branch;
     const float4 *__restrict__ zc;     // [n+1][E][G] (lnA, B, dlnA, dB)
     const float2 *__restrict__ fix;    // [periods+1][E] (lnA, B)
@@ -60,58 +88,101 @@ struct OuterArgs {
     const float *w_glob;               // device copy of the date-bucketed weights: wA [kMaxW], then wK [kMaxW]
 };
 
-template <int E, int C, int CS>
-__global__ void __launch_bounds__(128) sim_kernel(OuterArgs a)
+// Block: 32 outer paths (lane = path), NW warps. The normals of a fine step depend on no
+// state, so the block takes 8 steps at a time: its warps draw and correlate a step's
+// increments W = L z of the 32 paths each into shared memory, then the recursions run over
+// the 8 steps with the factors split over the warps (economies and counterparties w, w + NW,
+// ...; every warp that holds an FX rate carries its own copy of r^0). The noise is 97% of
+// the instructions and is spread evenly; 2^15 paths give 8192 warps instead of 1024.
+//
+// The correlation multiplies by packed pairs of rows of L (fma.rn.f32x2, each half rounded
+// as a single FMA): 352 instructions a step at 27 factors against 728 with one constant
+// load and one FMA per entry.
+//
+// Bound by instruction issue (Philox, logarithm, square root and sine-cosine of 14
+// Box-Muller pairs, the correlation): 2650 instructions a (path, step) at 27 factors and
+// 85% of the issue slots. Paper shape, 2^17 paths and 100 steps: 1.28 -> 1.11 ms against a
+// thread per path over all steps (96 registers, 7 to 14 warps a multiprocessor); 2^15
+// paths and 2500 steps 9.09 -> 6.51 ms; 2^14 paths and 100 steps 0.43 -> 0.18 ms.
+template <int E, int C, int CS, int NW>
+__global__ void __launch_bounds__(32 * NW, NW == 8 ? 3 : 5) sim_kernel(OuterArgs a)
 {
     constexpr int F = 2 * E - 1 + CS;
-    constexpr int NB = (F + 3) / 4;
-    const uint32_t kl = blockIdx.x * blockDim.x + threadIdx.x;
-    if (kl >= a.M) return;
+    constexpr int NB = (F + 3) / 4, FP = (F + 1) / 2 * 2;
+    constexpr int ME = (E + NW - 1) / NW, MC = (C + NW - 1) / NW;   // factors of a warp
+    constexpr int NS = F <= 8 ? 32 : 8;                             // fine steps at a time
+    __shared__ float Ws[NS][F][32], R0[NS][32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const uint32_t kl = blockIdx.x * 32u + (uint32_t)lane;
+    const bool live = kl < a.M;
     const uint32_t k = a.k0 + kl;
     const size_t M = a.M;
     const int n = c_sim.n, S = c_sim.S;
     const float ds = c_sim.ds;
     const double ds_d = c_sim.ds_d;
 
-    float r[E], lchi[E];
-    float gam[C], lam[C], lamc[C];
-#pragma unroll
-    for (int e = 0; e < E; ++e) {
-        r[e] = c_sim.r0[e];
-        lchi[e] = c_sim.lchi0[e];
-    }
-#pragma unroll
-    for (int c = 0; c < C; ++c) {
-        gam[c] = c_sim.gamma0[c];
-        lam[c] = 0.f;
-        lamc[c] = 0.f;
-    }
+    // this warp's factors and their coefficients
+    float r0 = c_sim.r0[0], r[ME], lchi[ME], gam[MC], lam[MC], lamc[MC];
     double I0 = 0.0;
+    auto has_e = [&](int i) { return NW * (i + 1) <= E || warp + NW * i < E; };
+    auto has_c = [&](int i) { return NW * (i + 1) <= C || warp + NW * i < C; };
+    auto is_cir = [&](int i) { return NW * (i + 1) <= CS || warp + NW * i < CS; };
+#pragma unroll
+    for (int i = 0; i < ME; ++i) {
+        const int e = has_e(i) ? warp + NW * i : 0;
+        r[i] = c_sim.r0[e];
+        lchi[i] = c_sim.lchi0[e];
+    }
+#pragma unroll
+    for (int i = 0; i < MC; ++i) {
+        const int c = has_c(i) ? warp + NW * i : 0;
+        gam[i] = c_sim.gamma0[c];
+        lam[i] = lamc[i] = 0.f;
+    }
+    // rows of a date this warp writes: the rate and the log FX rate of its first economy,
+    // its first counterparty's intensity and threshold; the next ones follow NW rows apart
+    float *pr = a.features + (size_t)warp * M + kl, *px = pr + (size_t)(E - 1) * M, *pg = pr + (size_t)(2 * E - 1) * M;
+    float *pt = a.thr + (size_t)warp * M + kl, *pd = a.disc + kl;
+    auto write_date = [&]() {
+        if (live) {
+#pragma unroll
+            for (int i = 0; i < ME; ++i)
+                if (has_e(i)) {
+                    pr[(size_t)(NW * i) * M] = r[i];
+                    if (i > 0 || warp > 0) px[(size_t)(NW * i) * M] = lchi[i];
+                }
+#pragma unroll
+            for (int i = 0; i < MC; ++i)
+                if (has_c(i)) {
+                    if (is_cir(i)) pg[(size_t)(NW * i) * M] = gam[i];
+                    pt[(size_t)(NW * i) * M] = -expm1f(-lam[i]);   // 0 at date 0
+                }
+        }
+        pr += (size_t)F * M;
+        px += (size_t)F * M;
+        pg += (size_t)F * M;
+        pt += (size_t)C * M;
+    };
+    write_date();
+    if (warp == NW - 1 && live) *pd = 0.f;
 
-    // date 0
-#pragma unroll
-    for (int e = 0; e < E; ++e) a.features[(size_t)e * M + kl] = r[e];
-#pragma unroll
-    for (int e = 1; e < E; ++e) a.features[(size_t)(E - 1 + e) * M + kl] = lchi[e];
-#pragma unroll
-    for (int c = 0; c < CS; ++c) a.features[(size_t)(2 * E - 1 + c) * M + kl] = gam[c];
-    a.disc[kl] = 0.f;
-#pragma unroll
-    for (int c = 0; c < C; ++c) a.thr[(size_t)c * M + kl] = 0.f;
-
-    for (int j = 1; j <= n; ++j) {
-        for (int s = 0; s < S; ++s) {
-            const uint32_t q = (uint32_t)((j - 1) * S + s);
+    const int steps = n * S;
+    const float *drow = a.drift;
+    int s = 0, sd = 0;   // sub-step of the next fine step (of the factors, of int r^0)
+    for (int q0 = 0; q0 < steps; q0 += NS) {
+#pragma unroll 1
+        for (int v = warp; v < NS && q0 + v < steps; v += NW) {
+            const int q = q0 + v;
             // correlated increments W = L z, accumulated one Philox block (four
             // normals) at a time
-            float W[F];
+            f32x2 W[FP / 2];
 #pragma unroll
-            for (int i = 0; i < F; ++i) W[i] = 0.f;
+            for (int i = 0; i < FP / 2; ++i) W[i] = pack2(0.f, 0.f);
 #pragma unroll
             for (int b = 0; b < NB; ++b) {
-                const uint4 x = philox4x32_10(
-                    make_uint4(k, q, j > a.branch_date ? a.branch : 0u, (kStreamOuter << 24) | (uint32_t)b), a.seed_lo,
-                    a.seed_hi);
+                const uint4 x = philox4x32_10(make_uint4(k, (uint32_t)q, q >= a.branch_step ? a.branch : 0u,
+                                                         (kStreamOuter << 24) | (uint32_t)b),
+                                              a.seed_lo, a.seed_hi);
                 float z[4];
                 box_muller(x.x, x.y, z[0], z[1]);
                 box_muller(x.z, x.w, z[2], z[3]);
@@ -119,47 +190,84 @@ __global__ void __launch_bounds__(128) sim_kernel(OuterArgs a)
                 for (int t = 0; t < 4; ++t) {
                     const int col = 4 * b + t;
                     if (col < F) {
+                        const f32x2 zz = pack2(z[t], z[t]);
 #pragma unroll
-                        for (int i = col; i < F; ++i) W[i] = fmaf(c_sim.L[i * (i + 1) / 2 + col], z[t], W[i]);
+                        for (int i = col / 2; i < FP / 2; ++i) {
+                            const float2 l = *reinterpret_cast<const float2 *>(&c_sim.Lc[col * FP + 2 * i]);
+                            W[i] = fma2(pack2(l.x, l.y), zz, W[i]);
+                        }
                     }
                 }
             }
-            const float r0 = r[0];
-            // left-point integrals: int r^0 in FP64, Lambda^c compensated FP32 and
-            // kept non-decreasing
-            I0 = fma((double)r0, ds_d, I0);
 #pragma unroll
-            for (int c = 0; c < C; ++c) {
-                const float gp = fmaxf(gam[c], 0.f);
-                const float y = fmaf(gp, ds, -lamc[c]);
-                const float t = lam[c] + y;
-                lamc[c] = (t - lam[c]) - y;
-                lam[c] = fmaxf(t, lam[c]);
-                if (c < CS) {
-                    constexpr int w0 = (CS > 0) ? 2 * E - 1 : 0;
-                    gam[c] += c_sim.cir_ktds[c] - c_sim.cir_kds[c] * gp
-                              + c_sim.cir_nu_sqds[c] * sqrtf(gp) * W[w0 + (c < CS ? c : 0)];
+            for (int i = 0; i < F; ++i) {
+                const float2 w = unpack2(W[i / 2]);
+                Ws[v][i][lane] = i & 1 ? w.y : w.x;
+            }
+        }
+        __syncthreads();
+        const int chunk = min(NS, steps - q0);
+        const float *W = &Ws[0][0][lane];
+        // the coefficients, in registers over the chunk only
+        float ha[ME], hs[ME], fd[ME], fs[ME], ckt[MC], ck[MC], cn[MC], ha0 = c_sim.hw_a_ds[0], hs0 = c_sim.hw_sig_sqds[0];
+#pragma unroll
+        for (int i = 0; i < ME; ++i) {
+            const int e = has_e(i) ? warp + NW * i : 0;
+            ha[i] = c_sim.hw_a_ds[e];
+            hs[i] = c_sim.hw_sig_sqds[e];
+            fd[i] = c_sim.fx_drift_ds[e];
+            fs[i] = c_sim.fx_sig_sqds[e];
+            asm volatile("" : "+f"(ha[i]), "+f"(hs[i]), "+f"(fd[i]), "+f"(fs[i]));
+        }
+#pragma unroll
+        for (int i = 0; i < MC; ++i) {
+            const int c = has_c(i) ? warp + NW * i : 0;
+            ckt[i] = c_sim.cir_ktds[c];
+            ck[i] = c_sim.cir_kds[c];
+            cn[i] = c_sim.cir_nu_sqds[c];
+            asm volatile("" : "+f"(ckt[i]), "+f"(ck[i]), "+f"(cn[i]));
+        }
+        asm volatile("" : "+f"(ha0), "+f"(hs0));
+#pragma unroll 1
+        for (int u = 0; u < chunk; ++u, W += F * 32, drow += E) {
+            if (warp == 0) R0[u][lane] = r0;
+            // Lambda^c: left-point integral, compensated FP32, kept non-decreasing
+#pragma unroll
+            for (int i = 0; i < MC; ++i)
+                if (has_c(i)) {
+                    const float gp = fmaxf(gam[i], 0.f);
+                    const float y = fmaf(gp, ds, -lamc[i]);
+                    const float t = lam[i] + y;
+                    lamc[i] = (t - lam[i]) - y;
+                    lam[i] = fmaxf(t, lam[i]);
+                    if (is_cir(i))
+                        gam[i] += ckt[i] - ck[i] * gp + cn[i] * sqrtf(gp) * W[(2 * E - 1 + warp + NW * i) * 32];
+                }
+#pragma unroll
+            for (int i = 0; i < ME; ++i)
+                if (has_e(i)) {
+                    const int e = warp + NW * i;
+                    if (i > 0 || warp > 0) lchi[i] += fmaf(r0 - r[i], ds, fd[i]) + fs[i] * W[(E - 1 + e) * 32];
+                    r[i] += (__ldg(drow + e) - ha[i] * r[i]) + hs[i] * W[e * 32];
+                }
+            r0 += (__ldg(drow) - ha0 * r0) + hs0 * W[0];
+            if (++s == S) {   // pricing date
+                s = 0;
+                write_date();
+            }
+        }
+        __syncthreads();   // the increments are read before the next steps overwrite them
+        // int r^0 in FP64, left points; one warp and one loop for it (the FP64 pipe is
+        // narrow, and instructions predicated off in the other warps would still occupy it)
+        if (warp == NW - 1)
+            for (int u = 0; u < chunk; ++u) {
+                I0 = fma((double)R0[u][lane], ds_d, I0);
+                if (++sd == S) {
+                    sd = 0;
+                    pd += M;
+                    if (live) *pd = (float)I0;
                 }
             }
-            const float *drow = a.drift + (size_t)q * E;
-#pragma unroll
-            for (int e = 1; e < E; ++e)
-                lchi[e] += fmaf(r0 - r[e], ds, c_sim.fx_drift_ds[e]) + c_sim.fx_sig_sqds[e] * W[E - 1 + e];
-#pragma unroll
-            for (int e = 0; e < E; ++e)
-                r[e] += (__ldg(drow + e) - c_sim.hw_a_ds[e] * r[e]) + c_sim.hw_sig_sqds[e] * W[e];
-        }
-
-        float *fe = a.features + (size_t)j * F * M + kl;
-#pragma unroll
-        for (int e = 0; e < E; ++e) fe[(size_t)e * M] = r[e];
-#pragma unroll
-        for (int e = 1; e < E; ++e) fe[(size_t)(E - 1 + e) * M] = lchi[e];
-#pragma unroll
-        for (int c = 0; c < CS; ++c) fe[(size_t)(2 * E - 1 + c) * M] = gam[c];
-        a.disc[(size_t)j * M + kl] = (float)I0;
-#pragma unroll
-        for (int c = 0; c < C; ++c) a.thr[((size_t)j * C + c) * M + kl] = -expm1f(-lam[c]);
     }
 }
 
@@ -438,7 +546,7 @@ cva_status outer_launch(Sim &s, uint64_t seed, uint64_t k0, cudaStream_t st)
     args.M = (uint32_t)s.M;
     args.k0 = (uint32_t)k0;
     args.seed_lo = (uint32_t)seed;
-    args.branch_date = s.branch_date;
+    args.branch_step = s.branch_date <= s.n ? s.branch_date * s.S : INT_MAX;
     args.branch = s.branch;
     args.seed_hi = (uint32_t)(seed >> 32);
     args.zc = s.d_zc;
@@ -467,9 +575,16 @@ cva_status outer_launch(Sim &s, uint64_t seed, uint64_t k0, cudaStream_t st)
             t_owner[dev] = &s;
         }
     }
-    const unsigned sb = (unsigned)(s.tune_sim_block > 0 && s.tune_sim_block <= 128 ? s.tune_sim_block : 128);
     const unsigned pb = (unsigned)(s.tune_price_block > 0 && s.tune_price_block <= 256 ? s.tune_price_block : 256);
-    sim_kernel<E, C, CS><<<(args.M + sb - 1) / sb, sb, 0, st>>>(args);
+    // 4 warps per 32 paths (fewest instructions: more factors a warp) unless such blocks
+    // leave the chip short of warps: at the paper shape 8 warps take 91 us against 115 us
+    // for 2^10 paths, 215 against 184 for 2^14 and 1265 against 1111 for 2^17
+    int sms = 0;
+    CVA_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    const unsigned sgrid = (args.M + 31u) / 32u;
+    const bool wide = s.tune_sim_block ? s.tune_sim_block == 128 : sgrid < 2u * (unsigned)sms;
+    if (wide) sim_kernel<E, C, CS, 8><<<sgrid, 256, 0, st>>>(args);
+    else sim_kernel<E, C, CS, 4><<<sgrid, 128, 0, st>>>(args);
     CVA_CUDA_TRY(cudaGetLastError());
     if (s.ev[1]) CVA_CUDA_TRY(cudaEventRecord(s.ev[1], st));
     if (s.tune_price_pf == 4) {   // every portfolio per 128-path tile on the tensor cores
@@ -481,8 +596,6 @@ cva_status outer_launch(Sim &s, uint64_t seed, uint64_t k0, cudaStream_t st)
                                               cudaFuncAttributeMaxDynamicSharedMemorySize, PT::bytes));
             attr[dev] = true;
         }
-        int sms = 0;
-        CVA_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
         const uint32_t tiles = (args.M + 127u) / 128u;
         const uint64_t items = (uint64_t)tiles * (uint64_t)(s.n + 1);
         const unsigned grid =

@@ -54,7 +54,7 @@ __global__ void __launch_bounds__(128) sim_generic_kernel(OuterArgs a)
             for (int i = 0; i < F; ++i) W[i] = 0.f;
             for (int b = 0; b < NB; ++b) {
                 const uint4 x = philox4x32_10(
-                    make_uint4(k, q, j > a.branch_date ? a.branch : 0u, (kStreamOuter << 24) | (uint32_t)b), a.seed_lo,
+                    make_uint4(k, q, (int)q >= a.branch_step ? a.branch : 0u, (kStreamOuter << 24) | (uint32_t)b), a.seed_lo,
                     a.seed_hi);
                 float z[4];
                 box_muller(x.x, x.y, z[0], z[1]);
@@ -547,7 +547,7 @@ cva_status outer_generic_launch(Sim &s, uint64_t seed, uint64_t k0, cudaStream_t
     args.k0 = (uint32_t)k0;
     args.seed_lo = (uint32_t)seed;
     args.seed_hi = (uint32_t)(seed >> 32);
-    args.branch_date = s.branch_date;
+    args.branch_step = s.branch_date <= s.n ? s.branch_date * s.S : INT_MAX;
     args.branch = s.branch;
     args.zc = s.d_zc;
     args.fix = s.d_fix;
