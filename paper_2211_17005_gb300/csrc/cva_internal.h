@@ -89,7 +89,7 @@ struct Sim {
     unsigned char *d_const_img = nullptr;
     // tile shapes, set by cva_autotune (sim_block 0: by the number of paths)
     int tune_sim_block = 0, tune_price_block = 256, tune_inner_P = 0, tune_lsq_chunks = 2432;
-    int tune_price_pf = 1;         // portfolios per pricing block (1, 2 or 3, dividing n_pf; 0: all, from shared memory)
+    int tune_price_pf = 0;         // portfolios per pricing block (1, 2 or 3, dividing n_pf; 0: the largest of them; 4: tensor cores)
     // scratch of the portfolio-grouped regression, owned by the simulation
     double *d_lsq = nullptr;
     size_t lsq_cap = 0;

@@ -10,7 +10,7 @@
 // int r^0 (FP64) and Lambda^c (compensated FP32). At each pricing date it
 // stores the state Y_j, int r^0 and the threshold 1 - exp(-Lambda_c(t_j)).
 //
-// price_kernel (one thread per outer path, pricing date and portfolio): the
+// price_kernel (two outer paths per thread, a period's pricing dates per block): the
 // portfolio MtM per counterparty from the App. B swap formula, regrouped exactly by
 // (counterparty, currency, reset date), and the exposure (1-R_c) beta_j MtM^+.
 // It reads the state of date j and the short rates of the last reset date
@@ -22,6 +22,7 @@
 #include <algorithm>
 #include <climits>
 #include <mutex>
+#include <type_traits>
 
 #include "cva_internal.h"
 #include "rng.cuh"
@@ -271,237 +272,169 @@ __global__ void __launch_bounds__(32 * NW, NW == 8 ? 3 : 5) sim_kernel(OuterArgs
     }
 }
 
-// NPB portfolios per block (blockIdx.z picks the group): the bond prices of a
-// (path, date) serve the group's portfolios, and the group's date-bucketed weights
-// (NPB C E G pairs) must stay within the constant cache; the autotuner chooses NPB.
-template <int E, int C, int CS, int G, int NPB>
-__global__ void __launch_bounds__(256) price_kernel(OuterArgs a)
-{
-    constexpr int F = 2 * E - 1 + CS;
-    const uint32_t kl = blockIdx.x * blockDim.x + threadIdx.x;
-    const int j = blockIdx.y, pf0 = blockIdx.z * NPB;
-    if (kl >= a.M) return;
-    const size_t M = a.M;
-    const int n = c_sim.n, ppp = c_sim.ppp;
-    if (j == 0) {   // no default at t_0: exposures of date 0 are never used
-#pragma unroll
-        for (int pb = 0; pb < NPB; ++pb)
-#pragma unroll
-            for (int c = 0; c < C; ++c) {
-                a.expo[((size_t)((pf0 + pb) * (n + 1)) * C + c) * M + kl] = 0.f;
-                if (a.mtm) a.mtm[((size_t)((pf0 + pb) * (n + 1)) * C + c) * M + kl] = 0.f;
-            }
-        return;
-    }
-    const int p = __ldg(a.date_p + j);          // t_j in (p delta, (p+1) delta]
-    const float *fe = a.features + (size_t)j * F * M + kl;
-    const float *ffix = a.features + (size_t)(p * ppp) * F * M + kl;   // state at the last reset
-    const float2 *fx = a.fix + (size_t)p * E;
-    const float beta = expf(-__ldg(a.disc + (size_t)j * M + kl));
+// Pricing on the FMA pipe: two paths per thread in packed FP32 pairs, the dates of one
+// period (p delta, (p+1) delta] per block, NPB portfolios per block (blockIdx.z picks the
+// group).
+//
+// A period's dates share the number LV = G - p of live reset dates, so the block runs the
+// instantiation for it: bond prices and weight products of dead reset dates (45% of them
+// on average) are not computed, and the loops over reset dates are unrolled without a
+// test. All packed operations round each half as the scalar one (fma.rn.f32x2), and the
+// terms left out are products with 0, so every split, period and portfolio grouping gives
+// the same bits. The economies are a real loop: the code of one instantiation stays
+// within the instruction cache (fully unrolled over economies and reset dates, a third of
+// the warps waited for instructions).
+//
+// The group's weights wait in shared memory, negated and doubled (w, w) as the packed
+// multiply wants them, two reset dates in a 16-byte broadcast load. The MtM enters as
+//   acc = sum_h (-wA)(-D_h) + sum_g (-wK) Z_g,
+// with -D_h = Z_{h-1} expm1(x_h), which is what the chain of bond prices produces.
+struct PriceShape {
+    int dates_per_block, splits;   // a period's dates in `splits` blocks of dates_per_block
+};
 
-    float mt[NPB][C];
-#pragma unroll
-    for (int pb = 0; pb < NPB; ++pb)
-#pragma unroll
-        for (int c = 0; c < C; ++c) mt[pb][c] = 0.f;
-#pragma unroll
-    for (int e = 0; e < E; ++e) {
-        const float re = __ldg(fe + (size_t)e * M);
-        // running floating coupon fixed at t_- = p delta: 1/ZC_{t_-}(t_+) - 1
-        const float2 f2 = __ldg(fx + e);
-        const float fixm1 = expm1f(fmaf(f2.y, __ldg(ffix + (size_t)e * M), -f2.x));
-        const float4 *tab = a.zc + ((size_t)j * E + e) * G;
-        // Z[g] = ZC_t((g+1) delta) for live reset dates (g >= p), chained from the
-        // first one: Z[g] = Z[g-1] (1 + expm1(x_g)), x_g = ln ZC_t((g+1) delta) -
-        // ln ZC_t(g delta). D[h] = ZC_t(h delta) - ZC_t((h+1) delta) = -Z[h-1] expm1(x_h)
-        // keeps full relative accuracy of each bond-price difference; D[p] carries the
-        // running floating coupon ZC_t(t_+) (1/ZC_{t_-}(t_+) - 1).
-        const float4 tp = __ldg(tab + (p < G ? p : G - 1));   // p >= G: every swap has matured
-        const float z_first = expf(fmaf(-tp.y, re, tp.x));
-        float Z[G], D[G];
-#pragma unroll
-        for (int g = 0; g < G; ++g) {
-            if (g < p) {
-                Z[g] = 0.f;
-                D[g] = 0.f;
-            } else if (g == p) {
-                Z[g] = z_first;
-                D[g] = z_first * fixm1;
-            } else {
-                const float4 t4 = __ldg(tab + g);
-                const float zp = Z[g > 0 ? g - 1 : 0];
-                const float em = expm1_small(fmaf(-t4.w, re, t4.z));
-                D[g] = -zp * em;
-                Z[g] = fmaf(zp, em, zp);
-            }
-        }
-        const float chi = (e == 0) ? 1.f : expf(__ldg(fe + (size_t)(E - 1 + (e > 0 ? e : 1)) * M));
-#pragma unroll
-        for (int pb = 0; pb < NPB; ++pb)
-#pragma unroll
-            for (int c = 0; c < C; ++c) {
-                const int base = (((pf0 + pb) * C + c) * E + e) * G;
-                float acc = 0.f;
-#pragma unroll
-                for (int h = 0; h < G; ++h) acc = fmaf(c_w.wA[base + h], D[h], acc);
-#pragma unroll
-                for (int g = 0; g < G; ++g) acc = fmaf(-c_w.wK[base + g], Z[g], acc);
-                mt[pb][c] = fmaf(chi, acc, mt[pb][c]);
-            }
+// fn(LV) for the run-time LV in 1..G (0: nothing is live)
+template <int G, int LV = G, class Fn>
+__device__ __forceinline__ void with_live(int lv, Fn &&fn)
+{
+    if constexpr (LV >= 0) {
+        if (lv == LV) fn(std::integral_constant<int, LV>{});
+        else with_live<G, LV - 1>(lv, fn);
     }
-#pragma unroll
-    for (int pb = 0; pb < NPB; ++pb)
-#pragma unroll
-        for (int c = 0; c < C; ++c) {
-            const size_t o = ((size_t)((pf0 + pb) * (n + 1) + j) * C + c) * M + kl;
-            a.expo[o] = c_sim.lgd[c] * beta * fmaxf(mt[pb][c], 0.f);
-            if (a.mtm) a.mtm[o] = mt[pb][c];
-        }
 }
 
-// Every portfolio of the simulation priced by one thread, for PT outer paths of a
-// pricing date at a time, with the date-bucketed weights staged once per block in
-// shared memory: each (path, date) computes its bond prices once for all
-// portfolios, and each weight, read with one broadcast load, feeds the thread's PT
-// paths. The state of the next economy is requested while the current one is
-// priced. The FMA order per path is price_kernel's, so the outputs are the same bits.
-// Block: 256 / PT threads = paths [256 b, 256 b + 256) (thread t takes t + u 256/PT,
-// u < PT), dates [dpb y, dpb y + dpb). Shared memory: NPF C E GP float2 (wA, wK)
-// pairs, GP = G rounded up to even so that every row of pairs is 16-byte aligned.
-template <int E, int C, int CS, int G, int NPF, int PT>
-__global__ void __launch_bounds__(256 / PT, 2) price_smem_kernel(OuterArgs a, int dates_per_block)
+// expm1_small of both halves: the series for both, the library function for a half
+// outside its range
+__device__ __forceinline__ f32x2 expm1_small2(f32x2 x)
 {
-    constexpr int F = 2 * E - 1 + CS, GP = (G + 1) / 2 * 2, NPAIR = NPF * C * E * GP, NT = 256 / PT;
-    extern __shared__ float4 price_smem[];
-    float2 *wsm = reinterpret_cast<float2 *>(price_smem);
-    for (int i = threadIdx.x; i < NPAIR; i += blockDim.x) {
-        const int h = i % GP, row = i / GP;   // row = (pf C + c) E + e
-        wsm[i] = h < G ? make_float2(__ldg(a.w_glob + row * G + h), __ldg(a.w_glob + kMaxW + row * G + h))
-                       : make_float2(0.f, 0.f);
+    f32x2 p = pack2(1.f / 40320.f, 1.f / 40320.f);
+    p = fma2(p, x, pack2(1.f / 5040.f, 1.f / 5040.f));
+    p = fma2(p, x, pack2(1.f / 720.f, 1.f / 720.f));
+    p = fma2(p, x, pack2(1.f / 120.f, 1.f / 120.f));
+    p = fma2(p, x, pack2(1.f / 24.f, 1.f / 24.f));
+    p = fma2(p, x, pack2(1.f / 6.f, 1.f / 6.f));
+    p = fma2(p, x, pack2(0.5f, 0.5f));
+    p = fma2(p, x, pack2(1.f, 1.f));
+    f32x2 r = mul2(p, x);
+    const float2 xs = unpack2(x);
+    if (fmaxf(fabsf(xs.x), fabsf(xs.y)) > 0.25f) {
+        float2 v = unpack2(r);
+        if (fabsf(xs.x) > 0.25f) v.x = expm1f(xs.x);
+        if (fabsf(xs.y) > 0.25f) v.y = expm1f(xs.y);
+        r = pack2(v.x, v.y);
     }
-    __syncthreads();
+    return r;
+}
+
+template <int E, int C, int CS, int G, int NPB>
+__global__ void __launch_bounds__(256, NPB == 1 ? 3 : 2) price_kernel(OuterArgs a, PriceShape ps)
+{
+    constexpr int F = 2 * E - 1 + CS, R = NPB * C;   // rows of weights per economy
+    extern __shared__ __align__(16) unsigned char price_smem[];
+    f32x2 *w_s = reinterpret_cast<f32x2 *>(price_smem);      // [E][R][2 LV] (-wA, then -wK), doubled
+    const int tid = threadIdx.x, nthr = blockDim.x, pf0 = (int)blockIdx.z * NPB;
     const size_t M = a.M;
     const int n = c_sim.n, ppp = c_sim.ppp;
-    uint32_t kk[PT];
-    bool has[PT];
-#pragma unroll
-    for (int t = 0; t < PT; ++t) {
-        const uint32_t k = blockIdx.x * 256u + (uint32_t)(t * NT) + threadIdx.x;
-        has[t] = k < a.M;
-        kk[t] = has[t] ? k : (blockIdx.x * 256u + threadIdx.x < a.M ? blockIdx.x * 256u + threadIdx.x : 0u);
-    }
-    if (!has[0]) return;
-    const int j0 = (int)blockIdx.y * dates_per_block;
-    for (int j = j0; j < j0 + dates_per_block && j <= n; ++j) {
-        if (j == 0) {   // no default at t_0: exposures of date 0 are never used
-#pragma unroll
-            for (int pf = 0; pf < NPF; ++pf)
-#pragma unroll
-                for (int c = 0; c < C; ++c)
-#pragma unroll
-                    for (int t = 0; t < PT; ++t) {
-                        if (!has[t]) continue;
-                        const size_t o = ((size_t)(pf * (n + 1)) * C + c) * M + kk[t];
-                        a.expo[o] = 0.f;
-                        if (a.mtm) a.mtm[o] = 0.f;
-                    }
-            continue;
+    const int p = (int)blockIdx.y / ps.splits, part = (int)blockIdx.y % ps.splits;
+    const int j0 = p * ppp + 1 + part * ps.dates_per_block;
+    const int j1 = min(min(j0 + ps.dates_per_block, (p + 1) * ppp + 1), n + 1);   // dates [j0, j1)
+    const uint32_t k0 = blockIdx.x * 2u * (uint32_t)nthr + (uint32_t)tid, k1 = k0 + (uint32_t)nthr;
+    const bool live0 = k0 < a.M, live1 = k1 < a.M;
+    const uint32_t r0 = live0 ? k0 : 0u, r1 = live1 ? k1 : r0;   // paths read
+    auto store = [&](int j, int row, float2 mt, float2 ex) {     // row = pb C + c
+        const size_t o = ((size_t)((pf0 + row / C) * (n + 1) + j) * C + row % C) * M;
+        if (live0) a.expo[o + k0] = ex.x;
+        if (live1) a.expo[o + k1] = ex.y;
+        if (a.mtm) {
+            if (live0) a.mtm[o + k0] = mt.x;
+            if (live1) a.mtm[o + k1] = mt.y;
         }
-        const int p = __ldg(a.date_p + j);          // t_j in (p delta, (p+1) delta]
-        const float2 *fx = a.fix + (size_t)p * E;
-        const float *fe = a.features + (size_t)j * F * M;
-        const float *ffix = a.features + (size_t)(p * ppp) * F * M;   // state at the last reset
-        float beta[PT], mt[PT][NPF][C];
-        float nre[PT], nfix[PT], nchi[PT];   // the next economy's state, requested one economy ahead
+    };
+    if (blockIdx.y == 0)   // no default at t_0: exposures of date 0 are never used
+        for (int row = 0; row < R; ++row) store(0, row, make_float2(0.f, 0.f), make_float2(0.f, 0.f));
+
+    with_live<G>(p < G ? G - p : 0, [&](auto lv_) {
+        constexpr int LV = decltype(lv_)::value;
+        if constexpr (LV == 0) {   // every swap has matured
+            for (int j = j0; j < j1; ++j)
+                for (int row = 0; row < R; ++row) store(j, row, make_float2(0.f, 0.f), make_float2(0.f, 0.f));
+            return;
+        } else {
+            constexpr int P0 = G - LV;   // = p
+            for (int i = tid; i < E * R * 2 * LV; i += nthr) {
+                const int q = i % (2 * LV), row = i / (2 * LV) % R, e = i / (2 * LV * R);
+                const int wrow = ((pf0 * C + row) * E + e) * G + P0;
+                const float w = q < LV ? __ldg(a.w_glob + wrow + q) : __ldg(a.w_glob + kMaxW + wrow + q - LV);
+                w_s[i] = pack2(-w, -w);
+            }
+            __syncthreads();
+            const float *ffix = a.features + (size_t)(p * ppp) * F * M;   // state at the last reset
+            const float2 *fx = a.fix + (size_t)p * E;
+            for (int j = j0; j < j1; ++j) {
+                const float *fe = a.features + (size_t)j * F * M;
+                const float4 *tab = a.zc + (size_t)j * E * G + P0;
+                f32x2 mt[R];
 #pragma unroll
-        for (int t = 0; t < PT; ++t) {
-            beta[t] = expf(-__ldg(a.disc + (size_t)j * M + kk[t]));
-            nre[t] = __ldg(fe + kk[t]);
-            nfix[t] = __ldg(ffix + kk[t]);
-            nchi[t] = 0.f;
-#pragma unroll
-            for (int pf = 0; pf < NPF; ++pf)
-#pragma unroll
-                for (int c = 0; c < C; ++c) mt[t][pf][c] = 0.f;
-        }
+                for (int i = 0; i < R; ++i) mt[i] = pack2(0.f, 0.f);
+                const float *dj = a.disc + (size_t)j * M;
+                const float beta0 = expf(-__ldg(dj + r0)), beta1 = expf(-__ldg(dj + r1));
+                float re0 = __ldg(fe + r0), re1 = __ldg(fe + r1), rf0 = __ldg(ffix + r0), rf1 = __ldg(ffix + r1);
+                float lc0 = 0.f, lc1 = 0.f;
+                const f32x2 *w = w_s;
 #pragma unroll 1
-        for (int e = 0; e < E; ++e) {
-            float re[PT], rfix[PT], lchi[PT];
+                for (int e = 0; e < E; ++e, tab += G, w += R * 2 * LV) {
+                    // bond prices Z[g] = ZC_t((p + g + 1) delta) of the live reset dates, chained
+                    // from the first: Z[g] = Z[g-1] (1 + expm1(x_g)), x_g = ln ZC_t of this date
+                    // - ln ZC_t of the one before. D[g] = ZC_t of the date before - Z[g] = -Z[g-1]
+                    // expm1(x_g) keeps full relative accuracy; D[0] carries the running floating
+                    // coupon ZC_t(t_+) (1/ZC_{t_-}(t_+) - 1). X holds -D, then Z.
+                    f32x2 X[2 * LV];
+                    const float2 f2 = __ldg(fx + e);
+                    const float4 tp = __ldg(tab);
+                    const float z0 = expf(fmaf(-tp.y, re0, tp.x)), z1 = expf(fmaf(-tp.y, re1, tp.x));
+                    X[0] = pack2(-(z0 * expm1f(fmaf(f2.y, rf0, -f2.x))), -(z1 * expm1f(fmaf(f2.y, rf1, -f2.x))));
+                    X[LV] = pack2(z0, z1);
+                    const f32x2 re = pack2(re0, re1);
+                    const f32x2 chi = e == 0 ? pack2(1.f, 1.f) : pack2(expf(lc0), expf(lc1));
+                    if (e + 1 < E) {   // the next economy's state, ahead of this one's products
+                        fe += M;
+                        ffix += M;
+                        re0 = __ldg(fe + r0);
+                        re1 = __ldg(fe + r1);
+                        rf0 = __ldg(ffix + r0);
+                        rf1 = __ldg(ffix + r1);
+                        lc0 = __ldg(fe + (size_t)(E - 1) * M + r0);
+                        lc1 = __ldg(fe + (size_t)(E - 1) * M + r1);
+                    }
 #pragma unroll
-            for (int t = 0; t < PT; ++t) {
-                re[t] = nre[t];
-                rfix[t] = nfix[t];
-                lchi[t] = nchi[t];
-                if (e + 1 < E) {
-                    nre[t] = __ldg(fe + (size_t)(e + 1) * M + kk[t]);
-                    nfix[t] = __ldg(ffix + (size_t)(e + 1) * M + kk[t]);
-                    nchi[t] = __ldg(fe + (size_t)(E + e) * M + kk[t]);   // log chi^{e+1}
-                }
-            }
-            const float2 f2 = __ldg(fx + e);
-            const float4 *tab = a.zc + ((size_t)j * E + e) * G;
-            const float4 tp = __ldg(tab + (p < G ? p : G - 1));   // p >= G: every swap has matured
-            float Z[PT][G], D[PT][G], chi[PT];
-#pragma unroll
-            for (int t = 0; t < PT; ++t) {
-                const float fixm1 = expm1f(fmaf(f2.y, rfix[t], -f2.x));
-                const float z_first = expf(fmaf(-tp.y, re[t], tp.x));
-#pragma unroll
-                for (int g = 0; g < G; ++g) {
-                    if (g < p) {
-                        Z[t][g] = 0.f;
-                        D[t][g] = 0.f;
-                    } else if (g == p) {
-                        Z[t][g] = z_first;
-                        D[t][g] = z_first * fixm1;
-                    } else {
+                    for (int g = 1; g < LV; ++g) {
                         const float4 t4 = __ldg(tab + g);
-                        const float zp = Z[t][g > 0 ? g - 1 : 0];
-                        const float em = expm1_small(fmaf(-t4.w, re[t], t4.z));
-                        D[t][g] = -zp * em;
-                        Z[t][g] = fmaf(zp, em, zp);
+                        const f32x2 em = expm1_small2(fma2(pack2(-t4.w, -t4.w), re, pack2(t4.z, t4.z)));
+                        X[g] = mul2(X[LV + g - 1], em);
+                        X[LV + g] = fma2(X[LV + g - 1], em, X[LV + g - 1]);
+                    }
+#pragma unroll
+                    for (int i = 0; i < R; ++i) {
+                        f32x2 acc = pack2(0.f, 0.f);
+#pragma unroll
+                        for (int q = 0; q < 2 * LV; q += 2) {
+                            const ulonglong2 w2 = *reinterpret_cast<const ulonglong2 *>(w + i * 2 * LV + q);
+                            acc = fma2(w2.x, X[q], acc);
+                            acc = fma2(w2.y, X[q + 1], acc);
+                        }
+                        mt[i] = fma2(chi, acc, mt[i]);
                     }
                 }
-                chi[t] = (e == 0) ? 1.f : expf(lchi[t]);
+                ffix -= (size_t)(E - 1) * M;
+#pragma unroll
+                for (int i = 0; i < R; ++i) {
+                    const float2 m = unpack2(mt[i]);
+                    const float l = c_sim.lgd[i % C];
+                    store(j, i, m, make_float2(l * beta0 * fmaxf(m.x, 0.f), l * beta1 * fmaxf(m.y, 0.f)));
+                }
             }
-#pragma unroll
-            for (int pf = 0; pf < NPF; ++pf)
-#pragma unroll
-                for (int c = 0; c < C; ++c) {
-                    const float4 *wr = reinterpret_cast<const float4 *>(wsm + ((pf * C + c) * E + e) * GP);
-                    float wa[GP], wk[GP];
-#pragma unroll
-                    for (int q = 0; q < GP / 2; ++q) {
-                        const float4 w4 = wr[q];
-                        wa[2 * q] = w4.x;
-                        wk[2 * q] = w4.y;
-                        wa[2 * q + 1] = w4.z;
-                        wk[2 * q + 1] = w4.w;
-                    }
-#pragma unroll
-                    for (int t = 0; t < PT; ++t) {
-                        float acc = 0.f;
-#pragma unroll
-                        for (int h = 0; h < G; ++h) acc = fmaf(wa[h], D[t][h], acc);
-#pragma unroll
-                        for (int g = 0; g < G; ++g) acc = fmaf(-wk[g], Z[t][g], acc);
-                        mt[t][pf][c] = fmaf(chi[t], acc, mt[t][pf][c]);
-                    }
-                }
         }
-#pragma unroll
-        for (int t = 0; t < PT; ++t) {
-            if (!has[t]) continue;
-#pragma unroll
-            for (int pf = 0; pf < NPF; ++pf)
-#pragma unroll
-                for (int c = 0; c < C; ++c) {
-                    const size_t o = ((size_t)(pf * (n + 1) + j) * C + c) * M + kk[t];
-                    a.expo[o] = c_sim.lgd[c] * beta[t] * fmaxf(mt[t][pf][c], 0.f);
-                    if (a.mtm) a.mtm[o] = mt[t][pf][c];
-                }
-        }
-    }
+    });
 }
 
 #include "price_tc.cuh"
@@ -605,27 +538,28 @@ cva_status outer_launch(Sim &s, uint64_t seed, uint64_t k0, cudaStream_t st)
         if (!capturing) CVA_CUDA_TRY(cudaEventRecord(t_last[dev], st));
         return CVA_OK;
     }
-    if (s.tune_price_pf == 0) {   // every portfolio per thread, weights in shared memory
-        constexpr int GP = (G + 1) / 2 * 2;
-        constexpr size_t smem = (size_t)NPF * C * E * GP * sizeof(float2);
-        static_assert(smem <= 48 * 1024, "portfolio weights exceed the default shared-memory limit");
-        const int dpb = 8;
-        const dim3 sgrid((args.M + 255u) / 256u, (unsigned)((s.n + 1 + dpb - 1) / dpb));
-        if (pb == 256) price_smem_kernel<E, C, CS, G, NPF, 1><<<sgrid, 256, smem, st>>>(args, dpb);
-        else price_smem_kernel<E, C, CS, G, NPF, 2><<<sgrid, 128, smem, st>>>(args, dpb);
-        CVA_CUDA_TRY(cudaGetLastError());
-        if (!capturing) CVA_CUDA_TRY(cudaEventRecord(t_last[dev], st));
-        return CVA_OK;
+    // portfolios per block: as set, or (0) the largest of 3, 2, 1 that divides their number
+    // (bond prices are computed once per block)
+    const int ppb = s.tune_price_pf ? (NPF % s.tune_price_pf == 0 ? s.tune_price_pf : 1)
+                                    : (NPF % 3 == 0 ? 3 : NPF % 2 == 0 ? 2 : 1);
+    const unsigned tiles = (args.M + 2 * pb - 1) / (2 * pb), periods = (unsigned)((s.n + s.ppp - 1) / s.ppp);
+    // a period's dates share one block's weights; split them while the blocks do not fill
+    // the chip four times
+    PriceShape ps = {s.ppp, 1};
+    while ((uint64_t)tiles * periods * (NPF / ppb) * ps.splits < 4u * (unsigned)sms && ps.dates_per_block > 1) {
+        ps.dates_per_block = (ps.dates_per_block + 1) / 2;
+        ps.splits = (s.ppp + ps.dates_per_block - 1) / ps.dates_per_block;
     }
-    const int ppb = ((s.tune_price_pf == 2 || s.tune_price_pf == 3) && NPF % s.tune_price_pf == 0) ? s.tune_price_pf : 1;
-    const dim3 pgrid((args.M + pb - 1) / pb, (unsigned)s.n + 1u, (unsigned)(NPF / ppb));
+    const dim3 pgrid(tiles, periods * (unsigned)ps.splits, (unsigned)(NPF / ppb));
+    const size_t psmem = (size_t)E * ppb * C * 2 * G * sizeof(f32x2);
+    static_assert(E * 3 * C * 2 * G * sizeof(f32x2) <= 48 * 1024, "portfolio weights exceed the default shared-memory limit");
     if constexpr (NPF % 3 == 0) {
-        if (ppb == 3) price_kernel<E, C, CS, G, 3><<<pgrid, pb, 0, st>>>(args);
+        if (ppb == 3) price_kernel<E, C, CS, G, 3><<<pgrid, pb, psmem, st>>>(args, ps);
     }
     if constexpr (NPF % 2 == 0) {
-        if (ppb == 2) price_kernel<E, C, CS, G, 2><<<pgrid, pb, 0, st>>>(args);
+        if (ppb == 2) price_kernel<E, C, CS, G, 2><<<pgrid, pb, psmem, st>>>(args, ps);
     }
-    if (ppb == 1) price_kernel<E, C, CS, G, 1><<<pgrid, pb, 0, st>>>(args);
+    if (ppb == 1) price_kernel<E, C, CS, G, 1><<<pgrid, pb, psmem, st>>>(args, ps);
     CVA_CUDA_TRY(cudaGetLastError());
     if (!capturing) CVA_CUDA_TRY(cudaEventRecord(t_last[dev], st));
     return CVA_OK;
