@@ -1,11 +1,10 @@
 // Grouped least-squares regression of eq. (e:forw), one group per pricing date:
 //   w = argmin_w sum_k (xi_k - w^T phi(Y_k))^2.
-// The augmented Gram matrix [phi, xi]^T [phi, xi] of the basis centred on path
-// 0's state is accumulated from FP32 products in FP32 runs of 512 rows per thread,
-// then in FP64 (per thread, per block, then across blocks in a fixed order), and
-// solved by a Jacobi-scaled Cholesky factorisation in FP64. The pass over the
-// features and targets is the only HBM traffic: every byte is read once. For the
-// linear basis the tiles are copied by cp.async into two buffers (lsq_gram_async).
+// The augmented Gram matrix [phi, xi]^T [phi, xi] of the basis centred on path 0's
+// state is accumulated by gram.cuh (FP32 products in short FP32 runs, then FP64 in a
+// fixed order; every byte of the features and targets is read once) and solved by a
+// Jacobi-scaled Cholesky factorisation in FP64. A second pass over the features makes
+// the predictions, from the last group back, whose features are still in L2.
 #include <cuda.h>
 #include <cudaTypedefs.h>
 #include <math.h>
@@ -14,12 +13,11 @@
 #include <vector>
 
 #include "cva_internal.h"
+#include "gram.cuh"
 
 namespace cva {
 
 namespace {
-
-constexpr int kGramThreads = 256;
 
 struct LsqArgs {
     const float *feat0;
@@ -30,7 +28,8 @@ struct LsqArgs {
     size_t pred_stride;
     int F, m, basis, chunks;
     uint32_t M, rows_per_chunk;
-    double *part;         // [groups][chunks][NUT*16]
+    double *part;         // [groups][chunks][stride] (gram.cuh)
+    size_t stride;
     double *coef;         // [groups][nt][m] centred basis
     double *coef_raw;     // [groups][nt][m] raw basis
     int *status;          // [groups] dropped columns
@@ -46,392 +45,48 @@ __device__ __forceinline__ float centre_of(const LsqArgs &a, const float *feat, 
     return a.centre ? __ldg(a.centre + f) : __ldg(feat + (size_t)f * a.M);
 }
 
-// value of augmented column `col` at row k (columns m..m+nt-1 are the targets);
-// c0[f] is path 0's value of factor f (the centring of the basis)
-__device__ __forceinline__ float basis_value(const LsqArgs &a, const float *feat, const float *targ,
-                                            const float *c0, int col, uint32_t k)
-{
-    if (col >= a.m) return __ldg(targ + (size_t)(col - a.m) * a.targ_tstride + k);
-    if (col == 0) return 1.f;
-    if (a.basis == CVA_BASIS_POLY2) {
-        const float d = __ldg(feat + k) - c0[0];
-        return col == 1 ? d : d * d;
-    }
-    return __ldg(feat + (size_t)(col - 1) * a.M + k) - c0[col - 1];
-}
-
-template <int MP, int TR>
-__global__ void __launch_bounds__(kGramThreads) lsq_gram(LsqArgs a)
-{
-    constexpr int NBLK = MP / 4, NUT = NBLK * (NBLK + 1) / 2, RS = MP + 4;
-    constexpr int NRG = kGramThreads / NUT;
-    extern __shared__ __align__(16) unsigned char smem[];
-    float *tile = reinterpret_cast<float *>(smem);          // [TR][RS]
-    const int g = blockIdx.y, chunk = blockIdx.x, tid = threadIdx.x;
-    const float *feat = a.feat0 + (size_t)g * a.feat_stride;
-    const float *targ = a.targ0 + (size_t)g * a.targ_stride;
-    const uint32_t r_begin = (uint32_t)chunk * a.rows_per_chunk;
-    const uint32_t r_end = min(a.M, r_begin + a.rows_per_chunk);
-    const int mA = a.m + a.nt;
-
-    // this thread's 4x4 block (bi <= bj) and row group
-    const int b = tid % NUT, rg = tid / NUT;
-    int bi = 0, bj = 0;
-    {
-        int t = b;
-        for (int i = 0; i < NBLK; ++i) {
-            if (t < NBLK - i) {
-                bi = i;
-                bj = i + t;
-                break;
-            }
-            t -= NBLK - i;
-        }
-    }
-    __shared__ float c0[40];
-    for (int f = tid; f < (a.basis == CVA_BASIS_POLY2 ? 1 : a.F); f += kGramThreads) c0[f] = centre_of(a, feat, f);
-    double dacc[16];
-    float acc[16];
-#pragma unroll
-    for (int i = 0; i < 16; ++i) {
-        dacc[i] = 0.0;
-        acc[i] = 0.f;
-    }
-    int since_flush = 0;
-
-    for (uint32_t r0 = r_begin; r0 < r_end; r0 += TR) {
-        __syncthreads();
-        for (int i = tid; i < MP * TR; i += kGramThreads) {
-            const int col = i / TR, r = i % TR;
-            const uint32_t k = r0 + r;
-            float v = 0.f;
-            if (col < mA && k < r_end) v = basis_value(a, feat, targ, c0, col, k);
-            tile[r * RS + col] = v;
-        }
-        __syncthreads();
-        if (rg < NRG) {
-            for (int r = rg; r < TR; r += NRG) {
-                const float4 x = *reinterpret_cast<const float4 *>(tile + r * RS + 4 * bi);
-                const float4 y = *reinterpret_cast<const float4 *>(tile + r * RS + 4 * bj);
-                const float xv[4] = {x.x, x.y, x.z, x.w}, yv[4] = {y.x, y.y, y.z, y.w};
-#pragma unroll
-                for (int u = 0; u < 4; ++u)
-#pragma unroll
-                    for (int v = 0; v < 4; ++v) acc[u * 4 + v] = fmaf(xv[u], yv[v], acc[u * 4 + v]);
-                if (++since_flush == 512) {
-#pragma unroll
-                    for (int i = 0; i < 16; ++i) {
-                        dacc[i] += (double)acc[i];
-                        acc[i] = 0.f;
-                    }
-                    since_flush = 0;
-                }
-            }
-        }
-    }
-#pragma unroll
-    for (int i = 0; i < 16; ++i) dacc[i] += (double)acc[i];
-
-    // reduce the row groups in a fixed order
-    __syncthreads();
-    double *red = reinterpret_cast<double *>(smem);        // [NRG][NUT*16]
-    if (rg < NRG)
-#pragma unroll
-        for (int i = 0; i < 16; ++i) red[(size_t)rg * NUT * 16 + b * 16 + i] = dacc[i];
-    __syncthreads();
-    double *out = a.part + ((size_t)g * a.chunks + chunk) * NUT * 16;
-    for (int e = tid; e < NUT * 16; e += kGramThreads) {
-        double s = 0.0;
-        for (int q = 0; q < NRG; ++q) s += red[(size_t)q * NUT * 16 + e];
-        out[e] = s;
-    }
-}
-
-__device__ __forceinline__ void cp_async4_zfill(uint32_t saddr, const void *g, bool valid)
-{
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(saddr), "l"(g), "r"(valid ? 4 : 0) : "memory");
-}
-
-// lsq_gram for the linear basis [1, Y - Y^0] with the same arithmetic (the same rows
-// per thread in the same order, the same flushes), its tiles copied by cp.async into
-// two buffers so that the copies of the next tile run during the products of this
-// one; the state columns are centred on path 0 in place once a tile has landed.
-// Work blocks of lsq_gram_async per row group: for MP <= 12 the 4 x 4 blocks (bi <= bj)
-// of the upper triangle; for MP = 32 and 40 the 4 x 8 blocks (bi, bj8) that touch it
-// (2 bj8 + 1 >= bi), each a pair of 4 x 4 output blocks: three 16-byte operand reads
-// per row for 32 FMAs instead of two for 16, so that a row costs a quarter of the
-// issue slots.
-template <int MP>
-struct GramWork {
-    static constexpr int NBLK = MP / 4, NUT = NBLK * (NBLK + 1) / 2;
-    static constexpr bool wide = MP >= 32;
-    static constexpr int count8()
-    {
-        int n = 0;
-        for (int bi = 0; bi < NBLK; ++bi) n += MP / 8 - bi / 2;
-        return n;
-    }
-    static constexpr int NW = wide ? count8() : NUT;          // work blocks
-    static constexpr int NRG = kGramThreads / NW;             // row groups
-    static constexpr int NA = wide ? 32 : 16;                 // accumulators per thread
-};
-
-// index of the 4 x 4 output block (bi <= bj) in the partial's block order
-__host__ __device__ constexpr int gram_blk(int NBLK, int bi, int bj)
-{
-    return bi * NBLK - bi * (bi - 1) / 2 + (bj - bi);
-}
-
-template <int MP, int TR>
-__global__ void __launch_bounds__(kGramThreads) lsq_gram_async(LsqArgs a)
-{
-    using GW = GramWork<MP>;
-    constexpr int NBLK = MP / 4, NUT = NBLK * (NBLK + 1) / 2, RS = MP + 4, TS = TR * RS;
-    constexpr int NRG = GW::NRG, NW = GW::NW, NA = GW::NA;
-    extern __shared__ __align__(16) unsigned char smem[];
-    float *tiles = reinterpret_cast<float *>(smem);          // [2][TR][RS]
-    const int g = blockIdx.y, chunk = blockIdx.x, tid = threadIdx.x;
-    const float *feat = a.feat0 + (size_t)g * a.feat_stride;
-    const float *targ = a.targ0 + (size_t)g * a.targ_stride;
-    const uint32_t r_begin = (uint32_t)chunk * a.rows_per_chunk;
-    const uint32_t r_end = min(a.M, r_begin + a.rows_per_chunk);
-    const int mA = a.m + a.nt, F = a.F, nload = a.F + a.nt;   // copied columns 1..F+nt: state, targets
-    const int b = tid % NW, rg = tid / NW;
-    int bi = 0, bj = 0;   // 4 x 4: block (bi, bj); 4 x 8: rows 4 bi.., columns 8 bj..
-    {
-        int t = b;
-        for (int i = 0; i < NBLK; ++i) {
-            const int w = GW::wide ? MP / 8 - i / 2 : NBLK - i;
-            if (t < w) {
-                bi = i;
-                bj = (GW::wide ? i / 2 : i) + t;
-                break;
-            }
-            t -= w;
-        }
-    }
-    __shared__ float c0[40];
-    for (int f = tid; f < F; f += kGramThreads) c0[f] = centre_of(a, feat, f);
-    for (int e = tid; e < 2 * TR; e += kGramThreads)       // padding columns stay zero
-        for (int c = mA; c < MP; ++c) tiles[e * RS + c] = 0.f;
-    __syncthreads();
-    const uint32_t sbase = (uint32_t)__cvta_generic_to_shared(tiles);
-    auto issue = [&](uint32_t r0, int buf) {
-        for (int e = tid; e < nload * TR; e += kGramThreads) {
-            const int lc = e / TR, r = e % TR;
-            const uint32_t k = r0 + r;
-            const bool ok = k < r_end;
-            const float *src = lc < F ? feat + (size_t)lc * a.M : targ + (size_t)(lc - F) * a.targ_tstride;
-            cp_async4_zfill(sbase + (uint32_t)(buf * TS + r * RS + 1 + lc) * 4u, src + (ok ? k : 0u), ok);
-        }
-        asm volatile("cp.async.commit_group;" ::: "memory");
-    };
-    double dacc[NA];
-    float acc[NA];
-#pragma unroll
-    for (int i = 0; i < NA; ++i) {
-        dacc[i] = 0.0;
-        acc[i] = 0.f;
-    }
-    int since_flush = 0;
-    if (r_begin < r_end) issue(r_begin, 0);
-    int buf = 0;
-    for (uint32_t r0 = r_begin; r0 < r_end; r0 += TR, buf ^= 1) {
-        asm volatile("cp.async.wait_all;" ::: "memory");
-        __syncthreads();                          // tile r0 is in buffer buf; buf ^ 1 is free
-        float *tile = tiles + buf * TS;
-        for (int e = tid; e < (F + 1) * TR; e += kGramThreads) {
-            const int col = e / TR, r = e % TR;
-            const bool ok = r0 + r < r_end;
-            float *v = tile + r * RS + col;
-            if (col == 0) *v = ok ? 1.f : 0.f;
-            else if (ok) *v -= c0[col - 1];
-        }
-        __syncthreads();
-        if (r0 + TR < r_end) issue(r0 + TR, buf ^ 1);
-        if (rg < NRG) {
-            for (int r = rg; r < TR; r += NRG) {
-                const float4 x = *reinterpret_cast<const float4 *>(tile + r * RS + 4 * bi);
-                const float xv[4] = {x.x, x.y, x.z, x.w};
-                float yv[NA / 4];
-                if constexpr (GW::wide) {
-                    const float4 y0 = *reinterpret_cast<const float4 *>(tile + r * RS + 8 * bj);
-                    const float4 y1 = *reinterpret_cast<const float4 *>(tile + r * RS + 8 * bj + 4);
-                    yv[0] = y0.x; yv[1] = y0.y; yv[2] = y0.z; yv[3] = y0.w;
-                    yv[4] = y1.x; yv[5] = y1.y; yv[6] = y1.z; yv[7] = y1.w;
-                } else {
-                    const float4 y = *reinterpret_cast<const float4 *>(tile + r * RS + 4 * bj);
-                    yv[0] = y.x; yv[1] = y.y; yv[2] = y.z; yv[3] = y.w;
-                }
-#pragma unroll
-                for (int u = 0; u < 4; ++u)
-#pragma unroll
-                    for (int v = 0; v < NA / 4; ++v) acc[u * (NA / 4) + v] = fmaf(xv[u], yv[v], acc[u * (NA / 4) + v]);
-                if (++since_flush == 512) {
-#pragma unroll
-                    for (int i = 0; i < NA; ++i) {
-                        dacc[i] += (double)acc[i];
-                        acc[i] = 0.f;
-                    }
-                    since_flush = 0;
-                }
-            }
-        }
-    }
-#pragma unroll
-    for (int i = 0; i < NA; ++i) dacc[i] += (double)acc[i];
-    __syncthreads();
-    double *red = reinterpret_cast<double *>(smem);        // [NRG][NUT*16]
-    if (rg < NRG) {
-        if constexpr (GW::wide) {   // the halves of the 4 x 8 block on or above the diagonal
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const int bj4 = 2 * bj + h;
-                if (bj4 < bi) continue;
-                double *dst = red + (size_t)rg * NUT * 16 + gram_blk(NBLK, bi, bj4) * 16;
-#pragma unroll
-                for (int u = 0; u < 4; ++u)
-#pragma unroll
-                    for (int v = 0; v < 4; ++v) dst[u * 4 + v] = dacc[u * 8 + 4 * h + v];
-            }
-        } else {
-#pragma unroll
-            for (int i = 0; i < 16; ++i) red[(size_t)rg * NUT * 16 + b * 16 + i] = dacc[i];
-        }
-    }
-    __syncthreads();
-    double *out = a.part + ((size_t)g * a.chunks + chunk) * NUT * 16;
-    for (int e = tid; e < NUT * 16; e += kGramThreads) {
-        double s = 0.0;
-        for (int q = 0; q < NRG; ++q) s += red[(size_t)q * NUT * 16 + e];
-        out[e] = s;
-    }
-}
-
-// Launch the Gram kernel of width MP and tile TR: the cp.async form for the linear
-// basis, the plain form (per-element basis values) for [1, r, r^2]. The dynamic shared
-// memory limit is raised outside stream capture (a call before capture sets it).
-template <int MP, int TR>
-cva_status launch_gram(const LsqArgs &a, dim3 grid, cudaStream_t st)
-{
-    constexpr int NUT = (MP / 4) * (MP / 4 + 1) / 2, NRG = GramWork<MP>::NRG;
-    if (a.basis == CVA_BASIS_LINEAR) {
-        const size_t tiles = 2 * (size_t)TR * (MP + 4) * sizeof(float), red = (size_t)NRG * NUT * 16 * sizeof(double);
-        const size_t smem = tiles > red ? tiles : red;
-        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-        CVA_CUDA_TRY(cudaStreamIsCapturing(st, &cap));
-        if (cap == cudaStreamCaptureStatusNone)
-            CVA_CUDA_TRY(cudaFuncSetAttribute(lsq_gram_async<MP, TR>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                              (int)smem));
-        lsq_gram_async<MP, TR><<<grid, kGramThreads, smem, st>>>(a);
-    } else {
-        lsq_gram<MP, TR><<<grid, kGramThreads, (size_t)TR * (MP + 4) * sizeof(float), st>>>(a);
-    }
-    CVA_CUDA_TRY(cudaGetLastError());
-    return CVA_OK;
-}
-
-template <int MP>
+// The normal equations of a group: the chunks added in order, solved for every target
+// column, the coefficients in the centred and in the raw basis.
 __global__ void __launch_bounds__(256) lsq_solve(LsqArgs a)
 {
-    constexpr int NBLK = MP / 4, NUT = NBLK * (NBLK + 1) / 2;
-    __shared__ double blocks[NUT * 16];
-    __shared__ double A[MP * MP];
-    __shared__ double sc[MP];
-    __shared__ int drop[MP];
+    constexpr int LD = 41;
+    __shared__ double A[40 * LD], w[400], sc[40];   // m + nt <= 40
+    __shared__ int drop[40];
     const int g = blockIdx.x, tid = threadIdx.x, m = a.m, mA = m + a.nt;
-    for (int e = tid; e < NUT * 16; e += blockDim.x) {
-        double s = 0.0;
-        const double *p = a.part + (size_t)g * a.chunks * NUT * 16 + e;
-        for (int c = 0; c < a.chunks; ++c) s += p[(size_t)c * NUT * 16];
-        blocks[e] = s;
-    }
-    __syncthreads();
-    // unpack the upper-triangular 4x4 blocks into the dense augmented matrix
-    for (int e = tid; e < NUT * 16; e += blockDim.x) {
-        int t = e / 16, bi = 0;
-        while (t >= NBLK - bi) {
-            t -= NBLK - bi;
-            ++bi;
+    for (int i = tid >> 4; i < m; i += 16)
+        for (int j = i + (tid & 15); j < mA; j += 16) {
+            const double *p = a.part + (size_t)g * a.chunks * a.stride + tri_index(mA, i, j);
+            double s = 0.0;
+#pragma unroll 8
+            for (int c = 0; c < a.chunks; ++c) s += p[(size_t)c * a.stride];
+            A[j * LD + i] = s;
         }
-        const int bj = bi + t, i = 4 * bi + (e % 16) / 4, j = 4 * bj + e % 4;
-        if (i < mA && j < mA) {
-            A[i * MP + j] = blocks[e];
-            A[j * MP + i] = blocks[e];
-        }
-    }
     __syncthreads();
-    // Jacobi scaling, then a right-looking Cholesky factorisation of the scaled normal
-    // matrix by the whole block (L overwrites the lower triangle); a column whose pivot
-    // vanishes is dropped: its part of L is zero and its coefficient 0
-    for (int r = tid; r < m; r += blockDim.x) {
-        const double d = A[r * MP + r];
-        drop[r] = !(d > 0.0);
-        sc[r] = drop[r] ? 0.0 : 1.0 / sqrt(d);
-    }
-    __syncthreads();
-    for (int e = tid; e < m * m; e += blockDim.x) {
-        const int r = e / m, c = e % m;
-        if (c <= r) A[r * MP + c] *= sc[r] * sc[c];
-    }
-    __syncthreads();
-    for (int j = 0; j < m; ++j) {
-        if (tid == 0) {
-            const double s = A[j * MP + j];
-            if (drop[j] || !(s > 1e-12)) {
-                drop[j] = 1;
-                A[j * MP + j] = 1.0;
-            } else {
-                A[j * MP + j] = sqrt(s);
-            }
-        }
-        __syncthreads();
-        const double inv = drop[j] ? 0.0 : 1.0 / A[j * MP + j];
-        for (int r = j + 1 + tid; r < m; r += blockDim.x) A[r * MP + j] *= inv;
-        __syncthreads();
-        const int t = m - j - 1;
-        for (int e = tid; e < t * t; e += blockDim.x) {
-            const int r = j + 1 + e / t, c = j + 1 + e % t;
-            if (c <= r) A[r * MP + c] -= A[r * MP + j] * A[c * MP + j];
-        }
-        __syncthreads();
-    }
-    if (tid == 0) {
-        int dropped = 0;
-        for (int r = 0; r < m; ++r) dropped += drop[r];
-        a.status[g] = dropped;
-    }
-    // one thread per target column: the two triangular solves and the coefficients
-    if (tid >= a.nt) return;
-    const int t = tid, rhs = m + t;
+    const int dropped = solve_normal<LD>(A, m, a.nt, w, sc, drop);
+    if (tid == 0) a.status[g] = dropped;
     const float *feat = a.feat0 + (size_t)g * a.feat_stride;
-    double y[MP], w[MP];
-    for (int i = 0; i < m; ++i) {               // L y = D^{-1/2} b
-        double s = A[i * MP + rhs] * sc[i];
-        for (int p = 0; p < i; ++p) s -= A[i * MP + p] * y[p];
-        y[i] = drop[i] ? 0.0 : s / A[i * MP + i];
-    }
-    for (int i = m - 1; i >= 0; --i) {         // L^T z = y, w = D^{-1/2} z
-        double s = y[i];
-        for (int p = i + 1; p < m; ++p) s -= A[p * MP + i] * w[p];
-        w[i] = drop[i] ? 0.0 : s / A[i * MP + i];
-    }
-    for (int i = 0; i < m; ++i) w[i] *= sc[i];
-    double *co = a.coef + ((size_t)g * a.nt + t) * m, *cr = a.coef_raw + ((size_t)g * a.nt + t) * m;
-    for (int i = 0; i < m; ++i) co[i] = w[i];
-    if (a.basis == CVA_BASIS_POLY2) {
-        const double c = (double)centre_of(a, feat, 0);
-        cr[0] = w[0] - w[1] * c + w[2] * c * c;
-        cr[1] = w[1] - 2.0 * w[2] * c;
-        cr[2] = w[2];
-    } else {
-        double w0 = w[0];
-        for (int f = 0; f < a.F; ++f) {
-            const double c = (double)centre_of(a, feat, f);
-            w0 -= w[1 + f] * c;
-            cr[1 + f] = w[1 + f];
+    for (int t = tid >> 5; t < a.nt; t += 8) {   // a warp per target column
+        const int lane = tid & 31;
+        double *co = a.coef + ((size_t)g * a.nt + t) * m, *cr = a.coef_raw + ((size_t)g * a.nt + t) * m;
+        const double *wt = w + t * m;
+        for (int i = lane; i < m; i += 32) co[i] = wt[i];
+        if (a.basis == CVA_BASIS_POLY2) {
+            if (lane == 0) {
+                const double c = (double)centre_of(a, feat, 0);
+                cr[0] = wt[0] - wt[1] * c + wt[2] * c * c;
+                cr[1] = wt[1] - 2.0 * wt[2] * c;
+                cr[2] = wt[2];
+            }
+        } else {
+            double s = 0.0;   // sum of the shifts, lanes over the factors
+            for (int f = lane; f < a.F; f += 32) {
+                cr[1 + f] = wt[1 + f];
+                s = fma(wt[1 + f], (double)centre_of(a, feat, f), s);
+            }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+            if (lane == 0) cr[0] = wt[0] - s;
         }
-        cr[0] = w0;
     }
 }
 
@@ -443,7 +98,7 @@ __global__ void __launch_bounds__(256) lsq_predict(LsqArgs a)
 {
     __shared__ float cs[40 * 40];   // [nt][m], m + nt <= 40
     __shared__ float f0[40];        // path 0's state: the centring of the basis
-    const int g = blockIdx.y, nt = a.nt, m = a.m;
+    const int g = (int)(gridDim.y - 1 - blockIdx.y), nt = a.nt, m = a.m;   // from the last group back
     const double *co = a.coef + (size_t)g * nt * m;
     const float *feat = a.feat0 + (size_t)g * a.feat_stride;
     for (int i = threadIdx.x; i < nt * m; i += blockDim.x) cs[i] = (float)co[i];
@@ -464,6 +119,7 @@ __global__ void __launch_bounds__(256) lsq_predict(LsqArgs a)
         float acc[8];
 #pragma unroll
         for (int u = 0; u < 8; ++u) acc[u] = u < tn ? cs[(t0 + u) * m] : 0.f;
+#pragma unroll 9
         for (int f = 0; f < a.F; ++f) {
             const float x = __ldg(feat + (size_t)f * a.M + k) - f0[f];
 #pragma unroll
@@ -482,7 +138,7 @@ __global__ void __launch_bounds__(256) lsq_predict4(LsqArgs a)
 {
     __shared__ float cs[40 * 40];   // [nt][m], m + nt <= 40
     __shared__ float f0[40];
-    const int g = blockIdx.y, nt = a.nt, m = a.m;
+    const int g = (int)(gridDim.y - 1 - blockIdx.y), nt = a.nt, m = a.m;   // from the last group back
     const double *co = a.coef + (size_t)g * nt * m;
     const float *feat = a.feat0 + (size_t)g * a.feat_stride;
     for (int i = threadIdx.x; i < nt * m; i += blockDim.x) cs[i] = (float)co[i];
@@ -499,7 +155,7 @@ __global__ void __launch_bounds__(256) lsq_predict4(LsqArgs a)
             const float c = u < tn ? cs[(t0 + u) * m] : 0.f;
             acc[u] = make_float4(c, c, c, c);
         }
-#pragma unroll 4
+#pragma unroll 9
         for (int f = 0; f < a.F; ++f) {
             const float4 v = __ldg(reinterpret_cast<const float4 *>(feat + (size_t)f * a.M + k));
             const float c0 = f0[f];
@@ -545,21 +201,65 @@ LsqScratch g_lsq[64];
 
 }  // namespace
 
-// Launch the grouped regression with the given scratch ([groups] x (chunks x NUT x 16 +
-// 2 x nt x m) doubles + groups ints); chunk_target sets the blocks per launch.
-static size_t lsq_scratch_doubles(int groups, int m, int nt, uint64_t chunks, int NUT)
+// Scratch of the grouped regression: [groups][chunks][stride] Gram partials, their sums
+// where the chunks are many ([groups][stride]), 2 [groups][nt][m] coefficients, groups ints.
+struct LsqPlan {
+    int m, rows;                // unknowns; rows of the Gram matrix (with the target's own for one target)
+    size_t stride;              // doubles of a partial
+    uint64_t rows_per_chunk, chunks;
+    bool reduce;                // add the chunks in a launch of their own
+    size_t doubles;
+};
+
+static LsqPlan lsq_plan(int F, int basis, int nt, uint64_t M, int groups, int target)
 {
-    return (size_t)groups * chunks * NUT * 16 + 2 * (size_t)groups * nt * m + (size_t)groups;
+    LsqPlan p;
+    p.m = basis == CVA_BASIS_POLY2 ? 3 : F + 1;
+    p.rows = p.m + (nt == 1);
+    p.stride = (size_t)tri_index(p.m + nt, p.rows - 1, p.m + nt - 1) + 1;
+    // 1024 rows a block at least, 512 where that would leave multiprocessors without work
+    gram_chunks(M, groups, target > 0 ? target : 2432, (uint64_t)groups * ((M + 1023) / 1024) < 304 ? 512 : 1024,
+                &p.rows_per_chunk, &p.chunks);
+    p.reduce = p.chunks > 48;
+    p.doubles = (size_t)groups * (p.chunks + p.reduce) * p.stride + 2 * (size_t)groups * nt * p.m + (size_t)groups;
+    return p;
 }
 
-static int lsq_width(int m, int nt) { return (m + nt <= 4) ? 4 : (m + nt <= 12) ? 12 : (m + nt <= 32) ? 32 : 40; }
-
-static uint64_t lsq_chunks(uint64_t M, int groups, int chunk_target)
+// the Gram partials of every group (columns of the basis, then the targets)
+static cva_status lsq_gram(const LsqArgs &a, int rows, int groups, cudaStream_t st)
 {
-    const uint64_t max_chunks = (M + 1023) / 1024;
-    uint64_t chunks = ((uint64_t)chunk_target + groups - 1) / groups;
-    if (chunks > max_chunks) chunks = max_chunks;
-    return chunks < 1 ? 1 : chunks;
+    GramArgs q;
+    q.feat0 = a.feat0;
+    q.feat_stride = a.feat_stride;
+    q.centre = a.centre;
+    q.F = a.F;
+    q.ext[0] = a.targ0;
+    q.ext_gstride[0] = a.targ_stride;
+    q.ext_cstride[0] = a.targ_tstride;
+    q.n_ext[0] = a.nt;
+    q.ext[1] = nullptr;
+    q.ext_gstride[1] = q.ext_cstride[1] = 0;
+    q.n_ext[1] = 0;
+    q.M = a.M;
+    q.rows_per_chunk = a.rows_per_chunk;
+    q.chunks = a.chunks;
+    q.cols = a.m + a.nt;
+    q.rows = rows;
+    q.part = a.part;
+    q.stride = a.stride;
+    if (a.basis == CVA_BASIS_LINEAR) return launch_gram(q, groups, st);
+    const dim3 grid((unsigned)a.chunks, (unsigned)groups);
+    switch (a.nt) {
+    case 1: poly_gram_kernel<1><<<grid, 256, 0, st>>>(q); break;
+    case 2: poly_gram_kernel<2><<<grid, 256, 0, st>>>(q); break;
+    case 3: poly_gram_kernel<3><<<grid, 256, 0, st>>>(q); break;
+    case 4: poly_gram_kernel<4><<<grid, 256, 0, st>>>(q); break;
+    case 5: poly_gram_kernel<5><<<grid, 256, 0, st>>>(q); break;
+    case 6: poly_gram_kernel<6><<<grid, 256, 0, st>>>(q); break;
+    default: return fail(CVA_ENOTSUP, "regress: at most 6 targets on the quadratic basis");
+    }
+    CVA_CUDA_TRY(cudaGetLastError());
+    return CVA_OK;
 }
 
 cva_status lsq_launch(const LsqJob &j, double *scratch, size_t scratch_cap, double *coef_host, cudaStream_t st)
@@ -571,10 +271,8 @@ cva_status lsq_launch(const LsqJob &j, double *scratch, size_t scratch_cap, doub
     const int m = (j.basis == CVA_BASIS_POLY2) ? 3 : j.F + 1;
     if (j.F < 1) return fail(CVA_EINVAL, "regress: need one factor");
     if (m + j.nt > 40) return fail(CVA_ENOTSUP, "regress: basis columns + targets must be <= 40");
-    const int MP = lsq_width(m, j.nt);
-    const int NUT = (MP / 4) * (MP / 4 + 1) / 2;
-    const uint64_t chunks = lsq_chunks(j.M, j.groups, j.chunk_target > 0 ? j.chunk_target : 2432);
-    if (lsq_scratch_doubles(j.groups, m, j.nt, chunks, NUT) > scratch_cap) return fail(CVA_ENOMEM, "regress: scratch too small");
+    const LsqPlan p = lsq_plan(j.F, j.basis, j.nt, j.M, j.groups, j.chunk_target);
+    if (p.doubles > scratch_cap) return fail(CVA_ENOMEM, "regress: scratch too small");
     LsqArgs a;
     a.feat0 = j.feat0;
     a.feat_stride = j.feat_stride;
@@ -588,28 +286,25 @@ cva_status lsq_launch(const LsqJob &j, double *scratch, size_t scratch_cap, doub
     a.F = j.F;
     a.m = m;
     a.basis = j.basis;
-    a.chunks = (int)chunks;
+    a.chunks = (int)p.chunks;
     a.M = (uint32_t)j.M;
-    a.rows_per_chunk = (uint32_t)((j.M + chunks - 1) / chunks);
+    a.rows_per_chunk = (uint32_t)p.rows_per_chunk;
     a.part = scratch;
-    a.coef = a.part + (size_t)j.groups * chunks * NUT * 16;
+    a.stride = p.stride;
+    a.coef = a.part + (size_t)j.groups * (p.chunks + p.reduce) * p.stride;
     a.coef_raw = a.coef + (size_t)j.groups * j.nt * m;
     a.status = reinterpret_cast<int *>(a.coef_raw + (size_t)j.groups * j.nt * m);
-    const dim3 ggrid((unsigned)chunks, (unsigned)j.groups);
-    cva_status gr;
-    switch (MP) {
-    case 4: gr = launch_gram<4, 1024>(a, ggrid, st); break;
-    case 12: gr = launch_gram<12, 512>(a, ggrid, st); break;
-    case 32: gr = launch_gram<32, 256>(a, ggrid, st); break;
-    default: gr = launch_gram<40, 256>(a, ggrid, st); break;
-    }
+    const cva_status gr = lsq_gram(a, p.rows, j.groups, st);
     if (gr != CVA_OK) return gr;
-    switch (MP) {
-    case 4: lsq_solve<4><<<j.groups, 256, 0, st>>>(a); break;
-    case 12: lsq_solve<12><<<j.groups, 256, 0, st>>>(a); break;
-    case 32: lsq_solve<32><<<j.groups, 256, 0, st>>>(a); break;
-    default: lsq_solve<40><<<j.groups, 256, 0, st>>>(a); break;
+    if (p.reduce) {
+        double *sums = a.part + (size_t)j.groups * p.chunks * p.stride;
+        gram_reduce_kernel<<<dim3((unsigned)((p.stride + 31) / 32), (unsigned)j.groups), 256, 0, st>>>(a.part, a.chunks,
+                                                                                                   a.stride, sums);
+        CVA_CUDA_TRY(cudaGetLastError());
+        a.part = sums;
+        a.chunks = 1;
     }
+    lsq_solve<<<j.groups, 256, 0, st>>>(a);
     CVA_CUDA_TRY(cudaGetLastError());
     if (j.pred0) {
         cva_status pr = lsq_predict_launch(a, j.groups, st);
@@ -629,10 +324,7 @@ cva_status lsq_launch(const LsqJob &j, double *scratch, size_t scratch_cap, doub
 
 size_t lsq_scratch_need(const LsqJob &j)
 {
-    const int m = (j.basis == CVA_BASIS_POLY2) ? 3 : j.F + 1;
-    const int MP = lsq_width(m, j.nt);
-    const int NUT = (MP / 4) * (MP / 4 + 1) / 2;
-    return lsq_scratch_doubles(j.groups, m, j.nt, lsq_chunks(j.M, j.groups, j.chunk_target > 0 ? j.chunk_target : 2432), NUT);
+    return lsq_plan(j.F, j.basis, j.nt, j.M, j.groups, j.chunk_target).doubles;
 }
 
 cva_status lsq_grouped_strided(const float *feat0, size_t feat_stride, const float *targ0,
@@ -746,10 +438,9 @@ cva_status lsq_normal_partial(const float *targ, const float *feat, int F, uint6
     if (r != CVA_OK) return r;
     if (!targ || !gram_host) return fail(CVA_EINVAL, "regress: bad arguments");
     const int m = (basis == CVA_BASIS_POLY2) ? 3 : F + 1, mA = m + 1;
-    const int MP = lsq_width(m, 1), NBLK = MP / 4, NUT = NBLK * (NBLK + 1) / 2;
-    const uint64_t chunks = lsq_chunks(M, 1, 2432);
+    const LsqPlan p = lsq_plan(F, basis, 1, M, 1, 2432);
     double *part = nullptr;
-    r = lsq_scratch_get((size_t)(chunks + 1) * NUT * 16, st, &part);
+    r = lsq_scratch_get((size_t)(p.chunks + 1) * p.stride, st, &part);
     if (r != CVA_OK) return r;
     LsqArgs a;
     a.feat0 = feat;
@@ -761,43 +452,30 @@ cva_status lsq_normal_partial(const float *targ, const float *feat, int F, uint6
     a.F = F;
     a.m = m;
     a.basis = basis;
-    a.chunks = (int)chunks;
+    a.chunks = (int)p.chunks;
     a.M = (uint32_t)M;
-    a.rows_per_chunk = (uint32_t)((M + chunks - 1) / chunks);
+    a.rows_per_chunk = (uint32_t)p.rows_per_chunk;
     a.part = part;
+    a.stride = p.stride;
     a.coef = a.coef_raw = nullptr;
     a.status = nullptr;
     a.centre = centre;
-    const dim3 ggrid((unsigned)chunks, 1u);
-    switch (MP) {
-    case 4: r = launch_gram<4, 1024>(a, ggrid, st); break;
-    case 12: r = launch_gram<12, 512>(a, ggrid, st); break;
-    default: r = launch_gram<32, 256>(a, ggrid, st); break;
-    }
-    if (r == CVA_OK) r = sum_columns_fp64(part, (int)chunks, NUT * 16, part + (size_t)chunks * NUT * 16, st);
-    std::vector<double> blocks((size_t)NUT * 16);
+    r = lsq_gram(a, p.rows, 1, st);
+    double *sums = part + (size_t)p.chunks * p.stride;
+    if (r == CVA_OK) r = sum_columns_fp64(part, a.chunks, (int)p.stride, sums, st);
+    std::vector<double> tri(p.stride);
     if (r == CVA_OK) {
-        cudaError_t e = cudaMemcpyAsync(blocks.data(), part + (size_t)chunks * NUT * 16, sizeof(double) * NUT * 16,
-                                        cudaMemcpyDeviceToHost, st);
+        cudaError_t e = cudaMemcpyAsync(tri.data(), sums, sizeof(double) * p.stride, cudaMemcpyDeviceToHost, st);
         if (e == cudaSuccess) e = cudaStreamSynchronize(st);
         if (e != cudaSuccess) r = cuda_fail(e, "regress: copy of the normal matrix");
     }
     const cva_status rr = lsq_scratch_release(st);
     if (r != CVA_OK) return r;
     if (rr != CVA_OK) return rr;
-    // the upper-triangular 4x4 blocks -> the dense symmetric (m+1) x (m+1) matrix
-    for (int e = 0; e < NUT * 16; ++e) {
-        int t = e / 16, bi = 0;
-        while (t >= NBLK - bi) {
-            t -= NBLK - bi;
-            ++bi;
-        }
-        const int bj = bi + t, i = 4 * bi + (e % 16) / 4, j = 4 * bj + e % 4;
-        if (i < mA && j < mA) {
-            gram_host[(size_t)i * mA + j] = blocks[e];
-            gram_host[(size_t)j * mA + i] = blocks[e];
-        }
-    }
+    // the packed upper triangle -> the dense symmetric (m+1) x (m+1) matrix
+    for (int i = 0; i < mA; ++i)
+        for (int j = i; j < mA; ++j)
+            gram_host[(size_t)i * mA + j] = gram_host[(size_t)j * mA + i] = tri[tri_index(mA, i, j)];
     return CVA_OK;
 }
 
@@ -932,16 +610,6 @@ StaticSetup g_static[64];
 PFN_cuCtxGetCurrent_v4000 g_ctx_current = nullptr;
 PFN_cuCtxGetId_v12000 g_ctx_id = nullptr;
 
-// dynamic shared memory of the linear-basis Gram kernel at width MP (launch_gram's size)
-template <int MP, int TR>
-cva_status static_gram_attr()
-{
-    constexpr int NUT = (MP / 4) * (MP / 4 + 1) / 2, NRG = GramWork<MP>::NRG;
-    const size_t tiles = 2 * (size_t)TR * (MP + 4) * sizeof(float), red = (size_t)NRG * NUT * 16 * sizeof(double);
-    CVA_CUDA_TRY(cudaFuncSetAttribute(lsq_gram_async<MP, TR>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)(tiles > red ? tiles : red)));
-    return CVA_OK;
-}
 }  // namespace
 
 // Set-up of the allocation-free path on the current device, once per device and
@@ -975,9 +643,11 @@ static cva_status static_scratch(double **out)
         void *p = nullptr;
         const cudaError_t e = cudaGetSymbolAddress(&p, g_static_scratch);
         if (e != cudaSuccess) return cuda_fail(e, "cudaGetSymbolAddress(g_static_scratch)");
-        cva_status r = static_gram_attr<12, 512>();
-        if (r == CVA_OK) r = static_gram_attr<32, 256>();
-        if (r != CVA_OK) return r;
+        // the shared-memory limits of the Gram kernels its shapes use (up to 32 columns)
+        const int smem = 3 * 32 * 256 * (int)sizeof(float);
+        for (auto kern : {gram_kernel<512, 320, 2, true>, gram_kernel<512, 320, 2, false>, gram_kernel<256, 320, 2, true>,
+                          gram_kernel<256, 320, 2, false>})
+            CVA_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
         su.ptr = static_cast<double *>(p);
         su.ctx_id = id;
     }
@@ -996,10 +666,11 @@ cva_status lsq_batched_static(const float *targ0, const float *feat0, int groups
     if (basis == CVA_BASIS_LINEAR && (F < 1 || m + 1 > 32))
         return fail(CVA_ENOTSUP, "regress_static: linear basis supports 1 <= F <= 30");
     if (basis == CVA_BASIS_POLY2 && F < 1) return fail(CVA_EINVAL, "regress_static: need one factor");
-    const int MP = lsq_width(m, 1);
-    const size_t NUT = (size_t)(MP / 4) * (MP / 4 + 1) / 2;
+    // room reserved per chunk: the triangle in 4 x 4 blocks of 4, 12 or 32 columns, an
+    // upper bound of what a partial takes
+    const int MP = m + 1 <= 4 ? 4 : m + 1 <= 12 ? 12 : 32;
     const size_t per_group_fixed = 2 * (size_t)m + 1;          // coefficients (two bases) + status
-    const size_t per_chunk = NUT * 16;
+    const size_t per_chunk = (size_t)(MP / 4) * (MP / 4 + 1) / 2 * 16;
     const size_t max_groups = kStaticScratchDoubles / (per_chunk + per_group_fixed);
     if ((size_t)groups > max_groups || groups > 1024)
         return fail(CVA_EINVAL, "regress_static: " + std::to_string(groups) + " groups exceed the static scratch (at most " +
@@ -1016,12 +687,10 @@ cva_status lsq_batched_static(const float *targ0, const float *feat0, int groups
     cva_status r = static_scratch(&scratch);
     if (r != CVA_OK) return r;
 
-    const uint64_t max_chunks = (M + 1023) / 1024;
-    uint64_t chunks = (2432 + groups - 1) / groups;
     const uint64_t fit = (kStaticScratchDoubles - (size_t)groups * per_group_fixed) / ((size_t)groups * per_chunk);
-    if (chunks > fit) chunks = fit;
-    if (chunks > max_chunks) chunks = max_chunks;
-    if (chunks < 1) chunks = 1;
+    uint64_t rows_per_chunk, chunks;
+    gram_chunks(M, groups, (int)std::min<uint64_t>(2432, fit * (uint64_t)groups), 1024, &rows_per_chunk, &chunks);
+    const int rows = m + 1;
 
     LsqArgs a;
     a.feat0 = feat0;
@@ -1035,25 +704,15 @@ cva_status lsq_batched_static(const float *targ0, const float *feat0, int groups
     a.basis = basis;
     a.chunks = (int)chunks;
     a.M = (uint32_t)M;
-    a.rows_per_chunk = (uint32_t)((M + chunks - 1) / chunks);
+    a.rows_per_chunk = (uint32_t)rows_per_chunk;
     a.part = scratch;
-    a.coef = a.part + (size_t)groups * chunks * per_chunk;
+    a.stride = (size_t)tri_index(rows, rows - 1, rows - 1) + 1;
+    a.coef = a.part + (size_t)groups * chunks * a.stride;
     a.coef_raw = a.coef + (size_t)groups * m;
     a.status = reinterpret_cast<int *>(a.coef_raw + (size_t)groups * m);
-
-    const dim3 ggrid((unsigned)chunks, (unsigned)groups);
-    cva_status gr = CVA_OK;
-    switch (MP) {
-    case 4: gr = launch_gram<4, 1024>(a, ggrid, st); break;
-    case 12: gr = launch_gram<12, 512>(a, ggrid, st); break;
-    default: gr = launch_gram<32, 256>(a, ggrid, st); break;
-    }
+    const cva_status gr = lsq_gram(a, rows, groups, st);
     if (gr != CVA_OK) return gr;
-    switch (MP) {
-    case 4: lsq_solve<4><<<groups, 256, 0, st>>>(a); break;
-    case 12: lsq_solve<12><<<groups, 256, 0, st>>>(a); break;
-    default: lsq_solve<32><<<groups, 256, 0, st>>>(a); break;
-    }
+    lsq_solve<<<groups, 256, 0, st>>>(a);
     CVA_CUDA_TRY(cudaGetLastError());
     if (pred0) {
         cva_status pr = lsq_predict_launch(a, groups, st);
