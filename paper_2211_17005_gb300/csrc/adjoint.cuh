@@ -1,8 +1,8 @@
-// Adjoint (reverse-mode) sensitivities of the smooth CVA_0 (one thread per outer
-// path), included by outer.cuh so that it reads the same constant-memory tables.
+// Adjoint (reverse-mode) sensitivities of the smooth CVA_0, included by outer.cuh so that
+// it reads the same constant-memory tables.
 //
-// The sampled default indicators have zero pathwise derivative, so the kernel
-// differentiates the smooth functional the oversimulated average estimates: the
+// The sampled default indicators have zero pathwise derivative, so the function
+// differentiated is the smooth functional the oversimulated average estimates: the
 // exact discrete conditional default probabilities e^{-Lambda(t_{j-1})} -
 // e^{-Lambda(t_j)} (the intensity form of eq. (eq:CVAint)):
 //   J_k = sum_c sum_{j=1..n} V_c(j) (e^{-Lambda_c(j-1)} - e^{-Lambda_c(j)}),
@@ -11,497 +11,376 @@
 // sigma^chi_e (e >= 1), CIR kappa_c, theta_c, nu_c (gamma_0 held fixed; fixed
 // rates of the swaps held at their base-curve par values).
 //
-// Forward sweep: the Euler scheme of the simulation kernel, storing the full
-// state every K pricing dates and the short rates at every reset date. Reverse
-// sweep, segment by segment from the last: restore the checkpoint, recompute the
-// segment's sub-steps (the Philox counters regenerate the normals), then walk
-// the dates backwards: the adjoint of the pricing at t_j (App. B swap formula in
-// its date-bucketed form, bond prices, FX conversion, exposure and survival
-// terms) followed by the adjoint of every Euler sub-step of (t_{j-1}, t_j].
+// Three kernels over a range of outer paths:
+//   sim_kernel<ADJ>      the states, discount integrals and survival factors e^{-Lambda} of
+//                        every date, and of every fine step the increments W and the
+//                        intensities before it;
+//   adj_price_kernel     the pricing at every date, which depends on that date's state only:
+//                        V_c and, in reverse, what the date adds to the adjoints of its
+//                        rates, log FX rates, discount integral and fixings, and to the
+//                        parameters of the bond tables;
+//   adj_reverse_kernel   the adjoint recursions over the fine steps from the last, in which
+//                        the factors are independent but for r^0.
+// Keeping the states and increments (40 KB a path at 100 dates and 27 factors) instead of
+// recomputing them from checkpoints lets the pricing, the bulk of the work, run over all
+// (path, date) pairs at once, and draws the normals once instead of three times. One
+// thread per path with checkpoints held 255 registers and local arrays and took 23.0 ms at
+// 2^17 paths; the calling code bounds the memory by taking the paths in ranges.
 #pragma once
 
 namespace cva {
 namespace {
 
-struct AdjArgs {
-    uint32_t M, k0, seed_lo, seed_hi;
-    int K, nseg;
-    int forward_only;                   // 1: the smooth CVA_0 of the forward sweep only
+struct AdjSplitArgs {
+    uint32_t M;
     const float4 *__restrict__ zc;      // [n+1][E][G] (lnA, B, dlnA, dB)
     const float2 *__restrict__ fix;     // [periods+1][E] (lnA, B)
-    const int *__restrict__ date_p;     // [n+1]
-    const float *__restrict__ drift;    // [n*S][E]
     const float4 *__restrict__ dzc;     // [n+1][E][G] d/df, d/dsigma of (lnA, dlnA)
     const float2 *__restrict__ dfix;    // [periods+1][E] d/df, d/dsigma of lnA at the fixing
     const float2 *__restrict__ ddrift;  // [n*S][E] d drift/df, d drift/dsigma^r (quanto included)
     const float *__restrict__ rho;      // [E] correlation of r^e and log chi^e (entry 0 unused)
     const float *__restrict__ sig;      // [E] sigma^r, [E] sigma^chi, [C] kappa, [C] theta, [C] nu
-    float *ckpt;                        // [nseg][2E+3C][M]
-    double *ckpt_I0;                    // [nseg][M]
-    float *fixr;                        // [periods+1][E][M]
-    double *part;                       // [blocks][npar + 1]
+    const float *w_glob;                // the weights
+    const float *features, *disc;       // [n+1][F][M], [n+1][M]
+    const float *surv;                  // [n+1][C][M] e^{-Lambda}
+    const float *inc, *gpre;            // [n*S][F][M] increments, [n*S][C][M] intensities before a fine step
+    float *V;                           // [n+1][C][M]
+    float *rbin, *lbin, *ibin;          // [n][E][M] (lbin row 0: the sum of the others), [n][M]: row j-1 = date j
+    float *fixin;                       // [periods * splits][E][M]
+    double *part_p;                     // [blocks][2E + 1]: f_e, sigma^r_e of the bond tables, J
+    double *part_r;                     // [blocks][NPAR]
 };
 
-template <int E, int C, int CS, int G, int KMAX, int SMAX>
-__global__ void __launch_bounds__(128) adjoint_kernel(AdjArgs a)
+template <int E, int C, int CS, int G, bool REV>
+__global__ void __launch_bounds__(128) adj_price_kernel(AdjSplitArgs a, PriceShape ps)
 {
-    constexpr int F = 2 * E - 1 + CS;
-    constexpr int NB = (F + 3) / 4;
-    constexpr int NV = 2 * E + 3 * C;          // checkpointed floats: r, lchi, gam, lam, lamc
-    constexpr int NPAR = 3 * E - 1 + 3 * C;
-    constexpr int PF = 0, PSR = E, PSX = 2 * E - 1, PK = 3 * E - 1, PT = PK + C, PN = PT + C;   // PSX + e for e >= 1
-    __shared__ float pb_s[NPAR * 128];
-    __shared__ double red_s[128];
+    constexpr int F = 2 * E - 1 + CS, NT = 128;
+    extern __shared__ __align__(16) unsigned char adj_smem[];
+    f32x2 *w_s = reinterpret_cast<f32x2 *>(adj_smem);            // [E][C][2 LV] (-wA, -wK), doubled
+    f32x2 *rf_s = w_s + E * C * 2 * G;                           // [E][NT] adjoints of the fixings
+    float *par_s = reinterpret_cast<float *>(rf_s + E * NT);     // [2E][NT] parameter adjoints, both paths
+    __shared__ double j_s[NT];
     const int tid = threadIdx.x;
-    const uint32_t kl = blockIdx.x * blockDim.x + tid;
-    const bool active = kl < a.M;
-    const uint32_t k = a.k0 + kl;
     const size_t M = a.M;
-    const int n = c_sim.n, S = c_sim.S, ppp = c_sim.ppp, K = a.K;
-    const float ds = c_sim.ds, sqds = c_sim.sqds;
-    const double ds_d = c_sim.ds_d;
-    float *pb = pb_s + tid;                    // this thread's parameter adjoints, stride 128
-    for (int i = 0; i < NPAR; ++i) pb[i * 128] = 0.f;
+    const int n = c_sim.n, ppp = c_sim.ppp;
+    const int p = (int)blockIdx.y / ps.splits, part = (int)blockIdx.y % ps.splits;
+    const int j0 = p * ppp + 1 + part * ps.dates_per_block;
+    const int j1 = min(min(j0 + ps.dates_per_block, (p + 1) * ppp + 1), n + 1);   // dates [j0, j1)
+    const uint32_t k0 = blockIdx.x * 2u * NT + (uint32_t)tid, k1 = k0 + NT;
+    const bool live0 = k0 < a.M, live1 = k1 < a.M;
+    const uint32_t r0 = live0 ? k0 : 0u, r1 = live1 ? k1 : r0;   // paths read
+    auto put = [&](float *row, float x, float y) {
+        if (live0) row[k0] = x;
+        if (live1) row[k1] = y;
+    };
     double J = 0.0;
-
-    if (active) {
-        // ---------------- forward sweep: checkpoints and fixings ----------------
-        float r[E], lchi[E], gam[C], lam[C], lamc[C];
+    if (REV)
         for (int e = 0; e < E; ++e) {
-            r[e] = c_sim.r0[e];
-            lchi[e] = c_sim.lchi0[e];
+            rf_s[e * NT + tid] = pack2(0.f, 0.f);
+            par_s[2 * e * NT + tid] = par_s[(2 * e + 1) * NT + tid] = 0.f;
         }
-        for (int c = 0; c < C; ++c) {
-            gam[c] = c_sim.gamma0[c];
-            lam[c] = 0.f;
-            lamc[c] = 0.f;
-        }
-        double I0 = 0.0;
-        float lam_prev[C];
-        for (int c = 0; c < C; ++c) lam_prev[c] = 0.f;
-        for (int j = 0; j <= n; ++j) {
-            if (j > 0) {
-                for (int s = 0; s < S; ++s) {
-                    const uint32_t q = (uint32_t)((j - 1) * S + s);
-                    float W[F];
-#pragma unroll
-                    for (int i = 0; i < F; ++i) W[i] = 0.f;
-#pragma unroll
-                    for (int b = 0; b < NB; ++b) {
-                        const uint4 x = philox4x32_10(make_uint4(k, q, 0u, (kStreamOuter << 24) | (uint32_t)b),
-                                                      a.seed_lo, a.seed_hi);
-                        float z[4];
-                        box_muller(x.x, x.y, z[0], z[1]);
-                        box_muller(x.z, x.w, z[2], z[3]);
-#pragma unroll
-                        for (int t = 0; t < 4; ++t) {
-                            const int col = 4 * b + t;
-                            if (col < F) {
-#pragma unroll
-                                for (int i = col; i < F; ++i) W[i] = fmaf(c_sim.L[i * (i + 1) / 2 + col], z[t], W[i]);
-                            }
-                        }
-                    }
-                    const float r0 = r[0];
-                    I0 = fma((double)r0, ds_d, I0);
-#pragma unroll
-                    for (int c = 0; c < C; ++c) {
-                        const float gp = fmaxf(gam[c], 0.f);
-                        const float y = fmaf(gp, ds, -lamc[c]);
-                        const float t = lam[c] + y;
-                        lamc[c] = (t - lam[c]) - y;
-                        lam[c] = fmaxf(t, lam[c]);
-                        if (c < CS) {
-                            constexpr int w0 = (CS > 0) ? 2 * E - 1 : 0;
-                            gam[c] += c_sim.cir_ktds[c] - c_sim.cir_kds[c] * gp
-                                      + c_sim.cir_nu_sqds[c] * sqrtf(gp) * W[w0 + (c < CS ? c : 0)];
-                        }
-                    }
-                    const float *drow = a.drift + (size_t)q * E;
-#pragma unroll
-                    for (int e = 1; e < E; ++e)
-                        lchi[e] += fmaf(r0 - r[e], ds, c_sim.fx_drift_ds[e]) + c_sim.fx_sig_sqds[e] * W[E - 1 + e];
-#pragma unroll
-                    for (int e = 0; e < E; ++e)
-                        r[e] += (__ldg(drow + e) - c_sim.hw_a_ds[e] * r[e]) + c_sim.hw_sig_sqds[e] * W[e];
-                }
-            }
-            if (j % ppp == 0)
-                for (int e = 0; e < E; ++e) a.fixr[((size_t)(j / ppp) * E + e) * M + kl] = r[e];
-            if (a.forward_only && j > 0) {
-                // smooth CVA_0 term of date j: V_c(j) (e^{-Lambda_c(j-1)} - e^{-Lambda_c(j)})
-                const int p = __ldg(a.date_p + j);
-                const float beta = expf(-(float)I0);
-                float mt[C];
-                for (int c = 0; c < C; ++c) mt[c] = 0.f;
-                for (int e = 0; e < E; ++e) {
-                    const float re = r[e];
-                    const float2 f2 = __ldg(a.fix + (size_t)p * E + e);
-                    const float fixm1 = expm1f(fmaf(f2.y, a.fixr[((size_t)p * E + e) * M + kl], -f2.x));
-                    const float4 *tab = a.zc + ((size_t)j * E + e) * G;
-                    float Z[G], D[G];
-                    const float4 tp = __ldg(tab + (p < G ? p : G - 1));
-                    const float z_first = expf(fmaf(-tp.y, re, tp.x));
-#pragma unroll
-                    for (int g = 0; g < G; ++g) {
-                        if (g < p) {
-                            Z[g] = 0.f;
-                            D[g] = 0.f;
-                        } else if (g == p) {
-                            Z[g] = z_first;
-                            D[g] = z_first * fixm1;
-                        } else {
-                            const float4 t4 = __ldg(tab + g);
-                            const float zp = Z[g > 0 ? g - 1 : 0];
-                            const float em = expm1_small(fmaf(-t4.w, re, t4.z));
-                            D[g] = -zp * em;
-                            Z[g] = fmaf(zp, em, zp);
-                        }
-                    }
-                    const float chi = (e == 0) ? 1.f : expf(lchi[e]);
-#pragma unroll
-                    for (int c = 0; c < C; ++c) {
-                        const int base = (c * E + e) * G;
-                        float acc = 0.f;
-#pragma unroll
-                        for (int h = 0; h < G; ++h) acc = fmaf(c_w.wA[base + h], D[h], acc);
-#pragma unroll
-                        for (int g = 0; g < G; ++g) acc = fmaf(-c_w.wK[base + g], Z[g], acc);
-                        mt[c] = fmaf(chi, acc, mt[c]);
-                    }
-                }
-                for (int c = 0; c < C; ++c) {
-                    const float V = c_sim.lgd[c] * beta * fmaxf(mt[c], 0.f);
-                    J += (double)V * (double)(expf(-lam_prev[c]) - expf(-lam[c]));
-                }
-            }
-            for (int c = 0; c < C; ++c) lam_prev[c] = lam[c];
-            if (j % K == 0 && j / K < a.nseg) {
-                float *cp = a.ckpt + (size_t)(j / K) * NV * M + kl;
-                int v = 0;
-                for (int e = 0; e < E; ++e) cp[(size_t)(v++) * M] = r[e];
-                for (int e = 0; e < E; ++e) cp[(size_t)(v++) * M] = lchi[e];
-                for (int c = 0; c < C; ++c) cp[(size_t)(v++) * M] = gam[c];
-                for (int c = 0; c < C; ++c) cp[(size_t)(v++) * M] = lam[c];
-                for (int c = 0; c < C; ++c) cp[(size_t)(v++) * M] = lamc[c];
-                a.ckpt_I0[(size_t)(j / K) * M + kl] = I0;
-            }
-        }
-
-        if (!a.forward_only) {
-        // ---------------- reverse sweep ----------------
-        float rb[E], lb[E], gb[C], Lb[C], rfb[E], Vnext[C];
-        for (int e = 0; e < E; ++e) rb[e] = lb[e] = rfb[e] = 0.f;
-        for (int c = 0; c < C; ++c) gb[c] = Lb[c] = Vnext[c] = 0.f;
-        float Ib = 0.f;
-        // segment storage (local memory): pre-states of every sub-step, states of every date
-        float st_g[KMAX * SMAX][C];
-        float dt_r[KMAX + 1][E], dt_l[KMAX + 1][E], dt_lam[KMAX + 1][C];
-        double dt_I0[KMAX + 1];
-        for (int seg = a.nseg - 1; seg >= 0; --seg) {
-            const int d0 = seg * K, d1 = min(d0 + K, n);
-            {
-                const float *cp = a.ckpt + (size_t)seg * NV * M + kl;
-                int v = 0;
-                for (int e = 0; e < E; ++e) r[e] = cp[(size_t)(v++) * M];
-                for (int e = 0; e < E; ++e) lchi[e] = cp[(size_t)(v++) * M];
-                for (int c = 0; c < C; ++c) gam[c] = cp[(size_t)(v++) * M];
-                for (int c = 0; c < C; ++c) lam[c] = cp[(size_t)(v++) * M];
-                for (int c = 0; c < C; ++c) lamc[c] = cp[(size_t)(v++) * M];
-                I0 = a.ckpt_I0[(size_t)seg * M + kl];
-            }
-            for (int e = 0; e < E; ++e) {
-                dt_r[0][e] = r[e];
-                dt_l[0][e] = lchi[e];
-            }
-            for (int c = 0; c < C; ++c) dt_lam[0][c] = lam[c];
-            dt_I0[0] = I0;
-            for (int j = d0 + 1; j <= d1; ++j) {
-                for (int s = 0; s < S; ++s) {
-                    const int qs = (j - d0 - 1) * S + s;
-                    for (int c = 0; c < C; ++c) st_g[qs][c] = gam[c];
-                    const uint32_t q = (uint32_t)((j - 1) * S + s);
-                    float W[F];
-#pragma unroll
-                    for (int i = 0; i < F; ++i) W[i] = 0.f;
-#pragma unroll
-                    for (int b = 0; b < NB; ++b) {
-                        const uint4 x = philox4x32_10(make_uint4(k, q, 0u, (kStreamOuter << 24) | (uint32_t)b),
-                                                      a.seed_lo, a.seed_hi);
-                        float z[4];
-                        box_muller(x.x, x.y, z[0], z[1]);
-                        box_muller(x.z, x.w, z[2], z[3]);
-#pragma unroll
-                        for (int t = 0; t < 4; ++t) {
-                            const int col = 4 * b + t;
-                            if (col < F) {
-#pragma unroll
-                                for (int i = col; i < F; ++i) W[i] = fmaf(c_sim.L[i * (i + 1) / 2 + col], z[t], W[i]);
-                            }
-                        }
-                    }
-                    const float r0 = r[0];
-                    I0 = fma((double)r0, ds_d, I0);
-#pragma unroll
-                    for (int c = 0; c < C; ++c) {
-                        const float gp = fmaxf(gam[c], 0.f);
-                        const float y = fmaf(gp, ds, -lamc[c]);
-                        const float t = lam[c] + y;
-                        lamc[c] = (t - lam[c]) - y;
-                        lam[c] = fmaxf(t, lam[c]);
-                        if (c < CS) {
-                            constexpr int w0 = (CS > 0) ? 2 * E - 1 : 0;
-                            gam[c] += c_sim.cir_ktds[c] - c_sim.cir_kds[c] * gp
-                                      + c_sim.cir_nu_sqds[c] * sqrtf(gp) * W[w0 + (c < CS ? c : 0)];
-                        }
-                    }
-                    const float *drow = a.drift + (size_t)q * E;
-#pragma unroll
-                    for (int e = 1; e < E; ++e)
-                        lchi[e] += fmaf(r0 - r[e], ds, c_sim.fx_drift_ds[e]) + c_sim.fx_sig_sqds[e] * W[E - 1 + e];
-#pragma unroll
-                    for (int e = 0; e < E; ++e)
-                        r[e] += (__ldg(drow + e) - c_sim.hw_a_ds[e] * r[e]) + c_sim.hw_sig_sqds[e] * W[e];
-                }
-                for (int e = 0; e < E; ++e) {
-                    dt_r[j - d0][e] = r[e];
-                    dt_l[j - d0][e] = lchi[e];
-                }
-                for (int c = 0; c < C; ++c) dt_lam[j - d0][c] = lam[c];
-                dt_I0[j - d0] = I0;
-            }
-
-            for (int j = d1; j > d0; --j) {
-                const int jj = j - d0;
-                // ---- pricing at t_j: forward ----
-                const int p = __ldg(a.date_p + j);
-                const float beta = expf(-(float)dt_I0[jj]);
-                float mt[C];
-                for (int c = 0; c < C; ++c) mt[c] = 0.f;
-                for (int e = 0; e < E; ++e) {
-                    const float re = dt_r[jj][e];
-                    const float2 f2 = __ldg(a.fix + (size_t)p * E + e);
-                    const float rfix = a.fixr[((size_t)p * E + e) * M + kl];
-                    const float fixm1 = expm1f(fmaf(f2.y, rfix, -f2.x));
-                    const float4 *tab = a.zc + ((size_t)j * E + e) * G;
-                    float Z[G], D[G];
-                    const float4 tp = __ldg(tab + (p < G ? p : G - 1));
-                    const float z_first = expf(fmaf(-tp.y, re, tp.x));
-#pragma unroll
-                    for (int g = 0; g < G; ++g) {
-                        if (g < p) {
-                            Z[g] = 0.f;
-                            D[g] = 0.f;
-                        } else if (g == p) {
-                            Z[g] = z_first;
-                            D[g] = z_first * fixm1;
-                        } else {
-                            const float4 t4 = __ldg(tab + g);
-                            const float zp = Z[g > 0 ? g - 1 : 0];
-                            const float em = expm1_small(fmaf(-t4.w, re, t4.z));
-                            D[g] = -zp * em;
-                            Z[g] = fmaf(zp, em, zp);
-                        }
-                    }
-                    const float chi = (e == 0) ? 1.f : expf(dt_l[jj][e]);
-#pragma unroll
-                    for (int c = 0; c < C; ++c) {
-                        const int base = (c * E + e) * G;
-                        float acc = 0.f;
-#pragma unroll
-                        for (int h = 0; h < G; ++h) acc = fmaf(c_w.wA[base + h], D[h], acc);
-#pragma unroll
-                        for (int g = 0; g < G; ++g) acc = fmaf(-c_w.wK[base + g], Z[g], acc);
-                        mt[c] = fmaf(chi, acc, mt[c]);
-                    }
-                }
-                // ---- survival terms and exposure adjoints ----
-                float mtb[C];
-                for (int c = 0; c < C; ++c) {
-                    const float V = c_sim.lgd[c] * beta * fmaxf(mt[c], 0.f);
-                    const float Sp = expf(-dt_lam[jj - 1][c]), Sc = expf(-dt_lam[jj][c]);
-                    J += (double)V * (double)(Sp - Sc);
-                    const float Vb = Sp - Sc;
-                    Lb[c] += Sc * (V - Vnext[c]);
-                    Vnext[c] = V;
-                    mtb[c] = mt[c] > 0.f ? Vb * c_sim.lgd[c] * beta : 0.f;
-                    Ib -= Vb * V;
-                }
-                // ---- pricing at t_j: reverse, economy by economy ----
-                for (int e = 0; e < E; ++e) {
-                    const float re = dt_r[jj][e];
-                    const float2 f2 = __ldg(a.fix + (size_t)p * E + e);
-                    const float rfix = a.fixr[((size_t)p * E + e) * M + kl];
-                    const float fixm1 = expm1f(fmaf(f2.y, rfix, -f2.x));
-                    const float4 *tab = a.zc + ((size_t)j * E + e) * G;
-                    const float4 *dtab = a.dzc + ((size_t)j * E + e) * G;
-                    float Z[G], D[G], EM[G];
-                    const int pc = p < G ? p : G - 1;
-                    const float4 tp = __ldg(tab + pc);
-                    const float z_first = expf(fmaf(-tp.y, re, tp.x));
-#pragma unroll
-                    for (int g = 0; g < G; ++g) {
-                        EM[g] = 0.f;
-                        if (g < p) {
-                            Z[g] = 0.f;
-                            D[g] = 0.f;
-                        } else if (g == p) {
-                            Z[g] = z_first;
-                            D[g] = z_first * fixm1;
-                        } else {
-                            const float4 t4 = __ldg(tab + g);
-                            const float zp = Z[g > 0 ? g - 1 : 0];
-                            const float em = expm1_small(fmaf(-t4.w, re, t4.z));
-                            EM[g] = em;
-                            D[g] = -zp * em;
-                            Z[g] = fmaf(zp, em, zp);
-                        }
-                    }
-                    const float chi = (e == 0) ? 1.f : expf(dt_l[jj][e]);
-                    float Db[G], Zb[G];
-#pragma unroll
-                    for (int g = 0; g < G; ++g) Db[g] = Zb[g] = 0.f;
-                    float chib = 0.f;
-#pragma unroll
-                    for (int c = 0; c < C; ++c) {
-                        const int base = (c * E + e) * G;
-                        float acc = 0.f;
-#pragma unroll
-                        for (int h = 0; h < G; ++h) acc = fmaf(c_w.wA[base + h], D[h], acc);
-#pragma unroll
-                        for (int g = 0; g < G; ++g) acc = fmaf(-c_w.wK[base + g], Z[g], acc);
-                        chib = fmaf(mtb[c], acc, chib);
-                        const float accb = mtb[c] * chi;
-#pragma unroll
-                        for (int h = 0; h < G; ++h) Db[h] = fmaf(accb, c_w.wA[base + h], Db[h]);
-#pragma unroll
-                        for (int g = 0; g < G; ++g) Zb[g] = fmaf(-accb, c_w.wK[base + g], Zb[g]);
-                    }
-                    if (e > 0) lb[e] += chib * chi;
-                    float rbe = 0.f, pf = 0.f, ps = 0.f;
-#pragma unroll
-                    for (int g = G - 1; g >= 0; --g) {
-                        if (g > p) {
-                            const float zp = Z[g - 1 >= 0 ? g - 1 : 0];
-                            const float em = EM[g];
-                            Zb[g - 1 >= 0 ? g - 1 : 0] += Zb[g] * (1.f + em) - Db[g] * em;
-                            const float xb = (Zb[g] - Db[g]) * zp * (1.f + em);
-                            const float4 t4 = __ldg(tab + g);
-                            const float4 d4 = __ldg(dtab + g);
-                            rbe -= xb * t4.w;
-                            pf += xb * d4.z;
-                            ps += xb * d4.w;
-                        } else if (g == p) {
-                            Zb[g] += Db[g] * fixm1;
-                            const float fixb = Db[g] * Z[g];
-                            const float yb = Zb[g] * Z[g];
-                            const float4 d4 = __ldg(dtab + g);
-                            rbe -= yb * tp.y;
-                            pf += yb * d4.x;
-                            ps += yb * d4.y;
-                            const float ub = fixb * (1.f + fixm1);
-                            const float2 df2 = __ldg(a.dfix + (size_t)p * E + e);
-                            rfb[e] += ub * f2.y;
-                            pf -= ub * df2.x;
-                            ps -= ub * df2.y;
-                        }
-                    }
-                    rb[e] += rbe;
-                    pb[(PF + e) * 128] += pf;
-                    pb[(PSR + e) * 128] += ps;
-                }
-                // ---- Euler sub-steps of (t_{j-1}, t_j], in reverse ----
-                for (int s = S - 1; s >= 0; --s) {
-                    const int qs = (jj - 1) * S + s;
-                    const uint32_t q = (uint32_t)((j - 1) * S + s);
-                    float W[F];
-#pragma unroll
-                    for (int i = 0; i < F; ++i) W[i] = 0.f;
-#pragma unroll
-                    for (int b = 0; b < NB; ++b) {
-                        const uint4 x = philox4x32_10(make_uint4(k, q, 0u, (kStreamOuter << 24) | (uint32_t)b),
-                                                      a.seed_lo, a.seed_hi);
-                        float z[4];
-                        box_muller(x.x, x.y, z[0], z[1]);
-                        box_muller(x.z, x.w, z[2], z[3]);
-#pragma unroll
-                        for (int t = 0; t < 4; ++t) {
-                            const int col = 4 * b + t;
-                            if (col < F) {
-#pragma unroll
-                                for (int i = col; i < F; ++i) W[i] = fmaf(c_sim.L[i * (i + 1) / 2 + col], z[t], W[i]);
-                            }
-                        }
-                    }
-                    const float2 *dd = a.ddrift + (size_t)q * E;
-                    // parameter adjoints of this sub-step
-#pragma unroll
+    with_live<G>(p < G ? G - p : 0, [&](auto lv_) {
+        constexpr int LV = decltype(lv_)::value;
+        if constexpr (LV == 0) {   // every swap has matured: no exposure, no adjoints
+            if (REV)
+                for (int j = j0; j < j1; ++j) {
+                    for (int c = 0; c < C; ++c) put(a.V + ((size_t)j * C + c) * M, 0.f, 0.f);
                     for (int e = 0; e < E; ++e) {
-                        const float2 d2 = __ldg(dd + e);
-                        pb[(PF + e) * 128] += rb[e] * d2.x;
-                        pb[(PSR + e) * 128] += rb[e] * fmaf(sqds, W[e], d2.y);
+                        put(a.rbin + ((size_t)(j - 1) * E + e) * M, 0.f, 0.f);
+                        put(a.lbin + ((size_t)(j - 1) * E + e) * M, 0.f, 0.f);
                     }
-#pragma unroll
-                    for (int e = 1; e < E; ++e) {
-                        const float sx = __ldg(a.sig + E + e), sr = __ldg(a.sig + e);
-                        pb[(PSX + e) * 128] += lb[e] * fmaf(sqds, W[E - 1 + e], -sx * ds)
-                                               - rb[e] * __ldg(a.rho + e) * sr * ds;
-                    }
-                    float rb0_extra = Ib * ds;
-#pragma unroll
-                    for (int e = 1; e < E; ++e) rb0_extra = fmaf(lb[e], ds, rb0_extra);
-#pragma unroll
-                    for (int e = 0; e < E; ++e) {
-                        float v = rb[e] - rb[e] * c_sim.hw_a_ds[e];
-                        if (e > 0) v -= lb[e] * ds;
-                        else v += rb0_extra;
-                        rb[e] = v;
-                    }
-#pragma unroll
-                    for (int c = 0; c < C; ++c) {
-                        const float g = st_g[qs][c];
-                        const float gp = fmaxf(g, 0.f);
-                        float gbn = gb[c];
-                        if (c < CS) {
-                            constexpr int w0 = (CS > 0) ? 2 * E - 1 : 0;
-                            const float Wc = W[w0 + (c < CS ? c : 0)];
-                            const float kap = __ldg(a.sig + 2 * E + c), th = __ldg(a.sig + 2 * E + C + c);
-                            pb[(PK + c) * 128] += gb[c] * (th - gp) * ds;
-                            pb[(PT + c) * 128] += gb[c] * kap * ds;
-                            pb[(PN + c) * 128] += gb[c] * sqrtf(gp) * sqds * Wc;
-                            if (g > 0.f)
-                                gbn = gb[c] * (1.f - c_sim.cir_kds[c] + c_sim.cir_nu_sqds[c] * Wc * 0.5f * rsqrtf(g));
-                        }
-                        if (g > 0.f) gbn += Lb[c] * ds;
-                        gb[c] = gbn;
-                    }
+                    put(a.ibin + (size_t)(j - 1) * M, 0.f, 0.f);
                 }
-                // the state at t_{j-1}: a reset date receives the adjoint of its fixing
-                if ((j - 1) % ppp == 0)
-                    for (int e = 0; e < E; ++e) {
-                        rb[e] += rfb[e];
-                        rfb[e] = 0.f;
-                    }
+        } else {
+            constexpr int P0 = G - LV;   // = p
+            for (int i = tid; i < E * C * 2 * LV; i += NT) {
+                const int q = i % (2 * LV), row = i / (2 * LV) % C, e = i / (2 * LV * C), wrow = (row * E + e) * G + P0;
+                const float w = q < LV ? __ldg(a.w_glob + wrow + q) : __ldg(a.w_glob + kMaxW + wrow + q - LV);
+                w_s[i] = pack2(-w, -w);
             }
-        }
-        // r_0 = f
-        for (int e = 0; e < E; ++e) pb[(PF + e) * 128] += rb[e];
-        }
-    }
-
-    // ---- block reduction of the parameter adjoints and of J (FP64, fixed order) ----
-    __syncthreads();
-    double *out = a.part + (size_t)blockIdx.x * (NPAR + 1);
-    for (int i = 0; i <= NPAR; ++i) {
-        red_s[tid] = (i < NPAR) ? (double)pb_s[i * 128 + tid] : J;
-        __syncthreads();
-        for (int s = 64; s > 0; s >>= 1) {
-            if (tid < s) red_s[tid] += red_s[tid + s];
             __syncthreads();
+            const float *ffix = a.features + (size_t)(p * ppp) * F * M;   // state at the last reset
+            const float2 *fx = a.fix + (size_t)p * E;
+            // bond prices of economy e (price_kernel's): X holds -D, then Z; em[g] = expm1(x_g)
+            auto bonds = [&](int e, const float4 *tab, f32x2 re, f32x2 rfix, f32x2 (&X)[2 * LV], f32x2 (&em)[LV], f32x2 &fixm1) {
+                const float2 f2 = __ldg(fx + e), r = unpack2(re), rf = unpack2(rfix);
+                const float4 tp = __ldg(tab);
+                const float z0 = expf(fmaf(-tp.y, r.x, tp.x)), z1 = expf(fmaf(-tp.y, r.y, tp.x));
+                const float m0 = expm1f(fmaf(f2.y, rf.x, -f2.x)), m1 = expm1f(fmaf(f2.y, rf.y, -f2.x));
+                fixm1 = pack2(m0, m1);
+                X[0] = pack2(-(z0 * m0), -(z1 * m1));
+                X[LV] = pack2(z0, z1);
+                em[0] = pack2(0.f, 0.f);
+#pragma unroll
+                for (int g = 1; g < LV; ++g) {
+                    const float4 t4 = __ldg(tab + g);
+                    em[g] = expm1_small2(fma2(pack2(-t4.w, -t4.w), re, pack2(t4.z, t4.z)));
+                    X[g] = mul2(X[LV + g - 1], em[g]);
+                    X[LV + g] = fma2(X[LV + g - 1], em[g], X[LV + g - 1]);
+                }
+            };
+            for (int j = j0; j < j1; ++j) {
+                const float *fe = a.features + (size_t)j * F * M;
+                const float4 *tab = a.zc + (size_t)j * E * G + P0;
+                f32x2 mt[C];
+#pragma unroll
+                for (int c = 0; c < C; ++c) mt[c] = pack2(0.f, 0.f);
+#pragma unroll 1
+                for (int e = 0; e < E; ++e) {
+                    f32x2 X[2 * LV], em[LV], fixm1;
+                    const f32x2 re = pack2(__ldg(fe + (size_t)e * M + r0), __ldg(fe + (size_t)e * M + r1));
+                    const f32x2 rf = pack2(__ldg(ffix + (size_t)e * M + r0), __ldg(ffix + (size_t)e * M + r1));
+                    const float *lc = fe + (size_t)(E - 1 + (e > 0 ? e : 1)) * M;
+                    const f32x2 chi = e == 0 ? pack2(1.f, 1.f) : pack2(expf(__ldg(lc + r0)), expf(__ldg(lc + r1)));
+                    bonds(e, tab + e * G, re, rf, X, em, fixm1);
+                    const f32x2 *w = w_s + e * C * 2 * LV;
+#pragma unroll
+                    for (int c = 0; c < C; ++c) {
+                        f32x2 acc = pack2(0.f, 0.f);
+#pragma unroll
+                        for (int q = 0; q < 2 * LV; q += 2) {
+                            const ulonglong2 w2 = *reinterpret_cast<const ulonglong2 *>(w + c * 2 * LV + q);
+                            acc = fma2(w2.x, X[q], acc);
+                            acc = fma2(w2.y, X[q + 1], acc);
+                        }
+                        mt[c] = fma2(chi, acc, mt[c]);
+                    }
+                }
+                // exposures, survival terms and the adjoints of the MtM and of int r^0
+                const float b0 = expf(-__ldg(a.disc + (size_t)j * M + r0)), b1 = expf(-__ldg(a.disc + (size_t)j * M + r1));
+                f32x2 mtb[C];
+                float ib0 = 0.f, ib1 = 0.f;
+#pragma unroll
+                for (int c = 0; c < C; ++c) {
+                    const float2 m = unpack2(mt[c]);
+                    const float l = c_sim.lgd[c];
+                    const float V0 = l * b0 * fmaxf(m.x, 0.f), V1 = l * b1 * fmaxf(m.y, 0.f);
+                    const float *s1 = a.surv + ((size_t)j * C + c) * M, *s0 = s1 - (size_t)C * M;
+                    const float d0 = __ldg(s0 + r0) - __ldg(s1 + r0), d1 = __ldg(s0 + r1) - __ldg(s1 + r1);
+                    if (live0) J += (double)V0 * (double)d0;
+                    if (live1) J += (double)V1 * (double)d1;
+                    if (REV) {
+                        put(a.V + ((size_t)j * C + c) * M, V0, V1);
+                        mtb[c] = pack2(m.x > 0.f ? d0 * l * b0 : 0.f, m.y > 0.f ? d1 * l * b1 : 0.f);
+                        ib0 -= d0 * V0;
+                        ib1 -= d1 * V1;
+                    }
+                }
+                if (!REV) continue;
+                put(a.ibin + (size_t)(j - 1) * M, ib0, ib1);
+                float lb0 = 0.f, lb1 = 0.f;
+#pragma unroll 1
+                for (int e = 0; e < E; ++e) {
+                    f32x2 X[2 * LV], em[LV], fixm1, u[2 * LV];
+                    const f32x2 re = pack2(__ldg(fe + (size_t)e * M + r0), __ldg(fe + (size_t)e * M + r1));
+                    const f32x2 rf = pack2(__ldg(ffix + (size_t)e * M + r0), __ldg(ffix + (size_t)e * M + r1));
+                    const float *lc = fe + (size_t)(E - 1 + (e > 0 ? e : 1)) * M;
+                    const f32x2 chi = e == 0 ? pack2(1.f, 1.f) : pack2(expf(__ldg(lc + r0)), expf(__ldg(lc + r1)));
+                    bonds(e, tab + e * G, re, rf, X, em, fixm1);
+                    // u = sum_c (adjoint of MtM_c) w_c: times chi the adjoint of X
+                    const f32x2 *w = w_s + e * C * 2 * LV;
+#pragma unroll
+                    for (int q = 0; q < 2 * LV; ++q) u[q] = pack2(0.f, 0.f);
+#pragma unroll
+                    for (int c = 0; c < C; ++c)
+#pragma unroll
+                        for (int q = 0; q < 2 * LV; q += 2) {
+                            const ulonglong2 w2 = *reinterpret_cast<const ulonglong2 *>(w + c * 2 * LV + q);
+                            u[q] = fma2(w2.x, mtb[c], u[q]);
+                            u[q + 1] = fma2(w2.y, mtb[c], u[q + 1]);
+                        }
+                    f32x2 chib = pack2(0.f, 0.f);
+#pragma unroll
+                    for (int q = 0; q < 2 * LV; ++q) {
+                        chib = fma2(u[q], X[q], chib);
+                        u[q] = mul2(u[q], chi);
+                    }
+                    // -D_g = Z_{g-1} em_g, Z_g = Z_{g-1} (1 + em_g), em_g = expm1(x_g), x_g = dlnA - dB r
+                    const f32x2 one = pack2(1.f, 1.f);
+                    f32x2 rb = pack2(0.f, 0.f), pf = rb, psg = rb;
+                    const float4 *dtab = a.dzc + ((size_t)j * E + e) * G + P0;
+#pragma unroll
+                    for (int g = LV - 1; g >= 1; --g) {
+                        const f32x2 em1 = fma2(em[g], one, one);
+                        const f32x2 xb = mul2(mul2(fma2(u[LV + g], one, u[g]), X[LV + g - 1]), em1);
+                        u[LV + g - 1] = fma2(u[LV + g], em1, fma2(u[g], em[g], u[LV + g - 1]));
+                        const float4 t4 = __ldg(tab + e * G + g), d4 = __ldg(dtab + g);
+                        rb = fma2(xb, pack2(-t4.w, -t4.w), rb);
+                        pf = fma2(xb, pack2(d4.z, d4.z), pf);
+                        psg = fma2(xb, pack2(d4.w, d4.w), psg);
+                    }
+                    // the first live date: -D_0 = -Z_0 fixm1, Z_0 = exp(lnA - B r)
+                    {
+                        const f32x2 ndb = u[0];   // adjoint of -D_0
+                        const float2 nd = unpack2(ndb);
+                        const f32x2 db = pack2(-nd.x, -nd.y);
+                        const f32x2 yb = mul2(fma2(db, fixm1, u[LV]), X[LV]);
+                        const f32x2 ub = mul2(mul2(db, X[LV]), fma2(fixm1, one, one));
+                        const float4 tp = __ldg(tab + e * G), d4 = __ldg(dtab);
+                        const float2 f2 = __ldg(fx + e), df2 = __ldg(a.dfix + (size_t)p * E + e);
+                        rb = fma2(yb, pack2(-tp.y, -tp.y), rb);
+                        pf = fma2(yb, pack2(d4.x, d4.x), pf);
+                        psg = fma2(yb, pack2(d4.y, d4.y), psg);
+                        pf = fma2(ub, pack2(-df2.x, -df2.x), pf);
+                        psg = fma2(ub, pack2(-df2.y, -df2.y), psg);
+                        rf_s[e * NT + tid] = fma2(ub, pack2(f2.y, f2.y), rf_s[e * NT + tid]);
+                    }
+                    const float2 rb2 = unpack2(rb), pf2 = unpack2(pf), ps2 = unpack2(psg);
+                    put(a.rbin + ((size_t)(j - 1) * E + e) * M, rb2.x, rb2.y);
+                    par_s[2 * e * NT + tid] += (live0 ? pf2.x : 0.f) + (live1 ? pf2.y : 0.f);
+                    par_s[(2 * e + 1) * NT + tid] += (live0 ? ps2.x : 0.f) + (live1 ? ps2.y : 0.f);
+                    if (e > 0) {
+                        const float2 l2 = unpack2(mul2(chib, chi));
+                        put(a.lbin + ((size_t)(j - 1) * E + e) * M, l2.x, l2.y);
+                        lb0 += l2.x;
+                        lb1 += l2.y;
+                    }
+                }
+                put(a.lbin + (size_t)(j - 1) * E * M, lb0, lb1);
+            }
         }
-        if (tid == 0) out[i] = red_s[0];
-        __syncthreads();
+    });
+    if (REV)
+        for (int e = 0; e < E; ++e) {
+            const float2 v = unpack2(rf_s[e * NT + tid]);
+            put(a.fixin + ((size_t)blockIdx.y * E + e) * M, v.x, v.y);
+        }
+    // block sums in FP64, fixed order: a warp per value
+    j_s[tid] = J;
+    __syncthreads();
+    double *out = a.part_p + ((size_t)blockIdx.y * gridDim.x + blockIdx.x) * (2 * E + 1);
+    const int lane = tid & 31;
+    for (int v = REV ? tid >> 5 : 2 * E + (tid >> 5); v <= 2 * E; v += NT / 32) {
+        double s = 0.0;
+        for (int i = lane; i < NT; i += 32) s += v < 2 * E ? (double)par_s[v * NT + i] : j_s[i];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if (lane == 0) out[v] = s;
     }
+}
+
+// Block: 32 outer paths (lane = path), NW warps with the factors split over them as in
+// sim_kernel; the economy of index 0 alone needs the others, through the sum of their
+// log-FX adjoints, which adj_price_kernel provides. Bound by HBM (80 floats a (path, step)).
+template <int E, int C, int CS, int NW>
+__global__ void __launch_bounds__(32 * NW) adj_reverse_kernel(AdjSplitArgs a, int splits)
+{
+    constexpr int F = 2 * E - 1 + CS, NPAR = 3 * E - 1 + 3 * C;
+    constexpr int ME = (E + NW - 1) / NW, MC = (C + NW - 1) / NW;
+    constexpr int PF = 0, PSR = E, PSX = 2 * E - 1, PK = 3 * E - 1, PT = PK + C, PN = PT + C;   // PSX + e for e >= 1
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const uint32_t kl = blockIdx.x * 32u + (uint32_t)lane;
+    const bool live = kl < a.M;
+    const size_t M = a.M;
+    const uint32_t kr = live ? kl : 0u;   // a valid path to read for a lane past M
+    const int n = c_sim.n, S = c_sim.S, ppp = c_sim.ppp;
+    const float ds = c_sim.ds, sqds = c_sim.sqds;
+    auto has_e = [&](int i) { return NW * (i + 1) <= E || warp + NW * i < E; };
+    auto has_c = [&](int i) { return NW * (i + 1) <= C || warp + NW * i < C; };
+    float rb[ME], lb[ME], pf[ME], psr[ME], psx[ME], gb[MC], Lb[MC], Vn[MC], pk[MC], pt[MC], pn[MC];
+    float Ib = 0.f, lbs = 0.f;
+#pragma unroll
+    for (int i = 0; i < ME; ++i) rb[i] = lb[i] = pf[i] = psr[i] = psx[i] = 0.f;
+#pragma unroll
+    for (int i = 0; i < MC; ++i) gb[i] = Lb[i] = Vn[i] = pk[i] = pt[i] = pn[i] = 0.f;
+    for (int j = n; j >= 1; --j) {
+        // what the pricing at t_j adds, and the survival terms
+        const float *rin = a.rbin + (size_t)(j - 1) * E * M + kr, *lin = a.lbin + (size_t)(j - 1) * E * M + kr;
+        const float *sv = a.surv + (size_t)j * C * M + kr, *vv = a.V + (size_t)j * C * M + kr;
+#pragma unroll
+        for (int i = 0; i < ME; ++i)
+            if (has_e(i)) {
+                const int e = warp + NW * i;
+                rb[i] += __ldg(rin + (size_t)e * M);
+                if (e > 0) lb[i] += __ldg(lin + (size_t)e * M);
+            }
+        if (warp == 0) {
+            Ib += __ldg(a.ibin + (size_t)(j - 1) * M + kr);
+            lbs += __ldg(lin);
+        }
+#pragma unroll
+        for (int i = 0; i < MC; ++i)
+            if (has_c(i)) {
+                const int c = warp + NW * i;
+                const float v = __ldg(vv + (size_t)c * M);
+                Lb[i] += __ldg(sv + (size_t)c * M) * (v - Vn[i]);
+                Vn[i] = v;
+            }
+        for (int s = S - 1; s >= 0; --s) {   // Euler sub-steps of (t_{j-1}, t_j], in reverse
+            const int q = (j - 1) * S + s;
+            const float *W = a.inc + (size_t)q * F * M + kr, *gp_ = a.gpre + (size_t)q * C * M + kr;
+            const float2 *dd = a.ddrift + (size_t)q * E;
+#pragma unroll
+            for (int i = 0; i < ME; ++i)
+                if (has_e(i)) {
+                    const int e = warp + NW * i;
+                    const float2 d2 = __ldg(dd + e);
+                    pf[i] += rb[i] * d2.x;
+                    psr[i] += rb[i] * fmaf(sqds, __ldg(W + (size_t)e * M), d2.y);
+                    float v = rb[i] - rb[i] * c_sim.hw_a_ds[e];
+                    if (e > 0) {
+                        const float sx = __ldg(a.sig + E + e), sr = __ldg(a.sig + e);
+                        psx[i] += lb[i] * fmaf(sqds, __ldg(W + (size_t)(E - 1 + e) * M), -sx * ds)
+                                  - rb[i] * __ldg(a.rho + e) * sr * ds;
+                        v -= lb[i] * ds;
+                    } else {
+                        v += fmaf(lbs, ds, Ib * ds);
+                    }
+                    rb[i] = v;
+                }
+#pragma unroll
+            for (int i = 0; i < MC; ++i)
+                if (has_c(i)) {
+                    const int c = warp + NW * i;
+                    const float g = __ldg(gp_ + (size_t)c * M), gp = fmaxf(g, 0.f);
+                    float gbn = gb[i];
+                    if (NW * (i + 1) <= CS || c < CS) {
+                        const float Wc = __ldg(W + (size_t)(2 * E - 1 + c) * M);
+                        const float kap = __ldg(a.sig + 2 * E + c), th = __ldg(a.sig + 2 * E + C + c);
+                        pk[i] += gb[i] * (th - gp) * ds;
+                        pt[i] += gb[i] * kap * ds;
+                        pn[i] += gb[i] * sqrtf(gp) * sqds * Wc;
+                        if (g > 0.f)
+                            gbn = gb[i] * (1.f - c_sim.cir_kds[c] + c_sim.cir_nu_sqds[c] * Wc * 0.5f * rsqrtf(g));
+                    }
+                    if (g > 0.f) gbn += Lb[i] * ds;
+                    gb[i] = gbn;
+                }
+        }
+        // the state at t_{j-1}: a reset date receives the adjoints of its fixing
+        if ((j - 1) % ppp == 0) {
+            const int p = (j - 1) / ppp;
+#pragma unroll
+            for (int i = 0; i < ME; ++i)
+                if (has_e(i))
+                    for (int b = 0; b < splits; ++b)
+                        rb[i] += __ldg(a.fixin + ((size_t)(p * splits + b) * E + warp + NW * i) * M + kr);
+        }
+    }
+    // sums over the block's paths, FP64
+    double *out = a.part_r + (size_t)blockIdx.x * NPAR;
+    auto total = [&](float x, int at) {
+        double s = live ? (double)x : 0.0;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if (lane == 0) out[at] = s;
+    };
+#pragma unroll
+    for (int i = 0; i < ME; ++i)
+        if (has_e(i)) {
+            const int e = warp + NW * i;
+            total(pf[i] + rb[i], PF + e);   // r_0 = f
+            total(psr[i], PSR + e);
+            if (e > 0) total(psx[i], PSX + e);
+        }
+#pragma unroll
+    for (int i = 0; i < MC; ++i)
+        if (has_c(i)) {
+            const int c = warp + NW * i;
+            total(pk[i], PK + c);
+            total(pt[i], PT + c);
+            total(pn[i], PN + c);
+        }
 }
 
 }  // namespace

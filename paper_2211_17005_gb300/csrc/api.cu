@@ -869,6 +869,10 @@ cva_status cva_mlp_regress_all(const cva_sim *sim, int pf, int hidden, int n_bat
 
 int cva_grad_num_params(int E, int C) { return 3 * E - 1 + 3 * C; }
 
+// device memory the adjoint of a compiled shape may take for its arrays: 2^15 paths at the
+// paper shape (40 KB a path), which fill the chip; larger path counts run in ranges
+constexpr size_t kAdjScratch = (size_t)1400 << 20;
+
 cva_status cva_par_rates(const cva_model_desc *model, const cva_portfolio_desc *pf, double *rates_host)
 {
     int F = 0, CS = 0;
@@ -957,6 +961,30 @@ cva_status cva_grad_cva0(const cva_model_desc *model, const cva_portfolio_desc *
     const size_t Mz = M;
     const unsigned blocks = (unsigned)((M + 127) / 128);
     cudaStream_t cs = reinterpret_cast<cudaStream_t>(stream);
+    // the compiled shapes take the paths in equal ranges whose arrays fit kAdjScratch; the
+    // run-time shapes take them at once, with checkpoints
+    uint64_t ranges = 1, Mr = M;
+    const size_t nsum = s.generic ? (size_t)NPAR + 1 : (size_t)(2 * E + 1 + NPAR);
+    if (!s.generic) {
+        for (;;) {
+            Mr = (M + ranges - 1) / ranges;
+            st = launch_adjoint(s, b, seed, k0, (uint32_t)Mr, cs);   // without scratch: its size
+            if (st != CVA_OK) {
+                cva_sim_destroy(hs);
+                return st;
+            }
+            if (b.scratch_bytes <= kAdjScratch || Mr <= 256) break;
+            ranges = std::max(ranges + 1, ranges * (b.scratch_bytes / kAdjScratch));
+        }
+        Mr = (Mr + 255) / 256 * 256;   // whole blocks
+        ranges = (M + Mr - 1) / Mr;
+        size_t most = 0;   // the full ranges and the last one
+        for (uint64_t m : {std::min<uint64_t>(Mr, M), M - (ranges - 1) * Mr}) {
+            launch_adjoint(s, b, seed, k0, (uint32_t)m, cs);
+            most = std::max(most, b.scratch_bytes);
+        }
+        b.scratch_bytes = most;
+    }
     auto cleanup = [&]() {
         cudaFree(b.dzc);
         cudaFree(b.dfix);
@@ -968,14 +996,17 @@ cva_status cva_grad_cva0(const cva_model_desc *model, const cva_portfolio_desc *
         cudaFree(b.fixr);
         cudaFree(b.part);
         cudaFree(b.sum);
+        cudaFree(b.scratch);
         cva_sim_destroy(hs);
     };
     if (dev_alloc(&b.dzc, dzc.size()) != CVA_OK || dev_alloc(&b.dfix, dfix.size()) != CVA_OK ||
         dev_alloc(&b.ddrift, ddrift.size()) != CVA_OK || dev_alloc(&b.rho, rho.size()) != CVA_OK ||
-        dev_alloc(&b.sig, sig.size()) != CVA_OK || dev_alloc(&b.ckpt, (size_t)b.nseg * NV * Mz) != CVA_OK ||
-        dev_alloc(&b.ckpt_I0, (size_t)b.nseg * Mz) != CVA_OK ||
-        dev_alloc(&b.fixr, (size_t)(periods + 1) * E * Mz) != CVA_OK ||
-        dev_alloc(&b.part, (size_t)blocks * (NPAR + 1)) != CVA_OK || dev_alloc(&b.sum, (size_t)NPAR + 1) != CVA_OK) {
+        dev_alloc(&b.sig, sig.size()) != CVA_OK || dev_alloc(&b.sum, nsum * ranges) != CVA_OK ||
+        (s.generic && (dev_alloc(&b.ckpt, (size_t)b.nseg * NV * Mz) != CVA_OK ||
+                       dev_alloc(&b.ckpt_I0, (size_t)b.nseg * Mz) != CVA_OK ||
+                       dev_alloc(&b.fixr, (size_t)(periods + 1) * E * Mz) != CVA_OK ||
+                       dev_alloc(&b.part, (size_t)blocks * (NPAR + 1)) != CVA_OK)) ||
+        (!s.generic && dev_alloc(&b.scratch, b.scratch_bytes) != CVA_OK)) {
         cleanup();
         return CVA_ENOMEM;
     }
@@ -989,18 +1020,44 @@ cva_status cva_grad_cva0(const cva_model_desc *model, const cva_portfolio_desc *
             cleanup();
             return cuda_fail(e, "grad: table upload");
         }
-    st = launch_adjoint(s, b, seed, k0, (uint32_t)M, cs);
-    if (st == CVA_OK) st = sum_columns_fp64(b.part, (int)blocks, NPAR + 1, b.sum, cs);
-    std::vector<double> h(NPAR + 1);
+    if (s.generic) {
+        st = launch_adjoint(s, b, seed, k0, (uint32_t)M, cs);
+        if (st == CVA_OK) st = sum_columns_fp64(b.part, (int)blocks, NPAR + 1, b.sum, cs);
+    } else {
+        double *sums = b.sum;
+        for (uint64_t r = 0; r < ranges && st == CVA_OK; ++r) {
+            const uint64_t first = r * Mr;
+            b.sum = sums + r * nsum;
+            st = launch_adjoint(s, b, seed, k0 + first, (uint32_t)std::min(Mr, M - first), cs);
+        }
+        b.sum = sums;
+    }
+    std::vector<double> h(nsum * ranges);
     if (st == CVA_OK) {
         cudaError_t e = cudaMemcpyAsync(h.data(), b.sum, h.size() * sizeof(double), cudaMemcpyDeviceToHost, cs);
         if (e == cudaSuccess) e = cudaStreamSynchronize(cs);
         if (e != cudaSuccess) st = cuda_fail(e, "grad: read-back");
     }
     if (st == CVA_OK) {
-        *cva0_host = h[NPAR] / (double)M;
+        std::vector<double> g((size_t)NPAR + 1, 0.0);   // parameters in the order of cva_grad_cva0, then J
+        for (uint64_t r = 0; r < ranges; ++r) {
+            const double *v = h.data() + r * nsum;
+            if (s.generic) {
+                for (int i = 0; i <= NPAR; ++i) g[i] += v[i];
+                continue;
+            }
+            if (!forward_only) {
+                for (int i = 0; i < NPAR; ++i) g[i] += v[2 * E + 1 + i];
+                for (int e = 0; e < E; ++e) {
+                    g[e] += v[2 * e];
+                    g[E + e] += v[2 * e + 1];
+                }
+            }
+            g[NPAR] += v[2 * E];
+        }
+        *cva0_host = g[NPAR] / (double)M;
         if (grad_host && !forward_only)
-            for (int i = 0; i < NPAR; ++i) grad_host[i] = h[i] / (double)M;
+            for (int i = 0; i < NPAR; ++i) grad_host[i] = g[i] / (double)M;
     }
     cleanup();
     return st;

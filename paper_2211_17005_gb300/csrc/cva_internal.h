@@ -120,7 +120,9 @@ struct AdjBuffers {
     double *ckpt_I0 = nullptr;  // [nseg][M]
     float *fixr = nullptr;      // [periods+1][E][M]
     double *part = nullptr;     // [blocks][npar+1]
-    double *sum = nullptr;      // [npar+1]
+    double *sum = nullptr;      // [npar+1]; the compiled shapes': [2E + 1 + npar] per range of paths
+    unsigned char *scratch = nullptr;   // the compiled shapes' arrays of one range of paths
+    size_t scratch_bytes = 0;
 };
 
 // One compiled shape of the outer-path kernel (outer_*.cu).
@@ -128,7 +130,7 @@ struct OuterInst {
     int E, C, CS, G, NPF;
     cva_status (*launch)(Sim &s, uint64_t seed, uint64_t k0, cudaStream_t st);
     void (*forget)(const Sim *s);
-    cva_status (*adjoint)(Sim &s, const AdjBuffers &b, uint64_t seed, uint64_t k0, uint32_t M, cudaStream_t st);
+    cva_status (*adjoint)(Sim &s, AdjBuffers &b, uint64_t seed, uint64_t k0, uint32_t M, cudaStream_t st);
 };
 
 // Kernel launchers (sim.cu).
@@ -136,7 +138,7 @@ cva_status launch_outer(Sim &s, uint64_t seed, uint64_t k0, cudaStream_t st);
 cva_status launch_inner(Sim &s, uint64_t seed, uint64_t k0, cudaStream_t st);
 void forget_const_owner(const Sim *s);
 bool outer_supported(int E, int C, int CS, int G, int NPF, int *Ginst);
-cva_status launch_adjoint(Sim &s, const AdjBuffers &b, uint64_t seed, uint64_t k0, uint32_t M, cudaStream_t st);
+cva_status launch_adjoint(Sim &s, AdjBuffers &b, uint64_t seed, uint64_t k0, uint32_t M, cudaStream_t st);
 cva_status sum_columns_fp64(const double *part, int rows, int cols, double *out, cudaStream_t st);
 // Block sums of the Prop. 1 statistics (sim.cu): part [blocks][n][3].
 cva_status launch_oversim(const Sim &s, int pf, const float *pred, uint64_t seed, double *part, unsigned blocks,
@@ -210,6 +212,10 @@ cva_status lsq_normal_partial(const float *targ, const float *feat, int F, uint6
                               double *gram_host, cudaStream_t st);
 cva_status lsq_solve_normal_host(const double *gram, int F, int basis, const double *centre, double *coef_centred,
                                  double *coef_raw, int *dropped);
+// Predictions of `groups` linear fits: group g's F + 1 coefficients in its basis centred on
+// path 0 at coef + g coef_stride.
+cva_status lsq_predict_groups(const float *feat0, size_t feat_stride, int F, uint64_t M, int groups, const double *coef,
+                              size_t coef_stride, float *pred0, size_t pred_stride, cudaStream_t st);
 cva_status lsq_predict_centred(const float *feat, int F, uint64_t M, int basis, const float *centre,
                                const double *coef_centred_host, float *pred, cudaStream_t st);
 cva_status twin_l2_fp64(const float *phi, const float *xi1, const float *xi2, uint64_t M, double *out2,

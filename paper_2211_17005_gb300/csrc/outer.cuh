@@ -87,6 +87,7 @@ struct OuterArgs {
     const float *__restrict__ drift;   // [n*S][E]
     float *features, *disc, *thr, *expo, *mtm;
     const float *w_glob;               // device copy of the date-bucketed weights: wA [kMaxW], then wK [kMaxW]
+    float *inc, *gpre;                 // the adjoint's: [n*S][F][M] increments, [n*S][C][M] intensities before a fine step
 };
 
 // Block: 32 outer paths (lane = path), NW warps. The normals of a fine step depend on no
@@ -100,12 +101,15 @@ struct OuterArgs {
 // as a single FMA): 352 instructions a step at 27 factors against 728 with one constant
 // load and one FMA per entry.
 //
+// ADJ: the adjoint's forward sweep, which keeps e^{-Lambda} in the place of the thresholds,
+// and the increments and intensities of every fine step.
+//
 // Bound by instruction issue (Philox, logarithm, square root and sine-cosine of 14
 // Box-Muller pairs, the correlation): 2650 instructions a (path, step) at 27 factors and
 // 85% of the issue slots. Paper shape, 2^17 paths and 100 steps: 1.28 -> 1.11 ms against a
 // thread per path over all steps (96 registers, 7 to 14 warps a multiprocessor); 2^15
 // paths and 2500 steps 9.09 -> 6.51 ms; 2^14 paths and 100 steps 0.43 -> 0.18 ms.
-template <int E, int C, int CS, int NW>
+template <int E, int C, int CS, int NW, bool ADJ>
 __global__ void __launch_bounds__(32 * NW, NW == 8 ? 3 : 5) sim_kernel(OuterArgs a)
 {
     constexpr int F = 2 * E - 1 + CS;
@@ -156,7 +160,8 @@ __global__ void __launch_bounds__(32 * NW, NW == 8 ? 3 : 5) sim_kernel(OuterArgs
             for (int i = 0; i < MC; ++i)
                 if (has_c(i)) {
                     if (is_cir(i)) pg[(size_t)(NW * i) * M] = gam[i];
-                    pt[(size_t)(NW * i) * M] = -expm1f(-lam[i]);   // 0 at date 0
+                    // threshold (0 at date 0) or survival factor
+                    pt[(size_t)(NW * i) * M] = ADJ ? expf(-lam[i]) : -expm1f(-lam[i]);
                 }
         }
         pr += (size_t)F * M;
@@ -204,6 +209,7 @@ __global__ void __launch_bounds__(32 * NW, NW == 8 ? 3 : 5) sim_kernel(OuterArgs
             for (int i = 0; i < F; ++i) {
                 const float2 w = unpack2(W[i / 2]);
                 Ws[v][i][lane] = i & 1 ? w.y : w.x;
+                if (ADJ && live) a.inc[((size_t)q * F + i) * M + kl] = i & 1 ? w.y : w.x;
             }
         }
         __syncthreads();
@@ -236,6 +242,7 @@ __global__ void __launch_bounds__(32 * NW, NW == 8 ? 3 : 5) sim_kernel(OuterArgs
 #pragma unroll
             for (int i = 0; i < MC; ++i)
                 if (has_c(i)) {
+                    if (ADJ && live) a.gpre[((size_t)(q0 + u) * C + warp + NW * i) * M + kl] = gam[i];
                     const float gp = fmaxf(gam[i], 0.f);
                     const float y = fmaf(gp, ds, -lamc[i]);
                     const float t = lam[i] + y;
@@ -469,13 +476,25 @@ static void outer_forget(const Sim *s)
         if (o == s) o = nullptr;
 }
 
+// a period's dates share one block's weights; they are split while `blocks` blocks do not
+// fill the chip four times
+static PriceShape price_shape(uint64_t blocks, int ppp, int sms)
+{
+    PriceShape ps = {ppp, 1};
+    while (blocks * ps.splits < 4u * (unsigned)sms && ps.dates_per_block > 1) {
+        ps.dates_per_block = (ps.dates_per_block + 1) / 2;
+        ps.splits = (ppp + ps.dates_per_block - 1) / ps.dates_per_block;
+    }
+    return ps;
+}
+
 template <int E, int C, int CS, int G, int NPF>
 cva_status outer_launch(Sim &s, uint64_t seed, uint64_t k0, cudaStream_t st)
 {
     int dev = 0;
     CVA_CUDA_TRY(cudaGetDevice(&dev));
     if (dev < 0 || dev >= 64) return fail(CVA_EINVAL, "device index out of range");
-    OuterArgs args;
+    OuterArgs args = {};
     args.M = (uint32_t)s.M;
     args.k0 = (uint32_t)k0;
     args.seed_lo = (uint32_t)seed;
@@ -516,8 +535,8 @@ cva_status outer_launch(Sim &s, uint64_t seed, uint64_t k0, cudaStream_t st)
     CVA_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     const unsigned sgrid = (args.M + 31u) / 32u;
     const bool wide = s.tune_sim_block ? s.tune_sim_block == 128 : sgrid < 2u * (unsigned)sms;
-    if (wide) sim_kernel<E, C, CS, 8><<<sgrid, 256, 0, st>>>(args);
-    else sim_kernel<E, C, CS, 4><<<sgrid, 128, 0, st>>>(args);
+    if (wide) sim_kernel<E, C, CS, 8, false><<<sgrid, 256, 0, st>>>(args);
+    else sim_kernel<E, C, CS, 4, false><<<sgrid, 128, 0, st>>>(args);
     CVA_CUDA_TRY(cudaGetLastError());
     if (s.ev[1]) CVA_CUDA_TRY(cudaEventRecord(s.ev[1], st));
     if (s.tune_price_pf == 4) {   // every portfolio per 128-path tile on the tensor cores
@@ -543,13 +562,7 @@ cva_status outer_launch(Sim &s, uint64_t seed, uint64_t k0, cudaStream_t st)
     const int ppb = s.tune_price_pf ? (NPF % s.tune_price_pf == 0 ? s.tune_price_pf : 1)
                                     : (NPF % 3 == 0 ? 3 : NPF % 2 == 0 ? 2 : 1);
     const unsigned tiles = (args.M + 2 * pb - 1) / (2 * pb), periods = (unsigned)((s.n + s.ppp - 1) / s.ppp);
-    // a period's dates share one block's weights; split them while the blocks do not fill
-    // the chip four times
-    PriceShape ps = {s.ppp, 1};
-    while ((uint64_t)tiles * periods * (NPF / ppb) * ps.splits < 4u * (unsigned)sms && ps.dates_per_block > 1) {
-        ps.dates_per_block = (ps.dates_per_block + 1) / 2;
-        ps.splits = (s.ppp + ps.dates_per_block - 1) / ps.dates_per_block;
-    }
+    const PriceShape ps = price_shape((uint64_t)tiles * periods * (NPF / ppb), s.ppp, sms);
     const dim3 pgrid(tiles, periods * (unsigned)ps.splits, (unsigned)(NPF / ppb));
     const size_t psmem = (size_t)E * ppb * C * 2 * G * sizeof(f32x2);
     static_assert(E * 3 * C * 2 * G * sizeof(f32x2) <= 48 * 1024, "portfolio weights exceed the default shared-memory limit");
@@ -565,35 +578,72 @@ cva_status outer_launch(Sim &s, uint64_t seed, uint64_t k0, cudaStream_t st)
     return CVA_OK;
 }
 
+// The adjoint of one range of paths; `b` holds the tables, the scratch and the sums that
+// this range adds. sums_only: the scratch this range needs, nothing launched.
 template <int E, int C, int CS, int G>
-cva_status adjoint_launch(Sim &s, const AdjBuffers &b, uint64_t seed, uint64_t k0, uint32_t M, cudaStream_t st)
+cva_status adjoint_launch(Sim &s, AdjBuffers &b, uint64_t seed, uint64_t k0, uint32_t M, cudaStream_t st)
 {
-    constexpr int KMAX = 16, SMAX = 4;
+    constexpr int KMAX = 16, SMAX = 4, F = 2 * E - 1 + CS, NPAR = 3 * E - 1 + 3 * C;
     if (b.K < 1 || b.K > KMAX || s.S > SMAX) return fail(CVA_ENOTSUP, "adjoint: checkpoint interval <= 16, sub-steps <= 4");
-    int dev = 0;
+    int dev = 0, sms = 0;
     CVA_CUDA_TRY(cudaGetDevice(&dev));
     if (dev < 0 || dev >= 64) return fail(CVA_EINVAL, "device index out of range");
-    AdjArgs a;
+    CVA_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    const size_t n = s.n, q = n * s.S, Mz = M;
+    const unsigned tiles = (M + 255u) / 256u, periods = (unsigned)((s.n + s.ppp - 1) / s.ppp), rblocks = (M + 31u) / 32u;
+    const PriceShape ps = price_shape((uint64_t)tiles * periods, s.ppp, sms);
+    const size_t pblocks = (size_t)tiles * periods * ps.splits;
+    // scratch: the block sums (FP64), then the arrays of the range
+    size_t off = 0;
+    auto take = [&](size_t bytes) {
+        const size_t at = off;
+        off += (bytes + 255) / 256 * 256;
+        return b.scratch ? b.scratch + at : nullptr;
+    };
+    AdjSplitArgs a = {};
+    a.part_p = reinterpret_cast<double *>(take(pblocks * (2 * E + 1) * 8));
+    a.part_r = reinterpret_cast<double *>(take((size_t)rblocks * NPAR * 8));
+    float *features = reinterpret_cast<float *>(take((n + 1) * F * Mz * 4));
+    float *disc = reinterpret_cast<float *>(take((n + 1) * Mz * 4));
+    float *surv = reinterpret_cast<float *>(take((n + 1) * C * Mz * 4));
+    float *inc = reinterpret_cast<float *>(take(q * F * Mz * 4));
+    float *gpre = reinterpret_cast<float *>(take(q * C * Mz * 4));
+    a.V = reinterpret_cast<float *>(take((n + 1) * C * Mz * 4));
+    a.rbin = reinterpret_cast<float *>(take(n * E * Mz * 4));
+    a.lbin = reinterpret_cast<float *>(take(n * E * Mz * 4));
+    a.ibin = reinterpret_cast<float *>(take(n * Mz * 4));
+    a.fixin = reinterpret_cast<float *>(take((size_t)periods * ps.splits * E * Mz * 4));
+    if (!b.scratch) {
+        b.scratch_bytes = off;
+        return CVA_OK;
+    }
+    if (off > b.scratch_bytes) return fail(CVA_ENOMEM, "adjoint: scratch too small");
     a.M = M;
-    a.k0 = (uint32_t)k0;
-    a.seed_lo = (uint32_t)seed;
-    a.seed_hi = (uint32_t)(seed >> 32);
-    a.K = b.K;
-    a.nseg = b.nseg;
-    a.forward_only = b.forward_only;
     a.zc = s.d_zc;
     a.fix = s.d_fix;
-    a.date_p = s.d_date_p;
-    a.drift = s.d_drift;
     a.dzc = b.dzc;
     a.dfix = b.dfix;
     a.ddrift = b.ddrift;
     a.rho = b.rho;
     a.sig = b.sig;
-    a.ckpt = b.ckpt;
-    a.ckpt_I0 = b.ckpt_I0;
-    a.fixr = b.fixr;
-    a.part = b.part;
+    a.w_glob = reinterpret_cast<const float *>(s.d_const_img + sizeof(SimConsts));
+    a.features = features;
+    a.disc = disc;
+    a.surv = surv;
+    a.inc = inc;
+    a.gpre = gpre;
+    OuterArgs o = {};
+    o.M = M;
+    o.k0 = (uint32_t)k0;
+    o.seed_lo = (uint32_t)seed;
+    o.seed_hi = (uint32_t)(seed >> 32);
+    o.branch_step = INT_MAX;
+    o.drift = s.d_drift;
+    o.features = features;
+    o.disc = disc;
+    o.thr = surv;
+    o.inc = inc;
+    o.gpre = gpre;
     std::lock_guard<std::mutex> lk(t_const_mu);
     if (!t_last[dev]) CVA_CUDA_TRY(cudaEventCreateWithFlags(&t_last[dev], cudaEventDisableTiming));
     else CVA_CUDA_TRY(cudaStreamWaitEvent(st, t_last[dev], 0));
@@ -601,10 +651,26 @@ cva_status adjoint_launch(Sim &s, const AdjBuffers &b, uint64_t seed, uint64_t k
         CVA_CUDA_TRY(upload_consts(s, st));
         t_owner[dev] = &s;
     }
-    adjoint_kernel<E, C, CS, G, KMAX, SMAX><<<(M + 127u) / 128u, 128, 0, st>>>(a);
+    if (rblocks < 2u * (unsigned)sms) sim_kernel<E, C, CS, 8, true><<<rblocks, 256, 0, st>>>(o);
+    else sim_kernel<E, C, CS, 4, true><<<rblocks, 128, 0, st>>>(o);
     CVA_CUDA_TRY(cudaGetLastError());
+    const dim3 pgrid(tiles, periods * (unsigned)ps.splits);
+    const size_t psmem = (size_t)E * C * 2 * G * sizeof(f32x2) + (size_t)E * 128 * 16;
+    static_assert(E * C * 2 * G * sizeof(f32x2) + E * 128 * 16 <= 47 * 1024, "adjoint pricing: default shared-memory limit");
+    if (b.forward_only) {
+        adj_price_kernel<E, C, CS, G, false><<<pgrid, 128, psmem, st>>>(a, ps);
+        CVA_CUDA_TRY(cudaGetLastError());
+    } else {
+        adj_price_kernel<E, C, CS, G, true><<<pgrid, 128, psmem, st>>>(a, ps);
+        CVA_CUDA_TRY(cudaGetLastError());
+        adj_reverse_kernel<E, C, CS, 4><<<rblocks, 128, 0, st>>>(a, ps.splits);
+        CVA_CUDA_TRY(cudaGetLastError());
+    }
     CVA_CUDA_TRY(cudaEventRecord(t_last[dev], st));
-    return CVA_OK;
+    // the range's sums: [2E + 1] of the pricing, then [NPAR] of the recursions
+    cva_status r = sum_columns_fp64(a.part_p, (int)pblocks, 2 * E + 1, b.sum, st);
+    if (r == CVA_OK && !b.forward_only) r = sum_columns_fp64(a.part_r, (int)rblocks, NPAR, b.sum + 2 * E + 1, st);
+    return r;
 }
 
 }  // namespace

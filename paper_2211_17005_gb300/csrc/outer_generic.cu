@@ -162,6 +162,25 @@ __global__ void __launch_bounds__(256) price_generic_kernel(OuterArgs a)
 // parameter adjoints live in dynamic shared memory, NPAR x 128 floats.
 constexpr int kAdjKMax = 16, kAdjSMax = 4;
 
+struct AdjArgs {
+    uint32_t M, k0, seed_lo, seed_hi;
+    int K, nseg;
+    int forward_only;                   // 1: the smooth CVA_0 of the forward sweep only
+    const float4 *__restrict__ zc;      // [n+1][E][G] (lnA, B, dlnA, dB)
+    const float2 *__restrict__ fix;     // [periods+1][E] (lnA, B)
+    const int *__restrict__ date_p;     // [n+1]
+    const float *__restrict__ drift;    // [n*S][E]
+    const float4 *__restrict__ dzc;     // [n+1][E][G] d/df, d/dsigma of (lnA, dlnA)
+    const float2 *__restrict__ dfix;    // [periods+1][E] d/df, d/dsigma of lnA at the fixing
+    const float2 *__restrict__ ddrift;  // [n*S][E] d drift/df, d drift/dsigma^r (quanto included)
+    const float *__restrict__ rho;      // [E] correlation of r^e and log chi^e (entry 0 unused)
+    const float *__restrict__ sig;      // [E] sigma^r, [E] sigma^chi, [C] kappa, [C] theta, [C] nu
+    float *ckpt;                        // [nseg][2E+3C][M]
+    double *ckpt_I0;                    // [nseg][M]
+    float *fixr;                        // [periods+1][E][M]
+    double *part;                       // [blocks][npar + 1]
+};
+
 // bond prices Z and their differences D (and the expm1 factors EM) of economy e at
 // date j for one path: the chained form of price_kernel
 __device__ __forceinline__ void bonds_generic(const AdjArgs &a, int j, int e, int p, float re, float fixm1,
@@ -488,7 +507,7 @@ __global__ void __launch_bounds__(128) adjoint_generic_kernel(AdjArgs a)
     }
 }
 
-cva_status adjoint_generic_launch(Sim &s, const AdjBuffers &b, uint64_t seed, uint64_t k0, uint32_t M, cudaStream_t st)
+cva_status adjoint_generic_launch(Sim &s, AdjBuffers &b, uint64_t seed, uint64_t k0, uint32_t M, cudaStream_t st)
 {
     if (b.K < 1 || b.K > kAdjKMax || s.S > kAdjSMax)
         return fail(CVA_ENOTSUP, "adjoint: checkpoint interval <= 16, sub-steps <= 4");
@@ -542,7 +561,7 @@ cva_status outer_generic_launch(Sim &s, uint64_t seed, uint64_t k0, cudaStream_t
     int dev = 0;
     CVA_CUDA_TRY(cudaGetDevice(&dev));
     if (dev < 0 || dev >= 64) return fail(CVA_EINVAL, "device index out of range");
-    OuterArgs args;
+    OuterArgs args = {};
     args.M = (uint32_t)s.M;
     args.k0 = (uint32_t)k0;
     args.seed_lo = (uint32_t)seed;

@@ -120,14 +120,22 @@ __global__ void __launch_bounds__(kRedThreads) relerr_stage1(const float *__rest
     if (threadIdx.x == 0) part[blockIdx.x] = make_double2(s, q);
 }
 
-// out[c] = sum over rows r of part[r][c], in row order (one thread per column)
-__global__ void sum_cols(const double *__restrict__ part, int rows, int cols, double *__restrict__ out)
+// out[c] = sum over rows r of part[r][c]: a block per column, a fixed tree
+__global__ void __launch_bounds__(kRedThreads) sum_cols(const double *__restrict__ part, int rows, int cols,
+                                                        double *__restrict__ out)
 {
-    const int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= cols) return;
+    __shared__ double sh[kRedThreads];
+    const int c = blockIdx.x, tid = threadIdx.x;
     double s = 0.0;
-    for (int r = 0; r < rows; ++r) s += part[(size_t)r * cols + c];
-    out[c] = s;
+#pragma unroll 4
+    for (int r = tid; r < rows; r += kRedThreads) s += part[(size_t)r * cols + c];
+    sh[tid] = s;
+    __syncthreads();
+    for (int o = kRedThreads / 2; o > 0; o >>= 1) {
+        if (tid < o) sh[tid] += sh[tid + o];
+        __syncthreads();
+    }
+    if (tid == 0) out[c] = sh[0];
 }
 
 std::mutex g_red_mu;
@@ -150,7 +158,7 @@ cva_status philox_blocks(const uint32_t *ctr, uint32_t *out, uint64_t n, uint64_
 
 cva_status sum_columns_fp64(const double *part, int rows, int cols, double *out, cudaStream_t st)
 {
-    sum_cols<<<(cols + 127) / 128, 128, 0, st>>>(part, rows, cols, out);
+    sum_cols<<<cols, kRedThreads, 0, st>>>(part, rows, cols, out);
     CVA_CUDA_TRY(cudaGetLastError());
     return CVA_OK;
 }

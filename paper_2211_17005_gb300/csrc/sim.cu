@@ -392,7 +392,7 @@ static const OuterInst *generic_outer()
     return p;
 }
 
-cva_status launch_adjoint(Sim &s, const AdjBuffers &b, uint64_t seed, uint64_t k0, uint32_t M, cudaStream_t st)
+cva_status launch_adjoint(Sim &s, AdjBuffers &b, uint64_t seed, uint64_t k0, uint32_t M, cudaStream_t st)
 {
     if (s.generic) return generic_outer()->adjoint(s, b, seed, k0, M, st);
     const OuterInst *o = find_outer(s.E, s.C, s.CS, s.G, s.NPF);
