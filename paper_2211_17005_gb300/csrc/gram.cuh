@@ -72,47 +72,59 @@ __global__ void __launch_bounds__(MAXT, MINB) gram_kernel(GramArgs a)
         const int s = i / ((NC - a.cols) * TR), o = i % ((NC - a.cols) * TR);
         tiles[(s * NC + a.cols) * TR + o] = 0.f;
     }
+    for (int i = tid; i < 3 * TR; i += nthr) tiles[(i / TR) * NC * TR + i % TR] = 1.f;
     __syncthreads();
     const uint32_t sbase = (uint32_t)__cvta_generic_to_shared(tiles);
     const int ntiles = r_begin < r_end ? (int)((r_end - r_begin + TR - 1) / TR) : 0;
-    constexpr int PW = VEC ? 4 : 1, NPC = TR / PW;   // rows of a piece, pieces of a column
+    const int nwarps = nthr >> 5;
+    constexpr int PW = VEC ? 4 : 1, PL = TR / PW / 32;   // rows of a piece, pieces of a lane
+    // a warp copies whole columns, its lanes the pieces lane, lane + 32, ...
     auto issue = [&](int t) {
         if (t < ntiles) {
-            const uint32_t r0 = r_begin + (uint32_t)t * TR;
-            const int s = t % 3;
-            for (int i = tid; i < ncopy * NPC; i += nthr) {
-                const int cc = i / NPC, q = i % NPC;
-                const uint32_t r = r0 + (uint32_t)(q * PW);
-                const bool ok = r < r_end;
-                const uint32_t to = sbase + (uint32_t)((s * NC + 1 + cc) * TR + q * PW) * 4u;
-                const float *from = src[cc] + (ok ? r : 0u);
-                if (VEC)
-                    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(to), "l"(from), "r"(ok ? 16 : 0)
-                                 : "memory");
-                else
-                    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(to), "l"(from), "r"(ok ? 4 : 0)
-                                 : "memory");
+            const uint32_t r0 = r_begin + (uint32_t)t * TR + (uint32_t)(lane * PW);
+            const uint32_t to0 = sbase + (uint32_t)((t % 3) * NC * TR + lane * PW) * 4u;
+            for (int cc = warp; cc < ncopy; cc += nwarps) {
+                const float *from = src[cc] + r0;
+                const uint32_t to = to0 + (uint32_t)((1 + cc) * TR) * 4u;
+#pragma unroll
+                for (int i = 0; i < PL; ++i) {
+                    const bool ok = r0 + (uint32_t)(i * 32 * PW) < r_end;
+                    if (VEC)
+                        asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(to + i * 512u),
+                                     "l"(ok ? from + i * 128 : src[cc]), "r"(ok ? 16 : 0)
+                                     : "memory");
+                    else
+                        asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(to + i * 128u),
+                                     "l"(ok ? from + i * 32 : src[cc]), "r"(ok ? 4 : 0)
+                                     : "memory");
+                }
             }
         }
         asm volatile("cp.async.commit_group;" ::: "memory");
     };
-    // this thread's pieces of the state columns of tile t: centred, zero past the end
+    // this lane's pieces of the state columns of tile t: centred, zero past the end (as the
+    // constant column is in the last tile)
     auto finish = [&](int t) {
-        const uint32_t r0 = r_begin + (uint32_t)t * TR;
-        float *tile = tiles + (size_t)(t % 3) * NC * TR;
-        for (int i = tid; i < nstate * NPC; i += nthr) {
-            const int cc = i / NPC, q = i % NPC;
-            const float c = r0 + (uint32_t)(q * PW) < r_end ? c0[cc] : 0.f;
-            float *v = tile + (1 + cc) * TR + q * PW;
-            if (VEC) {
-                float4 x = *reinterpret_cast<float4 *>(v);
-                x = make_float4(x.x - c, x.y - c, x.z - c, x.w - c);
-                *reinterpret_cast<float4 *>(v) = x;
-            } else {
-                *v -= c;
+        const uint32_t r0 = r_begin + (uint32_t)t * TR + (uint32_t)(lane * PW);
+        float *tile = tiles + (size_t)(t % 3) * NC * TR + lane * PW;
+        for (int cc = warp; cc < nstate; cc += nwarps) {
+            const float c1 = c0[cc];
+            float *v = tile + (1 + cc) * TR;
+#pragma unroll
+            for (int i = 0; i < PL; ++i) {
+                const float c = r0 + (uint32_t)(i * 32 * PW) < r_end ? c1 : 0.f;
+                if (VEC) {
+                    float4 x = *reinterpret_cast<float4 *>(v + i * 128);
+                    x = make_float4(x.x - c, x.y - c, x.z - c, x.w - c);
+                    *reinterpret_cast<float4 *>(v + i * 128) = x;
+                } else {
+                    v[i * 32] -= c;
+                }
             }
         }
-        for (int r = tid; r < TR; r += nthr) tile[r] = r0 + (uint32_t)r < r_end ? 1.f : 0.f;
+        if (t + 1 == ntiles)
+            for (int r = tid; r < TR; r += nthr)
+                tiles[(size_t)(t % 3) * NC * TR + r] = r_begin + (uint32_t)(t * TR + r) < r_end ? 1.f : 0.f;
     };
     // this warp's block (bi <= bj) and row group
     int bi = 0, bj = 0;
@@ -330,61 +342,59 @@ __global__ void __launch_bounds__(256) gram_reduce_kernel(const double *part, in
 
 // Normal equations A w = b of m unknowns and nt right-hand sides by the whole block
 // (256 threads): A [m + nt][LD] in shared memory, lower triangle, the right-hand sides as
-// rows m.. ; Jacobi scaling, right-looking Cholesky with the right-hand sides carried along
-// as further rows (their rows of L are the forward solutions), then one warp per
-// right-hand side for the back substitution. A column whose pivot vanishes is dropped:
-// its part of L is zero and its coefficient 0. w [nt][m] receives the solutions in the
-// unscaled basis; returns the number of dropped columns.
+// rows m.. ; Jacobi scaling, then the right-looking factorisation L D L^T with the right-hand
+// sides carried along as further rows, then one warp per right-hand side for the back
+// substitution. A column whose pivot vanishes is dropped: its part of L is zero and its
+// coefficient 0. w [nt][m] receives the solutions in the unscaled basis; returns the number
+// of dropped columns.
 //
-// Bound by the FP64 pipe (two lanes a clock and multiprocessor) and by the chain of
-// pivots: the reciprocal root of a pivot is an FP32 estimate and two Newton steps in FP64
-// instead of FP64 square root and division.
+// Bound by the FP64 pipe (two lanes a clock and multiprocessor) and by the chain of pivots,
+// so one warp alone computes a pivot's reciprocal, by Newton steps on an FP32 estimate
+// (scaled pivots lie in (1e-12, 1]), and nothing is divided or rooted in FP64. 28 unknowns:
+// 118 us with FP64 square roots and divisions and one thread's triangular solves.
 template <int LD>
 __device__ int solve_normal(double *A, int m, int nt, double *w, double *sc, int *drop)
 {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    auto rsqrt64 = [](double s) {
-        double y = (double)rsqrtf((float)s);
-        const double h = 0.5 * s;
-        y = fma(y, fma(-h * y, y, 0.5), y);
-        return fma(y, fma(-h * y, y, 0.5), y);
-    };
+    __shared__ double s_inv[2];
     for (int r = tid; r < m; r += blockDim.x) {
         const double d = A[r * LD + r];
         drop[r] = !(d > 0.0);
-        sc[r] = drop[r] ? 0.0 : 1.0 / sqrt(d);
+        sc[r] = drop[r] ? 0.0 : rsqrt(d);
     }
     __syncthreads();
     for (int r = tid >> 4; r < m + nt; r += blockDim.x >> 4)
         for (int c = tid & 15; c < m && c <= r; c += 16) A[r * LD + c] *= sc[c] * (r < m ? sc[r] : 1.0);
     __syncthreads();
     for (int j = 0; j < m; ++j) {
-        // every warp computes the pivot's reciprocal root; column j of L stays unscaled
-        // in A (A[r][j] = L[r][j] l) until the update below has used it
-        const double s = A[j * LD + j];
-        const bool out = drop[j] || !(s > 1e-12);
-        const double inv = out ? 0.0 : rsqrt64(s), inv2 = inv * inv;
-        for (int r = j + 1 + (tid >> 4); r < m + nt; r += blockDim.x >> 4) {
-            const double lr = A[r * LD + j] * inv2;
-            for (int c = j + 1 + (tid & 15); c < m && c <= r; c += 16) A[r * LD + c] = fma(-lr, A[c * LD + j], A[r * LD + c]);
+        if (warp == 0) {
+            const double s = A[j * LD + j];
+            const bool out = drop[j] || !(s > 1e-12);
+            double y = out ? 0.0 : (double)__frcp_rn((float)s);
+            y = fma(y, fma(-s, y, 1.0), y);
+            y = fma(y, fma(-s, y, 1.0), y);
+            __syncwarp();
+            if (lane == 0) {
+                s_inv[j & 1] = y;
+                drop[j] = out;
+                A[j * LD + j] = y;   // the reciprocal of the pivot
+            }
         }
         __syncthreads();
-        for (int r = j + 1 + tid; r < m + nt; r += blockDim.x) A[r * LD + j] *= inv;
-        if (tid == 0) {
-            drop[j] = out;
-            A[j * LD + j] = inv;   // the reciprocal of L[j][j]
+        const double inv = s_inv[j & 1];
+        for (int r = j + 1 + (tid >> 4); r < m + nt; r += blockDim.x >> 4) {
+            const double lr = -A[r * LD + j] * inv;
+            for (int c = j + 1 + (tid & 15); c < m && c <= r; c += 16) A[r * LD + c] = fma(lr, A[c * LD + j], A[r * LD + c]);
         }
-        // (the next column's update reads column j + 1 only)
+        __syncthreads();
     }
-    __syncthreads();
-    // L^T z = y, w = S z: lanes over the unknowns, two each
+    // L^T x = D^{-1} c, w = S x: lanes over the unknowns, two each
     for (int t = warp; t < nt; t += blockDim.x >> 5) {
         double y0 = lane < m ? A[(m + t) * LD + lane] : 0.0, y1 = lane + 32 < m ? A[(m + t) * LD + lane + 32] : 0.0;
         for (int i = m - 1; i >= 0; --i) {
-            const double yi = __shfl_sync(0xffffffffu, i >= 32 ? y1 : y0, i & 31);
-            const double z = yi * A[i * LD + i];   // 0 for a dropped column
+            const double z = __shfl_sync(0xffffffffu, i >= 32 ? y1 : y0, i & 31) * A[i * LD + i];   // 0 if dropped
             if (lane < i) y0 = fma(-A[i * LD + lane], z, y0);
-            if (lane + 32 < i) y1 = fma(-A[i * LD + lane + 32], z, y1);
+            if (i > 32 && lane + 32 < i) y1 = fma(-A[i * LD + lane + 32], z, y1);
             if (lane == (i & 31)) w[t * m + i] = z * sc[i];
         }
     }

@@ -36,6 +36,7 @@ struct LsqArgs {
     int nt = 1;                 // target columns sharing one normal matrix
     size_t targ_tstride = 0;    // floats between a group's targets
     size_t pred_tstride = 0;    // floats between a group's predictions
+    size_t coef_stride = 0;     // doubles between groups' coefficients (0: nt m)
     const float *centre = nullptr;   // [F] (poly2: [1]) centring state; null: path 0 of the group
 };
 
@@ -99,7 +100,7 @@ __global__ void __launch_bounds__(256) lsq_predict(LsqArgs a)
     __shared__ float cs[40 * 40];   // [nt][m], m + nt <= 40
     __shared__ float f0[40];        // path 0's state: the centring of the basis
     const int g = (int)(gridDim.y - 1 - blockIdx.y), nt = a.nt, m = a.m;   // from the last group back
-    const double *co = a.coef + (size_t)g * nt * m;
+    const double *co = a.coef + (size_t)g * (a.coef_stride ? a.coef_stride : (size_t)nt * m);
     const float *feat = a.feat0 + (size_t)g * a.feat_stride;
     for (int i = threadIdx.x; i < nt * m; i += blockDim.x) cs[i] = (float)co[i];
     const int nf = a.basis == CVA_BASIS_POLY2 ? 1 : a.F;
@@ -119,7 +120,7 @@ __global__ void __launch_bounds__(256) lsq_predict(LsqArgs a)
         float acc[8];
 #pragma unroll
         for (int u = 0; u < 8; ++u) acc[u] = u < tn ? cs[(t0 + u) * m] : 0.f;
-#pragma unroll 9
+#pragma unroll 4
         for (int f = 0; f < a.F; ++f) {
             const float x = __ldg(feat + (size_t)f * a.M + k) - f0[f];
 #pragma unroll
@@ -133,13 +134,15 @@ __global__ void __launch_bounds__(256) lsq_predict(LsqArgs a)
 // The linear-basis predictions of lsq_predict for 4 consecutive paths per thread:
 // 16-byte feature loads and prediction stores, the same FMA order per path (so the
 // same bits). Needs M, the strides and the base addresses to be multiples of 4
-// floats (checked by lsq_predict_launch).
+// floats (checked by lsq_predict_launch). TM: targets a thread carries at a time, 1 or 8
+// (one target leaves the registers to loads in flight).
+template <int TM>
 __global__ void __launch_bounds__(256) lsq_predict4(LsqArgs a)
 {
     __shared__ float cs[40 * 40];   // [nt][m], m + nt <= 40
     __shared__ float f0[40];
     const int g = (int)(gridDim.y - 1 - blockIdx.y), nt = a.nt, m = a.m;   // from the last group back
-    const double *co = a.coef + (size_t)g * nt * m;
+    const double *co = a.coef + (size_t)g * (a.coef_stride ? a.coef_stride : (size_t)nt * m);
     const float *feat = a.feat0 + (size_t)g * a.feat_stride;
     for (int i = threadIdx.x; i < nt * m; i += blockDim.x) cs[i] = (float)co[i];
     for (int f = threadIdx.x; f < a.F; f += blockDim.x) f0[f] = centre_of(a, feat, f);
@@ -147,21 +150,21 @@ __global__ void __launch_bounds__(256) lsq_predict4(LsqArgs a)
     const uint32_t k = 4u * (blockIdx.x * blockDim.x + threadIdx.x);
     if (k >= a.M) return;
     float *out = a.pred0 + (size_t)g * a.pred_stride + k;
-    for (int t0 = 0; t0 < nt; t0 += 8) {
-        const int tn = nt - t0 < 8 ? nt - t0 : 8;
-        float4 acc[8];
+    for (int t0 = 0; t0 < nt; t0 += TM) {
+        const int tn = nt - t0 < TM ? nt - t0 : TM;
+        float4 acc[TM];
 #pragma unroll
-        for (int u = 0; u < 8; ++u) {
+        for (int u = 0; u < TM; ++u) {
             const float c = u < tn ? cs[(t0 + u) * m] : 0.f;
             acc[u] = make_float4(c, c, c, c);
         }
-#pragma unroll 9
+#pragma unroll (TM == 1 ? 9 : 4)
         for (int f = 0; f < a.F; ++f) {
             const float4 v = __ldg(reinterpret_cast<const float4 *>(feat + (size_t)f * a.M + k));
             const float c0 = f0[f];
             const float x0 = v.x - c0, x1 = v.y - c0, x2 = v.z - c0, x3 = v.w - c0;
 #pragma unroll
-            for (int u = 0; u < 8; ++u)
+            for (int u = 0; u < TM; ++u)
                 if (u < tn) {
                     const float c = cs[(t0 + u) * m + 1 + f];
                     acc[u].x = fmaf(c, x0, acc[u].x);
@@ -182,7 +185,7 @@ cva_status lsq_predict_launch(const LsqArgs &a, int groups, cudaStream_t st)
                       a.pred_tstride % 4 == 0 && (reinterpret_cast<uintptr_t>(a.feat0) & 15u) == 0 &&
                       (reinterpret_cast<uintptr_t>(a.pred0) & 15u) == 0;
     if (wide)
-        lsq_predict4<<<dim3((unsigned)((a.M / 4 + 255) / 256), (unsigned)groups), 256, 0, st>>>(a);
+        (a.nt == 1 ? lsq_predict4<1> : lsq_predict4<8>)<<<dim3((unsigned)((a.M / 4 + 255) / 256), (unsigned)groups), 256, 0, st>>>(a);
     else
         lsq_predict<<<dim3((unsigned)((a.M + 255) / 256), (unsigned)groups), 256, 0, st>>>(a);
     CVA_CUDA_TRY(cudaGetLastError());
@@ -542,6 +545,24 @@ cva_status lsq_solve_normal_host(const double *gram, int F, int basis, const dou
     }
     if (dropped) *dropped = nd;
     return CVA_OK;
+}
+
+cva_status lsq_predict_groups(const float *feat0, size_t feat_stride, int F, uint64_t M, int groups, const double *coef,
+                              size_t coef_stride, float *pred0, size_t pred_stride, cudaStream_t st)
+{
+    LsqArgs a = {};
+    a.feat0 = feat0;
+    a.feat_stride = feat_stride;
+    a.pred0 = pred0;
+    a.pred_stride = pred_stride;
+    a.F = F;
+    a.m = F + 1;
+    a.basis = CVA_BASIS_LINEAR;
+    a.M = (uint32_t)M;
+    a.coef = const_cast<double *>(coef);
+    a.coef_stride = coef_stride;
+    a.nt = 1;
+    return lsq_predict_launch(a, groups, st);
 }
 
 cva_status lsq_predict_centred(const float *feat, int F, uint64_t M, int basis, const float *centre,
