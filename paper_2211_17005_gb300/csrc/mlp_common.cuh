@@ -510,12 +510,23 @@ __global__ void __launch_bounds__(256) mlp_stats_kernel(const float *feat, int F
     const float *x = feat + (size_t)d * date_stride + (size_t)f * M;
     const float c = __ldg(x);
     float s1 = 0.f, s2 = 0.f;
-    for (uint32_t r = 4u * tid; r < M; r += 4u * blockDim.x) {
-        const float4 v = __ldg(reinterpret_cast<const float4 *>(x + r));
+    auto add = [&](const float4 v) {
         const float a0 = v.x - c, a1 = v.y - c, a2 = v.z - c, a3 = v.w - c;
         s1 += (a0 + a1) + (a2 + a3);
         s2 += (a0 * a0 + a1 * a1) + (a2 * a2 + a3 * a3);
+    };
+    // one block per factor and date, so a thread's chain of loads sets the time: sixteen in
+    // flight ahead of the sums (2^20 paths: 467 us with one)
+    const uint32_t step = 4u * blockDim.x;
+    uint32_t r = 4u * tid;
+    for (; r + 15u * step < M; r += 16u * step) {
+        float4 v[16];
+#pragma unroll
+        for (int i = 0; i < 16; ++i) v[i] = __ldg(reinterpret_cast<const float4 *>(x + r + i * step));
+#pragma unroll
+        for (int i = 0; i < 16; ++i) add(v[i]);
     }
+    for (; r < M; r += step) add(__ldg(reinterpret_cast<const float4 *>(x + r)));
     double t1 = s1, t2 = s2;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
