@@ -12,7 +12,7 @@
 // rates of the swaps held at their base-curve par values).
 //
 // Three kernels over a range of outer paths:
-//   sim_kernel<ADJ>      the states, discount integrals and survival factors e^{-Lambda} of
+//   sim_kernel (adjoint) the states, discount integrals and survival factors e^{-Lambda} of
 //                        every date, and of every fine step the increments W and the
 //                        intensities before it;
 //   adj_price_kernel     the pricing at every date, which depends on that date's state only:

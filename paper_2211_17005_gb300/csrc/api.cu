@@ -98,6 +98,7 @@ void free_sim(Sim *s)
     cudaFree(s->d_mtm);
     cudaFree(s->d_targets);
     cudaFree(s->d_idx);
+    cudaFree(s->d_ckpt);
     cudaFree(s->d_const_img);
     cudaFree(s->d_lsq);
     cudaFree(s->d_alive_stats);
@@ -405,12 +406,29 @@ cva_status cva_nested_reference(cva_sim *sim, uint64_t seed, uint64_t k0, int pf
     if (copies < 1 || copies >= (1 << 24)) return fail(CVA_EINVAL, "nested: copies must be in [1, 2^24)");
     const cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
     const float *row = s.d_targets + ((size_t)pf * s.n + date) * s.M;
-    for (int b = 1; b <= copies; ++b) {
-        cva_status r = cva_simulate_twin(sim, seed, k0, date, (uint32_t)b, stream);
-        if (r == CVA_OK) r = accumulate_mean(out_dev, row, s.M, b == 1, b == copies, copies, st);
-        if (r != CVA_OK) return r;
+    // The copies share everything up to the branch date: the first one saves its running
+    // integrals there and the others start from it. (The run-time shapes, and a captured call
+    // before the buffer exists, run every copy from date 0; the bits are the same.)
+    bool restart = !s.generic && date > 0 && copies > 1;
+    if (restart && !s.d_ckpt) {
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        CVA_CUDA_TRY(cudaStreamIsCapturing(st, &cap));
+        if (cap != cudaStreamCaptureStatusNone) restart = false;
+        else if (cudaMalloc(&s.d_ckpt, s.M * (2 * (size_t)s.C * sizeof(float) + sizeof(double))) != cudaSuccess) {
+            (void)cudaGetLastError();
+            s.d_ckpt = nullptr;
+            restart = false;
+        }
     }
-    return CVA_OK;
+    cva_status r = CVA_OK;
+    for (int b = 1; b <= copies && r == CVA_OK; ++b) {
+        if (restart) (b == 1 ? s.save_date : s.start_date) = date;
+        r = cva_simulate_twin(sim, seed, k0, date, (uint32_t)b, stream);
+        s.save_date = -1;
+        s.start_date = 0;
+        if (r == CVA_OK) r = accumulate_mean(out_dev, row, s.M, b == 1, b == copies, copies, st);
+    }
+    return r;
 }
 
 cva_status cva_relative_rmse(const float *phi_dev, const float *ref_dev, uint64_t M, double *out2, void *stream)

@@ -106,6 +106,10 @@ struct Sim {
     // word; 0 (and no branch date) for the simulation itself
     int branch_date = 1 << 30;
     uint32_t branch = 0;
+    // nested reference: later copies start at the branch date, from the states of the first
+    // copy and the running integrals it saved there (compiled shapes)
+    int start_date = 0, save_date = -1;
+    float *d_ckpt = nullptr;       // [2C][M] Lambda and its compensation, then [M] doubles int r^0
 };
 
 // Device buffers of the adjoint sweep (adjoint.cuh).

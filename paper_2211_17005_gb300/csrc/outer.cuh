@@ -77,6 +77,8 @@ __device__ __forceinline__ float expm1_small(float x)
     return p * x;
 }
 
+enum class SimMode { plain, adjoint, restart };
+
 struct OuterArgs {
     uint32_t M, k0, seed_lo, seed_hi;
     int branch_step;                   // fine steps q >= branch_step draw with counter word `branch`
@@ -87,6 +89,12 @@ struct OuterArgs {
     const float *__restrict__ drift;   // [n*S][E]
     float *features, *disc, *thr, *expo, *mtm;
     const float *w_glob;               // device copy of the date-bucketed weights: wA [kMaxW], then wK [kMaxW]
+    // a run that starts at pricing date `start` > 0 takes the state there from features and
+    // ckpt, which a run with save_date = start has left: [2C][M] Lambda and its compensation,
+    // ckpt_I0 [M] int r^0
+    int start, save_date;
+    float *ckpt;
+    double *ckpt_I0;
     float *inc, *gpre;                 // the adjoint's: [n*S][F][M] increments, [n*S][C][M] intensities before a fine step
 };
 
@@ -101,20 +109,23 @@ struct OuterArgs {
 // as a single FMA): 352 instructions a step at 27 factors against 728 with one constant
 // load and one FMA per entry.
 //
-// ADJ: the adjoint's forward sweep, which keeps e^{-Lambda} in the place of the thresholds,
-// and the increments and intensities of every fine step.
+// Modes: adjoint, its forward sweep, which keeps e^{-Lambda} in the place of the thresholds,
+// and the increments and intensities of every fine step; restart, a run that starts at a
+// pricing date or saves what such a run needs (separate instances: their pointers would
+// spill the plain one's registers).
 //
 // Bound by instruction issue (Philox, logarithm, square root and sine-cosine of 14
 // Box-Muller pairs, the correlation): 2650 instructions a (path, step) at 27 factors and
 // 85% of the issue slots. Paper shape, 2^17 paths and 100 steps: 1.28 -> 1.11 ms against a
 // thread per path over all steps (96 registers, 7 to 14 warps a multiprocessor); 2^15
 // paths and 2500 steps 9.09 -> 6.51 ms; 2^14 paths and 100 steps 0.43 -> 0.18 ms.
-template <int E, int C, int CS, int NW, bool ADJ>
+template <int E, int C, int CS, int NW, SimMode MODE>
 __global__ void __launch_bounds__(32 * NW, NW == 8 ? 3 : 5) sim_kernel(OuterArgs a)
 {
     constexpr int F = 2 * E - 1 + CS;
     constexpr int NB = (F + 3) / 4, FP = (F + 1) / 2 * 2;
     constexpr int ME = (E + NW - 1) / NW, MC = (C + NW - 1) / NW;   // factors of a warp
+    constexpr bool ADJ = MODE == SimMode::adjoint, CKPT = MODE == SimMode::restart;
     constexpr int NS = F <= 8 ? 32 : 8;                             // fine steps at a time
     __shared__ float Ws[NS][F][32], R0[NS][32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -144,12 +155,42 @@ __global__ void __launch_bounds__(32 * NW, NW == 8 ? 3 : 5) sim_kernel(OuterArgs
         gam[i] = c_sim.gamma0[c];
         lam[i] = lamc[i] = 0.f;
     }
+    const int start = CKPT ? a.start : 0;
+    if (start > 0) {
+        const float *fe = a.features + (size_t)start * F * M + (live ? kl : 0u);
+        const uint32_t kr = live ? kl : 0u;
+        r0 = __ldg(fe);
+#pragma unroll
+        for (int i = 0; i < ME; ++i)
+            if (has_e(i)) {
+                const int e = warp + NW * i;
+                r[i] = __ldg(fe + (size_t)e * M);
+                if (e > 0) lchi[i] = __ldg(fe + (size_t)(E - 1 + e) * M);
+            }
+#pragma unroll
+        for (int i = 0; i < MC; ++i)
+            if (has_c(i)) {
+                const int c = warp + NW * i;
+                if (is_cir(i)) gam[i] = __ldg(fe + (size_t)(2 * E - 1 + c) * M);
+                lam[i] = a.ckpt[(size_t)c * M + kr];
+                lamc[i] = a.ckpt[(size_t)(C + c) * M + kr];
+            }
+        I0 = a.ckpt_I0[kr];
+    }
     // rows of a date this warp writes: the rate and the log FX rate of its first economy,
     // its first counterparty's intensity and threshold; the next ones follow NW rows apart
     float *pr = a.features + (size_t)warp * M + kl, *px = pr + (size_t)(E - 1) * M, *pg = pr + (size_t)(2 * E - 1) * M;
     float *pt = a.thr + (size_t)warp * M + kl, *pd = a.disc + kl;
+    int date = 0;
     auto write_date = [&]() {
         if (live) {
+            if (CKPT && date == a.save_date)
+#pragma unroll
+                for (int i = 0; i < MC; ++i)
+                    if (has_c(i)) {
+                        a.ckpt[(size_t)(warp + NW * i) * M + kl] = lam[i];
+                        a.ckpt[(size_t)(C + warp + NW * i) * M + kl] = lamc[i];
+                    }
 #pragma unroll
             for (int i = 0; i < ME; ++i)
                 if (has_e(i)) {
@@ -168,14 +209,24 @@ __global__ void __launch_bounds__(32 * NW, NW == 8 ? 3 : 5) sim_kernel(OuterArgs
         px += (size_t)F * M;
         pg += (size_t)F * M;
         pt += (size_t)C * M;
+        ++date;
     };
-    write_date();
-    if (warp == NW - 1 && live) *pd = 0.f;
-
-    const int steps = n * S;
-    const float *drow = a.drift;
+    const int steps = n * S, first = start * S;
+    const float *drow = a.drift + (size_t)first * E;
+    if (start > 0) {   // the dates up to the start are in place
+        pr += (size_t)(start + 1) * F * M;
+        px += (size_t)(start + 1) * F * M;
+        pg += (size_t)(start + 1) * F * M;
+        pt += (size_t)(start + 1) * C * M;
+        pd += (size_t)start * M;
+        date = start + 1;
+    } else {
+        write_date();
+        if (warp == NW - 1 && live) *pd = 0.f;
+    }
+    int jd = start;   // dates of int r^0 written so far
     int s = 0, sd = 0;   // sub-step of the next fine step (of the factors, of int r^0)
-    for (int q0 = 0; q0 < steps; q0 += NS) {
+    for (int q0 = first; q0 < steps; q0 += NS) {
 #pragma unroll 1
         for (int v = warp; v < NS && q0 + v < steps; v += NW) {
             const int q = q0 + v;
@@ -273,7 +324,11 @@ __global__ void __launch_bounds__(32 * NW, NW == 8 ? 3 : 5) sim_kernel(OuterArgs
                 if (++sd == S) {
                     sd = 0;
                     pd += M;
-                    if (live) *pd = (float)I0;
+                    ++jd;
+                    if (live) {
+                        *pd = (float)I0;
+                        if (CKPT && jd == a.save_date) a.ckpt_I0[kl] = I0;
+                    }
                 }
             }
     }
@@ -298,6 +353,7 @@ __global__ void __launch_bounds__(32 * NW, NW == 8 ? 3 : 5) sim_kernel(OuterArgs
 // with -D_h = Z_{h-1} expm1(x_h), which is what the chain of bond prices produces.
 struct PriceShape {
     int dates_per_block, splits;   // a period's dates in `splits` blocks of dates_per_block
+    int start = 0;                 // dates up to this one are priced already
 };
 
 // fn(LV) for the run-time LV in 1..G (0: nothing is live)
@@ -343,8 +399,9 @@ __global__ void __launch_bounds__(256, NPB == 1 ? 3 : 2) price_kernel(OuterArgs 
     const size_t M = a.M;
     const int n = c_sim.n, ppp = c_sim.ppp;
     const int p = (int)blockIdx.y / ps.splits, part = (int)blockIdx.y % ps.splits;
-    const int j0 = p * ppp + 1 + part * ps.dates_per_block;
-    const int j1 = min(min(j0 + ps.dates_per_block, (p + 1) * ppp + 1), n + 1);   // dates [j0, j1)
+    const int jp = p * ppp + 1 + part * ps.dates_per_block, j0 = max(jp, ps.start + 1);
+    const int j1 = min(min(jp + ps.dates_per_block, (p + 1) * ppp + 1), n + 1);   // dates [j0, j1)
+    if (j0 >= j1 && blockIdx.y > 0) return;
     const uint32_t k0 = blockIdx.x * 2u * (uint32_t)nthr + (uint32_t)tid, k1 = k0 + (uint32_t)nthr;
     const bool live0 = k0 < a.M, live1 = k1 < a.M;
     const uint32_t r0 = live0 ? k0 : 0u, r1 = live1 ? k1 : r0;   // paths read
@@ -480,7 +537,7 @@ static void outer_forget(const Sim *s)
 // fill the chip four times
 static PriceShape price_shape(uint64_t blocks, int ppp, int sms)
 {
-    PriceShape ps = {ppp, 1};
+    PriceShape ps = {ppp, 1, 0};
     while (blocks * ps.splits < 4u * (unsigned)sms && ps.dates_per_block > 1) {
         ps.dates_per_block = (ps.dates_per_block + 1) / 2;
         ps.splits = (ppp + ps.dates_per_block - 1) / ps.dates_per_block;
@@ -498,6 +555,10 @@ cva_status outer_launch(Sim &s, uint64_t seed, uint64_t k0, cudaStream_t st)
     args.M = (uint32_t)s.M;
     args.k0 = (uint32_t)k0;
     args.seed_lo = (uint32_t)seed;
+    args.start = s.start_date;
+    args.save_date = s.save_date;
+    args.ckpt = s.d_ckpt;
+    args.ckpt_I0 = reinterpret_cast<double *>(s.d_ckpt + 2 * (size_t)C * s.M);
     args.branch_step = s.branch_date <= s.n ? s.branch_date * s.S : INT_MAX;
     args.branch = s.branch;
     args.seed_hi = (uint32_t)(seed >> 32);
@@ -535,24 +596,33 @@ cva_status outer_launch(Sim &s, uint64_t seed, uint64_t k0, cudaStream_t st)
     CVA_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     const unsigned sgrid = (args.M + 31u) / 32u;
     const bool wide = s.tune_sim_block ? s.tune_sim_block == 128 : sgrid < 2u * (unsigned)sms;
-    if (wide) sim_kernel<E, C, CS, 8, false><<<sgrid, 256, 0, st>>>(args);
-    else sim_kernel<E, C, CS, 4, false><<<sgrid, 128, 0, st>>>(args);
+    const bool restart = s.start_date > 0 || s.save_date >= 0;
+    if (restart && wide) sim_kernel<E, C, CS, 8, SimMode::restart><<<sgrid, 256, 0, st>>>(args);
+    else if (restart) sim_kernel<E, C, CS, 4, SimMode::restart><<<sgrid, 128, 0, st>>>(args);
+    else if (wide) sim_kernel<E, C, CS, 8, SimMode::plain><<<sgrid, 256, 0, st>>>(args);
+    else sim_kernel<E, C, CS, 4, SimMode::plain><<<sgrid, 128, 0, st>>>(args);
     CVA_CUDA_TRY(cudaGetLastError());
     if (s.ev[1]) CVA_CUDA_TRY(cudaEventRecord(s.ev[1], st));
     if (s.tune_price_pf == 4) {   // every portfolio per 128-path tile on the tensor cores
-        using PT = PriceTc<E, G, NPF, C>;
+        constexpr int bytes = price_tc_bytes<E, NPF, C, G>();
         static bool attr[64] = {};
         if (!attr[dev]) {
             if (capturing) return fail(CVA_EINVAL, "price: run once before capturing (kernel attribute)");
             CVA_CUDA_TRY(cudaFuncSetAttribute(price_tc_kernel<E, C, CS, G, NPF>,
-                                              cudaFuncAttributeMaxDynamicSharedMemorySize, PT::bytes));
+                                              cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
             attr[dev] = true;
         }
-        const uint32_t tiles = (args.M + 127u) / 128u;
-        const uint64_t items = (uint64_t)tiles * (uint64_t)(s.n + 1);
-        const unsigned grid =
-            (unsigned)std::min<uint64_t>((items + kPriceSlots - 1) / kPriceSlots, (uint64_t)sms);
-        price_tc_kernel<E, C, CS, G, NPF><<<grid, 128 * kPriceSlots, PT::bytes, st>>>(args, tiles);
+        // at least six path tiles per slot and part of a period, so that the last round of
+        // tiles is a small part of them
+        const uint32_t tiles = (args.M + 127u) / 128u, slots = (uint32_t)sms * kPriceSlots;
+        const unsigned periods = (unsigned)((s.n + s.ppp - 1) / s.ppp);
+        PriceShape ps = {s.ppp, 1, s.start_date};
+        while ((uint64_t)tiles * ps.splits < 6ull * slots && ps.dates_per_block > 1) {
+            ps.dates_per_block = (ps.dates_per_block + 1) / 2;
+            ps.splits = (s.ppp + ps.dates_per_block - 1) / ps.dates_per_block;
+        }
+        const dim3 tgrid(std::min((tiles + kPriceSlots - 1) / kPriceSlots, (uint32_t)sms), periods * (unsigned)ps.splits);
+        price_tc_kernel<E, C, CS, G, NPF><<<tgrid, 128 * kPriceSlots, bytes, st>>>(args, tiles, ps);
         CVA_CUDA_TRY(cudaGetLastError());
         if (!capturing) CVA_CUDA_TRY(cudaEventRecord(t_last[dev], st));
         return CVA_OK;
@@ -562,7 +632,8 @@ cva_status outer_launch(Sim &s, uint64_t seed, uint64_t k0, cudaStream_t st)
     const int ppb = s.tune_price_pf ? (NPF % s.tune_price_pf == 0 ? s.tune_price_pf : 1)
                                     : (NPF % 3 == 0 ? 3 : NPF % 2 == 0 ? 2 : 1);
     const unsigned tiles = (args.M + 2 * pb - 1) / (2 * pb), periods = (unsigned)((s.n + s.ppp - 1) / s.ppp);
-    const PriceShape ps = price_shape((uint64_t)tiles * periods * (NPF / ppb), s.ppp, sms);
+    PriceShape ps = price_shape((uint64_t)tiles * periods * (NPF / ppb), s.ppp, sms);
+    ps.start = s.start_date;
     const dim3 pgrid(tiles, periods * (unsigned)ps.splits, (unsigned)(NPF / ppb));
     const size_t psmem = (size_t)E * ppb * C * 2 * G * sizeof(f32x2);
     static_assert(E * 3 * C * 2 * G * sizeof(f32x2) <= 48 * 1024, "portfolio weights exceed the default shared-memory limit");
@@ -651,8 +722,8 @@ cva_status adjoint_launch(Sim &s, AdjBuffers &b, uint64_t seed, uint64_t k0, uin
         CVA_CUDA_TRY(upload_consts(s, st));
         t_owner[dev] = &s;
     }
-    if (rblocks < 2u * (unsigned)sms) sim_kernel<E, C, CS, 8, true><<<rblocks, 256, 0, st>>>(o);
-    else sim_kernel<E, C, CS, 4, true><<<rblocks, 128, 0, st>>>(o);
+    if (rblocks < 2u * (unsigned)sms) sim_kernel<E, C, CS, 8, SimMode::adjoint><<<rblocks, 256, 0, st>>>(o);
+    else sim_kernel<E, C, CS, 4, SimMode::adjoint><<<rblocks, 128, 0, st>>>(o);
     CVA_CUDA_TRY(cudaGetLastError());
     const dim3 pgrid(tiles, periods * (unsigned)ps.splits);
     const size_t psmem = (size_t)E * C * 2 * G * sizeof(f32x2) + (size_t)E * 128 * 16;
