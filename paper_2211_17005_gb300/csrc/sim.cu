@@ -432,7 +432,10 @@ static cudaError_t launch_inner_t(InnerArgs &args, int tune, int sms, int dev, c
     // tiles of 8, 16, 32 paths) replaces the first rule as far as it fits.
     auto threads_of = [&](int lg) {
         const uint64_t want = (uint64_t)args.N << lg;
-        return want >= 512 ? 512 : want >= 256 ? 256 : 128;
+        const int t = want >= 512 ? 512 : want >= 256 ? 256 : 128;
+        // half the queues where that lets a second block in
+        const auto two = [&](int threads) { return inner_smem(lg, threads, C, args.n, args.NPF, packed) <= 108 * 1024; };
+        return t == 512 && !two(512) && two(256) ? 256 : t;
     };
     auto smem_of = [&](int lg) { return inner_smem(lg, threads_of(lg), C, args.n, args.NPF, packed); };
     int lg = tune == 2 ? 3 : tune == 4 ? 4 : 5;
