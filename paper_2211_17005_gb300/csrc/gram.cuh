@@ -43,7 +43,7 @@ __host__ __device__ constexpr int tri_index(int cols, int i, int j) { return i *
 // for 128 FMAs. FP32 runs of at most 256 rows a lane are reduced over the lanes by a
 // butterfly (five more roundings) and added in FP64.
 //
-// Bound by the FMA issue (640 multiply-adds a row at 29 columns; 528 are needed) and the
+// Bound by the FMA issue (528 multiply-adds a row at 29 columns; 435 are needed) and the
 // read of the data, about equal. The tiles were transposed to rows before, with eight-way
 // bank conflicts in the copies and in the centring pass: 29 columns of 2^17 rows at 99
 // dates took 1276 us.
@@ -175,13 +175,23 @@ __global__ void __launch_bounds__(MAXT, MINB) gram_kernel(GramArgs a)
             float2 x[8];
 #pragma unroll
             for (int u = 0; u < 8; ++u) x[u] = *reinterpret_cast<const float2 *>(px + u * TR + it * 64);
+            if (bi == bj) {   // a diagonal block: its upper triangle, of its own columns
 #pragma unroll
-            for (int v = 0; v < 8; ++v) {
-                const float2 y = *reinterpret_cast<const float2 *>(py + v * TR + it * 64);
+                for (int v = 0; v < 8; ++v) {
 #pragma unroll
-                for (int u = 0; u < 8; ++u) acc[u][v] = fmaf(x[u].x, y.x, acc[u][v]);
+                    for (int u = 0; u <= v; ++u) acc[u][v] = fmaf(x[u].x, x[v].x, acc[u][v]);
 #pragma unroll
-                for (int u = 0; u < 8; ++u) acc[u][v] = fmaf(x[u].y, y.y, acc[u][v]);
+                    for (int u = 0; u <= v; ++u) acc[u][v] = fmaf(x[u].y, x[v].y, acc[u][v]);
+                }
+            } else {
+#pragma unroll
+                for (int v = 0; v < 8; ++v) {
+                    const float2 y = *reinterpret_cast<const float2 *>(py + v * TR + it * 64);
+#pragma unroll
+                    for (int u = 0; u < 8; ++u) acc[u][v] = fmaf(x[u].x, y.x, acc[u][v]);
+#pragma unroll
+                    for (int u = 0; u < 8; ++u) acc[u][v] = fmaf(x[u].y, y.y, acc[u][v]);
+                }
             }
             if (++run == 128) {
                 run = 0;
