@@ -106,10 +106,10 @@ __global__ void __launch_bounds__(256) alive_stats_kernel(AliveArgs a)
     const int p = tid & (PT - 1), c = tid >> lg;
     const uint32_t kl = tile0 + (uint32_t)p;
     const bool live = c < C && kl < M;
-    for (int i = 0; i < n; ++i) {
-        dq[i * nthr] = 0.f;
-        dn[i * nthr] = 0;
-    }
+    for (uint32_t i = tid; i < (uint32_t)(n * nthr * 4) / 16; i += nthr)   // (whole warps: a multiple of 128 bytes a date)
+        reinterpret_cast<uint4 *>(smem + sh.dq)[i] = make_uint4(0u, 0u, 0u, 0u);
+    for (uint32_t i = tid; i < (uint32_t)(n * nthr * 2) / 16; i += nthr)
+        reinterpret_cast<uint4 *>(smem + sh.dn)[i] = make_uint4(0u, 0u, 0u, 0u);
     for (int i = tid; i < n * NP; i += nthr) pair[i] = 0;
     for (int i = tid; i < n << lg; i += nthr) {
         const uint32_t k = tile0 + (uint32_t)(i & (PT - 1));
@@ -142,16 +142,22 @@ __global__ void __launch_bounds__(256) alive_stats_kernel(AliveArgs a)
                 list[found * nthr] = (uint8_t)l;
                 ++found;
             }
-            if (ic < n) dn[ic * nthr] += 1;
         }
         for (int t = 0; t < found; ++t) {
             const uint8_t *js = row + list[t * nthr] * C;
             const int ic = js[c];
             float v[C], later = 0.f;
             int jd[C];
+            if constexpr (C == 8) {   // the draw's steps in one load
+                const uint2 w = *reinterpret_cast<const uint2 *>(js);
+#pragma unroll
+                for (int d = 0; d < 8; ++d) jd[d] = ((d < 4 ? w.x : w.y) >> (8 * (d & 3))) & 255u;
+            } else {
+#pragma unroll
+                for (int d = 0; d < C; ++d) jd[d] = js[d];
+            }
 #pragma unroll
             for (int d = 0; d < C; ++d) {
-                jd[d] = js[d];
                 v[d] = jd[d] > ic && jd[d] <= n ? __ldg(a.expo + ((size_t)jd[d] * C + d) * M + kl) : 0.f;
             }
 #pragma unroll
@@ -160,7 +166,10 @@ __global__ void __launch_bounds__(256) alive_stats_kernel(AliveArgs a)
                 if (d > c && j < n) atomicAdd(&pair[j * NP + c * (2 * C - c - 1) / 2 + (d - c - 1)], 1);
                 later += v[d];
             }
-            if (ic < n) dq[ic * nthr] += later;
+            if (ic < n) {
+                dq[ic * nthr] += later;
+                dn[ic * nthr] += 1;
+            }
 #pragma unroll
             for (int d = 0; d < C; ++d)
                 if (jd[d] > ic && jd[d] < n) dq[jd[d] * nthr] -= v[d];
@@ -169,13 +178,22 @@ __global__ void __launch_bounds__(256) alive_stats_kernel(AliveArgs a)
     __syncthreads();
     float q = 0.f;
     uint32_t defaults = 0u;
+#pragma unroll 4
     for (int i = 1; i < n; ++i) {
         q += dq[i * nthr];
         defaults += dn[i * nthr];
+        dq[i * nthr] = live ? q * binv[(i << lg) + p] : 0.f;
         if (live) a.dstat[((size_t)i * C + c) * M + kl] = (float)defaults;
-        float s = live ? q * binv[(i << lg) + p] : 0.f;
-        for (int o = PT / 2; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-        if (p == 0 && c < C) a.qsum[((size_t)i * NQ + NP + c) * a.nblk + blockIdx.x] = s;
+    }
+    __syncthreads();
+    // q_c over the tile's paths: a thread per (date, c), which starts at a path of its own so
+    // that a warp's reads spread over the banks
+    for (int t = tid; t < (n - 1) * C; t += nthr) {
+        const int i = 1 + t / C, d = t % C;
+        const float *src = reinterpret_cast<const float *>(smem + sh.dq) + i * nthr + (d << lg);
+        float s = 0.f;
+        for (int u = 0; u < PT; ++u) s += src[(u + tid) & (PT - 1)];
+        a.qsum[((size_t)i * NQ + NP + d) * a.nblk + blockIdx.x] = s;
     }
     for (int t = tid; t < NP; t += nthr) {
         int s = 0;
