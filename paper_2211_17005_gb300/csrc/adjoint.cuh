@@ -283,32 +283,80 @@ __global__ void __launch_bounds__(32 * NW) adj_reverse_kernel(AdjSplitArgs a, in
     for (int i = 0; i < ME; ++i) rb[i] = lb[i] = pf[i] = psr[i] = psx[i] = 0.f;
 #pragma unroll
     for (int i = 0; i < MC; ++i) gb[i] = Lb[i] = Vn[i] = pk[i] = pt[i] = pn[i] = 0.f;
-    for (int j = n; j >= 1; --j) {
-        // what the pricing at t_j adds, and the survival terms
-        const float *rin = a.rbin + (size_t)(j - 1) * E * M + kr, *lin = a.lbin + (size_t)(j - 1) * E * M + kr;
-        const float *sv = a.surv + (size_t)j * C * M + kr, *vv = a.V + (size_t)j * C * M + kr;
+    // what a fine step and a date read, requested one ahead of their use: nothing in the
+    // recursions' inputs depends on them, and a step's own work is short
+    float We[ME] = {}, Wx[ME] = {}, Wc[MC] = {}, gq[MC] = {}, ri[ME] = {}, li[ME] = {}, sv[MC] = {}, vv[MC] = {}, ibn = 0.f,
+          lsn = 0.f;
+    auto load_step = [&](int q) {
+        const float *W = a.inc + (size_t)q * F * M + kr, *g = a.gpre + (size_t)q * C * M + kr;
 #pragma unroll
         for (int i = 0; i < ME; ++i)
             if (has_e(i)) {
                 const int e = warp + NW * i;
-                rb[i] += __ldg(rin + (size_t)e * M);
-                if (e > 0) lb[i] += __ldg(lin + (size_t)e * M);
+                We[i] = __ldg(W + (size_t)e * M);
+                Wx[i] = e > 0 ? __ldg(W + (size_t)(E - 1 + e) * M) : 0.f;
+            }
+#pragma unroll
+        for (int i = 0; i < MC; ++i)
+            if (has_c(i)) {
+                const int c = warp + NW * i;
+                gq[i] = __ldg(g + (size_t)c * M);
+                Wc[i] = NW * (i + 1) <= CS || c < CS ? __ldg(W + (size_t)(2 * E - 1 + c) * M) : 0.f;
+            }
+    };
+    auto load_date = [&](int j) {
+        const float *rin = a.rbin + (size_t)(j - 1) * E * M + kr, *lin = a.lbin + (size_t)(j - 1) * E * M + kr;
+        const float *s = a.surv + (size_t)j * C * M + kr, *v = a.V + (size_t)j * C * M + kr;
+#pragma unroll
+        for (int i = 0; i < ME; ++i)
+            if (has_e(i)) {
+                const int e = warp + NW * i;
+                ri[i] = __ldg(rin + (size_t)e * M);
+                li[i] = e > 0 ? __ldg(lin + (size_t)e * M) : 0.f;
             }
         if (warp == 0) {
-            Ib += __ldg(a.ibin + (size_t)(j - 1) * M + kr);
-            lbs += __ldg(lin);
+            ibn = __ldg(a.ibin + (size_t)(j - 1) * M + kr);
+            lsn = __ldg(lin);
         }
 #pragma unroll
         for (int i = 0; i < MC; ++i)
             if (has_c(i)) {
                 const int c = warp + NW * i;
-                const float v = __ldg(vv + (size_t)c * M);
-                Lb[i] += __ldg(sv + (size_t)c * M) * (v - Vn[i]);
-                Vn[i] = v;
+                sv[i] = __ldg(s + (size_t)c * M);
+                vv[i] = __ldg(v + (size_t)c * M);
             }
+    };
+    load_date(n);
+    load_step(n * S - 1);
+    for (int j = n; j >= 1; --j) {
+        // what the pricing at t_j adds, and the survival terms
+#pragma unroll
+        for (int i = 0; i < ME; ++i) {
+            rb[i] += ri[i];
+            lb[i] += li[i];
+        }
+        Ib += ibn;
+        lbs += lsn;
+#pragma unroll
+        for (int i = 0; i < MC; ++i) {
+            Lb[i] += sv[i] * (vv[i] - Vn[i]);
+            Vn[i] = vv[i];
+        }
+        if (j > 1) load_date(j - 1);
         for (int s = S - 1; s >= 0; --s) {   // Euler sub-steps of (t_{j-1}, t_j], in reverse
             const int q = (j - 1) * S + s;
-            const float *W = a.inc + (size_t)q * F * M + kr, *gp_ = a.gpre + (size_t)q * C * M + kr;
+            float we[ME], wx[ME], wc[MC], g_[MC];
+#pragma unroll
+            for (int i = 0; i < ME; ++i) {
+                we[i] = We[i];
+                wx[i] = Wx[i];
+            }
+#pragma unroll
+            for (int i = 0; i < MC; ++i) {
+                wc[i] = Wc[i];
+                g_[i] = gq[i];
+            }
+            if (q > 0) load_step(q - 1);
             const float2 *dd = a.ddrift + (size_t)q * E;
 #pragma unroll
             for (int i = 0; i < ME; ++i)
@@ -316,12 +364,11 @@ __global__ void __launch_bounds__(32 * NW) adj_reverse_kernel(AdjSplitArgs a, in
                     const int e = warp + NW * i;
                     const float2 d2 = __ldg(dd + e);
                     pf[i] += rb[i] * d2.x;
-                    psr[i] += rb[i] * fmaf(sqds, __ldg(W + (size_t)e * M), d2.y);
+                    psr[i] += rb[i] * fmaf(sqds, we[i], d2.y);
                     float v = rb[i] - rb[i] * c_sim.hw_a_ds[e];
                     if (e > 0) {
                         const float sx = __ldg(a.sig + E + e), sr = __ldg(a.sig + e);
-                        psx[i] += lb[i] * fmaf(sqds, __ldg(W + (size_t)(E - 1 + e) * M), -sx * ds)
-                                  - rb[i] * __ldg(a.rho + e) * sr * ds;
+                        psx[i] += lb[i] * fmaf(sqds, wx[i], -sx * ds) - rb[i] * __ldg(a.rho + e) * sr * ds;
                         v -= lb[i] * ds;
                     } else {
                         v += fmaf(lbs, ds, Ib * ds);
@@ -332,16 +379,15 @@ __global__ void __launch_bounds__(32 * NW) adj_reverse_kernel(AdjSplitArgs a, in
             for (int i = 0; i < MC; ++i)
                 if (has_c(i)) {
                     const int c = warp + NW * i;
-                    const float g = __ldg(gp_ + (size_t)c * M), gp = fmaxf(g, 0.f);
+                    const float g = g_[i], gp = fmaxf(g, 0.f);
                     float gbn = gb[i];
                     if (NW * (i + 1) <= CS || c < CS) {
-                        const float Wc = __ldg(W + (size_t)(2 * E - 1 + c) * M);
                         const float kap = __ldg(a.sig + 2 * E + c), th = __ldg(a.sig + 2 * E + C + c);
                         pk[i] += gb[i] * (th - gp) * ds;
                         pt[i] += gb[i] * kap * ds;
-                        pn[i] += gb[i] * sqrtf(gp) * sqds * Wc;
+                        pn[i] += gb[i] * sqrtf(gp) * sqds * wc[i];
                         if (g > 0.f)
-                            gbn = gb[i] * (1.f - c_sim.cir_kds[c] + c_sim.cir_nu_sqds[c] * Wc * 0.5f * rsqrtf(g));
+                            gbn = gb[i] * (1.f - c_sim.cir_kds[c] + c_sim.cir_nu_sqds[c] * wc[i] * 0.5f * rsqrtf(g));
                     }
                     if (g > 0.f) gbn += Lb[i] * ds;
                     gb[i] = gbn;

@@ -734,7 +734,7 @@ cva_status adjoint_launch(Sim &s, AdjBuffers &b, uint64_t seed, uint64_t k0, uin
     } else {
         adj_price_kernel<E, C, CS, G, true><<<pgrid, 128, psmem, st>>>(a, ps);
         CVA_CUDA_TRY(cudaGetLastError());
-        adj_reverse_kernel<E, C, CS, 4><<<rblocks, 128, 0, st>>>(a, ps.splits);
+        adj_reverse_kernel<E, C, CS, 8><<<rblocks, 256, 0, st>>>(a, ps.splits);
         CVA_CUDA_TRY(cudaGetLastError());
     }
     CVA_CUDA_TRY(cudaEventRecord(t_last[dev], st));
