@@ -344,14 +344,12 @@ struct WNetT {
     }
 
     // ---- epilogues: thread = (row, half), 64 hidden columns each ----
-    // H1 = relu(D + b1) into B; the mask of h1 > 0 in m1
-    __device__ void epi1(uint32_t (&m1)[2]) const
+    // h1 = relu(D + b1), into B and left in v
+    __device__ void epi1(float (&v)[64]) const
     {
         unsigned char *b = smem + L::sB;
         const float4 *b1 = reinterpret_cast<const float4 *>(vec + L::vb1 + 64 * half);
-        float v[64];
         umma::tmem_ld64(taddr(L::cD + 64u * half), v);
-        m1[0] = m1[1] = 0u;
 #pragma unroll
         for (int g = 0; g < 16; ++g) {
             const float4 c = b1[g];
@@ -361,9 +359,15 @@ struct WNetT {
             v[4 * g + 3] = fmaxf(v[4 * g + 3] + c.w, 0.f);
         }
 #pragma unroll
-        for (int i = 0; i < 64; ++i) m1[i / 32] |= (v[i] > 0.f ? 1u : 0u) << (i % 32);
-#pragma unroll
         for (int g = 0; g < 8; ++g) *reinterpret_cast<uint4 *>(b + wrow_off(row, 64 * half + 8 * g, L::wB)) = pack8(v + 8 * g);
+    }
+
+    // the mask of h1 > 0
+    static __device__ void mask(const float (&v)[64], uint32_t (&m1)[2])
+    {
+        m1[0] = m1[1] = 0u;
+#pragma unroll
+        for (int i = 0; i < 64; ++i) m1[i / 32] |= (v[i] > 0.f ? 1u : 0u) << (i % 32);
     }
 
     // h2 = relu(D + b2) of this thread's 64 columns in place; returns their share of
@@ -401,17 +405,15 @@ struct WNetT {
     }
 
     // output, loss derivative and the output-layer backward of this thread's row:
-    // dH2 = dout w3 (h2 > 0) into A; column sums of h2 dout over the warp's rows
-    // (dw3) and, in the first warpgroup, of dout (db3) and dpred (dmu)
-    __device__ void out_back2(int pos, float y, float inv_batch, float *gsl) const
+    // dH2 = dout w3 (h2 > 0) into A; h2 is left in v
+    __device__ void out_back2(int pos, float y, float inv_batch, float (&v)[64], float &dout, float &dpred) const
     {
         unsigned char *a = smem + L::sA;
         const float4 *w3 = reinterpret_cast<const float4 *>(vec + L::vw3 + 64 * half);
-        float v[64];
         const float out = zeta(layer2(v));
         const float pred = (pos ? fmaxf(out, 0.f) : out) + vec[L::vmu];
-        const float dpred = 2.f * (pred - y) * inv_batch;
-        const float dout = pos ? (out > 0.f ? dpred : 0.f) : dpred;
+        dpred = 2.f * (pred - y) * inv_batch;
+        dout = pos ? (out > 0.f ? dpred : 0.f) : dpred;
 #pragma unroll
         for (int g = 0; g < 8; ++g) {
             const float4 w0 = w3[2 * g], w1 = w3[2 * g + 1];
@@ -421,6 +423,12 @@ struct WNetT {
             for (int i = 0; i < 8; ++i) d[i] = v[8 * g + i] > 0.f ? dout * wv[i] : 0.f;
             *reinterpret_cast<uint4 *>(a + wrow_off(row, 64 * half + 8 * g, L::wA)) = pack8(d);
         }
+    }
+
+    // column sums of h2 dout over the warp's rows (dw3) and, in the first warpgroup, of
+    // dout (db3) and dpred (dmu)
+    __device__ void out_sums(float (&v)[64], float dout, float dpred, float *gsl) const
+    {
 #pragma unroll
         for (int i = 0; i < 64; ++i) v[i] *= dout;
         const float2 cs = column_sums64(v, lane);
@@ -453,8 +461,9 @@ struct WNetT {
     __device__ bool forward12(uint32_t (&m1)[2], bool in_ok, Side side)
     {
         if (!mma([&] { gemm_rows(L::cD, L::sB, L::wB, L::cX, L::sW1, kIn, L::U); }, in_ok, side)) return false;
-        epi1(m1);
-        return mma([&] { gemm_rows(L::cD, L::sB, L::wB, 0, L::sW2, L::U, L::U); });
+        float v[64];
+        epi1(v);
+        return mma([&] { gemm_rows(L::cD, L::sB, L::wB, 0, L::sW2, L::U, L::U); }, true, [&] { mask(v, m1); });
     }
 
     // constant columns of B: ones after H1 (first warpgroup) and after X (second)
@@ -602,8 +611,10 @@ __global__ void __launch_bounds__(kWThreads, 1) wide_train_kernel(WTrainArgs a, 
                 if (has_next) n.prefetch(&tm, a.targ, a.F, next);
             });
             if (ok) {
-                n.out_back2(a.pos, y, inv_batch, my_gsl);
-                ok = n.mma([&] { n.gemm_w2t(WL::cD); });
+                // the output layer's column sums run while the tensor core works on GEMM3
+                float v[64], dout, dpred;
+                n.out_back2(a.pos, y, inv_batch, v, dout, dpred);
+                ok = n.mma([&] { n.gemm_w2t(WL::cD); }, true, [&] { n.out_sums(v, dout, dpred, my_gsl); });
             }
             if (ok) {
                 n.back1(m1);
