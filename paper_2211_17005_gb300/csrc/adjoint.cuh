@@ -58,7 +58,9 @@ __global__ void __launch_bounds__(128) adj_price_kernel(AdjSplitArgs a, PriceSha
     extern __shared__ __align__(16) unsigned char adj_smem[];
     f32x2 *w_s = reinterpret_cast<f32x2 *>(adj_smem);            // [E][C][2 LV] (-wA, -wK), doubled
     f32x2 *rf_s = w_s + E * C * 2 * G;                           // [E][NT] adjoints of the fixings
-    float *par_s = reinterpret_cast<float *>(rf_s + E * NT);     // [2E][NT] parameter adjoints, both paths
+    f32x2 *fix_s = rf_s + E * NT;                                // [E][NT] running coupons at the fixing
+    float4 *tab_s = reinterpret_cast<float4 *>(fix_s + E * NT);  // [2][E][LV] the date's bond tables, their derivatives
+    float *par_s = reinterpret_cast<float *>(tab_s + 2 * E * G); // [2E][NT] parameter adjoints, both paths
     __shared__ double j_s[NT];
     const int tid = threadIdx.x;
     const size_t M = a.M;
@@ -73,7 +75,7 @@ __global__ void __launch_bounds__(128) adj_price_kernel(AdjSplitArgs a, PriceSha
         if (live0) row[k0] = x;
         if (live1) row[k1] = y;
     };
-    double J = 0.0;
+    SumPair J = {0.f, 0.f};
     if (REV)
         for (int e = 0; e < E; ++e) {
             rf_s[e * NT + tid] = pack2(0.f, 0.f);
@@ -98,41 +100,51 @@ __global__ void __launch_bounds__(128) adj_price_kernel(AdjSplitArgs a, PriceSha
                 const float w = q < LV ? __ldg(a.w_glob + wrow + q) : __ldg(a.w_glob + kMaxW + wrow + q - LV);
                 w_s[i] = pack2(-w, -w);
             }
-            __syncthreads();
-            const float *ffix = a.features + (size_t)(p * ppp) * F * M;   // state at the last reset
             const float2 *fx = a.fix + (size_t)p * E;
+            {   // 1/ZC_{t_-}(t_+) - 1, which the period's dates share
+                const float *ffix = a.features + (size_t)(p * ppp) * F * M;   // state at the last reset
+#pragma unroll 2
+                for (int e = 0; e < E; ++e) {
+                    const float2 f2 = __ldg(fx + e);
+                    fix_s[e * NT + tid] = pack2(expm1f(fmaf(f2.y, __ldg(ffix + (size_t)e * M + r0), -f2.x)),
+                                                expm1f(fmaf(f2.y, __ldg(ffix + (size_t)e * M + r1), -f2.x)));
+                }
+            }
             // bond prices of economy e (price_kernel's): X holds -D, then Z; em[g] = expm1(x_g)
-            auto bonds = [&](int e, const float4 *tab, f32x2 re, f32x2 rfix, f32x2 (&X)[2 * LV], f32x2 (&em)[LV], f32x2 &fixm1) {
-                const float2 f2 = __ldg(fx + e), r = unpack2(re), rf = unpack2(rfix);
-                const float4 tp = __ldg(tab);
+            auto bonds = [&](const float4 *tab, f32x2 re, f32x2 fixm1, f32x2 (&X)[2 * LV], f32x2 (&em)[LV]) {
+                const float2 r = unpack2(re), fm = unpack2(fixm1);
+                const float4 tp = tab[0];
                 const float z0 = expf(fmaf(-tp.y, r.x, tp.x)), z1 = expf(fmaf(-tp.y, r.y, tp.x));
-                const float m0 = expm1f(fmaf(f2.y, rf.x, -f2.x)), m1 = expm1f(fmaf(f2.y, rf.y, -f2.x));
-                fixm1 = pack2(m0, m1);
-                X[0] = pack2(-(z0 * m0), -(z1 * m1));
+                X[0] = pack2(-(z0 * fm.x), -(z1 * fm.y));
                 X[LV] = pack2(z0, z1);
                 em[0] = pack2(0.f, 0.f);
 #pragma unroll
                 for (int g = 1; g < LV; ++g) {
-                    const float4 t4 = __ldg(tab + g);
+                    const float4 t4 = tab[g];
                     em[g] = expm1_small2(fma2(pack2(-t4.w, -t4.w), re, pack2(t4.z, t4.z)));
                     X[g] = mul2(X[LV + g - 1], em[g]);
                     X[LV + g] = fma2(X[LV + g - 1], em[g], X[LV + g - 1]);
                 }
             };
             for (int j = j0; j < j1; ++j) {
+                __syncthreads();   // the weights, and every warp is done with the last date's tables
+                for (int i = tid; i < E * LV; i += NT) {
+                    const size_t o = ((size_t)j * E + i / LV) * G + P0 + i % LV;
+                    tab_s[i] = __ldg(a.zc + o);
+                    if (REV) tab_s[E * LV + i] = __ldg(a.dzc + o);
+                }
+                __syncthreads();
                 const float *fe = a.features + (size_t)j * F * M;
-                const float4 *tab = a.zc + (size_t)j * E * G + P0;
                 f32x2 mt[C];
 #pragma unroll
                 for (int c = 0; c < C; ++c) mt[c] = pack2(0.f, 0.f);
 #pragma unroll 1
                 for (int e = 0; e < E; ++e) {
-                    f32x2 X[2 * LV], em[LV], fixm1;
+                    f32x2 X[2 * LV], em[LV];
                     const f32x2 re = pack2(__ldg(fe + (size_t)e * M + r0), __ldg(fe + (size_t)e * M + r1));
-                    const f32x2 rf = pack2(__ldg(ffix + (size_t)e * M + r0), __ldg(ffix + (size_t)e * M + r1));
                     const float *lc = fe + (size_t)(E - 1 + (e > 0 ? e : 1)) * M;
                     const f32x2 chi = e == 0 ? pack2(1.f, 1.f) : pack2(expf(__ldg(lc + r0)), expf(__ldg(lc + r1)));
-                    bonds(e, tab + e * G, re, rf, X, em, fixm1);
+                    bonds(tab_s + e * LV, re, fix_s[e * NT + tid], X, em);
                     const f32x2 *w = w_s + e * C * 2 * LV;
 #pragma unroll
                     for (int c = 0; c < C; ++c) {
@@ -157,8 +169,11 @@ __global__ void __launch_bounds__(128) adj_price_kernel(AdjSplitArgs a, PriceSha
                     const float V0 = l * b0 * fmaxf(m.x, 0.f), V1 = l * b1 * fmaxf(m.y, 0.f);
                     const float *s1 = a.surv + ((size_t)j * C + c) * M, *s0 = s1 - (size_t)C * M;
                     const float d0 = __ldg(s0 + r0) - __ldg(s1 + r0), d1 = __ldg(s0 + r1) - __ldg(s1 + r1);
-                    if (live0) J += (double)V0 * (double)d0;
-                    if (live1) J += (double)V1 * (double)d1;
+                    // V d with its rounding error: as exact as FP64 without its narrow pipe
+                    const float t0 = live0 ? d0 : 0.f, t1 = live1 ? d1 : 0.f;
+                    const float q0 = __fmul_rn(V0, t0), q1 = __fmul_rn(V1, t1);
+                    J.add(q0, fmaf(V0, t0, -q0));
+                    J.add(q1, fmaf(V1, t1, -q1));
                     if (REV) {
                         put(a.V + ((size_t)j * C + c) * M, V0, V1);
                         mtb[c] = pack2(m.x > 0.f ? d0 * l * b0 : 0.f, m.y > 0.f ? d1 * l * b1 : 0.f);
@@ -171,12 +186,13 @@ __global__ void __launch_bounds__(128) adj_price_kernel(AdjSplitArgs a, PriceSha
                 float lb0 = 0.f, lb1 = 0.f;
 #pragma unroll 1
                 for (int e = 0; e < E; ++e) {
-                    f32x2 X[2 * LV], em[LV], fixm1, u[2 * LV];
+                    f32x2 X[2 * LV], em[LV], u[2 * LV];
+                    const f32x2 fixm1 = fix_s[e * NT + tid];
+                    const float4 *tab = tab_s + e * LV, *dtab = tab + E * LV;
                     const f32x2 re = pack2(__ldg(fe + (size_t)e * M + r0), __ldg(fe + (size_t)e * M + r1));
-                    const f32x2 rf = pack2(__ldg(ffix + (size_t)e * M + r0), __ldg(ffix + (size_t)e * M + r1));
                     const float *lc = fe + (size_t)(E - 1 + (e > 0 ? e : 1)) * M;
                     const f32x2 chi = e == 0 ? pack2(1.f, 1.f) : pack2(expf(__ldg(lc + r0)), expf(__ldg(lc + r1)));
-                    bonds(e, tab + e * G, re, rf, X, em, fixm1);
+                    bonds(tab, re, fixm1, X, em);
                     // u = sum_c (adjoint of MtM_c) w_c: times chi the adjoint of X
                     const f32x2 *w = w_s + e * C * 2 * LV;
 #pragma unroll
@@ -198,13 +214,12 @@ __global__ void __launch_bounds__(128) adj_price_kernel(AdjSplitArgs a, PriceSha
                     // -D_g = Z_{g-1} em_g, Z_g = Z_{g-1} (1 + em_g), em_g = expm1(x_g), x_g = dlnA - dB r
                     const f32x2 one = pack2(1.f, 1.f);
                     f32x2 rb = pack2(0.f, 0.f), pf = rb, psg = rb;
-                    const float4 *dtab = a.dzc + ((size_t)j * E + e) * G + P0;
 #pragma unroll
                     for (int g = LV - 1; g >= 1; --g) {
                         const f32x2 em1 = fma2(em[g], one, one);
                         const f32x2 xb = mul2(mul2(fma2(u[LV + g], one, u[g]), X[LV + g - 1]), em1);
                         u[LV + g - 1] = fma2(u[LV + g], em1, fma2(u[g], em[g], u[LV + g - 1]));
-                        const float4 t4 = __ldg(tab + e * G + g), d4 = __ldg(dtab + g);
+                        const float4 t4 = tab[g], d4 = dtab[g];
                         rb = fma2(xb, pack2(-t4.w, -t4.w), rb);
                         pf = fma2(xb, pack2(d4.z, d4.z), pf);
                         psg = fma2(xb, pack2(d4.w, d4.w), psg);
@@ -216,7 +231,7 @@ __global__ void __launch_bounds__(128) adj_price_kernel(AdjSplitArgs a, PriceSha
                         const f32x2 db = pack2(-nd.x, -nd.y);
                         const f32x2 yb = mul2(fma2(db, fixm1, u[LV]), X[LV]);
                         const f32x2 ub = mul2(mul2(db, X[LV]), fma2(fixm1, one, one));
-                        const float4 tp = __ldg(tab + e * G), d4 = __ldg(dtab);
+                        const float4 tp = tab[0], d4 = dtab[0];
                         const float2 f2 = __ldg(fx + e), df2 = __ldg(a.dfix + (size_t)p * E + e);
                         rb = fma2(yb, pack2(-tp.y, -tp.y), rb);
                         pf = fma2(yb, pack2(d4.x, d4.x), pf);
@@ -246,7 +261,7 @@ __global__ void __launch_bounds__(128) adj_price_kernel(AdjSplitArgs a, PriceSha
             put(a.fixin + ((size_t)blockIdx.y * E + e) * M, v.x, v.y);
         }
     // block sums in FP64, fixed order: a warp per value
-    j_s[tid] = J;
+    j_s[tid] = (double)J.hi + (double)J.lo;
     __syncthreads();
     double *out = a.part_p + ((size_t)blockIdx.y * gridDim.x + blockIdx.x) * (2 * E + 1);
     const int lane = tid & 31;

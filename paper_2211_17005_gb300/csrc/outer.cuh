@@ -61,6 +61,17 @@ __device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b)
     return r;
 }
 
+// a sum of FP32 terms and the rounding errors made in it: as exact as an FP64 sum
+struct SumPair {
+    float hi, lo;
+    __device__ void add(float p, float e = 0.f)   // p + e, e the error of p
+    {
+        const float s = hi + p, b = s - hi;
+        lo += ((hi - (s - b)) + (p - b)) + e;
+        hi = s;
+    }
+};
+
 // expm1(x) by its Taylor series to degree 8 for |x| <= 1/4 (relative error below
 // 2e-10 there, so the rounding of the FMAs dominates), library expm1f elsewhere.
 __device__ __forceinline__ float expm1_small(float x)
@@ -348,7 +359,9 @@ __global__ void __launch_bounds__(32 * NW, NW == 8 ? 3 : 5) sim_kernel(OuterArgs
 // the warps waited for instructions).
 //
 // The group's weights wait in shared memory, negated and doubled (w, w) as the packed
-// multiply wants them, two reset dates in a 16-byte broadcast load. The MtM enters as
+// multiply wants them, two reset dates in a 16-byte broadcast load; so do the date's bond
+// tables (read through L1 they were the longest wait) and, where they fit beside the
+// weights, the running coupons at the fixing, which the period's dates share. The MtM enters as
 //   acc = sum_h (-wA)(-D_h) + sum_g (-wK) Z_g,
 // with -D_h = Z_{h-1} expm1(x_h), which is what the chain of bond prices produces.
 struct PriceShape {
@@ -389,12 +402,24 @@ __device__ __forceinline__ f32x2 expm1_small2(f32x2 x)
     return r;
 }
 
+// shared memory of price_kernel: weights, the date's tables, the coupons where they fit
+template <int E, int C, int G, int NPB>
+struct PriceSmem {
+    static constexpr int weights = E * NPB * C * 2 * G * 8, tables = E * G * 16, coupons = E * 256 * 8;
+    static constexpr bool keep = weights + tables + coupons <= 48 * 1024;   // the default limit
+    static constexpr int bytes = weights + tables + (keep ? coupons : 0);
+    static_assert(bytes <= 48 * 1024, "portfolio weights exceed the default shared-memory limit");
+};
+
 template <int E, int C, int CS, int G, int NPB>
 __global__ void __launch_bounds__(256, NPB == 1 ? 3 : 2) price_kernel(OuterArgs a, PriceShape ps)
 {
+    using SM = PriceSmem<E, C, G, NPB>;
     constexpr int F = 2 * E - 1 + CS, R = NPB * C;   // rows of weights per economy
     extern __shared__ __align__(16) unsigned char price_smem[];
     f32x2 *w_s = reinterpret_cast<f32x2 *>(price_smem);      // [E][R][2 LV] (-wA, then -wK), doubled
+    float4 *tab_s = reinterpret_cast<float4 *>(price_smem + SM::weights);                          // [E][LV]
+    f32x2 *fix_s = reinterpret_cast<f32x2 *>(price_smem + SM::weights + SM::tables) + threadIdx.x;  // [E], stride 256
     const int tid = threadIdx.x, nthr = blockDim.x, pf0 = (int)blockIdx.z * NPB;
     const size_t M = a.M;
     const int n = c_sim.n, ppp = c_sim.ppp;
@@ -431,48 +456,57 @@ __global__ void __launch_bounds__(256, NPB == 1 ? 3 : 2) price_kernel(OuterArgs 
                 const float w = q < LV ? __ldg(a.w_glob + wrow + q) : __ldg(a.w_glob + kMaxW + wrow + q - LV);
                 w_s[i] = pack2(-w, -w);
             }
-            __syncthreads();
             const float *ffix = a.features + (size_t)(p * ppp) * F * M;   // state at the last reset
             const float2 *fx = a.fix + (size_t)p * E;
+            // 1/ZC_{t_-}(t_+) - 1 of economy e
+            auto coupon = [&](int e) {
+                const float2 f2 = __ldg(fx + e);
+                const float *f = ffix + (size_t)e * M;
+                return pack2(expm1f(fmaf(f2.y, __ldg(f + r0), -f2.x)), expm1f(fmaf(f2.y, __ldg(f + r1), -f2.x)));
+            };
+            if (SM::keep) {
+#pragma unroll 2
+                for (int e = 0; e < E; ++e) fix_s[e * 256] = coupon(e);
+            }
             for (int j = j0; j < j1; ++j) {
+                __syncthreads();   // the weights, and every warp is done with the last date's tables
+                for (int i = tid; i < E * LV; i += nthr) tab_s[i] = __ldg(a.zc + ((size_t)j * E + i / LV) * G + P0 + i % LV);
                 const float *fe = a.features + (size_t)j * F * M;
-                const float4 *tab = a.zc + (size_t)j * E * G + P0;
+                const float4 *tab = tab_s;
                 f32x2 mt[R];
 #pragma unroll
                 for (int i = 0; i < R; ++i) mt[i] = pack2(0.f, 0.f);
                 const float *dj = a.disc + (size_t)j * M;
                 const float beta0 = expf(-__ldg(dj + r0)), beta1 = expf(-__ldg(dj + r1));
-                float re0 = __ldg(fe + r0), re1 = __ldg(fe + r1), rf0 = __ldg(ffix + r0), rf1 = __ldg(ffix + r1);
+                float re0 = __ldg(fe + r0), re1 = __ldg(fe + r1);
                 float lc0 = 0.f, lc1 = 0.f;
                 const f32x2 *w = w_s;
+                __syncthreads();
 #pragma unroll 1
-                for (int e = 0; e < E; ++e, tab += G, w += R * 2 * LV) {
+                for (int e = 0; e < E; ++e, tab += LV, w += R * 2 * LV) {
                     // bond prices Z[g] = ZC_t((p + g + 1) delta) of the live reset dates, chained
                     // from the first: Z[g] = Z[g-1] (1 + expm1(x_g)), x_g = ln ZC_t of this date
                     // - ln ZC_t of the one before. D[g] = ZC_t of the date before - Z[g] = -Z[g-1]
                     // expm1(x_g) keeps full relative accuracy; D[0] carries the running floating
                     // coupon ZC_t(t_+) (1/ZC_{t_-}(t_+) - 1). X holds -D, then Z.
                     f32x2 X[2 * LV];
-                    const float2 f2 = __ldg(fx + e);
-                    const float4 tp = __ldg(tab);
+                    const float2 fm = unpack2(SM::keep ? fix_s[e * 256] : coupon(e));
+                    const float4 tp = tab[0];
                     const float z0 = expf(fmaf(-tp.y, re0, tp.x)), z1 = expf(fmaf(-tp.y, re1, tp.x));
-                    X[0] = pack2(-(z0 * expm1f(fmaf(f2.y, rf0, -f2.x))), -(z1 * expm1f(fmaf(f2.y, rf1, -f2.x))));
+                    X[0] = pack2(-(z0 * fm.x), -(z1 * fm.y));
                     X[LV] = pack2(z0, z1);
                     const f32x2 re = pack2(re0, re1);
                     const f32x2 chi = e == 0 ? pack2(1.f, 1.f) : pack2(expf(lc0), expf(lc1));
                     if (e + 1 < E) {   // the next economy's state, ahead of this one's products
                         fe += M;
-                        ffix += M;
                         re0 = __ldg(fe + r0);
                         re1 = __ldg(fe + r1);
-                        rf0 = __ldg(ffix + r0);
-                        rf1 = __ldg(ffix + r1);
                         lc0 = __ldg(fe + (size_t)(E - 1) * M + r0);
                         lc1 = __ldg(fe + (size_t)(E - 1) * M + r1);
                     }
 #pragma unroll
                     for (int g = 1; g < LV; ++g) {
-                        const float4 t4 = __ldg(tab + g);
+                        const float4 t4 = tab[g];
                         const f32x2 em = expm1_small2(fma2(pack2(-t4.w, -t4.w), re, pack2(t4.z, t4.z)));
                         X[g] = mul2(X[LV + g - 1], em);
                         X[LV + g] = fma2(X[LV + g - 1], em, X[LV + g - 1]);
@@ -489,7 +523,6 @@ __global__ void __launch_bounds__(256, NPB == 1 ? 3 : 2) price_kernel(OuterArgs 
                         mt[i] = fma2(chi, acc, mt[i]);
                     }
                 }
-                ffix -= (size_t)(E - 1) * M;
 #pragma unroll
                 for (int i = 0; i < R; ++i) {
                     const float2 m = unpack2(mt[i]);
@@ -613,11 +646,12 @@ cva_status outer_launch(Sim &s, uint64_t seed, uint64_t k0, cudaStream_t st)
             attr[dev] = true;
         }
         // at least six path tiles per slot and part of a period, so that the last round of
-        // tiles is a small part of them
+        // tiles is a small part of them; at most kPriceTcDates dates, whose tables a block keeps
         const uint32_t tiles = (args.M + 127u) / 128u, slots = (uint32_t)sms * kPriceSlots;
         const unsigned periods = (unsigned)((s.n + s.ppp - 1) / s.ppp);
         PriceShape ps = {s.ppp, 1, s.start_date};
-        while ((uint64_t)tiles * ps.splits < 6ull * slots && ps.dates_per_block > 1) {
+        while (ps.dates_per_block > kPriceTcDates ||
+               ((uint64_t)tiles * ps.splits < 6ull * slots && ps.dates_per_block > 1)) {
             ps.dates_per_block = (ps.dates_per_block + 1) / 2;
             ps.splits = (s.ppp + ps.dates_per_block - 1) / ps.dates_per_block;
         }
@@ -635,15 +669,13 @@ cva_status outer_launch(Sim &s, uint64_t seed, uint64_t k0, cudaStream_t st)
     PriceShape ps = price_shape((uint64_t)tiles * periods * (NPF / ppb), s.ppp, sms);
     ps.start = s.start_date;
     const dim3 pgrid(tiles, periods * (unsigned)ps.splits, (unsigned)(NPF / ppb));
-    const size_t psmem = (size_t)E * ppb * C * 2 * G * sizeof(f32x2);
-    static_assert(E * 3 * C * 2 * G * sizeof(f32x2) <= 48 * 1024, "portfolio weights exceed the default shared-memory limit");
     if constexpr (NPF % 3 == 0) {
-        if (ppb == 3) price_kernel<E, C, CS, G, 3><<<pgrid, pb, psmem, st>>>(args, ps);
+        if (ppb == 3) price_kernel<E, C, CS, G, 3><<<pgrid, pb, PriceSmem<E, C, G, 3>::bytes, st>>>(args, ps);
     }
     if constexpr (NPF % 2 == 0) {
-        if (ppb == 2) price_kernel<E, C, CS, G, 2><<<pgrid, pb, psmem, st>>>(args, ps);
+        if (ppb == 2) price_kernel<E, C, CS, G, 2><<<pgrid, pb, PriceSmem<E, C, G, 2>::bytes, st>>>(args, ps);
     }
-    if (ppb == 1) price_kernel<E, C, CS, G, 1><<<pgrid, pb, psmem, st>>>(args, ps);
+    if (ppb == 1) price_kernel<E, C, CS, G, 1><<<pgrid, pb, PriceSmem<E, C, G, 1>::bytes, st>>>(args, ps);
     CVA_CUDA_TRY(cudaGetLastError());
     if (!capturing) CVA_CUDA_TRY(cudaEventRecord(t_last[dev], st));
     return CVA_OK;
@@ -726,8 +758,9 @@ cva_status adjoint_launch(Sim &s, AdjBuffers &b, uint64_t seed, uint64_t k0, uin
     else sim_kernel<E, C, CS, 4, SimMode::adjoint><<<rblocks, 128, 0, st>>>(o);
     CVA_CUDA_TRY(cudaGetLastError());
     const dim3 pgrid(tiles, periods * (unsigned)ps.splits);
-    const size_t psmem = (size_t)E * C * 2 * G * sizeof(f32x2) + (size_t)E * 128 * 16;
-    static_assert(E * C * 2 * G * sizeof(f32x2) + E * 128 * 16 <= 47 * 1024, "adjoint pricing: default shared-memory limit");
+    // weights, fixing adjoints, coupons, tables, parameter adjoints
+    constexpr size_t psmem = (size_t)E * C * 2 * G * 8 + (size_t)E * 128 * (8 + 8 + 8) + 2 * (size_t)E * G * 16;
+    static_assert(psmem <= 47 * 1024, "adjoint pricing: default shared-memory limit");
     if (b.forward_only) {
         adj_price_kernel<E, C, CS, G, false><<<pgrid, 128, psmem, st>>>(a, ps);
         CVA_CUDA_TRY(cudaGetLastError());

@@ -30,13 +30,15 @@
 // accumulators, so that a date's MtM is read while the next date's is accumulated.
 //
 // Shared memory: W hi | W lo ([NN][KT] each, K-major core matrices), the X buffers
-// (Xhi | Xlo, [128][GK] each) of every slot, the coupons at the fixing [E][512]. TMEM:
-// two 128 x NN FP32 accumulators per slot.
+// (Xhi | Xlo, [128][GK] each) of every slot, the coupons at the fixing [E][512], the bond
+// tables of the block's dates (the rest of the multiprocessor's memory is too small an L1 to
+// hold them). TMEM: two 128 x NN FP32 accumulators per slot.
 //
 // Six portfolios (50 to 2000 swaps), 2^18 paths, 120 dates: 9.94 ms with every reset date,
 // one X buffer and a block barrier and vote per economy.
 constexpr uint32_t kPriceMbarPolls = 1u << 26;   // limit of a wait for the tensor core
 constexpr int kPriceSlots = 4;
+constexpr int kPriceTcDates = 6;                 // dates of a block at most
 
 template <int E, int NPF, int C, int LV>
 struct PriceTc {
@@ -48,9 +50,10 @@ struct PriceTc {
     static constexpr int sWhi = 0, sWlo = NN * KT * 4;
     static constexpr int sX = 2 * NN * KT * 4;            // buffer b of slot s at sX + (s bufs + b) xbuf
     static constexpr int xbuf = 2 * 128 * GK * 4;         // Xhi, then Xlo at + 128 GK 4
-    static constexpr int sFixBytes = E * 128 * kPriceSlots * 4;
-    static constexpr int bufs = sX + 2 * kPriceSlots * xbuf + sFixBytes <= 220 * 1024 ? 2 : 1;
-    static constexpr int sFix = sX + bufs * kPriceSlots * xbuf;
+    static constexpr int sFixBytes = E * 128 * kPriceSlots * 4, sTabBytes = kPriceTcDates * E * LV * 16;
+    static constexpr int bufs = sX + 2 * kPriceSlots * xbuf + sFixBytes + sTabBytes <= 224 * 1024 ? 2 : 1;
+    static constexpr int sTab = sX + bufs * kPriceSlots * xbuf;
+    static constexpr int sFix = sTab + sTabBytes;
     static constexpr int bytes = sFix + sFixBytes;
     static_assert(NN <= 64 && tmem_cols <= 512, "tensor memory");
     static_assert(bytes <= 224 * 1024, "shared memory");
@@ -82,13 +85,13 @@ __device__ __forceinline__ bool slot_all(bool p, int slot)
 template <int LV, int GK>
 __device__ __forceinline__ void price_row(float (&x)[GK], const float4 *tab, float re, float fixm1, float chi)
 {
-    const float4 tp = __ldg(tab);
+    const float4 tp = tab[0];
     float zp = expf(fmaf(-tp.y, re, tp.x));
     x[0] = chi * (zp * fixm1);
     x[LV] = chi * zp;
 #pragma unroll
     for (int g = 1; g < LV; ++g) {
-        const float4 t4 = __ldg(tab + g);
+        const float4 t4 = tab[g];
         const float em = expm1_small(fmaf(-t4.w, re, t4.z));
         x[g] = chi * (-zp * em);
         zp = fmaf(zp, em, zp);
@@ -154,6 +157,9 @@ __global__ void __launch_bounds__(128 * kPriceSlots, 1) price_tc_kernel(OuterArg
                 *reinterpret_cast<float *>(tsm + P::sWhi + off) = hi;
                 *reinterpret_cast<float *>(tsm + P::sWlo + off) = umma::tf32_round(w - hi);
             }
+            float4 *tab_s = reinterpret_cast<float4 *>(tsm + P::sTab);   // [date - j0][E][LV]
+            for (int i = tid; i < (j1 - j0) * E * LV; i += blockDim.x)
+                tab_s[i] = __ldg(a.zc + ((size_t)j0 * E + i / LV) * G + P0 + i % LV);
             // the X columns past the live ones stay zero
             for (int b = 0; b < BUFS; ++b)
                 for (int h = 0; h < 2; ++h)
@@ -190,17 +196,25 @@ __global__ void __launch_bounds__(128 * kPriceSlots, 1) price_tc_kernel(OuterArg
                 }
                 for (int j = j0; j < j1 && ok; ++j, ++item) {
                     const float *fe = a.features + (size_t)j * F * M + kr;
-                    const float4 *tab = a.zc + (size_t)j * E * G + P0;
+                    const float4 *tab = tab_s + (j - j0) * E * LV;
                     const float beta = expf(-__ldg(a.disc + (size_t)j * M + kr));
                     const uint32_t acc = tmem + (item & 1u) * P::acc_cols;
-                    // an economy's state is requested one economy ahead
-                    float n_r = __ldg(fe), n_lchi = 0.f;
+                    // an economy's state is requested two economies ahead (rate, log chi)
+                    float n_r[2], n_l[2];
+#pragma unroll
+                    for (int i = 0; i < 2; ++i) {
+                        const int e = i < E ? i : 0;
+                        n_r[i] = __ldg(fe + (size_t)e * M);
+                        n_l[i] = e > 0 ? __ldg(fe + (size_t)(E - 1 + e) * M) : 0.f;
+                    }
 #pragma unroll 1
-                    for (int e = 0; e < E; ++e, ++uses, tab += G) {
-                        const float re = n_r, chi = e == 0 ? 1.f : expf(n_lchi);
-                        if (e + 1 < E) {
-                            n_r = __ldg(fe + (size_t)(e + 1) * M);
-                            n_lchi = __ldg(fe + (size_t)(E + e) * M);   // log chi^{e+1}
+                    for (int e = 0; e < E; ++e, ++uses, tab += LV) {
+                        const float re = n_r[0], chi = e == 0 ? 1.f : expf(n_l[0]);
+                        n_r[0] = n_r[1];
+                        n_l[0] = n_l[1];
+                        if (e + 2 < E) {
+                            n_r[1] = __ldg(fe + (size_t)(e + 2) * M);
+                            n_l[1] = __ldg(fe + (size_t)(E + 1 + e) * M);   // log chi^{e+2}
                         }
                         float x[GK];
                         price_row<LV, GK>(x, tab, re, fix_s[e * 128 * kPriceSlots], chi);
