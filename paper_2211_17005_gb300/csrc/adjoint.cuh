@@ -52,7 +52,7 @@ struct AdjSplitArgs {
 };
 
 template <int E, int C, int CS, int G, bool REV>
-__global__ void __launch_bounds__(128) adj_price_kernel(AdjSplitArgs a, PriceShape ps)
+__global__ void __launch_bounds__(128, 4) adj_price_kernel(AdjSplitArgs a, PriceShape ps)
 {
     constexpr int F = 2 * E - 1 + CS, NT = 128;
     extern __shared__ __align__(16) unsigned char adj_smem[];

@@ -1,0 +1,180 @@
+"""Edges of the kernels' tiles: path counts around a tile and a warp, step counts that leave
+a partial chunk, draw counts around the staging and counter widths, every width of the
+normal equations. References are computed here in FP64 or are the same paths of a larger run."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2211_17005_gb300 import workload as W
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def api():
+    assert torch.cuda.is_available(), "GPU tests need CUDA"
+    from paper_2211_17005_gb300 import api as A, build
+    build.build()
+    return A
+
+
+def _clocks(api, seed, M, N, C):
+    """The draws' uniforms [M, N, C] (exact in FP32 and FP64)."""
+    out = np.empty((M, N, 4 * ((C + 3) // 4)))
+    k, l = np.meshgrid(np.arange(M), np.arange(N), indexing="ij")   # noqa: E741
+    for b in range((C + 3) // 4):
+        ctr = np.stack([k, l, np.zeros_like(k), np.full_like(k, (2 << 24) | b)], axis=-1).astype(np.uint32)
+        x = api.philox4x32_10(torch.from_numpy(ctr.reshape(-1, 4).view(np.int32)).cuda(), seed)
+        x = x.cpu().numpy().view(np.uint32).reshape(M, N, 4)
+        out[:, :, 4 * b:4 * b + 4] = ((x >> 9) + 0.5) * 2.0 ** -23
+    return out[:, :, :C]
+
+
+@pytest.mark.parametrize("name,M,N,n", [("small", 5, 70000, 50), ("small", 33, 1, 5), ("mixed", 37, 33, 250),
+                                        ("paper", 129, 3, 20), ("batched", 40, 65, 30)])
+def test_default_steps_and_targets_follow_from_thresholds_and_exposures(api, name, M, N, n):
+    wl = W.make(name, M=M, N=N, n_steps=n)
+    sim = api.Simulation(wl.model, wl.portfolios, wl.grid, M, N, keep_defaults=True)
+    sim.run(wl.seed)
+    C = wl.model.C
+    w = _clocks(api, wl.seed, M, N, C)
+    thr = sim.thresholds().cpu().numpy().astype(np.float64)
+    idx = sim.defaults().cpu().numpy()
+    expo = sim.exposures().cpu().numpy().astype(np.float64)
+    I0 = sim.discount_integral().cpu().numpy().astype(np.float64)
+    for k in range(M):
+        for c in range(C):
+            ref = 1 + np.searchsorted(thr[1:, c, k], w[k, :, c], side="left")
+            np.testing.assert_array_equal(idx[k, :, c], ref)
+    cnt = np.zeros((n + 2, C, M))
+    for c in range(C):
+        for k in range(M):
+            cnt[:, c, k] = np.bincount(idx[k, :, c], minlength=n + 2)[:n + 2]
+    got = sim.targets().cpu().numpy().astype(np.float64)
+    # nonnegative FP32 terms: every rounding of the n C additions and products is relative
+    rtol = (n * C + 16) * 2.0 ** -24
+    for pf in range(sim.n_pf):
+        loss = (expo[pf, 1:] * cnt[1:n + 1]).sum(1)
+        ref = np.exp(I0[:n]) * np.cumsum(loss[::-1], axis=0)[::-1] / N
+        np.testing.assert_allclose(got[pf], ref, rtol=rtol, atol=0)
+    bits = sim.targets().clone()
+    for inner in (2, 4, 8):   # other tiles, and 128 threads' paths per pricing block
+        sim.set_tiles(64, 128, inner, 2432, 1)
+        sim.run(wl.seed)
+        assert torch.equal(sim.targets(), bits)
+    sim.close()
+
+
+@pytest.mark.parametrize("M", [1, 31, 33, 257])
+@pytest.mark.parametrize("name,n,S", [("paper", 10, 3), ("small", 25, 1), ("mixed", 10, 1)])
+def test_paths_do_not_depend_on_the_tiles(api, name, n, S, M):
+    """A short run's paths equal the same paths of a longer one, with four and eight warps a block."""
+    big = W.make(name, M=700, N=2, n_steps=n, substeps=S)
+    a = api.Simulation(big.model, big.portfolios, big.grid, 700, 2)
+    a.run(big.seed)
+    b = api.Simulation(big.model, big.portfolios, big.grid, M, 2)
+    for tiles in (None, (64, 128, 0, 2432, 1), (128, 256, 0, 2432, 1)):
+        if tiles:
+            b.set_tiles(*tiles)
+        b.run(big.seed)
+        for what in ("features", "discount_integral", "thresholds", "exposures", "targets"):
+            assert torch.equal(getattr(b, what)(), getattr(a, what)()[..., :M]), (what, tiles)
+    a.close()
+    b.close()
+
+
+def _fit64(cols, y):
+    """Fitted values of the targets y [nt, M] on the columns [m, M] and a constant, FP64."""
+    A = np.concatenate([np.ones((1, cols.shape[1])), cols]).T
+    A = A / np.linalg.norm(A, axis=0)
+    return (A @ np.linalg.lstsq(A, y.T, rcond=None)[0]).T
+
+
+@pytest.mark.parametrize("F,M", [(1, 97), (6, 1024), (7, 1025), (14, 4099), (15, 4100), (22, 513), (23, 20000),
+                                 (27, 100003), (30, 2049)])
+@pytest.mark.parametrize("basis", ["linear", "poly2"])
+def test_fit_at_every_width_of_the_normal_equations(api, F, M, basis):
+    rng = np.random.default_rng(100 * F + M)
+    Y = (0.02 + 0.01 * rng.normal(size=(F, M))).astype(np.float32)
+    xi = (0.01 + (Y - 0.02).sum(0) + 0.005 * rng.normal(size=M)).astype(np.float32)
+    pred, coef = api.regress(torch.from_numpy(xi).cuda(), torch.from_numpy(Y).cuda(), basis=basis)
+    Y64 = Y.astype(np.float64)
+    d = Y64[0] - Y64[0].mean()
+    ref = _fit64(np.stack([d, d ** 2]) if basis == "poly2" else Y64, xi.astype(np.float64)[None])[0]
+    # FP32 runs of at most 256 products and five more additions: 261 roundings of 2^-24 in the
+    # normal equations, whose scaled condition number is below 7 here
+    assert np.sqrt(np.mean((pred.cpu().numpy() - ref) ** 2)) <= 261 * 2.0 ** -24 * 7 * np.sqrt(np.mean(xi.astype(np.float64) ** 2))
+    assert np.all(np.isfinite(coef))
+
+
+@pytest.mark.parametrize("basis", ["linear", "poly2"])
+def test_six_targets_share_the_normal_equations(api, basis):
+    wl = W.make("batched", M=1003, N=16, n_steps=20)
+    sim = api.Simulation(wl.model, wl.portfolios, wl.grid, wl.M, wl.N)
+    sim.run(wl.seed)
+    pred, _ = sim.regress_portfolios(basis)
+    j = 7
+    Y = sim.features()[j].cpu().numpy().astype(np.float64)
+    xi = sim.targets()[:, j].cpu().numpy().astype(np.float64)
+    d = Y[0] - Y[0].mean()
+    ref = _fit64(np.stack([d, d ** 2]) if basis == "poly2" else Y, xi)
+    gap = np.sqrt(np.mean((pred[:, j].cpu().numpy() - ref) ** 2, axis=1))
+    assert np.all(gap <= 261 * 2.0 ** -24 * 30 * np.sqrt(np.mean(xi ** 2, axis=1))), gap   # correlated factors
+    sim.close()
+
+
+@pytest.mark.parametrize("name,M,N,n", [("mixed", 203, 70, 20), ("small", 67, 5, 25), ("paper", 150, 64, 10)])
+def test_alive_statistics_around_the_staged_draws(api, name, M, N, n):
+    """The fit at X = 0 equals the least squares over the written-out M N rows."""
+    wl = W.make(name, M=M, N=N, n_steps=n)
+    sim = api.Simulation(wl.model, wl.portfolios, wl.grid, M, N, keep_defaults=True)
+    sim.run(wl.seed)
+    pred, _, dropped = sim.regress_alive(0)
+    j, C = n // 2, wl.model.C
+    idx = sim.defaults().cpu().numpy().astype(np.int64)
+    V = np.concatenate([sim.exposures()[0].cpu().numpy(), np.zeros((1, C, M), np.float32)]).astype(np.float64)
+    I0 = sim.discount_integral()[j].cpu().numpy().astype(np.float64)
+    loss = sum(np.where(idx[:, :, c] > j, V[idx[:, :, c], c, np.arange(M)[:, None]], 0.0) for c in range(C))
+    y = (loss * np.exp(I0)[:, None]).reshape(-1)
+    X = (idx <= j).astype(np.float64).reshape(-1, C)
+    f = sim.features()[j].cpu().numpy().astype(np.float64)
+    Y = np.repeat(((f - f.mean(1, keepdims=True)) / f.std(1, keepdims=True)).T, N, axis=0)
+    use = X.any(0)
+    assert dropped[j] == C - use.sum()
+    A = np.concatenate([np.ones((M * N, 1)), Y, X[:, use]], axis=1)
+    w = np.linalg.lstsq(A, y, rcond=None)[0]
+    ref = A[::N, :1 + f.shape[0]] @ w[:1 + f.shape[0]]
+    # as above; the indicators' columns are near multiples of one another at small samples
+    assert np.sqrt(np.mean((pred[j].cpu().numpy() - ref) ** 2)) <= 261 * 2.0 ** -24 * 60 * np.sqrt(np.mean(y ** 2))
+    sim.close()
+
+
+def test_adjoint_of_path_ranges_adds_up(api):
+    """Path counts that run in several ranges: the gradient is the mean of its parts'."""
+    wl = W.make("adjoint", M=70001, n_steps=100)
+    pf = api.frozen(wl.model, wl.portfolios[0])
+    c, g = api.grad_cva0(wl.model, pf, wl.grid, 70001, wl.seed)
+    parts = [(0, 30000), (30000, 39999), (69999, 2)]
+    cs, gs = zip(*(api.grad_cva0(wl.model, pf, wl.grid, m, wl.seed, k0=k) for k, m in parts))
+    wgt = np.array([m for _, m in parts]) / 70001
+    assert c == pytest.approx(float(np.dot(wgt, cs)), rel=1e-9)
+    ref = np.tensordot(wgt, np.stack(gs), axes=1)
+    # the parts split a period's dates over other blocks: FP32 sums of up to ten terms each
+    np.testing.assert_allclose(g, ref, rtol=1e-5, atol=1e-6 * np.abs(ref).max())
+
+
+@pytest.mark.parametrize("date", [0, 1, 13, 19])
+def test_nested_copies_start_at_the_branch_date(api, date):
+    wl = W.make("paper", M=130, N=16, n_steps=20, substeps=2)
+    sim = api.Simulation(wl.model, wl.portfolios, wl.grid, wl.M, wl.N)
+    got = sim.nested_reference(wl.seed, date, 3)
+    left = {w: getattr(sim, w)().clone() for w in ("features", "discount_integral", "thresholds", "exposures", "targets")}
+    acc = None
+    for b in (1, 2, 3):
+        sim.run_twin(wl.seed, date, b)
+        t = sim.targets()[0, date].clone()
+        acc = t if acc is None else acc + t
+    for w, v in left.items():   # the last copy stays, whole
+        assert torch.equal(getattr(sim, w)(), v), w
+    assert torch.allclose(got, acc / 3, rtol=3 * 2.0 ** -24, atol=0)
+    sim.close()
