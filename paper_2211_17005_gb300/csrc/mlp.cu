@@ -330,26 +330,16 @@ struct Net {
     }
 
     // ---- epilogues (thread = row of the tile) ----
-    // H1 = relu(D + b1) into B; the mask of h1 > 0 in m1
-    __device__ void epi1(uint32_t (&m1)[U / 32]) const
+    // H1 = relu(D + b1) into B
+    __device__ void epi1() const
     {
         unsigned char *b = smem + offB();
         const float4 *b1 = reinterpret_cast<const float4 *>(th + L::ob1);
         float v[64];
         umma::tmem_ld64(taddr(dcol()), v);
-        m1[0] = m1[1] = 0u;
 #pragma unroll
-        for (int g = 0; g < 16; ++g) {
-            const float4 c = b1[g];
-            v[4 * g + 0] = fmaxf(v[4 * g + 0] + c.x, 0.f);
-            v[4 * g + 1] = fmaxf(v[4 * g + 1] + c.y, 0.f);
-            v[4 * g + 2] = fmaxf(v[4 * g + 2] + c.z, 0.f);
-            v[4 * g + 3] = fmaxf(v[4 * g + 3] + c.w, 0.f);
-        }
-#pragma unroll
-        for (int i = 0; i < 64; ++i) m1[i / 32] |= (v[i] > 0.f ? 1u : 0u) << (i % 32);
-#pragma unroll
-        for (int g = 0; g < 8; ++g) *reinterpret_cast<uint4 *>(b + row_off(row, 8 * g)) = pack8(v + 8 * g);
+        for (int g = 0; g < 8; ++g)
+            *reinterpret_cast<uint4 *>(b + row_off(row, 8 * g)) = bias_relu8(v + 8 * g, b1[2 * g], b1[2 * g + 1]);
     }
 
     // second hidden layer of this thread's row from its accumulator: h2 = relu(D + b2)
@@ -358,20 +348,10 @@ struct Net {
     {
         const float4 *b2 = reinterpret_cast<const float4 *>(th + L::ob2), *w3 = reinterpret_cast<const float4 *>(th + L::ow3);
         umma::tmem_ld64(taddr(dcol()), v);
-        float acc[4] = {th[L::ob3], 0.f, 0.f, 0.f};
-#pragma unroll
-        for (int g = 0; g < 16; ++g) {
-            const float4 c = b2[g], w = w3[g];
-            v[4 * g + 0] = fmaxf(v[4 * g + 0] + c.x, 0.f);
-            v[4 * g + 1] = fmaxf(v[4 * g + 1] + c.y, 0.f);
-            v[4 * g + 2] = fmaxf(v[4 * g + 2] + c.z, 0.f);
-            v[4 * g + 3] = fmaxf(v[4 * g + 3] + c.w, 0.f);
-            acc[0] = fmaf(v[4 * g + 0], w.x, acc[0]);
-            acc[1] = fmaf(v[4 * g + 1], w.y, acc[1]);
-            acc[2] = fmaf(v[4 * g + 2], w.z, acc[2]);
-            acc[3] = fmaf(v[4 * g + 3], w.w, acc[3]);
-        }
-        return (acc[0] + acc[1]) + (acc[2] + acc[3]);
+        f32x2 a01 = two(th[L::ob3], 0.f), a23 = two(0.f, 0.f);
+        bias_relu_dot64(v, b2, w3, a01, a23);
+        const float2 x = both(a01), y = both(a23);
+        return (x.x + x.y) + (y.x + y.y);
     }
 
     // output of this thread's row: zeta (+ relu if pos) + mu
@@ -396,16 +376,9 @@ struct Net {
         const float dpred = 2.f * (pred - y) * inv_batch;
         const float dout = pos ? (out > 0.f ? dpred : 0.f) : dpred;
 #pragma unroll
-        for (int g = 0; g < 8; ++g) {
-            const float4 w0 = w3[2 * g], w1 = w3[2 * g + 1];
-            const float wv[8] = {w0.x, w0.y, w0.z, w0.w, w1.x, w1.y, w1.z, w1.w};
-            float d[8];
-#pragma unroll
-            for (int i = 0; i < 8; ++i) d[i] = v[8 * g + i] > 0.f ? dout * wv[i] : 0.f;
-            *reinterpret_cast<uint4 *>(a + row_off(row, 8 * g)) = pack8(d);
-        }
-#pragma unroll
-        for (int i = 0; i < 64; ++i) v[i] *= dout;
+        for (int g = 0; g < 8; ++g)
+            *reinterpret_cast<uint4 *>(a + row_off(row, 8 * g)) = masked_scale8(v + 8 * g, dout, w3[2 * g], w3[2 * g + 1]);
+        scale64(v, dout);
         const float2 cs = column_sums64(v, lane);
         gsl[2 * lane] += cs.x;
         gsl[2 * lane + 1] += cs.y;
@@ -416,26 +389,27 @@ struct Net {
         }
     }
 
-    // dH1 = D (h1 > 0) into A
-    __device__ void back1(const uint32_t (&m1)[U / 32]) const
+    // dH1 = D (h1 > 0) into A, the mask from this thread's own part of H1 in B
+    __device__ void back1() const
     {
         unsigned char *a = smem + offA();
+        const unsigned char *b = smem + offB();
         float v[64];
         umma::tmem_ld64(taddr(dcol()), v);
 #pragma unroll
-        for (int i = 0; i < 64; ++i) v[i] = ((m1[i / 32] >> (i % 32)) & 1u) ? v[i] : 0.f;
-#pragma unroll
-        for (int g = 0; g < 8; ++g) *reinterpret_cast<uint4 *>(a + row_off(row, L::cDH1 + 8 * g)) = pack8(v + 8 * g);
+        for (int g = 0; g < 8; ++g)
+            *reinterpret_cast<uint4 *>(a + row_off(row, L::cDH1 + 8 * g)) =
+                masked8(v + 8 * g, *reinterpret_cast<const uint4 *>(b + row_off(row, 8 * g)));
     }
 
     // first two layers of the staged tile (staging status in_ok); D holds the second-layer
     // pre-activation after it. side() runs during the first GEMM, when every thread of
     // the slot is past the staging area (the next tile's copies may be requested).
     template <class Side>
-    __device__ bool forward12(uint32_t (&m1)[U / 32], bool in_ok, Side side)
+    __device__ bool forward12(bool in_ok, Side side)
     {
         if (!mma([&] { gemm_rows(dcol(), offB(), L::cX, L::sW1, kIn, U, false); }, in_ok, side)) return false;
-        epi1(m1);
+        epi1();
         return mma([&] { gemm_rows(dcol(), offB(), 0, L::sW2, U, U, false); });
     }
 
@@ -444,14 +418,13 @@ struct Net {
     __device__ bool train_tile(const TrainArgs &a, const CUtensorMap *tm, float y, bool in_ok, bool first,
                                float inv_batch, bool has_next, uint32_t next_path, float *gsl)
     {
-        uint32_t m1[U / 32];
-        if (!forward12(m1, in_ok, [&] {
+        if (!forward12(in_ok, [&] {
                 if (has_next) prefetch(tm, a.targ, a.F, next_path);
             }))
             return false;
         out_back2(a.pos, y, inv_batch, gsl);
         if (!mma([&] { gemm_rows_w2t(dcol(), offA()); })) return false;
-        back1(m1);
+        back1();
         return mma([&] { gemm_paths(wcol(), offA(), offB(), kRows, !first); });
     }
 
@@ -770,8 +743,7 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_sweep_kernel(SweepArgs a, con
         const uint32_t nt = t + stride;
         float y;
         const bool in_ok = n.stage_x(y);
-        uint32_t m1[U / 32];
-        ok = n.forward12(m1, in_ok, [&] {
+        ok = n.forward12(in_ok, [&] {
             if (nt < tiles) n.prefetch(&tm, a.targ, a.F, nt * kRows);
         });
         if (ok && a.mode != 1) {

@@ -22,14 +22,118 @@ constexpr uint32_t kMbarPolls = 1u << 26;
 
 __device__ __forceinline__ uint16_t bf16_bits(float x) { return __bfloat16_as_ushort(__float2bfloat16_rn(x)); }
 
+// (a, b) rounded to BF16, a in the low half: one instruction for the pair (two scalar
+// conversions and a merge otherwise)
 __device__ __forceinline__ uint32_t pack2(float a, float b)
 {
-    return (uint32_t)bf16_bits(a) | ((uint32_t)bf16_bits(b) << 16);
+    uint32_t r;
+    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(b), "f"(a));
+    return r;
+}
+
+// The epilogues of the trainers run two FP32 values at a time (each half rounded as the
+// scalar operation would): they are bound by the instructions an SM can issue.
+using f32x2 = unsigned long long;
+__device__ __forceinline__ f32x2 two(float a, float b)
+{
+    f32x2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ float2 both(f32x2 v)
+{
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+    return r;
+}
+__device__ __forceinline__ float2 add2(float a0, float a1, float b0, float b1)
+{
+    f32x2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(two(a0, a1)), "l"(two(b0, b1)));
+    return both(r);
+}
+__device__ __forceinline__ float2 mul2(float a0, float a1, float b0, float b1)
+{
+    f32x2 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(two(a0, a1)), "l"(two(b0, b1)));
+    return both(r);
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c)
+{
+    f32x2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+
+// max(x, 0) of a BF16 pair (0 for a NaN, as fmaxf gives); rounding to BF16 keeps the sign, so
+// it commutes with the ReLU
+__device__ __forceinline__ uint32_t relu_bf2(uint32_t w)
+{
+    asm("max.bf16x2 %0, %0, %1;" : "+r"(w) : "r"(0u));
+    return w;
+}
+// all ones in the halves of w that are above 0
+__device__ __forceinline__ uint32_t positive_bf2(uint32_t w)
+{
+    const uint32_t zero = 0u;
+    return __hgt2_mask(*reinterpret_cast<const __nv_bfloat162 *>(&w), *reinterpret_cast<const __nv_bfloat162 *>(&zero));
 }
 
 __device__ __forceinline__ uint4 pack8(const float *v)
 {
     return make_uint4(pack2(v[0], v[1]), pack2(v[2], v[3]), pack2(v[4], v[5]), pack2(v[6], v[7]));
+}
+
+// relu(v[i] + c[i]) of eight values as BF16 (c: two float4 of shared memory)
+__device__ __forceinline__ uint4 bias_relu8(const float *v, const float4 &c0, const float4 &c1)
+{
+    const float2 a = add2(v[0], v[1], c0.x, c0.y), b = add2(v[2], v[3], c0.z, c0.w);
+    const float2 d = add2(v[4], v[5], c1.x, c1.y), e = add2(v[6], v[7], c1.z, c1.w);
+    return make_uint4(relu_bf2(pack2(a.x, a.y)), relu_bf2(pack2(b.x, b.y)), relu_bf2(pack2(d.x, d.y)),
+                      relu_bf2(pack2(e.x, e.y)));
+}
+
+// v = relu(v + b) of 64 values in place and acc += w . v in four partial sums (a01, a23)
+__device__ __forceinline__ void bias_relu_dot64(float (&v)[64], const float4 *b, const float4 *w, f32x2 &a01, f32x2 &a23)
+{
+#pragma unroll
+    for (int g = 0; g < 16; ++g) {
+        const float4 c = b[g], u = w[g];
+        const float2 x = add2(v[4 * g], v[4 * g + 1], c.x, c.y), y = add2(v[4 * g + 2], v[4 * g + 3], c.z, c.w);
+        v[4 * g + 0] = fmaxf(x.x, 0.f);
+        v[4 * g + 1] = fmaxf(x.y, 0.f);
+        v[4 * g + 2] = fmaxf(y.x, 0.f);
+        v[4 * g + 3] = fmaxf(y.y, 0.f);
+        a01 = fma2(two(v[4 * g], v[4 * g + 1]), two(u.x, u.y), a01);
+        a23 = fma2(two(v[4 * g + 2], v[4 * g + 3]), two(u.z, u.w), a23);
+    }
+}
+
+// (v > 0 ? d w : 0) of eight values as BF16 (v >= 0: its BF16 is above 0 where it is)
+__device__ __forceinline__ uint4 masked_scale8(const float *v, float d, const float4 &w0, const float4 &w1)
+{
+    const float2 a = mul2(w0.x, w0.y, d, d), b = mul2(w0.z, w0.w, d, d);
+    const float2 c = mul2(w1.x, w1.y, d, d), e = mul2(w1.z, w1.w, d, d);
+    return make_uint4(pack2(a.x, a.y) & positive_bf2(pack2(v[0], v[1])), pack2(b.x, b.y) & positive_bf2(pack2(v[2], v[3])),
+                      pack2(c.x, c.y) & positive_bf2(pack2(v[4], v[5])), pack2(e.x, e.y) & positive_bf2(pack2(v[6], v[7])));
+}
+
+// (h > 0 ? v : 0) of eight values as BF16, h given as its BF16
+__device__ __forceinline__ uint4 masked8(const float *v, const uint4 &h)
+{
+    return make_uint4(pack2(v[0], v[1]) & positive_bf2(h.x), pack2(v[2], v[3]) & positive_bf2(h.y),
+                      pack2(v[4], v[5]) & positive_bf2(h.z), pack2(v[6], v[7]) & positive_bf2(h.w));
+}
+
+// v *= d
+__device__ __forceinline__ void scale64(float (&v)[64], float d)
+{
+#pragma unroll
+    for (int i = 0; i < 64; i += 2) {
+        const float2 x = mul2(v[i], v[i + 1], d, d);
+        v[i] = x.x;
+        v[i + 1] = x.y;
+    }
 }
 
 // Adam's parameter step lr m_hat / (sqrt(v_hat) + eps) (Kingma & Ba) with the bias

@@ -344,30 +344,16 @@ struct WNetT {
     }
 
     // ---- epilogues: thread = (row, half), 64 hidden columns each ----
-    // h1 = relu(D + b1), into B and left in v
-    __device__ void epi1(float (&v)[64]) const
+    // H1 = relu(D + b1) into B
+    __device__ void epi1() const
     {
         unsigned char *b = smem + L::sB;
         const float4 *b1 = reinterpret_cast<const float4 *>(vec + L::vb1 + 64 * half);
+        float v[64];
         umma::tmem_ld64(taddr(L::cD + 64u * half), v);
 #pragma unroll
-        for (int g = 0; g < 16; ++g) {
-            const float4 c = b1[g];
-            v[4 * g + 0] = fmaxf(v[4 * g + 0] + c.x, 0.f);
-            v[4 * g + 1] = fmaxf(v[4 * g + 1] + c.y, 0.f);
-            v[4 * g + 2] = fmaxf(v[4 * g + 2] + c.z, 0.f);
-            v[4 * g + 3] = fmaxf(v[4 * g + 3] + c.w, 0.f);
-        }
-#pragma unroll
-        for (int g = 0; g < 8; ++g) *reinterpret_cast<uint4 *>(b + wrow_off(row, 64 * half + 8 * g, L::wB)) = pack8(v + 8 * g);
-    }
-
-    // the mask of h1 > 0
-    static __device__ void mask(const float (&v)[64], uint32_t (&m1)[2])
-    {
-        m1[0] = m1[1] = 0u;
-#pragma unroll
-        for (int i = 0; i < 64; ++i) m1[i / 32] |= (v[i] > 0.f ? 1u : 0u) << (i % 32);
+        for (int g = 0; g < 8; ++g)
+            *reinterpret_cast<uint4 *>(b + wrow_off(row, 64 * half + 8 * g, L::wB)) = bias_relu8(v + 8 * g, b1[2 * g], b1[2 * g + 1]);
     }
 
     // h2 = relu(D + b2) of this thread's 64 columns in place; returns their share of
@@ -377,20 +363,10 @@ struct WNetT {
         const float4 *b2 = reinterpret_cast<const float4 *>(vec + L::vb2 + 64 * half),
                      *w3 = reinterpret_cast<const float4 *>(vec + L::vw3 + 64 * half);
         umma::tmem_ld64(taddr(L::cD + 64u * half), v);
-        float acc[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-        for (int g = 0; g < 16; ++g) {
-            const float4 c = b2[g], w = w3[g];
-            v[4 * g + 0] = fmaxf(v[4 * g + 0] + c.x, 0.f);
-            v[4 * g + 1] = fmaxf(v[4 * g + 1] + c.y, 0.f);
-            v[4 * g + 2] = fmaxf(v[4 * g + 2] + c.z, 0.f);
-            v[4 * g + 3] = fmaxf(v[4 * g + 3] + c.w, 0.f);
-            acc[0] = fmaf(v[4 * g + 0], w.x, acc[0]);
-            acc[1] = fmaf(v[4 * g + 1], w.y, acc[1]);
-            acc[2] = fmaf(v[4 * g + 2], w.z, acc[2]);
-            acc[3] = fmaf(v[4 * g + 3], w.w, acc[3]);
-        }
-        return (acc[0] + acc[1]) + (acc[2] + acc[3]);
+        f32x2 a01 = two(0.f, 0.f), a23 = two(0.f, 0.f);
+        bias_relu_dot64(v, b2, w3, a01, a23);
+        const float2 x = both(a01), y = both(a23);
+        return (x.x + x.y) + (y.x + y.y);
     }
 
     // zeta = w3 . h2 + b3 of this thread's row: the two halves' shares added in order
@@ -415,22 +391,15 @@ struct WNetT {
         dpred = 2.f * (pred - y) * inv_batch;
         dout = pos ? (out > 0.f ? dpred : 0.f) : dpred;
 #pragma unroll
-        for (int g = 0; g < 8; ++g) {
-            const float4 w0 = w3[2 * g], w1 = w3[2 * g + 1];
-            const float wv[8] = {w0.x, w0.y, w0.z, w0.w, w1.x, w1.y, w1.z, w1.w};
-            float d[8];
-#pragma unroll
-            for (int i = 0; i < 8; ++i) d[i] = v[8 * g + i] > 0.f ? dout * wv[i] : 0.f;
-            *reinterpret_cast<uint4 *>(a + wrow_off(row, 64 * half + 8 * g, L::wA)) = pack8(d);
-        }
+        for (int g = 0; g < 8; ++g)
+            *reinterpret_cast<uint4 *>(a + wrow_off(row, 64 * half + 8 * g, L::wA)) = masked_scale8(v + 8 * g, dout, w3[2 * g], w3[2 * g + 1]);
     }
 
     // column sums of h2 dout over the warp's rows (dw3) and, in the first warpgroup, of
     // dout (db3) and dpred (dmu)
     __device__ void out_sums(float (&v)[64], float dout, float dpred, float *gsl) const
     {
-#pragma unroll
-        for (int i = 0; i < 64; ++i) v[i] *= dout;
+        scale64(v, dout);
         const float2 cs = column_sums64(v, lane);
         gsl[2 * lane] += cs.x;
         gsl[2 * lane + 1] += cs.y;
@@ -443,27 +412,26 @@ struct WNetT {
         }
     }
 
-    // dH1 = D (h1 > 0) into A
-    __device__ void back1(const uint32_t (&m1)[2]) const
+    // dH1 = D (h1 > 0) into A, the mask from this thread's own part of H1 in B
+    __device__ void back1() const
     {
         unsigned char *a = smem + L::sA;
+        const unsigned char *b = smem + L::sB;
         float v[64];
         umma::tmem_ld64(taddr(L::cD + 64u * half), v);
 #pragma unroll
-        for (int i = 0; i < 64; ++i) v[i] = ((m1[i / 32] >> (i % 32)) & 1u) ? v[i] : 0.f;
-#pragma unroll
         for (int g = 0; g < 8; ++g)
-            *reinterpret_cast<uint4 *>(a + wrow_off(row, L::U + 64 * half + 8 * g, L::wA)) = pack8(v + 8 * g);
+            *reinterpret_cast<uint4 *>(a + wrow_off(row, L::U + 64 * half + 8 * g, L::wA)) =
+                masked8(v + 8 * g, *reinterpret_cast<const uint4 *>(b + wrow_off(row, 64 * half + 8 * g, L::wB)));
     }
 
     // first two layers of the staged tile; D holds the second-layer pre-activation
     template <class Side>
-    __device__ bool forward12(uint32_t (&m1)[2], bool in_ok, Side side)
+    __device__ bool forward12(bool in_ok, Side side)
     {
         if (!mma([&] { gemm_rows(L::cD, L::sB, L::wB, L::cX, L::sW1, kIn, L::U); }, in_ok, side)) return false;
-        float v[64];
-        epi1(v);
-        return mma([&] { gemm_rows(L::cD, L::sB, L::wB, 0, L::sW2, L::U, L::U); }, true, [&] { mask(v, m1); });
+        epi1();
+        return mma([&] { gemm_rows(L::cD, L::sB, L::wB, 0, L::sW2, L::U, L::U); });
     }
 
     // constant columns of B: ones after H1 (first warpgroup) and after X (second)
@@ -606,8 +574,7 @@ __global__ void __launch_bounds__(kWThreads, 1) wide_train_kernel(WTrainArgs a, 
             const uint32_t next = last ? path_of(st + 1, 0) : path_of(st, rd + 1);
             float y;
             const bool in_ok = n.stage_x(y);
-            uint32_t m1[2];
-            ok = n.forward12(m1, in_ok, [&] {
+            ok = n.forward12(in_ok, [&] {
                 if (has_next) n.prefetch(&tm, a.targ, a.F, next);
             });
             if (ok) {
@@ -617,7 +584,7 @@ __global__ void __launch_bounds__(kWThreads, 1) wide_train_kernel(WTrainArgs a, 
                 ok = n.mma([&] { n.gemm_w2t(WL::cD); }, true, [&] { n.out_sums(v, dout, dpred, my_gsl); });
             }
             if (ok) {
-                n.back1(m1);
+                n.back1();
                 const bool acc = rd > 0;
                 ok = n.mma([&] {
                     n.gemm_paths(WL::cW2, WL::sA, WL::wA, 0, WL::sB, WL::wB, 0, WL::U + 16, acc);
@@ -835,8 +802,7 @@ __global__ void __launch_bounds__(kWThreads, MinBlocks) wide_sweep_kernel(WSweep
         const uint32_t nt = t + stride;
         float y;
         const bool in_ok = n.stage_x(y);
-        uint32_t m1[2];
-        ok = n.forward12(m1, in_ok, [&] {
+        ok = n.forward12(in_ok, [&] {
             if (nt < tiles) n.prefetch(&tm, a.targ, a.F, nt * kRows);
         });
         if (!ok) break;
@@ -1036,16 +1002,9 @@ __global__ void __launch_bounds__(kWThreads, 1) wide_fwd_kernel(WSweepArgs a, co
         float v[64];
         umma::tmem_ld64(n.taddr(128u * (uint32_t)b + 64u * (uint32_t)n.half), v);
 #pragma unroll
-        for (int g = 0; g < 16; ++g) {
-            const float4 c = b1[g];
-            v[4 * g + 0] = fmaxf(v[4 * g + 0] + c.x, 0.f);
-            v[4 * g + 1] = fmaxf(v[4 * g + 1] + c.y, 0.f);
-            v[4 * g + 2] = fmaxf(v[4 * g + 2] + c.z, 0.f);
-            v[4 * g + 3] = fmaxf(v[4 * g + 3] + c.w, 0.f);
-        }
-#pragma unroll
         for (int g = 0; g < 8; ++g)
-            *reinterpret_cast<uint4 *>(bp + wrow_off(n.row, 64 * n.half + 8 * g, L::wB)) = pack8(v + 8 * g);
+            *reinterpret_cast<uint4 *>(bp + wrow_off(n.row, 64 * n.half + 8 * g, L::wB)) =
+                bias_relu8(v + 8 * g, b1[2 * g], b1[2 * g + 1]);
     };
     // this thread's share of w3 . relu(D[b] + b2) (four partial sums, the order of layer2)
     auto share_of = [&](int b) {
@@ -1053,20 +1012,10 @@ __global__ void __launch_bounds__(kWThreads, 1) wide_fwd_kernel(WSweepArgs a, co
                      *w3 = reinterpret_cast<const float4 *>(n.vec + L::vw3 + 64 * n.half);
         float v[64];
         umma::tmem_ld64(n.taddr(128u * (uint32_t)b + 64u * (uint32_t)n.half), v);
-        float acc[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-        for (int g = 0; g < 16; ++g) {
-            const float4 c = b2[g], w = w3[g];
-            v[4 * g + 0] = fmaxf(v[4 * g + 0] + c.x, 0.f);
-            v[4 * g + 1] = fmaxf(v[4 * g + 1] + c.y, 0.f);
-            v[4 * g + 2] = fmaxf(v[4 * g + 2] + c.z, 0.f);
-            v[4 * g + 3] = fmaxf(v[4 * g + 3] + c.w, 0.f);
-            acc[0] = fmaf(v[4 * g + 0], w.x, acc[0]);
-            acc[1] = fmaf(v[4 * g + 1], w.y, acc[1]);
-            acc[2] = fmaf(v[4 * g + 2], w.z, acc[2]);
-            acc[3] = fmaf(v[4 * g + 3], w.w, acc[3]);
-        }
-        return (acc[0] + acc[1]) + (acc[2] + acc[3]);
+        f32x2 a01 = two(0.f, 0.f), a23 = a01;
+        bias_relu_dot64(v, b2, w3, a01, a23);
+        const float2 x = both(a01), y = both(a23);
+        return (x.x + x.y) + (y.x + y.y);
     };
 
     const uint32_t tiles = a.M / kRows, stride = gridDim.x;
