@@ -160,6 +160,7 @@ struct Net {
     uint32_t tmem = 0;
     uint64_t *mbar, *sbar;         // tensor-core completion, input staging (this slot's)
     uint32_t phase = 0, sphase = 0;
+    bool good = true;              // no wait of this thread has given up
     bool pending = false;          // a staging copy was issued and not yet consumed
     int tid, warp, lane, slot, row;
     const float *th, *mean, *istd;
@@ -203,11 +204,12 @@ struct Net {
     }
 
     // one tensor-core step of this slot: operands written -> issue (row 0) ->
-    // completion; the result is the same for the whole slot
-    // side() runs in every thread of the slot after the slot barrier, while the
-    // tensor core works (it may request the next tile's inputs)
+    // completion. side() runs in every thread of the slot after the slot barrier, while
+    // the tensor core works (it may request the next tile's inputs). A wait that gives up
+    // clears `good`, and later ones are skipped; the slot votes once per tile (train_tile,
+    // forward12's callers).
     template <class Issue, class Side>
-    __device__ bool mma(Issue issue, bool pre_ok, Side side)
+    __device__ void mma(Issue issue, Side side)
     {
         umma::fence_proxy_async();
         umma::fence_before_sync();
@@ -218,15 +220,14 @@ struct Net {
             umma::commit(mbar);
         }
         side();
-        const bool done = umma::mbar_wait(mbar, phase, kMbarPolls);
+        if (good) good = umma::mbar_wait(mbar, phase, kMbarPolls);
         phase ^= 1u;
         umma::fence_after_sync();
-        return wg_all(done && pre_ok);
     }
     template <class Issue>
-    __device__ bool mma(Issue issue)
+    __device__ void mma(Issue issue)
     {
-        return mma(issue, true, [] {});
+        mma(issue, [] {});
     }
 
     // D = A B^T: A = K columns of the rows from column c0 (K-major), B = a K-major image [N][K]
@@ -289,10 +290,9 @@ struct Net {
 #pragma unroll
         for (int g = 0; g < kIn / 4; ++g) {
             const float4 m = mv[g], r = iv[g];
-            x[4 * g + 0] = (stage[(4 * g + 0) * kRows + row] - m.x) * r.x;
-            x[4 * g + 1] = (stage[(4 * g + 1) * kRows + row] - m.y) * r.y;
-            x[4 * g + 2] = (stage[(4 * g + 2) * kRows + row] - m.z) * r.z;
-            x[4 * g + 3] = (stage[(4 * g + 3) * kRows + row] - m.w) * r.w;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) x[4 * g + i] = stage[(4 * g + i) * kRows + row];
+            standardise4(x + 4 * g, m, r);
         }
         unsigned char *b = smem + offB();
 #pragma unroll
@@ -406,11 +406,12 @@ struct Net {
     // pre-activation after it. side() runs during the first GEMM, when every thread of
     // the slot is past the staging area (the next tile's copies may be requested).
     template <class Side>
-    __device__ bool forward12(bool in_ok, Side side)
+    __device__ void forward12(bool in_ok, Side side)
     {
-        if (!mma([&] { gemm_rows(dcol(), offB(), L::cX, L::sW1, kIn, U, false); }, in_ok, side)) return false;
+        good = good && in_ok;
+        mma([&] { gemm_rows(dcol(), offB(), L::cX, L::sW1, kIn, U, false); }, side);
         epi1();
-        return mma([&] { gemm_rows(dcol(), offB(), 0, L::sW2, U, U, false); });
+        mma([&] { gemm_rows(dcol(), offB(), 0, L::sW2, U, U, false); });
     }
 
     // forward + backward of one tile whose inputs stage_x has placed (target y, staging
@@ -418,14 +419,14 @@ struct Net {
     __device__ bool train_tile(const TrainArgs &a, const CUtensorMap *tm, float y, bool in_ok, bool first,
                                float inv_batch, bool has_next, uint32_t next_path, float *gsl)
     {
-        if (!forward12(in_ok, [&] {
-                if (has_next) prefetch(tm, a.targ, a.F, next_path);
-            }))
-            return false;
+        forward12(in_ok, [&] {
+            if (has_next) prefetch(tm, a.targ, a.F, next_path);
+        });
         out_back2(a.pos, y, inv_batch, gsl);
-        if (!mma([&] { gemm_rows_w2t(dcol(), offA()); })) return false;
+        mma([&] { gemm_rows_w2t(dcol(), offA()); });
         back1();
-        return mma([&] { gemm_paths(wcol(), offA(), offB(), kRows, !first); });
+        mma([&] { gemm_paths(wcol(), offA(), offB(), kRows, !first); });
+        return wg_all(good);
     }
 
     // this CTA's gradient partial (both slots' DW + the output-layer slots) into P, q order
@@ -743,9 +744,10 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_sweep_kernel(SweepArgs a, con
         const uint32_t nt = t + stride;
         float y;
         const bool in_ok = n.stage_x(y);
-        ok = n.forward12(in_ok, [&] {
+        n.forward12(in_ok, [&] {
             if (nt < tiles) n.prefetch(&tm, a.targ, a.F, nt * kRows);
         });
+        ok = n.wg_all(n.good);
         if (ok && a.mode != 1) {
             float out;
             const float pred = n.output(1, out);
@@ -764,7 +766,8 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_sweep_kernel(SweepArgs a, con
             *reinterpret_cast<uint4 *>(ar + row_off(n.row, U)) =
                 make_uint4(pack2(1.f, y - n.th[L::omu]), 0u, 0u, 0u);
             // G (+)= Z^T Z: M = the 128 columns of the rows (Z in the first U + 2), N = U + 16
-            ok = n.mma([&] { n.gemm_paths(n.wcol(), n.offA(), n.offA(), U + 16, !first); });
+            n.mma([&] { n.gemm_paths(n.wcol(), n.offA(), n.offA(), U + 16, !first); });
+            ok = n.wg_all(n.good);
         }
         if (!ok && n.row == 0) atomicExch(a.err, 2);
         first = false;

@@ -52,6 +52,12 @@ __device__ __forceinline__ float2 add2(float a0, float a1, float b0, float b1)
     asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(two(a0, a1)), "l"(two(b0, b1)));
     return both(r);
 }
+__device__ __forceinline__ float2 sub2(float a0, float a1, float b0, float b1)
+{
+    f32x2 r;
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(two(a0, a1)), "l"(two(b0, b1)));
+    return both(r);
+}
 __device__ __forceinline__ float2 mul2(float a0, float a1, float b0, float b1)
 {
     f32x2 r;
@@ -107,6 +113,17 @@ __device__ __forceinline__ void bias_relu_dot64(float (&v)[64], const float4 *b,
         a01 = fma2(two(v[4 * g], v[4 * g + 1]), two(u.x, u.y), a01);
         a23 = fma2(two(v[4 * g + 2], v[4 * g + 3]), two(u.z, u.w), a23);
     }
+}
+
+// (x[i] - m[i]) r[i] of four values
+__device__ __forceinline__ void standardise4(float *x, const float4 &m, const float4 &r)
+{
+    const float2 a = sub2(x[0], x[1], m.x, m.y), b = sub2(x[2], x[3], m.z, m.w);
+    const float2 c = mul2(a.x, a.y, r.x, r.y), d = mul2(b.x, b.y, r.z, r.w);
+    x[0] = c.x;
+    x[1] = c.y;
+    x[2] = d.x;
+    x[3] = d.y;
 }
 
 // (v > 0 ? d w : 0) of eight values as BF16 (v >= 0: its BF16 is above 0 where it is)

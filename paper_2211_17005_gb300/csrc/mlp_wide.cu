@@ -53,6 +53,7 @@ namespace cva {
 
 namespace {
 
+constexpr int kFwdThreads = 512;   // loss and prediction passes: two groups of 256
 constexpr int kWThreads = 256;
 constexpr uint32_t kGridPolls = 1u << 22;   // default limit of a grid-barrier wait (polls 32 ns apart)
 
@@ -99,16 +100,14 @@ struct WL {
 static_assert(WL::sStage % 128 == 0, "TMA destination must be 128-byte aligned");
 static_assert(WL::bytes <= 227 * 1024, "shared memory");
 
-// Pipelined forward layout of the loss and prediction passes: two B buffers and two
-// TMEM accumulators, so that the first GEMM of a CTA's next tile runs while the
-// output layer of its current tile is evaluated, and kStages staging buffers, so that
-// the inputs of the next kStages tiles are in flight (one CTA per SM).
+// Forward layout of the loss and prediction passes: a B buffer, a TMEM accumulator and two
+// staging buffers for each of the two groups of threads (one CTA per SM).
 struct WLP : WL {
     static constexpr int kStages = 4;
     static constexpr int stage_bytes = (kIn + 1) * kRows * 4;
     static constexpr int sA = -1;
     static constexpr int sB = 0;
-    static constexpr int sB1 = sB + kRows * wB * 2;               // the second B buffer
+    static constexpr int sB1 = sB + kRows * wB * 2;               // the second group's B buffer
     static constexpr int sW1 = sB1 + kRows * wB * 2;
     static constexpr int sW2 = sW1 + U * kIn * 2;
     static constexpr int sVec = sW2 + U * U * 2;
@@ -116,8 +115,8 @@ struct WLP : WL {
     static constexpr int sStats = sStage + kStages * stage_bytes;
     static constexpr int sGsl = sStats + 2 * kIn * 4;
     static constexpr int sOut = sGsl + 8 * 66 * 4;
-    static constexpr int bytes = sOut + 2 * kRows * 4;
-    static constexpr uint32_t tmem_cols = 256;                   // D of tile k at 128 (k & 1)
+    static constexpr int bytes = sOut + 4 * kRows * 4;           // [2 groups][2][128] half outputs
+    static constexpr uint32_t tmem_cols = 256;                   // D of group g at 128 g
 };
 static_assert(WLP::sStage % 128 == 0 && WLP::stage_bytes % 128 == 0 && WLP::sB1 % 1024 == 0,
               "TMA destinations and operand alignment");
@@ -331,10 +330,9 @@ struct WNetT {
         for (int g = 0; g < 4; ++g) {
             const int f0 = 16 * half + 4 * g;
             const float4 m = mv[f0 / 4], r = iv[f0 / 4];
-            x[4 * g + 0] = (stage[(f0 + 0) * kRows + row] - m.x) * r.x;
-            x[4 * g + 1] = (stage[(f0 + 1) * kRows + row] - m.y) * r.y;
-            x[4 * g + 2] = (stage[(f0 + 2) * kRows + row] - m.z) * r.z;
-            x[4 * g + 3] = (stage[(f0 + 3) * kRows + row] - m.w) * r.w;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) x[4 * g + i] = stage[(f0 + i) * kRows + row];
+            standardise4(x + 4 * g, m, r);
         }
         unsigned char *b = smem + L::sB;
         *reinterpret_cast<uint4 *>(b + wrow_off(row, L::cX + 16 * half, L::wB)) = pack8(x);
@@ -910,25 +908,31 @@ __global__ void __launch_bounds__(kWThreads, MinBlocks) wide_sweep_kernel(WSweep
     wide_teardown(n);
 }
 
-// Loss (mode 0) and prediction (mode 2) passes: the forward pass of the trainer's
-// tiles (both warpgroups on one tile, 64 hidden columns each) in a two-stage
-// pipeline over the CTA's tiles k = 0, 1, ...:
-//   stage tile k into B[k & 1] and issue D[k & 1] = X W1^T;
-//   wait for tile k - 1's second GEMM, evaluate its output layer and loss;
-//   wait for tile k's first GEMM, H1 = relu(D + b1) into B[k & 1], issue
-//   D[k & 1] = H1 W2^T.
-// Every row's arithmetic is the trainer's forward pass, and a CTA adds its rows'
-// losses in tile order, so the result does not depend on the pipeline.
-__global__ void __launch_bounds__(kWThreads, 1) wide_fwd_kernel(WSweepArgs a, const __grid_constant__ CUtensorMap tm)
+// Loss (mode 0) and prediction (mode 2) passes: the forward pass of the trainer's tiles.
+// Two groups of 256 threads (two threads per row, 64 hidden columns each) take the CTA's
+// tiles alternately, each with its own B buffer, accumulator and two staging buffers, so
+// that one group's epilogues run while the other waits for the tensor core: per tile
+//   B = X (staged during the previous tile's second GEMM), D = X W1^T;
+//   H1 = relu(D + b1) into B, D = H1 W2^T;
+//   the output layer and the loss of the rows.
+// Every row's arithmetic is the trainer's forward pass, and the losses are added in a fixed
+// order, so the result does not depend on the timing.
+//
+// Bound by the chain of a tile (two tensor-core round trips of about 0.8k cycles and two
+// epilogues) over two groups. One group with a two-stage pipeline took 697 us for 2^20 paths
+// on 24 SMs, longer than the 634 us epoch it runs beside.
+__global__ void __launch_bounds__(kFwdThreads, 1) wide_fwd_kernel(WSweepArgs a, const __grid_constant__ CUtensorMap tm)
 {
     using L = WLP;
     extern __shared__ __align__(1024) unsigned char smem[];
     __shared__ uint32_t s_tmem;
-    __shared__ __align__(8) uint64_t s_mbar[3];   // first GEMM, (unused staging), second GEMM
+    __shared__ __align__(8) uint64_t s_mbar[4];   // tensor-core completion of group g: [2 g]
     __shared__ __align__(8) uint64_t s_sbar[L::kStages];   // staging buffer s complete
-    __shared__ double s_red[8];
+    __shared__ double s_red[kFwdThreads / 32];
     __shared__ int s_flag[2];
     WNetT<L> n(smem, s_mbar);
+    const int grp = n.tid >> 8, gt = n.tid & 255;   // group, thread within it
+    n.half = (n.tid >> 7) & 1;
     wide_setup(n, &s_tmem, s_mbar, a.stats, a.F, false);
     if (n.tid == 0) {
         umma::mbar_init(&s_mbar[2], 1);
@@ -936,136 +940,130 @@ __global__ void __launch_bounds__(kWThreads, 1) wide_fwd_kernel(WSweepArgs a, co
         umma::fence_mbar_init();
     }
     // rows f >= F of every staging buffer stay zero (the copies fill rows < F)
-    for (int i = n.tid; i < L::kStages * (kIn + 1) * kRows; i += kWThreads) {
+    for (int i = n.tid; i < L::kStages * (kIn + 1) * kRows; i += kFwdThreads) {
         const int f = (i / kRows) % (kIn + 1);
         if (f >= a.F && f < kIn) n.stage[i] = 0.f;
     }
     wide_load_params(n, a.theta);
     wide_finish_setup(n, &s_tmem);
-    uint64_t *bar1 = &s_mbar[0], *bar2 = &s_mbar[2];
-    uint32_t ph1 = 0, ph2 = 0;
+    uint64_t *bar = &s_mbar[2 * grp];
+    uint32_t ph = 0;
+    bool ok = true, pend = false;   // pend: a GEMM issued and not yet waited for
+    unsigned char *const bp = smem + (grp ? L::sB1 : L::sB);
+    const int b_off = grp ? L::sB1 : L::sB;
+    const uint32_t dcol = 128u * (uint32_t)grp;
 
-    // tensor-core issue by thread 0 once every thread's operands are written
-    auto issue = [&](uint64_t *bar, auto f) {
+    auto group_sync = [&] { asm volatile("bar.sync %0, 256;" ::"r"(1 + grp) : "memory"); };
+    // tensor-core issue by the group's thread 0 once every thread's operands are written
+    auto issue = [&](auto f) {
         umma::fence_proxy_async();
         umma::fence_before_sync();
-        __syncthreads();
+        group_sync();
         umma::fence_after_sync();
-        if (n.tid == 0) {
+        if (gt == 0 && ok) {
             f();
             umma::commit(bar);
         }
+        pend = true;
     };
-    auto wait = [&](uint64_t *bar, uint32_t &ph) {
-        const bool d = umma::mbar_wait(bar, ph, kMbarPolls);
+    // (a wait that gave up is not repeated: every later one would run out too)
+    auto wait = [&] {
+        if (ok) ok = umma::mbar_wait(bar, ph, kMbarPolls);
         ph ^= 1u;
+        pend = !ok;
         umma::fence_after_sync();
-        return d;
     };
-    // the inputs of the CTA's tile j (paths path0 ...) into staging buffer j % kStages
-    // (one thread issues; called once no thread reads that buffer any more)
-    auto request = [&](uint32_t j, uint32_t path0) {
-        if (n.tid == 32) {
-            uint64_t *sb = &s_sbar[j % L::kStages];
-            const uint32_t dst = n.saddr(L::sStage + (int)(j % L::kStages) * L::stage_bytes);
-            umma::mbar_arrive_expect_tx(sb, (uint32_t)(a.F + 1) * kRows * 4u);
-            umma::tma_load_2d(dst, &tm, (int32_t)path0, 0, sb);
-            umma::bulk_g2s(dst + kIn * kRows * 4u, a.targ + path0, kRows * 4u, sb);
+    // the inputs of the group's tile i (paths path0 ...) into its staging buffer i % 2
+    // (one thread issues; called once no thread of the group reads that buffer any more)
+    auto request = [&](uint32_t i, uint32_t path0) {
+        if (gt == 32 && ok) {
+            const int q = 2 * grp + (int)(i & 1u);
+            const uint32_t dst = n.saddr(L::sStage + q * L::stage_bytes);
+            umma::mbar_arrive_expect_tx(&s_sbar[q], (uint32_t)(a.F + 1) * kRows * 4u);
+            umma::tma_load_2d(dst, &tm, (int32_t)path0, 0, &s_sbar[q]);
+            umma::bulk_g2s(dst + kIn * kRows * 4u, a.targ + path0, kRows * 4u, &s_sbar[q]);
         }
     };
-    // wait for tile j's inputs; this thread's 16 standardised inputs into the X columns
-    // of B[b]; y receives the target
-    auto stage_into = [&](uint32_t j, int b, float &y) {
-        const bool got = umma::mbar_wait(&s_sbar[j % L::kStages], (j / L::kStages) & 1u, kMbarPolls);
-        const float *stg = reinterpret_cast<const float *>(smem + L::sStage + (int)(j % L::kStages) * L::stage_bytes);
+    // wait for tile i's inputs; this thread's 16 standardised inputs into the X columns of B;
+    // y receives the target
+    auto stage_into = [&](uint32_t i, float &y) {
+        const int q = 2 * grp + (int)(i & 1u);
+        if (ok) ok = umma::mbar_wait(&s_sbar[q], (i >> 1) & 1u, kMbarPolls);
+        const float *stg = reinterpret_cast<const float *>(smem + L::sStage + q * L::stage_bytes);
         const float4 *mv = reinterpret_cast<const float4 *>(n.mean), *iv = reinterpret_cast<const float4 *>(n.istd);
         float x[16];
 #pragma unroll
         for (int g = 0; g < 4; ++g) {
             const int f0 = 16 * n.half + 4 * g;
             const float4 m = mv[f0 / 4], r = iv[f0 / 4];
-            x[4 * g + 0] = (stg[(f0 + 0) * kRows + n.row] - m.x) * r.x;
-            x[4 * g + 1] = (stg[(f0 + 1) * kRows + n.row] - m.y) * r.y;
-            x[4 * g + 2] = (stg[(f0 + 2) * kRows + n.row] - m.z) * r.z;
-            x[4 * g + 3] = (stg[(f0 + 3) * kRows + n.row] - m.w) * r.w;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) x[4 * g + i] = stg[(f0 + i) * kRows + n.row];
+            standardise4(x + 4 * g, m, r);
         }
-        unsigned char *bp = smem + (b ? L::sB1 : L::sB);
         *reinterpret_cast<uint4 *>(bp + wrow_off(n.row, L::cX + 16 * n.half, L::wB)) = pack8(x);
         *reinterpret_cast<uint4 *>(bp + wrow_off(n.row, L::cX + 16 * n.half + 8, L::wB)) = pack8(x + 8);
         y = stg[kIn * kRows + n.row];
-        return got;
     };
-    // H1 = relu(D[b] + b1) of this thread's 64 columns into B[b]
-    auto epi1_into = [&](int b) {
-        unsigned char *bp = smem + (b ? L::sB1 : L::sB);
+    // H1 = relu(D + b1) of this thread's 64 columns into B
+    auto epi1_into = [&] {
         const float4 *b1 = reinterpret_cast<const float4 *>(n.vec + L::vb1 + 64 * n.half);
         float v[64];
-        umma::tmem_ld64(n.taddr(128u * (uint32_t)b + 64u * (uint32_t)n.half), v);
+        umma::tmem_ld64(n.taddr(dcol + 64u * (uint32_t)n.half), v);
 #pragma unroll
         for (int g = 0; g < 8; ++g)
             *reinterpret_cast<uint4 *>(bp + wrow_off(n.row, 64 * n.half + 8 * g, L::wB)) =
                 bias_relu8(v + 8 * g, b1[2 * g], b1[2 * g + 1]);
     };
-    // this thread's share of w3 . relu(D[b] + b2) (four partial sums, the order of layer2)
-    auto share_of = [&](int b) {
+    // this thread's share of w3 . relu(D + b2) (four partial sums, the order of layer2)
+    auto share_of = [&] {
         const float4 *b2 = reinterpret_cast<const float4 *>(n.vec + L::vb2 + 64 * n.half),
                      *w3 = reinterpret_cast<const float4 *>(n.vec + L::vw3 + 64 * n.half);
         float v[64];
-        umma::tmem_ld64(n.taddr(128u * (uint32_t)b + 64u * (uint32_t)n.half), v);
+        umma::tmem_ld64(n.taddr(dcol + 64u * (uint32_t)n.half), v);
         f32x2 a01 = two(0.f, 0.f), a23 = a01;
         bias_relu_dot64(v, b2, w3, a01, a23);
         const float2 x = both(a01), y = both(a23);
         return (x.x + x.y) + (y.x + y.y);
     };
 
-    const uint32_t tiles = a.M / kRows, stride = gridDim.x;
-    const uint32_t K = blockIdx.x < tiles ? (tiles - 1 - blockIdx.x) / stride + 1 : 0;   // this CTA's tiles
+    // the group's tiles: first, first + stride, ...
+    const uint32_t tiles = a.M / kRows, stride = 2u * gridDim.x, first = blockIdx.x + (uint32_t)grp * gridDim.x;
+    const uint32_t K = first < tiles ? (tiles - 1 - first) / stride + 1 : 0;
+    auto path_of = [&](uint32_t i) { return (first + i * stride) * kRows; };
     double acc = 0.0;
-    bool ok = true, pend2 = false;   // pend2: a second GEMM issued and not yet waited for
-    float y_prev = 0.f, y = 0.f;
-    uint32_t requested = 0, consumed = 0;   // tiles whose inputs were requested / read
-    for (; requested < K && requested < (uint32_t)L::kStages; ++requested)
-        request(requested, (blockIdx.x + requested * stride) * kRows);
-    for (uint32_t k = 0; k <= K; ++k) {
-        const int b = (int)(k & 1u);
-        const uint32_t t = blockIdx.x + k * stride;
-        if (k < K) {
-            ok = stage_into(k, b, y) && ok;
-            ++consumed;
-            issue(bar1, [&] { n.gemm_rows(128u * (uint32_t)b, b ? L::sB1 : L::sB, L::wB, L::cX, L::sW1, kIn, L::U); });
-            if (requested < K) {   // every thread is past buffer k % kStages: tile k + kStages into it
-                request(requested, (blockIdx.x + requested * stride) * kRows);
-                ++requested;
+    float y = 0.f, y_next = 0.f;
+    float *so = reinterpret_cast<float *>(smem + L::sOut) + grp * 2 * kRows;
+    for (uint32_t i = 0; i < K && i < 2; ++i) request(i, path_of(i));
+    if (K > 0) stage_into(0, y_next);
+    for (uint32_t i = 0; i < K; ++i) {
+        y = y_next;
+        issue([&] { n.gemm_rows(dcol, b_off, L::wB, L::cX, L::sW1, kIn, L::U); });
+        if (i + 2 < K) request(i + 2, path_of(i + 2));   // every thread has read buffer i % 2
+        wait();
+        epi1_into();
+        issue([&] { n.gemm_rows(dcol, b_off, L::wB, 0, L::sW2, L::U, L::U); });
+        if (i + 1 < K) stage_into(i + 1, y_next);   // the X columns are free since the first GEMM
+        wait();
+        // zeta = w3 . h2 + b3: the two halves' shares added in order (the shares are read
+        // before the barriers of the next tile, which the next write follows)
+        so[n.half * kRows + n.row] = share_of();
+        group_sync();
+        const float pred = fmaxf((so[n.row] + so[kRows + n.row]) + n.vec[L::vb3], 0.f) + n.vec[L::vmu];
+        if (n.half == 0) {
+            if (a.mode == 2) {
+                if (a.pred) a.pred[path_of(i) + n.row] = pred;
+            } else {
+                acc += (double)((pred - y) * (pred - y));
             }
-        }
-        if (k > 0) {   // the output layer of tile k - 1
-            ok = wait(bar2, ph2) && ok;
-            pend2 = false;
-            const float pred = fmaxf(n.zeta(share_of(b ^ 1)), 0.f) + n.vec[L::vmu];
-            if (n.half == 0) {
-                if (a.mode == 2) {
-                    if (a.pred) a.pred[(t - stride) * kRows + n.row] = pred;
-                } else {
-                    acc += (double)((pred - y_prev) * (pred - y_prev));
-                }
-            }
-        }
-        if (k < K) {
-            ok = wait(bar1, ph1) && ok;
-            epi1_into(b);
-            issue(bar2, [&] { n.gemm_rows(128u * (uint32_t)b, b ? L::sB1 : L::sB, L::wB, 0, L::sW2, L::U, L::U); });
-            pend2 = true;
-        }
-        y_prev = y;
-        if (!__syncthreads_and(ok)) {
-            ok = false;
-            break;
         }
     }
-    if (pend2) (void)wait(bar2, ph2);   // a loop left early: no tensor-core work outlives the CTA
-    for (uint32_t j = consumed; j < requested; ++j)   // nor any input copy
-        (void)umma::mbar_wait(&s_sbar[j % L::kStages], (j / L::kStages) & 1u, kMbarPolls);
-    if (!ok && n.tid == 0) atomicExch(a.err, 2);
+    // after a wait that gave up: no tensor-core work and no input copy outlives the CTA
+    // (bounded)
+    if (pend) (void)umma::mbar_wait(bar, ph ^ 1u, kMbarPolls);
+    if (!ok)
+        for (int q = 2 * grp; q < 2 * grp + 2; ++q)
+            for (uint32_t par = 0; par < 2; ++par) (void)umma::mbar_wait(&s_sbar[q], par, kMbarPolls >> 6);
+    if (!ok && gt == 0) atomicExch(a.err, 2);
     umma::fence_before_sync();
     __syncthreads();
     umma::fence_after_sync();
@@ -1078,7 +1076,7 @@ __global__ void __launch_bounds__(kWThreads, 1) wide_fwd_kernel(WSweepArgs a, co
         __syncthreads();
         if (n.tid == 0) {
             double bsum = 0.0;
-            for (int w = 0; w < 8; ++w) bsum += s_red[w];
+            for (int w = 0; w < kFwdThreads / 32; ++w) bsum += s_red[w];
             a.part[blockIdx.x] = bsum;
             __threadfence();
             s_flag[0] = atomicAdd(a.count, 1u) == gridDim.x - 1;
@@ -1097,7 +1095,7 @@ __global__ void __launch_bounds__(kWThreads, 1) wide_fwd_kernel(WSweepArgs a, co
             }
             __syncthreads();
             if (s_flag[1])
-                for (int p = n.tid; p < L::NP; p += kWThreads) a.best[p] = __ldg(a.theta + p);
+                for (int p = n.tid; p < L::NP; p += kFwdThreads) a.best[p] = __ldg(a.theta + p);
         }
     }
     wide_teardown(n);
@@ -1311,7 +1309,7 @@ cva_status mlp_wide_fit_dates(const float *feat0, size_t feat_stride, const floa
                 CVA_CUDA_TRY(cudaEventRecord(w.ev_train, st));
                 CVA_CUDA_TRY(cudaStreamWaitEvent(sst, w.ev_train, 0));
             }
-            wide_fwd_kernel<<<e == epochs ? fwd_grid : side_grid, kWThreads, WLP::bytes, sst>>>(sw, tm);
+            wide_fwd_kernel<<<e == epochs ? fwd_grid : side_grid, kFwdThreads, WLP::bytes, sst>>>(sw, tm);
             CVA_CUDA_TRY(cudaGetLastError());
         }
         // the best parameters are known once the last loss pass ran: the next date (st)
@@ -1325,7 +1323,7 @@ cva_status mlp_wide_fit_dates(const float *feat0, size_t feat_stride, const floa
             pv.mode = 2;
             pv.theta = best[par];
             pv.pred = pred0 + (size_t)d * M;
-            wide_fwd_kernel<<<side_grid, kWThreads, WLP::bytes, sst>>>(pv, tm);
+            wide_fwd_kernel<<<side_grid, kFwdThreads, WLP::bytes, sst>>>(pv, tm);
             CVA_CUDA_TRY(cudaGetLastError());
         }
         if (d == 0)
