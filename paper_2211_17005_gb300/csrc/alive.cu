@@ -270,12 +270,14 @@ __global__ void __launch_bounds__(256) alive_solve_kernel(AliveArgs a)
     }
 }
 
+constexpr int kStatMaxSmem = 110 * 1024;   // two blocks a multiprocessor
+
 // paths per tile: 32 up to four counterparties, else 16 (128 threads), fewer where the
 // dates' columns would not fit shared memory twice over
 int stat_lg(int C, int n)
 {
     int lg = C <= 4 ? 5 : 4;
-    while (lg > 2 && stat_shape(lg, C, n).bytes > 110 * 1024) --lg;
+    while (lg > 2 && stat_shape(lg, C, n).bytes > kStatMaxSmem) --lg;
     return lg;
 }
 
@@ -283,9 +285,9 @@ template <int C>
 cva_status launch_stats(const AliveArgs &a, bool capturing, cudaStream_t st)
 {
     const StatShape sh = stat_shape(a.lg, C, a.n);
-    if (!capturing)
+    if (!capturing)   // (the most any date count takes, so that no call lowers another's limit)
         CVA_CUDA_TRY(cudaFuncSetAttribute(alive_stats_kernel<C>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                          (int)sh.bytes));
+                                          kStatMaxSmem));
     alive_stats_kernel<C><<<a.nblk, sh.threads, sh.bytes, st>>>(a);
     CVA_CUDA_TRY(cudaGetLastError());
     return CVA_OK;

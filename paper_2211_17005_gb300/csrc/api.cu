@@ -979,30 +979,29 @@ cva_status cva_grad_cva0(const cva_model_desc *model, const cva_portfolio_desc *
     const size_t Mz = M;
     const unsigned blocks = (unsigned)((M + 127) / 128);
     cudaStream_t cs = reinterpret_cast<cudaStream_t>(stream);
-    // the compiled shapes take the paths in equal ranges whose arrays fit kAdjScratch; the
+    // the compiled shapes take the paths in equal ranges whose arrays fit a limit; the
     // run-time shapes take them at once, with checkpoints
     uint64_t ranges = 1, Mr = M;
     const size_t nsum = s.generic ? (size_t)NPAR + 1 : (size_t)(2 * E + 1 + NPAR);
-    if (!s.generic) {
-        for (;;) {
+    auto plan = [&](size_t limit) -> cva_status {
+        for (ranges = 1;;) {
             Mr = (M + ranges - 1) / ranges;
-            st = launch_adjoint(s, b, seed, k0, (uint32_t)Mr, cs);   // without scratch: its size
-            if (st != CVA_OK) {
-                cva_sim_destroy(hs);
-                return st;
-            }
-            if (b.scratch_bytes <= kAdjScratch || Mr <= 256) break;
-            ranges = std::max(ranges + 1, ranges * (b.scratch_bytes / kAdjScratch));
+            const cva_status r = launch_adjoint(s, b, seed, k0, (uint32_t)Mr, cs);   // without scratch: its size
+            if (r != CVA_OK) return r;
+            if (b.scratch_bytes <= limit || Mr <= 256) break;
+            ranges = std::max(ranges + 1, ranges * (b.scratch_bytes / limit));
         }
         Mr = (Mr + 255) / 256 * 256;   // whole blocks
         ranges = (M + Mr - 1) / Mr;
         size_t most = 0;   // the full ranges and the last one
         for (uint64_t m : {std::min<uint64_t>(Mr, M), M - (ranges - 1) * Mr}) {
-            launch_adjoint(s, b, seed, k0, (uint32_t)m, cs);
+            const cva_status r = launch_adjoint(s, b, seed, k0, (uint32_t)m, cs);
+            if (r != CVA_OK) return r;
             most = std::max(most, b.scratch_bytes);
         }
         b.scratch_bytes = most;
-    }
+        return CVA_OK;
+    };
     auto cleanup = [&]() {
         cudaFree(b.dzc);
         cudaFree(b.dfix);
@@ -1017,14 +1016,25 @@ cva_status cva_grad_cva0(const cva_model_desc *model, const cva_portfolio_desc *
         cudaFree(b.scratch);
         cva_sim_destroy(hs);
     };
+    // less memory free than the arrays of the widest ranges: narrower ones
+    for (size_t limit = kAdjScratch; !s.generic && !b.scratch; limit /= 2) {
+        st = plan(limit);
+        if (st == CVA_OK && dev_alloc(&b.scratch, b.scratch_bytes) != CVA_OK) {
+            cudaGetLastError();   // (the failed allocation's)
+            if (Mr <= 256 || limit < 2) st = CVA_ENOMEM;
+        }
+        if (st != CVA_OK) {
+            cleanup();
+            return st;
+        }
+    }
     if (dev_alloc(&b.dzc, dzc.size()) != CVA_OK || dev_alloc(&b.dfix, dfix.size()) != CVA_OK ||
         dev_alloc(&b.ddrift, ddrift.size()) != CVA_OK || dev_alloc(&b.rho, rho.size()) != CVA_OK ||
         dev_alloc(&b.sig, sig.size()) != CVA_OK || dev_alloc(&b.sum, nsum * ranges) != CVA_OK ||
         (s.generic && (dev_alloc(&b.ckpt, (size_t)b.nseg * NV * Mz) != CVA_OK ||
                        dev_alloc(&b.ckpt_I0, (size_t)b.nseg * Mz) != CVA_OK ||
                        dev_alloc(&b.fixr, (size_t)(periods + 1) * E * Mz) != CVA_OK ||
-                       dev_alloc(&b.part, (size_t)blocks * (NPAR + 1)) != CVA_OK)) ||
-        (!s.generic && dev_alloc(&b.scratch, b.scratch_bytes) != CVA_OK)) {
+                       dev_alloc(&b.part, (size_t)blocks * (NPAR + 1)) != CVA_OK))) {
         cleanup();
         return CVA_ENOMEM;
     }

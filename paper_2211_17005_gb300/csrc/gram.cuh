@@ -6,6 +6,7 @@
 #include <stdint.h>
 
 #include <algorithm>
+#include <atomic>
 
 #include "cva_internal.h"
 
@@ -299,6 +300,33 @@ inline void gram_chunks(uint64_t M, int groups, int target, uint64_t min_rows, u
     *chunks = (M + *rows - 1) / *rows;
 }
 
+// Lets every form take the shared memory of its widest call, once per device: a limit that
+// followed the call's own width would be lowered under another thread's launch, or under a
+// captured call of a wider system. (Inside a capture it is left as it is.)
+inline cva_status gram_allow_smem(cudaStream_t st)
+{
+    static std::atomic<uint64_t> ready{0};
+    int dev = 0;
+    CVA_CUDA_TRY(cudaGetDevice(&dev));
+    const uint64_t bit = dev < 64 ? 1ull << dev : 0ull;
+    if (ready.load(std::memory_order_acquire) & bit) return CVA_OK;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    CVA_CUDA_TRY(cudaStreamIsCapturing(st, &cap));
+    if (cap != cudaStreamCaptureStatusNone) return CVA_OK;
+    auto allow = [](auto kern, size_t bytes) {
+        return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    };
+    constexpr size_t f = sizeof(float);
+    CVA_CUDA_TRY(allow(gram_kernel<512, 320, 2, true>, 3 * 16 * 512 * f));
+    CVA_CUDA_TRY(allow(gram_kernel<512, 320, 2, false>, 3 * 16 * 512 * f));
+    CVA_CUDA_TRY(allow(gram_kernel<256, 320, 2, true>, 3 * 32 * 256 * f));
+    CVA_CUDA_TRY(allow(gram_kernel<256, 320, 2, false>, 3 * 32 * 256 * f));
+    CVA_CUDA_TRY(allow(gram_kernel<256, 640, 1, true>, 3 * kGramMaxCols * 256 * f));
+    CVA_CUDA_TRY(allow(gram_kernel<256, 640, 1, false>, 3 * kGramMaxCols * 256 * f));
+    ready.fetch_or(bit, std::memory_order_release);
+    return CVA_OK;
+}
+
 // Launch: the widest form whose registers and tiles fit, two blocks per multiprocessor
 // up to 32 columns (10 warps), one beyond; 512-row tiles where three column blocks or
 // fewer leave shared memory for them. 16-byte copies where every column allows them.
@@ -318,11 +346,9 @@ inline cva_status launch_gram(GramArgs &a, int groups, cudaStream_t st)
     const int threads = 32 * a.nblk * a.RG;
     const int TR = nb <= 2 ? 512 : 256;
     const size_t smem = std::max((size_t)3 * nb * 8 * TR * sizeof(float), (size_t)a.nblk * a.RG * 64 * sizeof(double));
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    CVA_CUDA_TRY(cudaStreamIsCapturing(st, &cap));
+    const cva_status allowed = gram_allow_smem(st);
+    if (allowed != CVA_OK) return allowed;
     auto go = [&](auto kern) -> cva_status {
-        if (cap == cudaStreamCaptureStatusNone)
-            CVA_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
         kern<<<grid, threads, smem, st>>>(a);
         CVA_CUDA_TRY(cudaGetLastError());
         return CVA_OK;
