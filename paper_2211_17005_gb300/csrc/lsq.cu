@@ -220,8 +220,12 @@ static LsqPlan lsq_plan(int F, int basis, int nt, uint64_t M, int groups, int ta
     p.m = basis == CVA_BASIS_POLY2 ? 3 : F + 1;
     p.rows = p.m + (nt == 1);
     p.stride = (size_t)tri_index(p.m + nt, p.rows - 1, p.m + nt - 1) + 1;
-    // 1024 rows a block at least, 512 where that would leave multiprocessors without work
-    gram_chunks(M, groups, target > 0 ? target : 2432, (uint64_t)groups * ((M + 1023) / 1024) < 304 ? 512 : 1024,
+    // 1024 rows a block at least, 512 where that would leave multiprocessors without work; the
+    // quadratic basis takes a quarter of the blocks, whose reduction otherwise outweighs the
+    // few products of their rows (49 dates of 2^14 paths: 17 us with 784 blocks)
+    target = target > 0 ? target : 2432;
+    if (basis == CVA_BASIS_POLY2) target = std::max(target / 4, 1);
+    gram_chunks(M, groups, target, (uint64_t)groups * ((M + 1023) / 1024) < 304 ? 512 : 1024,
                 &p.rows_per_chunk, &p.chunks);
     p.reduce = p.chunks > 48;
     p.doubles = (size_t)groups * (p.chunks + p.reduce) * p.stride + 2 * (size_t)groups * nt * p.m + (size_t)groups;

@@ -29,19 +29,21 @@ __device__ __forceinline__ uint4 philox4x32_10(uint4 c, uint32_t k0, uint32_t k1
     return c;
 }
 
-// Uniform on (0,1): (m + 1/2) 2^-23 with m the top 23 bits; exact in binary32.
-__device__ __forceinline__ float uniform23(uint32_t x)
-{
-    return (__uint2float_rn(x >> 9) + 0.5f) * 1.1920928955078125e-07f;
-}
+// 1 + m 2^-23 with m the top 23 bits of x: the bits of m below the exponent of 1 (no
+// integer-to-float conversion, whose pipe is a quarter as wide).
+__device__ __forceinline__ float one_plus23(uint32_t x) { return __uint_as_float(0x3f800000u | (x >> 9)); }
 
-// Box-Muller on a pair of uniforms: (rad cos 2 pi u2, rad sin 2 pi u2).
+// Uniform on (0,1): (m + 1/2) 2^-23 = (1 + m 2^-23) - (1 - 2^-24); exact in binary32, as
+// both operands and the result are.
+__device__ __forceinline__ float uniform23(uint32_t x) { return one_plus23(x) - 0.99999994039535522f; }
+
+// Box-Muller on a pair of uniforms: (rad cos 2 pi u2, rad sin 2 pi u2). 2 u2 in one exact
+// multiply-add.
 __device__ __forceinline__ void box_muller(uint32_t a, uint32_t b, float &z0, float &z1)
 {
-    const float u1 = uniform23(a), u2 = uniform23(b);
-    const float rad = sqrtf(-2.0f * logf(u1));
+    const float rad = sqrtf(-2.0f * logf(uniform23(a)));
     float s, c;
-    sincospif(2.0f * u2, &s, &c);
+    sincospif(fmaf(2.0f, one_plus23(b), -1.9999998807907104f), &s, &c);
     z0 = rad * c;
     z1 = rad * s;
 }
