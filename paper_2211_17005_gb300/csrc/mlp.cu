@@ -434,6 +434,13 @@ struct Net {
     {
         const int q4 = warp & 3, wg = warp >> 2;
         const uint32_t lanes = (uint32_t)(q4 * 32) << 16;
+        // (by the warps with the fewest TMEM columns below)
+        if (const int t = tid - 64; t >= 0 && t < U + 2) {
+            float s = 0.f;
+#pragma unroll
+            for (int w = 0; w < 8; ++w) s += gsl[w * (U + 2) + t];
+            P[t < U ? L::ow3 + t : (t == U ? L::ob3 : L::omu)] = s;
+        }
         // every TMEM load of the thread is issued before the one wait; a chunk past the
         // thread's range reads allocated columns whose values are not used
         if (q4 < 2) {   // rows o < U: dW2[o][:] at columns [0, U), db2[o] at column U
@@ -487,13 +494,6 @@ struct Net {
                     }
                 }
         }
-        if (tid < U + 2) {
-            float s = 0.f;
-            for (int w = 0; w < 8; ++w) s += gsl[w * (U + 2) + tid];
-            P[tid < U ? L::ow3 + tid : (tid == U ? L::ob3 : L::omu)] = s;
-        }
-        __syncthreads();
-        for (int i = tid; i < 8 * (U + 2); i += kThreads) gsl[i] = 0.f;
     }
 };
 
@@ -551,14 +551,48 @@ __device__ void net_teardown(Net<U> &n)
 // Batch b covers paths [b * P, (b + 1) * P), P = tiles_per_batch * 128; in each
 // step the cluster's 2 CL slots take the batch's tiles round-robin.
 //
+// W consecutive words (aligned to them) in one access
+template <int W>
+__device__ __forceinline__ void load_words(const float *p, float *v)
+{
+    if constexpr (W == 4) {
+        const float4 x = *reinterpret_cast<const float4 *>(p);
+        v[0] = x.x, v[1] = x.y, v[2] = x.z, v[3] = x.w;
+    } else {
+        const float2 x = *reinterpret_cast<const float2 *>(p);
+        v[0] = x.x, v[1] = x.y;
+    }
+}
+template <int W>
+__device__ __forceinline__ void store_words(float *p, const float *v)
+{
+    if constexpr (W == 4) *reinterpret_cast<float4 *>(p) = make_float4(v[0], v[1], v[2], v[3]);
+    else *reinterpret_cast<float2 *>(p) = make_float2(v[0], v[1]);
+}
+template <int W>
+__device__ __forceinline__ void load_words_cg(const float *p, float *v)
+{
+#pragma unroll
+    for (int i = 0; i < W; i += 2) {
+        const float2 x = __ldcg(reinterpret_cast<const float2 *>(p + i));
+        v[i] = x.x, v[i + 1] = x.y;
+    }
+}
+template <int W>
+__device__ __forceinline__ void store_words_cg(float *p, const float *v)
+{
+#pragma unroll
+    for (int i = 0; i < W; i += 2) __stcg(reinterpret_cast<float2 *>(p + i), make_float2(v[i], v[i + 1]));
+}
+
 // The exchange of one Adam step moves data only by bulk copies between the CTAs'
 // shared memories, each completing on the receiver's mbarrier (no cluster-wide
 // barrier inside the step loop):
 //   1. every CTA writes its gradient partial (column order q) and copies slice c
 //      of it into CTA c's receive buffer, at row = its own rank;
 //   2. CTA c waits for the CL slices of its own slice, sums them in CTA order,
-//      applies Adam (moments in global memory, requested before the wait) and
-//      writes the new values into its own copy of the parameters;
+//      applies Adam (moments in registers where a thread's share fits) and writes
+//      the new values into its own copy of the parameters;
 //   3. CTA c copies that slice into every other CTA's copy of the parameters;
 //      every CTA waits for the other CL - 1 slices before its next step.
 // A CTA's next partial reaches an owner only after that CTA received the owner's
@@ -609,6 +643,34 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_train_kernel(TrainArgs a, con
     const uint32_t xbar_part = umma::smem_u32(&s_xbar[0]), xbar_par = umma::smem_u32(&s_xbar[1]);
     uint32_t ph_part = 0, ph_par = 0;
 
+    // the copies of an exchange: one lane of every warp at a time, the CTA after this one first
+    const uint32_t copy_i = (uint32_t)(n.warp + 8 * n.lane), copy_to = (rank + 1 + copy_i) % CL;
+
+    // Adam moments of this thread's part of the owned slice: 2 or 4 entries, in registers over
+    // the launch's steps where that covers the slice (clusters of 8 and 16), else in global
+    // memory (requested before the wait for the partials they meet)
+    const bool once = S <= 4 * kThreads;
+    float am[4] = {}, av[4] = {};
+    auto moments = [&](auto width, int q0, bool fresh) {
+        constexpr int W = decltype(width)::value;
+        if (q0 < hi && !fresh) {
+            load_words_cg<W>(a.adam_m + q0, am);
+            load_words_cg<W>(a.adam_v + q0, av);
+        } else {   // the moments of a date start at zero
+#pragma unroll
+            for (int i = 0; i < W; ++i) am[i] = av[i] = 0.f;
+        }
+    };
+    auto keep = [&](auto width, int q0) {
+        constexpr int W = decltype(width)::value;
+        if (q0 < hi) {
+            store_words_cg<W>(a.adam_m + q0, am);
+            store_words_cg<W>(a.adam_v + q0, av);
+        }
+    };
+    if (S <= 2 * kThreads) moments(std::integral_constant<int, 2>{}, lo + 2 * n.tid, a.step0 == 0);
+    else if (once) moments(std::integral_constant<int, 4>{}, lo + 4 * n.tid, a.step0 == 0);
+
     // bias corrections 1 - beta^t of Adam, as running powers of beta
     float b1t = powf(a.beta1, (float)a.step0), b2t = powf(a.beta2, (float)a.step0);
     bool ok = true, staged = false, in_ok_next = true;
@@ -632,10 +694,11 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_train_kernel(TrainArgs a, con
         n.write_partial(part, gsl, h0, h1);
         umma::fence_proxy_async();   // the partial is read by the bulk copies (async proxy)
         __syncthreads();
-        if (n.tid < (int)CL)   // slice c of this CTA's partial -> CTA c's receive buffer, row `rank`
-            umma::bulk_s2c(umma::map_rank(recv_s + rank * slice_bytes, (uint32_t)n.tid),
-                           part_s + (uint32_t)n.tid * slice_bytes, slice_bytes,
-                           umma::map_rank(xbar_part, (uint32_t)n.tid));
+        if (copy_i < CL) {   // slice c of this CTA's partial -> CTA c's receive buffer, row `rank`
+            umma::bulk_s2c(umma::map_rank(recv_s + rank * slice_bytes, copy_to), part_s + copy_to * slice_bytes,
+                           slice_bytes, umma::map_rank(xbar_part, copy_to));
+        }
+        for (int i = n.tid; i < 8 * (U + 2); i += kThreads) gsl[i] = 0.f;   // (read by write_partial)
 
         // the next step's first tile: its inputs into the X columns of B (free since the
         // weight-gradient GEMM completed) while the exchange runs
@@ -644,18 +707,10 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_train_kernel(TrainArgs a, con
             staged = true;
         }
 
-        // the owned slice: Adam moments requested before the wait for the partials
         const int step = a.step0 + st + 1;
-        const bool fresh = a.step0 == 0 && st == 0;   // the moments of a date start at zero
         b1t *= a.beta1;
         b2t *= a.beta2;
         const float inv_bc1 = 1.f / (1.f - b1t), inv_bc2 = 1.f / (1.f - b2t);
-        const int q_first = lo + 4 * n.tid;
-        float4 m4 = make_float4(0.f, 0.f, 0.f, 0.f), v4 = m4;
-        if (q_first < hi && !fresh) {
-            m4 = __ldcg(reinterpret_cast<const float4 *>(a.adam_m + q_first));
-            v4 = __ldcg(reinterpret_cast<const float4 *>(a.adam_v + q_first));
-        }
         if (n.tid == 0) umma::mbar_arrive_expect_tx(&s_xbar[0], (uint32_t)L::NPpad * 4u);
         if (!umma::mbar_wait(&s_xbar[0], ph_part, kMbarPolls)) {
             ok = false;
@@ -669,37 +724,40 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_train_kernel(TrainArgs a, con
             v = a.beta2 * v + (1.f - a.beta2) * g * g;
             return th[q] - adam_delta(m, v, inv_bc1, inv_bc2, a.lr, a.eps);
         };
-        for (int q0 = q_first; q0 < hi; q0 += 4 * kThreads) {
-            if (q0 != q_first && !fresh) {
-                m4 = __ldcg(reinterpret_cast<const float4 *>(a.adam_m + q0));
-                v4 = __ldcg(reinterpret_cast<const float4 *>(a.adam_v + q0));
-            } else if (q0 != q_first) {
-                m4 = v4 = make_float4(0.f, 0.f, 0.f, 0.f);
-            }
-            const float4 *rv = reinterpret_cast<const float4 *>(recv + (q0 - lo));
-            float4 pv[kMaxCluster];
+        auto update = [&](auto width) {   // W entries a thread
+            constexpr int W = decltype(width)::value;
+            for (int q0 = lo + W * n.tid; q0 < hi; q0 += W * kThreads) {
+                if (!once) {
+                    moments(std::integral_constant<int, W>{}, q0, a.step0 == 0 && st == 0);
+                }
+                float pv[kMaxCluster][W], g[W], t[W];
 #pragma unroll
-            for (int c = 0; c < kMaxCluster; ++c)   // all loads in flight
-                pv[c] = (uint32_t)c < CL ? rv[c * (S / 4)] : make_float4(0.f, 0.f, 0.f, 0.f);
-            float4 g = make_float4(0.f, 0.f, 0.f, 0.f);
+                for (int c = 0; c < kMaxCluster; ++c)   // all loads in flight
+                    if ((uint32_t)c < CL) {
+                        load_words<W>(recv + (q0 - lo) + c * S, pv[c]);
+                    } else {
 #pragma unroll
-            for (int c = 0; c < kMaxCluster; ++c) {   // fixed CTA order
-                g.x += pv[c].x;
-                g.y += pv[c].y;
-                g.z += pv[c].z;
-                g.w += pv[c].w;
+                        for (int i = 0; i < W; ++i) pv[c][i] = 0.f;
+                    }
+#pragma unroll
+                for (int i = 0; i < W; ++i) g[i] = 0.f;
+#pragma unroll
+                for (int c = 0; c < kMaxCluster; ++c)   // fixed CTA order
+#pragma unroll
+                    for (int i = 0; i < W; ++i) g[i] += pv[c][i];
+#pragma unroll
+                for (int i = 0; i < W; ++i) t[i] = adam(q0 + i, g[i], am[i], av[i]);
+                store_words<W>(th + q0, t);
+                if (!once) keep(std::integral_constant<int, W>{}, q0);
             }
-            const float4 t = make_float4(adam(q0, g.x, m4.x, v4.x), adam(q0 + 1, g.y, m4.y, v4.y),
-                                         adam(q0 + 2, g.z, m4.z, v4.z), adam(q0 + 3, g.w, m4.w, v4.w));
-            *reinterpret_cast<float4 *>(th + q0) = t;
-            __stcg(reinterpret_cast<float4 *>(a.adam_m + q0), m4);
-            __stcg(reinterpret_cast<float4 *>(a.adam_v + q0), v4);
-        }
+        };
+        if (S <= 2 * kThreads) update(std::integral_constant<int, 2>{});
+        else update(std::integral_constant<int, 4>{});
         umma::fence_proxy_async();   // the new slice is read by the bulk copies
         __syncthreads();
-        if (n.tid < (int)CL && n.tid != (int)rank)   // the new slice -> every other CTA's parameters
-            umma::bulk_s2c(umma::map_rank(th_s + (uint32_t)lo * 4u, (uint32_t)n.tid), th_s + (uint32_t)lo * 4u,
-                           slice_bytes, umma::map_rank(xbar_par, (uint32_t)n.tid));
+        if (copy_i + 1 < CL)   // the new slice -> every other CTA's parameters
+            umma::bulk_s2c(umma::map_rank(th_s + (uint32_t)lo * 4u, copy_to), th_s + (uint32_t)lo * 4u, slice_bytes,
+                           umma::map_rank(xbar_par, copy_to));
         if (n.tid == 0) umma::mbar_arrive_expect_tx(&s_xbar[1], (CL - 1u) * slice_bytes);
         if (!umma::mbar_wait(&s_xbar[1], ph_par, kMbarPolls)) {
             ok = false;
@@ -710,6 +768,8 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_train_kernel(TrainArgs a, con
         umma::fence_proxy_async();
         __syncthreads();
     }
+    if (S <= 2 * kThreads) keep(std::integral_constant<int, 2>{}, lo + 2 * n.tid);
+    else if (once) keep(std::integral_constant<int, 4>{}, lo + 4 * n.tid);
     for (int q = lo + n.tid; q < hi; q += kThreads) {
         if (q < L::NP) {
             a.params[L::p_of(q)] = th[q];
