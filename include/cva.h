@@ -323,24 +323,23 @@ CVA_API cva_status cva_regress_portfolios(cva_sim *sim, int basis, float *pred_d
  * draws where c has defaulted give the normal equations (FP64 accumulation), solved
  * by a Jacobi-scaled Cholesky factorisation in FP64; a column whose pivot vanishes
  * (no default of c by t_i in the whole sample) is dropped, with coefficient 0.
- * Needs a simulation created with CVA_KEEP_DEFAULTS after cva_simulate; C <= 8 (one
- * warp lane per counterparty pair), 1 + F + C <= 40 and N (5C + 6) bytes of draw tables must fit 160 KB of shared
- * memory (N <= 3400 at C = 8; else CVA_ENOTSUP).
+ * Needs a simulation created with CVA_KEEP_DEFAULTS after cva_simulate; C <= 8,
+ * 1 + F + C <= 40 and N (5C + 6) <= 160 KB (N <= 3400 at C = 8; else CVA_ENOTSUP).
  * pred_dev: float [n][M] (nullable; date 0 untouched) receives the fit at X_i = 0
  * (every counterparty alive). coef_host: double [n][1+F+C] (nullable; date 0
  * untouched) receives w_i in the raw basis [1, Y_i, X_i]. dropped_host: int [n]
  * (nullable) receives the number of dropped columns per date (0 at date 0). The
  * scratch (n C M floats of per-path default counts, the pair and loss sums of each
- * block of 8 paths, and the Gram partials) belongs to the simulation: the first call allocates it, so make one call before capturing this
- * one in a CUDA graph. Synchronises `stream` only when coef_host or dropped_host is
+ * tile of at most 32 paths, and the Gram partials) belongs to the simulation: the first
+ * call allocates it, so make one call before capturing this one in a CUDA graph. Synchronises `stream` only when coef_host or dropped_host is
  * given. */
 CVA_API cva_status cva_regress_alive(cva_sim *sim, int pf, float *pred_dev, double *coef_host, int *dropped_host,
                                      void *stream);
 
-/* Tile shapes of a simulation chosen by measurement: threads per block of the
- * path-simulation and pricing kernels, outer paths per block of the
- * inner-default kernel, and the number of blocks of the grouped regression
- * (basis `basis`). Each candidate runs on the simulation's own shapes (CUDA-event
+/* Tile shapes of a simulation chosen by measurement (the values of cva_set_tiles): warps
+ * per 32 paths of the path-simulation kernel, threads per block of the pricing kernel,
+ * the tile of the inner-default kernel, the number of blocks of the grouped regression
+ * (basis `basis`) and the pricing form. Each candidate runs on the simulation's own shapes (CUDA-event
  * timings, best of two after a warm-up); the choice is kept in the simulation and
  * cached per (device, shape) for the life of the process. report (nullable)
  * receives the choice as JSON. Runs the kernels; synchronises `stream`. */
@@ -353,10 +352,9 @@ CVA_API cva_status cva_autotune(cva_sim *sim, uint64_t seed, int basis, char *re
  * inner_paths_per_block in {0 (automatic), 2, 4, 8 (tiles of 8, 16 and 32 paths, as
  * far as they fit shared memory)}, lsq_chunk_target in
  * [152, 2^20], and the pricing form portfolios_per_price_block: 1, 2 or 3 dividing
- * the simulation's number of portfolios (a block prices that many portfolios,
- * weights in constant memory; price_block threads), 0 (every thread prices every
- * portfolio for 2 paths with price_block = 128 or 1 path with 256, weights staged in
- * shared memory) or 4 (every portfolio of 128-path tiles on the tensor cores: the
+ * the simulation's number of portfolios (a block of price_block threads, two paths a
+ * thread, prices that many portfolios for the dates of one coupon period, weights in
+ * shared memory), 0 (the largest of these) or 4 (every portfolio of 128-path tiles on the tensor cores: the
  * MtM as a TF32 product with each operand split into head and tail, FP32
  * accumulation). None of the shapes and forms 0-3 changes any result bit; form 4
  * rounds the MtM differently (within the oracle tolerances). Returns CVA_EINVAL
@@ -374,14 +372,16 @@ CVA_API cva_status cva_set_tiles(cva_sim *sim, int sim_block, int price_block, i
  * entries) receives dCVA_0/d theta in this order: curve levels f_e (E), rate
  * volatilities sigma^r_e (E), FX volatilities sigma^chi_e for e = 1..E-1, CIR
  * kappa_c (C), theta_c (C), nu_c (C) (gamma_0 and the swaps' fixed rates held
- * fixed); cva0_host receives the smooth CVA_0. The forward sweep keeps the
- * state every ckpt_every pricing dates (<= 16; sub-steps <= 4); the reverse sweep
- * recomputes each segment from its checkpoint. forward_only = 1 computes only
+ * fixed); cva0_host receives the smooth CVA_0. forward_only = 1 computes only
  * the smooth CVA_0 (grad_host may be NULL). Per-path adjoints are reduced in
  * FP64. The fast-path shapes of cva_sim_create with one portfolio, (E, C) = (1, 2
- * constant) and (10, 8 CIR), have compiled adjoint kernels; every other shape within
- * the limits of cva_sim_create runs the run-time-shape adjoint (same arithmetic,
- * slower: its per-path arrays live in local memory). A constant intensity's kappa_c,
+ * constant) and (10, 8 CIR), have compiled adjoint kernels: simulate, price with the
+ * pricing's derivatives, and sweep the Euler steps back, over ranges of paths whose
+ * arrays (every pricing date's state and derivatives) take up to 1.4 GB, less where that
+ * is not free. Every other shape within the limits of cva_sim_create runs the
+ * run-time-shape adjoint, slower (its per-path arrays live in local memory): its forward
+ * sweep keeps the state every ckpt_every pricing dates, and the reverse sweep recomputes
+ * each segment from its checkpoint. ckpt_every <= 16 and sub-steps <= 4 for both. A constant intensity's kappa_c,
  * theta_c and nu_c receive 0. Allocates and frees its buffers; synchronises `stream`. */
 CVA_API cva_status cva_grad_cva0(const cva_model_desc *model, const cva_portfolio_desc *pf,
                                  const cva_grid *grid, uint64_t M, uint64_t seed, uint64_t k0,

@@ -87,8 +87,9 @@ __host__ __device__ inline StatShape stat_shape(int lg, int C, int n)
 // tile's paths.
 //
 // Bound by latency and by shared memory for the columns (6 bytes per date and thread:
-// 12 warps a multiprocessor). A warp per path that re-read a draw's table at each of its
-// events, with a block barrier per date, took 3.1 ms at 2^17 paths, 64 draws, 100 dates.
+// 12 warps a multiprocessor). 2^17 paths, 64 draws, 100 dates: 1.31 ms; a warp per path that
+// re-read a draw's table at each of its events, with a block barrier per date, took 3.13 ms,
+// and this walk without the list of events 4.5 ms.
 template <int C>
 __global__ void __launch_bounds__(256) alive_stats_kernel(AliveArgs a)
 {

@@ -750,8 +750,8 @@ cva_status cva_autotune(cva_sim *sim, uint64_t seed, int basis, char *report, si
             s.tune_price_pf = save[4];
             return err == CVA_OK ? t : 1e30f;
         };
-        // portfolios per pricing block: the divisors of n_pf among 1, 2, 3 (weights in
-        // constant memory), or 0 (every portfolio per thread, weights in shared memory)
+        // pricing form: the tensor cores (4), or portfolios per block, the divisors of n_pf
+        // among 1, 2, 3 (0 is the largest of them)
         std::vector<int> ppf = {4, 0, 1};
         for (int v : {2, 3})
             if (s.NPF % v == 0) ppf.push_back(v);
@@ -759,8 +759,7 @@ cva_status cva_autotune(cva_sim *sim, uint64_t seed, int basis, char *report, si
         // the first pass needs valid outputs of the earlier kernels: simulate once
         cva_status r = cva_simulate(sim, seed, 0, stream);
         if (r != CVA_OK) return r;
-        // the pricing form (portfolios per block) before its block size: the best block
-        // size differs between the constant-memory and the shared-memory forms
+        // the pricing form before its block size, which the tensor-core form has none of
         for (int w : {0, 4, 1, 2, 3}) {
             float tb = 1e30f;
             for (int v : cand[w]) {
@@ -813,8 +812,8 @@ cva_status cva_set_tiles(cva_sim *sim, int sim_block, int price_block, int inner
     if (portfolios_per_price_block < 0 || portfolios_per_price_block > 4 ||
         (portfolios_per_price_block >= 1 && portfolios_per_price_block <= 3 &&
          s.NPF % portfolios_per_price_block != 0))
-        return fail(CVA_EINVAL, "pricing form must be 0 (shared memory), 1, 2 or 3 dividing the number of portfolios "
-                                "(constant memory) or 4 (tensor cores)");
+        return fail(CVA_EINVAL, "pricing form must be 0 (the largest group), 1, 2 or 3 dividing the number of portfolios "
+                                "or 4 (tensor cores)");
     s.tune_sim_block = sim_block;
     s.tune_price_block = price_block;
     s.tune_inner_P = inner_paths_per_block;

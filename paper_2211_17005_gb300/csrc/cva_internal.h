@@ -94,7 +94,7 @@ struct Sim {
     double *d_lsq = nullptr;
     size_t lsq_cap = 0;
     // scratch of the regression on (default indicators, state), owned by the simulation
-    float *d_alive_stats = nullptr;   // [n][2C + C(C-1)/2][M] per-path sums over the inner draws
+    float *d_alive_stats = nullptr;   // [n][C][M] per-path default counts, [n][C(C-1)/2 + C][tiles] pair and loss sums
     size_t alive_stats_cap = 0;
     double *d_alive = nullptr;        // Gram partials, coefficients, status
     size_t alive_cap = 0;
@@ -120,7 +120,7 @@ struct AdjBuffers {
     float2 *ddrift = nullptr;   // [n*S][E] d drift/df, d drift/dsigma^r
     float *rho = nullptr;       // [E]
     float *sig = nullptr;       // [2E + 3C]
-    float *ckpt = nullptr;      // [nseg][2E+3C][M]
+    float *ckpt = nullptr;      // [nseg][2E+3C][M] (this and the next three: run-time shapes)
     double *ckpt_I0 = nullptr;  // [nseg][M]
     float *fixr = nullptr;      // [periods+1][E][M]
     double *part = nullptr;     // [blocks][npar+1]

@@ -47,7 +47,8 @@ __host__ __device__ constexpr int tri_index(int cols, int i, int j) { return i *
 // Bound by the FMA issue (528 multiply-adds a row at 29 columns; 435 are needed) and the
 // read of the data, about equal. The tiles were transposed to rows before, with eight-way
 // bank conflicts in the copies and in the centring pass: 29 columns of 2^17 rows at 99
-// dates took 1276 us.
+// dates took 1276 us, now 599 us (2.5 TB/s of the data, 42% of the issue slots: the warps of a
+// block wait for each other's tiles).
 template <int TR, int MAXT, int MINB, bool VEC>
 __global__ void __launch_bounds__(MAXT, MINB) gram_kernel(GramArgs a)
 {
@@ -231,6 +232,8 @@ struct SumPair {
     }
 };
 
+// Bound by latency: 49 dates of 2^14 paths take 16 us (49 us as a case of the general kernel,
+// with its FP64 runs).
 template <int NT>
 __global__ void __launch_bounds__(256) poly_gram_kernel(GramArgs a)
 {
@@ -387,7 +390,8 @@ __global__ void __launch_bounds__(256) gram_reduce_kernel(const double *part, in
 // Bound by the FP64 pipe (two lanes a clock and multiprocessor) and by the chain of pivots,
 // so one warp alone computes a pivot's reciprocal, by Newton steps on an FP32 estimate
 // (scaled pivots lie in (1e-12, 1]), and nothing is divided or rooted in FP64. 28 unknowns:
-// 118 us with FP64 square roots and divisions and one thread's triangular solves.
+// 118 us with FP64 square roots and divisions and one thread's triangular solves, now 39 us
+// (99 systems in one launch).
 template <int LD>
 __device__ int solve_normal(double *A, int m, int nt, double *w, double *sc, int *drop)
 {

@@ -94,7 +94,8 @@ __global__ void __launch_bounds__(256) lsq_solve(LsqArgs a)
 // Predictions of every target column of group g (blockIdx.y) at one path per
 // thread: the features are read once per path for all nt columns, and the block
 // converts the group's FP64 coefficients to FP32 once (FP64 conversions run on
-// the slow FP64 pipe). The FMA order per column is the basis order.
+// the slow FP64 pipe). The FMA order per column is the basis order. Groups run from the last
+// back: the Gram has just read that one, so part of it is still in the L2 cache.
 __global__ void __launch_bounds__(256) lsq_predict(LsqArgs a)
 {
     __shared__ float cs[40 * 40];   // [nt][m], m + nt <= 40
@@ -135,7 +136,8 @@ __global__ void __launch_bounds__(256) lsq_predict(LsqArgs a)
 // 16-byte feature loads and prediction stores, the same FMA order per path (so the
 // same bits). Needs M, the strides and the base addresses to be multiples of 4
 // floats (checked by lsq_predict_launch). TM: targets a thread carries at a time, 1 or 8
-// (one target leaves the registers to loads in flight).
+// (one target leaves the registers to loads in flight). Bound by HBM: one target, 27 factors,
+// 2^17 paths and 99 dates 294 -> 216 us, 6.8 TB/s.
 template <int TM>
 __global__ void __launch_bounds__(256) lsq_predict4(LsqArgs a)
 {

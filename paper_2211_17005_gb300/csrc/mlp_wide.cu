@@ -920,7 +920,7 @@ __global__ void __launch_bounds__(kWThreads, MinBlocks) wide_sweep_kernel(WSweep
 //
 // Bound by the chain of a tile (two tensor-core round trips of about 0.8k cycles and two
 // epilogues) over two groups. One group with a two-stage pipeline took 697 us for 2^20 paths
-// on 24 SMs, longer than the 634 us epoch it runs beside.
+// on 24 SMs, longer than the 550 us epoch it runs beside; two groups take 442 us.
 __global__ void __launch_bounds__(kFwdThreads, 1) wide_fwd_kernel(WSweepArgs a, const __grid_constant__ CUtensorMap tm)
 {
     using L = WLP;

@@ -127,9 +127,9 @@ struct OuterArgs {
 //
 // Bound by instruction issue (Philox, logarithm, square root and sine-cosine of 14
 // Box-Muller pairs, the correlation): 2650 instructions a (path, step) at 27 factors and
-// 85% of the issue slots. Paper shape, 2^17 paths and 100 steps: 1.28 -> 1.11 ms against a
+// 85% of the issue slots. Paper shape, 2^17 paths and 100 steps: 1.28 -> 1.09 ms against a
 // thread per path over all steps (96 registers, 7 to 14 warps a multiprocessor); 2^15
-// paths and 2500 steps 9.09 -> 6.51 ms; 2^14 paths and 100 steps 0.43 -> 0.18 ms.
+// paths and 2500 steps 9.09 -> 6.3 ms; 2^14 paths and 100 steps 0.43 -> 0.18 ms.
 template <int E, int C, int CS, int NW, SimMode MODE>
 __global__ void __launch_bounds__(32 * NW, NW == 8 ? 3 : 5) sim_kernel(OuterArgs a)
 {
@@ -364,6 +364,11 @@ __global__ void __launch_bounds__(32 * NW, NW == 8 ? 3 : 5) sim_kernel(OuterArgs
 // weights, the running coupons at the fixing, which the period's dates share. The MtM enters as
 //   acc = sum_h (-wA)(-D_h) + sum_g (-wK) Z_g,
 // with -D_h = Z_{h-1} expm1(x_h), which is what the chain of bond prices produces.
+//
+// Bound by instruction issue and, within it, by shared-memory reads of the weights. Paper
+// shape, 2^17 paths, 101 dates: 2.19 ms with a thread per (path, date), every reset date and
+// the weights in constant memory, 1.19 ms with live dates and packed pairs, 1.00 ms with the
+// tables and coupons in shared memory.
 struct PriceShape {
     int dates_per_block, splits;   // a period's dates in `splits` blocks of dates_per_block
     int start = 0;                 // dates up to this one are priced already
@@ -682,7 +687,7 @@ cva_status outer_launch(Sim &s, uint64_t seed, uint64_t k0, cudaStream_t st)
 }
 
 // The adjoint of one range of paths; `b` holds the tables, the scratch and the sums that
-// this range adds. sums_only: the scratch this range needs, nothing launched.
+// this range adds. Without scratch only its size is computed, nothing launched.
 template <int E, int C, int CS, int G>
 cva_status adjoint_launch(Sim &s, AdjBuffers &b, uint64_t seed, uint64_t k0, uint32_t M, cudaStream_t st)
 {

@@ -9,7 +9,8 @@
 // c_sim.gpos[c] (the factors are r^0..r^{E-1}, log chi^1..log chi^{E-1}, then the
 // CIR intensities in counterparty order), or -1 for a constant intensity.
 // Three economies, five counterparties, four portfolios, 20011 paths, 40 dates: simulation
-// 177 us and pricing 273 us with a thread per path and per (path, date, portfolio).
+// 177 us and pricing 273 us with a thread per path and per (path, date, portfolio), now 68 and
+// 80 us.
 #include <atomic>
 
 #include "outer.cuh"

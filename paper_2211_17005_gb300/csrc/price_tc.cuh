@@ -34,8 +34,11 @@
 // tables of the block's dates (the rest of the multiprocessor's memory is too small an L1 to
 // hold them). TMEM: two 128 x NN FP32 accumulators per slot.
 //
-// Six portfolios (50 to 2000 swaps), 2^18 paths, 120 dates: 9.94 ms with every reset date,
-// one X buffer and a block barrier and vote per economy.
+// Bound by the latency of a slot's chain (bond prices, operand split, stores to shared memory,
+// the multiplication behind them) at 16 warps a multiprocessor. Six portfolios (50 to 2000
+// swaps), 2^18 paths, 120 dates: 9.94 ms with every reset date, one X buffer and a block
+// barrier and vote per economy, 7.99 ms by period with two, 5.74 ms with the tables and
+// coupons in shared memory.
 constexpr uint32_t kPriceMbarPolls = 1u << 26;   // limit of a wait for the tensor core
 constexpr int kPriceSlots = 4;
 constexpr int kPriceTcDates = 6;                 // dates of a block at most

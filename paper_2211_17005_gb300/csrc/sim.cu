@@ -64,6 +64,9 @@ __device__ __forceinline__ int lower_bound_pow2(Thr T, int n, float w)
 // ones that default (two draws' at most, in its own column of the queue), so that the
 // lower bounds run over queues a few entries long. The blocks of a multiprocessor are in
 // different phases, which overlaps the two bounds.
+// Paper shape, 2^17 paths, 64 draws, 100 dates: 0.40 ms; as two kernels with the counts in
+// global memory between them 0.55 + 0.17 ms. Six portfolios, 2^18 paths, 256 draws: 3.0 ms
+// against 2.2 + 1.45 ms.
 // IDX: the default steps are kept too (cva_sim's validation output).
 template <int C, bool IDX>
 __global__ void __launch_bounds__(512) inner_kernel(InnerArgs a)
