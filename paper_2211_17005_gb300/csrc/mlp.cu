@@ -80,8 +80,8 @@ struct Layout {
     static constexpr int oW1 = 0, ob1 = kIn * U, oW2 = ob1 + U, ob2 = oW2 + U * U, ow3 = ob2 + U,
                          ob3 = ow3 + U, omu = ob3 + 1;
     static constexpr int Z = U + 2;                   // refit: [h2 | 1] unknowns and the target column
-    // columns of the row buffers: B = [H1 | 1 0.. | X | 1 0..], A = [dH2 | dH1]
-    static constexpr int cOne1 = U, cX = U + 16, cOne2 = U + 48, cDH1 = U;
+    // columns of the row buffers: B = [H1 | 1 0.. | X], A = [dH2 | dH1]
+    static constexpr int cOne1 = U, cX = U + 16, cDH1 = U, cEnd = cX + kIn;
     // shared memory (bytes)
     static constexpr int sSlot = 65536;                         // slot s: A at s * sSlot, B at + 32768
     static constexpr int sW1 = 2 * sSlot;                       // W1 image [U][32], K-major
@@ -301,15 +301,13 @@ struct Net {
         return ok;
     }
 
-    // constant columns of B (ones after H1 and after X, zeros beside them), both slots
+    // constant columns of B (ones after H1, zeros beside them), both slots
     __device__ void init_constants()
     {
         const uint4 one = make_uint4((uint32_t)bf16_bits(1.f), 0u, 0u, 0u), zero = make_uint4(0u, 0u, 0u, 0u);
         unsigned char *b = smem + offB();
         *reinterpret_cast<uint4 *>(b + row_off(row, L::cOne1)) = one;
         *reinterpret_cast<uint4 *>(b + row_off(row, L::cOne1 + 8)) = zero;
-        *reinterpret_cast<uint4 *>(b + row_off(row, L::cOne2)) = one;
-        *reinterpret_cast<uint4 *>(b + row_off(row, L::cOne2 + 8)) = zero;
     }
 
     // BF16 images of W1 and W2 from the shared parameters (all 256 threads)
@@ -364,20 +362,24 @@ struct Net {
     }
 
     // output, loss derivative and the output-layer backward of this thread's row:
-    // dH2 = dout w3 (h2 > 0) into A; the column sums of h2 dout (dw3), of dout (db3)
-    // and of dpred (dmu) over the warp's rows into this warp's slots gsl
-    __device__ void out_back2(int pos, float y, float inv_batch, float *gsl) const
+    // dH2 = dout w3 (h2 > 0) into A; v receives h2 dout
+    __device__ void out_back2(int pos, float y, float inv_batch, float (&v)[64], float &dout, float &dpred) const
     {
         unsigned char *a = smem + offA();
         const float4 *w3 = reinterpret_cast<const float4 *>(th + L::ow3);
-        float v[64];
         const float out = layer2(v);
         const float pred = (pos ? fmaxf(out, 0.f) : out) + th[L::omu];
-        const float dpred = 2.f * (pred - y) * inv_batch;
-        const float dout = pos ? (out > 0.f ? dpred : 0.f) : dpred;
+        dpred = 2.f * (pred - y) * inv_batch;
+        dout = pos ? (out > 0.f ? dpred : 0.f) : dpred;
 #pragma unroll
         for (int g = 0; g < 8; ++g)
             *reinterpret_cast<uint4 *>(a + row_off(row, 8 * g)) = masked_scale8(v + 8 * g, dout, w3[2 * g], w3[2 * g + 1]);
+    }
+
+    // the column sums of h2 dout (dw3), of dout (db3) and of dpred (dmu) over the warp's
+    // rows into this warp's slots gsl
+    __device__ void out_sums(float (&v)[64], float dout, float dpred, float *gsl) const
+    {
         scale64(v, dout);
         const float2 cs = column_sums64(v, lane);
         gsl[2 * lane] += cs.x;
@@ -422,10 +424,11 @@ struct Net {
         forward12(in_ok, [&] {
             if (has_next) prefetch(tm, a.targ, a.F, next_path);
         });
-        out_back2(a.pos, y, inv_batch, gsl);
-        mma([&] { gemm_rows_w2t(dcol(), offA()); });
+        float v[64], dout, dpred;
+        out_back2(a.pos, y, inv_batch, v, dout, dpred);
+        mma([&] { gemm_rows_w2t(dcol(), offA()); }, [&] { out_sums(v, dout, dpred, gsl); });
         back1();
-        mma([&] { gemm_paths(wcol(), offA(), offB(), kRows, !first); });
+        mma([&] { gemm_paths(wcol(), offA(), offB(), L::cEnd, !first); });
         return wg_all(good);
     }
 
@@ -468,9 +471,9 @@ struct Net {
                         else if (col == U) P[L::ob2 + o] = g;
                     }
                 }
-        } else {        // rows U + i: dW1[i][:] at columns [cX, cX + 32), db1[i] at column cOne2
+        } else {        // rows U + i: dW1[i][:] at columns [cX, cX + 32), db1[i] at column cOne1
             const int i0 = (q4 - 2) * 32 + lane;
-            const int k0 = wg ? 7 : 5, k1 = wg ? 8 : 7;
+            const int k0 = wg ? 6 : 4, k1 = wg ? 7 : 6;
             float v0[2][16], v1[2][16];
 #pragma unroll
             for (int j = 0; j < 2; ++j) {
@@ -487,10 +490,10 @@ struct Net {
                 if (k0 + j < k1) {
 #pragma unroll
                     for (int i = 0; i < 16; ++i) {
-                        const int f = 16 * (k0 + j) + i - L::cX;
+                        const int col = 16 * (k0 + j) + i, f = col - L::cX;
                         const float g = (h0 ? v0[j][i] : 0.f) + (h1 ? v1[j][i] : 0.f);
-                        if (f < kIn) P[L::oW1 + f * U + i0] = g;
-                        else if (f == kIn) P[L::ob1 + i0] = g;
+                        if (f >= 0) P[L::oW1 + f * U + i0] = g;
+                        else if (col == L::cOne1) P[L::ob1 + i0] = g;
                     }
                 }
         }
@@ -668,7 +671,7 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_train_kernel(TrainArgs a, con
             store_words_cg<W>(a.adam_v + q0, av);
         }
     };
-    if (S <= 2 * kThreads) moments(std::integral_constant<int, 2>{}, lo + 2 * n.tid, a.step0 == 0);
+    if (CL == kMaxCluster) moments(std::integral_constant<int, 2>{}, lo + 2 * n.tid, a.step0 == 0);
     else if (once) moments(std::integral_constant<int, 4>{}, lo + 4 * n.tid, a.step0 == 0);
 
     // bias corrections 1 - beta^t of Adam, as running powers of beta
@@ -710,30 +713,33 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_train_kernel(TrainArgs a, con
         const int step = a.step0 + st + 1;
         b1t *= a.beta1;
         b2t *= a.beta2;
-        const float inv_bc1 = 1.f / (1.f - b1t), inv_bc2 = 1.f / (1.f - b2t);
+        float inv_bc1 = 1.f / (1.f - b1t), inv_bc2 = 1.f / (1.f - b2t);
+        asm volatile("" : "+f"(inv_bc1), "+f"(inv_bc2));   // (divided before the wait)
         if (n.tid == 0) umma::mbar_arrive_expect_tx(&s_xbar[0], (uint32_t)L::NPpad * 4u);
         if (!umma::mbar_wait(&s_xbar[0], ph_part, kMbarPolls)) {
             ok = false;
             atomicExch(a.err, 4);
         }
         ph_part ^= 1u;
-        auto adam = [&](int q, float g, float &m, float &v) -> float {
-            if (step == 1 && a.grad_out && q < L::NP) a.grad_out[L::p_of(q)] = g;
+        const bool keep_grad = step == 1 && a.grad_out;
+        // one entry: q its place, t its value now
+        auto adam = [&](int q, float t, float g, float &m, float &v) -> float {
+            if (keep_grad && q < L::NP) a.grad_out[L::p_of(q)] = g;
             if (q >= L::NP || (q < L::ob1 && q / U >= a.F)) return 0.f;   // padding stays zero
             m = a.beta1 * m + (1.f - a.beta1) * g;
             v = a.beta2 * v + (1.f - a.beta2) * g * g;
-            return th[q] - adam_delta(m, v, inv_bc1, inv_bc2, a.lr, a.eps);
+            return t - adam_delta(m, v, inv_bc1, inv_bc2, a.lr, a.eps);
         };
-        auto update = [&](auto width) {   // W entries a thread
+        auto update = [&](auto width, auto full) {   // W entries a thread; full: CL = kMaxCluster
             constexpr int W = decltype(width)::value;
+            constexpr bool FULL = decltype(full)::value;
             for (int q0 = lo + W * n.tid; q0 < hi; q0 += W * kThreads) {
-                if (!once) {
-                    moments(std::integral_constant<int, W>{}, q0, a.step0 == 0 && st == 0);
-                }
+                if (!FULL && !once) moments(width, q0, a.step0 == 0 && st == 0);
                 float pv[kMaxCluster][W], g[W], t[W];
+                load_words<W>(th + q0, t);
 #pragma unroll
                 for (int c = 0; c < kMaxCluster; ++c)   // all loads in flight
-                    if ((uint32_t)c < CL) {
+                    if (FULL || (uint32_t)c < CL) {
                         load_words<W>(recv + (q0 - lo) + c * S, pv[c]);
                     } else {
 #pragma unroll
@@ -746,13 +752,17 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_train_kernel(TrainArgs a, con
 #pragma unroll
                     for (int i = 0; i < W; ++i) g[i] += pv[c][i];
 #pragma unroll
-                for (int i = 0; i < W; ++i) t[i] = adam(q0 + i, g[i], am[i], av[i]);
+                for (int i = 0; i < W; ++i) t[i] = adam(q0 + i, t[i], g[i], am[i], av[i]);
                 store_words<W>(th + q0, t);
-                if (!once) keep(std::integral_constant<int, W>{}, q0);
+                if (!FULL && !once) keep(width, q0);
+                if (FULL) break;   // one pass covers the slice
             }
         };
-        if (S <= 2 * kThreads) update(std::integral_constant<int, 2>{});
-        else update(std::integral_constant<int, 4>{});
+        using W2 = std::integral_constant<int, 2>;
+        using W4 = std::integral_constant<int, 4>;
+        static_assert(L::NPpad / kMaxCluster <= 2 * kThreads, "one pass");
+        if (CL == kMaxCluster) update(W2{}, std::true_type{});
+        else update(W4{}, std::false_type{});
         umma::fence_proxy_async();   // the new slice is read by the bulk copies
         __syncthreads();
         if (copy_i + 1 < CL)   // the new slice -> every other CTA's parameters
@@ -768,7 +778,7 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_train_kernel(TrainArgs a, con
         umma::fence_proxy_async();
         __syncthreads();
     }
-    if (S <= 2 * kThreads) keep(std::integral_constant<int, 2>{}, lo + 2 * n.tid);
+    if (CL == kMaxCluster) keep(std::integral_constant<int, 2>{}, lo + 2 * n.tid);
     else if (once) keep(std::integral_constant<int, 4>{}, lo + 4 * n.tid);
     for (int q = lo + n.tid; q < hi; q += kThreads) {
         if (q < L::NP) {
