@@ -217,6 +217,7 @@ struct WNetT {
     uint32_t tmem = 0;
     uint64_t *mbar, *sbar;
     uint32_t phase = 0, sphase = 0;
+    bool good = true;              // no wait of this thread has given up
     bool pending = false;
     int tid, warp, lane, row, half;
     float *vec, *stage;
@@ -242,9 +243,10 @@ struct WNetT {
 
     // one tensor-core step of the CTA: operands written -> issue (thread 0) ->
     // completion; side() runs in every thread after the barrier while the tensor
-    // core works
+    // core works. A wait that gives up clears `good`, and later ones are skipped; the CTA
+    // votes once per tile (all_good).
     template <class Issue, class Side>
-    __device__ bool mma(Issue issue, bool pre_ok, Side side)
+    __device__ void mma(Issue issue, Side side)
     {
         umma::fence_proxy_async();
         umma::fence_before_sync();
@@ -255,16 +257,16 @@ struct WNetT {
             umma::commit(mbar);
         }
         side();
-        const bool done = umma::mbar_wait(mbar, phase, kMbarPolls);
+        if (good) good = umma::mbar_wait(mbar, phase, kMbarPolls);
         phase ^= 1u;
         umma::fence_after_sync();
-        return __syncthreads_and(done && pre_ok) != 0;
     }
     template <class Issue>
-    __device__ bool mma(Issue issue)
+    __device__ void mma(Issue issue)
     {
-        return mma(issue, true, [] {});
+        mma(issue, [] {});
     }
+    __device__ bool all_good() const { return __syncthreads_and(good) != 0; }
 
     // D = A B^T: A = K columns of a row buffer (width w, from column c0, K-major),
     // B = a K-major image [N][K]
@@ -373,9 +375,8 @@ struct WNetT {
         float *so = reinterpret_cast<float *>(smem + L::sOut);
         so[half * kRows + row] = share;
         __syncthreads();
-        const float z = (so[row] + so[kRows + row]) + vec[L::vb3];
-        __syncthreads();
-        return z;
+        // (written again one tile later, several barriers away)
+        return (so[row] + so[kRows + row]) + vec[L::vb3];
     }
 
     // output, loss derivative and the output-layer backward of this thread's row:
@@ -425,11 +426,12 @@ struct WNetT {
 
     // first two layers of the staged tile; D holds the second-layer pre-activation
     template <class Side>
-    __device__ bool forward12(bool in_ok, Side side)
+    __device__ void forward12(bool in_ok, Side side)
     {
-        if (!mma([&] { gemm_rows(L::cD, L::sB, L::wB, L::cX, L::sW1, kIn, L::U); }, in_ok, side)) return false;
+        good = good && in_ok;
+        mma([&] { gemm_rows(L::cD, L::sB, L::wB, L::cX, L::sW1, kIn, L::U); }, side);
         epi1();
-        return mma([&] { gemm_rows(L::cD, L::sB, L::wB, 0, L::sW2, L::U, L::U); });
+        mma([&] { gemm_rows(L::cD, L::sB, L::wB, 0, L::sW2, L::U, L::U); });
     }
 
     // constant columns of B: ones after H1 (first warpgroup) and after X (second)
@@ -566,29 +568,37 @@ __global__ void __launch_bounds__(kWThreads, 1) wide_train_kernel(WTrainArgs a, 
 
     if (my_rounds > 0) n.prefetch(&tm, a.targ, a.F, path_of(0, 0));
     for (int st = 0; st < a.n_steps; ++st) {
+        const int step = a.step0 + st + 1;
+        float inv_bc1 = 1.f, inv_bc2 = 1.f;   // Adam's bias corrections
+        auto corrections = [&] {
+            inv_bc1 = 1.f / (1.f - powf(a.beta1, (float)step));
+            inv_bc2 = 1.f / (1.f - powf(a.beta2, (float)step));
+            asm volatile("" : "+f"(inv_bc1), "+f"(inv_bc2));   // (here, not where they are used)
+        };
+        if (my_rounds == 0) corrections();
         for (int rd = 0; rd < my_rounds && ok; ++rd) {
             const bool last = rd + 1 == my_rounds;
             const bool has_next = !last || st + 1 < a.n_steps;
             const uint32_t next = last ? path_of(st + 1, 0) : path_of(st, rd + 1);
             float y;
             const bool in_ok = n.stage_x(y);
-            ok = n.forward12(in_ok, [&] {
+            n.forward12(in_ok, [&] {
                 if (has_next) n.prefetch(&tm, a.targ, a.F, next);
             });
-            if (ok) {
-                // the output layer's column sums run while the tensor core works on GEMM3
-                float v[64], dout, dpred;
-                n.out_back2(a.pos, y, inv_batch, v, dout, dpred);
-                ok = n.mma([&] { n.gemm_w2t(WL::cD); }, true, [&] { n.out_sums(v, dout, dpred, my_gsl); });
-            }
-            if (ok) {
-                n.back1();
-                const bool acc = rd > 0;
-                ok = n.mma([&] {
-                    n.gemm_paths(WL::cW2, WL::sA, WL::wA, 0, WL::sB, WL::wB, 0, WL::U + 16, acc);
-                    n.gemm_paths(WL::cW1, WL::sA, WL::wA, WL::U, WL::sB, WL::wB, WL::cX, kIn + 16, acc);
-                });
-            }
+            // the output layer's column sums run while the tensor core works on GEMM3, the
+            // bias corrections behind the weight gradients
+            float v[64], dout, dpred;
+            n.out_back2(a.pos, y, inv_batch, v, dout, dpred);
+            n.mma([&] { n.gemm_w2t(WL::cD); }, [&] { n.out_sums(v, dout, dpred, my_gsl); });
+            n.back1();
+            const bool acc = rd > 0;
+            n.mma([&] {
+                n.gemm_paths(WL::cW2, WL::sA, WL::wA, 0, WL::sB, WL::wB, 0, WL::U + 16, acc);
+                n.gemm_paths(WL::cW1, WL::sA, WL::wA, WL::U, WL::sB, WL::wB, WL::cX, kIn + 16, acc);
+            }, [&] {
+                if (last) corrections();
+            });
+            ok = n.all_good();
             if (!ok && n.tid == 0) atomicExch(a.err, 2);
         }
         umma::fence_before_sync();
@@ -658,9 +668,6 @@ __global__ void __launch_bounds__(kWThreads, 1) wide_train_kernel(WTrainArgs a, 
         // ranges of CTAs per group of four parameters, added in range order), Adam,
         // new FP32 values and their BF16 images
         {
-            const int step = a.step0 + st + 1;
-            const float inv_bc1 = 1.f / (1.f - powf(a.beta1, (float)step)),
-                        inv_bc2 = 1.f / (1.f - powf(a.beta2, (float)step));
             const int NG = (hi - lo) / 4;
             const int nsub = NG >= kWThreads ? 1 : (NG > 0 ? kWThreads / NG : 1);
             const int Pg = kWThreads / nsub;
@@ -800,9 +807,10 @@ __global__ void __launch_bounds__(kWThreads, MinBlocks) wide_sweep_kernel(WSweep
         const uint32_t nt = t + stride;
         float y;
         const bool in_ok = n.stage_x(y);
-        ok = n.forward12(in_ok, [&] {
+        n.forward12(in_ok, [&] {
             if (nt < tiles) n.prefetch(&tm, a.targ, a.F, nt * kRows);
         });
+        ok = n.all_good();
         if (!ok) break;
         float v[64];
         const float share = n.layer2(v);
@@ -831,7 +839,8 @@ __global__ void __launch_bounds__(kWThreads, MinBlocks) wide_sweep_kernel(WSweep
                 acc[2] += db * db;
             }
             // G (+)= Z^T Z: M = the 128 h2 columns, N = the first 144 columns of the rows
-            ok = n.mma([&] { n.gemm_paths(L::cW2, L::sA, L::wA, 0, L::sA, L::wA, 0, L::U + 16, !first); });
+            n.mma([&] { n.gemm_paths(L::cW2, L::sA, L::wA, 0, L::sA, L::wA, 0, L::U + 16, !first); });
+            ok = n.all_good();
         }
         if (!ok && n.tid == 0) atomicExch(a.err, 2);
         first = false;
