@@ -31,7 +31,8 @@ def _clocks(api, seed, M, N, C):
 
 
 @pytest.mark.parametrize("name,M,N,n", [("small", 5, 70000, 50), ("small", 33, 1, 5), ("mixed", 37, 33, 250),
-                                        ("paper", 129, 3, 20), ("batched", 40, 65, 30)])
+                                        ("paper", 129, 3, 20), ("paper", 70, 2, 100),
+                                        ("batched", 40, 65, 30)])
 def test_default_steps_and_targets_follow_from_thresholds_and_exposures(api, name, M, N, n):
     wl = W.make(name, M=M, N=N, n_steps=n)
     sim = api.Simulation(wl.model, wl.portfolios, wl.grid, M, N, keep_defaults=True)
