@@ -202,6 +202,13 @@ __global__ void __launch_bounds__(128 * kPriceSlots, 1) price_tc_kernel(OuterArg
                     const float4 *tab = tab_s + (j - j0) * E * LV;
                     const float beta = expf(-__ldg(a.disc + (size_t)j * M + kr));
                     const uint32_t acc = tmem + (item & 1u) * P::acc_cols;
+                    {   // the next date's states (the next tile's first), for its loads to find in the L2 cache
+                        const bool more = j + 1 < j1;
+                        const size_t jn = more ? (size_t)(j + 1) : (size_t)j0;
+                        const uint64_t kn = (uint64_t)(more ? t : t + step) * 128u + (uint32_t)(row & ~31);
+                        if (kn < a.M)
+                            prefetch_state<E>(a.features + jn * F * M, a.disc + jn * M, M, (uint32_t)kn, a.M);
+                    }
                     // an economy's state is requested two economies ahead (rate, log chi)
                     float n_r[2], n_l[2];
 #pragma unroll
