@@ -106,21 +106,20 @@ def price_instr_per_path_date(wl):
 
 # DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) per unit of work from one
 # ncu capture of each kernel in its current form (profiles/), scaled to a launch by
-# the units it processes. The simulation kernels were captured at 32768 paths of the
+# the units it processes. The simulation kernels were captured at 65536 paths of the
 # paper workload (part of their writes still sat in the 129 MB L2 when they ended,
-# so the scaled figures are lower bounds); the trainer at the benchmark's 2^17 paths.
+# so the scaled figures are lower bounds); the trainers at the benchmark's shapes.
 NCU_TRAFFIC = {
-    "sim_kernel": {"bytes_per_unit": (0.12e6 + 415.28e6) / (32768 * 100), "unit": "path-step",
-                   "profile": "profiles/sim_price_inner_kernels_paper_32k.md"},
-    "price_kernel": {"bytes_per_unit": (263.78e6 + 81.86e6) / (32768 * 100), "unit": "path-date",
-                     "profile": "profiles/sim_price_inner_kernels_paper_32k.md"},
-    # one launch = one epoch at one date; captured at 65536 paths, scaled by the paths
-    "mlp_train_kernel": {"bytes_per_unit": (7.506432e6 + 0.0) / 65536, "unit": "path",
-                         "profile": "profiles/mlp_train_kernel_paper_64k.md"},
-    # width 128: one launch = one epoch at one date; captured at 131072 paths (second
-    # launch of the capture), scaled by the paths
-    "wide_train_kernel": {"bytes_per_unit": (15.038720e6 + 0.005120e6) / 131072, "unit": "path",
-                          "profile": "profiles/wide_train_kernel_precision_128k.md"},
+    "sim_kernel": {"bytes_per_unit": (0.33e6 + 892.04e6) / (65536 * 100), "unit": "path-step",
+                   "profile": "profiles/kernels_64k.md"},
+    "price_kernel": {"bytes_per_unit": (556.50e6 + 189.07e6) / (65536 * 100), "unit": "path-date",
+                     "profile": "profiles/kernels_64k.md"},
+    # one launch = one epoch at one date; captured at 131072 paths
+    "mlp_train_kernel": {"bytes_per_unit": (14.83e6 + 0.0) / 131072, "unit": "path",
+                         "profile": "profiles/kernels_64k.md"},
+    # width 128: one launch = one epoch at one date; captured at 2^20 paths
+    "wide_train_kernel": {"bytes_per_unit": (117.81e6 + 3.05e6) / 1048576, "unit": "path",
+                          "profile": "profiles/kernels_64k.md"},
 }
 
 

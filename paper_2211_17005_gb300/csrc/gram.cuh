@@ -47,7 +47,7 @@ __host__ __device__ constexpr int tri_index(int cols, int i, int j) { return i *
 // Bound by the FMA issue (528 multiply-adds a row at 29 columns; 435 are needed) and the
 // read of the data, about equal. The tiles were transposed to rows before, with eight-way
 // bank conflicts in the copies and in the centring pass: 29 columns of 2^17 rows at 99
-// dates took 1276 us, now 599 us (2.5 TB/s of the data, 42% of the issue slots: the warps of a
+// dates took 1276 us, now 599 us (2.5 TB/s of the data, 59% of the issue slots: the warps of a
 // block wait for each other's tiles).
 template <int TR, int MAXT, int MINB, bool VEC>
 __global__ void __launch_bounds__(MAXT, MINB) gram_kernel(GramArgs a)
