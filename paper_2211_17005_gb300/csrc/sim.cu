@@ -50,6 +50,17 @@ __device__ __forceinline__ int lower_bound_pow2(Thr T, int n, float w)
     return pos + 1;
 }
 
+// A thread's draws between two stores of the staged steps: 32 bytes or so of them, so that few
+// counterparties do not mean many barriers (a multiple of 4: runs of whole 16 bytes).
+__host__ __device__ constexpr int idx_draws(int C) { return C >= 8 ? 4 : 32 / C / 4 * 4; }
+// Shared memory of the staged steps: [2^lg] rows of idx_draws (nthr >> lg) draws, 16 bytes more
+// each so that rows start in different banks; after thresholds, counters and queues.
+__host__ __device__ constexpr int idx_stage_pitch(int lg, int C, int nthr) { return idx_draws(C) * (nthr >> lg) * C + 16; }
+__host__ __device__ constexpr size_t idx_stage_offset(int rows, int cnt_words, int lg, int C, int nthr)
+{
+    return (4 * (((size_t)rows << lg) + (size_t)cnt_words + (size_t)2 * C * nthr) + 15) / 16 * 16;
+}
+
 // Clocks, counts and targets of a tile of PT = 2^lg outer paths in one block.
 //
 // A lane owns one path of the tile (lane mod PT) throughout, so shared memory is laid
@@ -67,7 +78,12 @@ __device__ __forceinline__ int lower_bound_pow2(Thr T, int n, float w)
 // Paper shape, 2^17 paths, 64 draws, 100 dates: 0.40 ms; as two kernels with the counts in
 // global memory between them 0.55 + 0.17 ms. Six portfolios, 2^18 paths, 256 draws: 3.0 ms
 // against 2.2 + 1.45 ms.
-// IDX: the default steps are kept too (cva_sim's validation output).
+// IDX: the default steps are kept too (cva_sim's validation output). They wait in shared memory,
+// some of a thread's draws at a time (idx_draws), and leave as whole runs of a path's row.
+// Stored from where they are found, a byte of another path's row per lane, they took longer
+// than the clocks: four counterparties, 65536 paths, 512 draws, 50 dates, the whole simulation
+// 1259 us, so 566 us (519 without the steps); the paper's shape with 256 draws and 20 dates
+// 1295 and 580 us.
 template <int C, bool IDX>
 __global__ void __launch_bounds__(512) inner_kernel(InnerArgs a)
 {
@@ -79,6 +95,8 @@ __global__ void __launch_bounds__(512) inner_kernel(InnerArgs a)
     uint32_t *cnt = reinterpret_cast<uint32_t *>(T + ((size_t)a.rows << lg));    // counts
     const int cnt_words = ((n * C + ps) >> ps) << lg;
     uint32_t *queue = cnt + cnt_words + tid;                                     // [2 C][nthr], this thread's column
+    uint8_t *stage = reinterpret_cast<uint8_t *>(smem + idx_stage_offset(a.rows, cnt_words, lg, C, nthr));   // IDX: [PT][pitch]
+    const int pitch = idx_stage_pitch(lg, C, nthr);
     const uint32_t M = a.M, tile0 = blockIdx.x << lg;
     const int p = tid & (PT - 1);
     const bool live = tile0 + (uint32_t)p < M;
@@ -105,28 +123,35 @@ __global__ void __launch_bounds__(512) inner_kernel(InnerArgs a)
         asm volatile("cp.async.commit_group;" ::: "memory");
     }
     for (int i = tid; i < cnt_words; i += nthr) cnt[i] = 0u;
+    const uint32_t none = (uint32_t)(n + 1) * 0x01010101u;   // no default, four times
+    if (IDX)
+        for (int i = tid; i < (pitch << lg) / 16; i += nthr)
+            reinterpret_cast<uint4 *>(stage)[i] = make_uint4(none, none, none, none);
     asm volatile("cp.async.wait_all;" ::: "memory");
     __syncthreads();
 
-    if (live) {
-        const uint32_t kl = tile0 + (uint32_t)p, k = a.k0 + kl, stride = (uint32_t)(nthr >> lg);
-        // w = (m + 1/2) 2^-23 <= T(n)  <=>  m < bound = floor(2^23 T(n) - 1/2) + 1, every
-        // operation exact (T <= 1; a NaN takes every clock, as the comparison of w would)
-        uint32_t bound[C];
+    const uint32_t k = a.k0 + tile0 + (uint32_t)p, stride = (uint32_t)(nthr >> lg);
+    // w = (m + 1/2) 2^-23 <= T(n)  <=>  m < bound = floor(2^23 T(n) - 1/2) + 1, every
+    // operation exact (T <= 1; a NaN takes every clock, as the comparison of w would)
+    uint32_t bound[C];
 #pragma unroll
-        for (int c = 0; c < C; ++c) {
-            const float t = T[(((n - 1) * C + c) << lg) + p] * 8388608.f;
-            bound[c] = t >= 0.5f ? (uint32_t)floorf(fminf(t, 8388608.f) - 0.5f) + 1u : t < 0.5f ? 0u : 8388608u;
-        }
-        const uint32_t Tp = (uint32_t)__cvta_generic_to_shared(T + p);
-        auto lds = [](uint32_t addr) {
-            float v;
-            asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(addr));
-            return v;
-        };
+    for (int c = 0; c < C; ++c) {
+        const float t = T[(((n - 1) * C + c) << lg) + p] * 8388608.f;
+        bound[c] = t >= 0.5f ? (uint32_t)floorf(fminf(t, 8388608.f) - 0.5f) + 1u : t < 0.5f ? 0u : 8388608u;
+    }
+    const uint32_t Tp = (uint32_t)__cvta_generic_to_shared(T + p);
+    auto lds = [](uint32_t addr) {
+        float v;
+        asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(addr));
+        return v;
+    };
+    // this thread's draws of [l0, l1)
+    auto draw = [&](uint32_t l0, uint32_t l1) {
         int queued = 0;
         bool even = false;
-        for (uint32_t l = (uint32_t)(tid >> lg); l < a.N; l += stride) {
+        for (uint32_t l = l0 + (uint32_t)(tid >> lg); l < l1; l += stride) {
+            // an entry: the draw's 23 bits, (IDX) which of the two draws, the counterparty
+            const uint32_t tag = IDX && even ? 16u : 0u;
 #pragma unroll
             for (int cb = 0; cb < (C + 3) / 4; ++cb) {
                 const uint4 x = philox4x32_10(make_uint4(k, l, a.branch, (kStreamInner << 24) | (uint32_t)cb),
@@ -137,24 +162,26 @@ __global__ void __launch_bounds__(512) inner_kernel(InnerArgs a)
                     const int c = 4 * cb + i;
                     if (c < C) {
                         const bool hit = (xs[i] >> 9) < bound[c];
-                        if (hit) queue[queued] = (xs[i] & ~0x1ffu) | (uint32_t)c;
+                        if (hit) queue[queued] = (xs[i] & ~0x1ffu) | tag | (uint32_t)c;
                         queued += hit ? nthr : 0;
-                        if (IDX && !hit) a.idx[((size_t)kl * a.N + l) * C + c] = (uint8_t)(n + 1);
                     }
                 }
             }
             even = !even;
-            if (!IDX && even && l + stride < a.N) continue;   // the queue holds two draws' defaults
+            if (even && l + stride < l1) continue;   // the queue holds two draws' defaults
+            // the first draw's place in the staged row
+            const uint32_t row = IDX ? (uint32_t)(p * pitch) + (l - l0 - (even ? 0u : stride)) * C : 0u;
             even = false;
             // four entries at a time: their searches interleave
             for (int t = 0; t < queued; t += 4 * nthr) {
                 float w[4];
-                uint32_t at[4];      // shared address of the search's lower end
+                uint32_t at[4], to[4];      // shared address of the search's lower end; place of the draw's steps
 #pragma unroll
                 for (int u = 0; u < 4; ++u) {
                     const uint32_t x = t + u * nthr < queued ? queue[t + u * nthr] : 0u;
                     w[u] = uniform23(x);
-                    at[u] = Tp + ((x & 0x1ffu) << (lg + 2));
+                    at[u] = Tp + ((x & (IDX ? 0xfu : 0x1ffu)) << (lg + 2));
+                    if (IDX) to[u] = row + (x & 16u ? stride * C : 0u);
                 }
                 // first j with T(j) >= w among 1..n (T(n) >= w): the halving of a range of
                 // n depends on n only, so its steps are the same for every lane
@@ -171,10 +198,40 @@ __global__ void __launch_bounds__(512) inner_kernel(InnerArgs a)
                     if (t + u * nthr < queued) {
                         const uint32_t ci = (at[u] - Tp) >> (lg + 2);   // step (at 0) x C + counterparty
                         atomicAdd(&cnt[((ci >> ps) << lg) + p], 1u << (16 * (ci & (uint32_t)ps)));
-                        if (IDX) a.idx[((size_t)kl * a.N + l) * C + ci % C] = (uint8_t)(ci / C + 1);
+                        if (IDX) stage[to[u] + ci % C] = (uint8_t)(ci / C + 1);
                     }
             }
             queued = 0;
+        }
+    };
+    if constexpr (!IDX) {
+        if (live) draw(0u, a.N);
+    } else {
+        const uint32_t span = idx_draws(C) * stride, paths = min((uint32_t)PT, M - tile0);
+        // the staged rows' first `bytes` bytes to the paths' rows from draw l0, W at a time; what
+        // was read is set back to "no default"
+        auto store = [&](auto word, uint32_t l0, uint32_t bytes) {
+            using W = decltype(word);
+            constexpr uint32_t B = sizeof(W);
+            const uint32_t per = bytes / B;
+            for (uint32_t i = tid; i < paths * per; i += nthr) {
+                const uint32_t q = i / per, o = i % per * B;
+                W *from = reinterpret_cast<W *>(stage + q * pitch + o);
+                *reinterpret_cast<W *>(a.idx + ((size_t)(tile0 + q) * a.N + l0) * C + o) = *from;
+                if constexpr (B == 16) *from = make_uint4(none, none, none, none);
+                else *from = (W)none;
+            }
+        };
+        for (uint32_t l0 = 0; l0 < a.N; l0 += span) {
+            const uint32_t nl = min(span, a.N - l0), bytes = nl * C;
+            if (live) draw(l0, l0 + nl);
+            __syncthreads();
+            // (span C is a multiple of 16, so only the rows' own length decides)
+            if ((a.N * (uint32_t)C) % 16 == 0) store(uint4{}, l0, bytes);
+            else if ((a.N * (uint32_t)C) % 4 == 0) store(uint32_t{}, l0, bytes);
+            else store(uint8_t{}, l0, bytes);
+            __syncthreads();
+            if (span > a.N - l0) break;   // (l0 + span may not fit 32 bits)
         }
     }
     __syncthreads();
@@ -411,11 +468,12 @@ cva_status launch_outer(Sim &s, uint64_t seed, uint64_t k0, cudaStream_t st)
     return o->launch(s, seed, k0, st);
 }
 
-// Shared memory of a tile: thresholds (later the portfolio sums), counters, queues.
-static size_t inner_smem(int lg, int threads, int C, int n, int NPF, bool packed)
+// Shared memory of a tile: thresholds (later the portfolio sums), counters, queues and (keep)
+// the staged steps.
+static size_t inner_smem(int lg, int threads, int C, int n, int NPF, bool packed, bool keep)
 {
-    const size_t rows = (size_t)n * std::max(C, NPF), words = packed ? ((size_t)n * C + 1) / 2 : (size_t)n * C;
-    return 4 * (((rows + words) << lg) + (size_t)2 * C * threads);
+    const int rows = n * std::max(C, NPF), words = (packed ? (n * C + 1) / 2 : n * C) << lg;
+    return idx_stage_offset(rows, words, lg, C, threads) + (keep ? (size_t)idx_stage_pitch(lg, C, threads) << lg : 0);
 }
 
 template <int C>
@@ -440,10 +498,10 @@ static cudaError_t launch_inner_t(InnerArgs &args, int tune, int sms, int dev, c
         const uint64_t want = std::max<uint64_t>(args.N, (uint64_t)args.n * C / 8) << lg;
         const int t = want >= 512 ? 512 : want >= 256 ? 256 : 128;
         // half the queues where that lets a second block in
-        const auto two = [&](int threads) { return inner_smem(lg, threads, C, args.n, args.NPF, packed) <= 108 * 1024; };
+        const auto two = [&](int threads) { return inner_smem(lg, threads, C, args.n, args.NPF, packed, keep) <= 108 * 1024; };
         return t == 512 && !two(512) && two(256) ? 256 : t;
     };
-    auto smem_of = [&](int lg) { return inner_smem(lg, threads_of(lg), C, args.n, args.NPF, packed); };
+    auto smem_of = [&](int lg) { return inner_smem(lg, threads_of(lg), C, args.n, args.NPF, packed, keep); };
     int lg = tune == 2 ? 3 : tune == 4 ? 4 : 5;
     while (tune == 0 && lg > 3 && (smem_of(lg) > 108 * 1024 || (args.M >> lg) < 2u * (unsigned)sms)) --lg;
     while (lg > 0 && smem_of(lg) > 216 * 1024) --lg;

@@ -179,3 +179,23 @@ def test_nested_copies_start_at_the_branch_date(api, date):
         assert torch.equal(getattr(sim, w)(), v), w
     assert torch.allclose(got, acc / 3, rtol=3 * 2.0 ** -24, atol=0)
     sim.close()
+
+
+@pytest.mark.parametrize("C,M,N", [(1, 70, 15), (1, 33, 64), (2, 37, 130), (3, 65, 127), (3, 40, 64), (4, 5, 2050),
+                                   (8, 33, 257), (8, 1, 1), (16, 19, 67)])
+def test_kept_default_steps_at_the_edges_of_the_staged_draws(api, C, M, N):
+    """Rows of N C bytes of every alignment, draw counts around the staged ones, every tile."""
+    model = W.single_swap_model(tuple(0.02 + 0.05 * c for c in range(C)))
+    pf = W._swaps(np.random.default_rng(C), 12, 1, C, 1.0, 5.0)
+    sim = api.Simulation(model, [pf], W.Grid(5.0, 20), M, N, keep_defaults=True)
+    for inner in (0, 2, 4, 8):
+        sim.set_tiles(128, 256, inner, 2432, 1)
+        sim.defaults().zero_()
+        sim.run(3)
+        w = _clocks(api, 3, M, N, C)
+        thr = sim.thresholds().cpu().numpy().astype(np.float64)
+        idx = sim.defaults().cpu().numpy()
+        for c in range(C):
+            ref = np.stack([1 + np.searchsorted(thr[1:, c, k], w[k, :, c], side="left") for k in range(M)])
+            np.testing.assert_array_equal(idx[:, :, c], ref)
+    sim.close()
