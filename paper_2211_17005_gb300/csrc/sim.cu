@@ -50,6 +50,11 @@ __device__ __forceinline__ int lower_bound_pow2(Thr T, int n, float w)
     return pos + 1;
 }
 
+// Draws whose defaults a thread's queue holds: two, and more where the counterparties are so few
+// that the searches would run one or two at a time. One counterparty, 65536 paths, 512 draws, 50
+// dates, clocks to targets: 250 us with two draws, 168 with eight (178 for the two kernels of a
+// warp per path before).
+__host__ __device__ constexpr int queue_draws(int C) { return C == 1 ? 8 : C == 2 ? 4 : 2; }
 // A thread's draws between two stores of the staged steps: 32 bytes or so of them, so that few
 // counterparties do not mean many barriers (a multiple of 4: runs of whole 16 bytes).
 __host__ __device__ constexpr int idx_draws(int C) { return C >= 8 ? 4 : 32 / C / 4 * 4; }
@@ -58,7 +63,7 @@ __host__ __device__ constexpr int idx_draws(int C) { return C >= 8 ? 4 : 32 / C 
 __host__ __device__ constexpr int idx_stage_pitch(int lg, int C, int nthr) { return idx_draws(C) * (nthr >> lg) * C + 16; }
 __host__ __device__ constexpr size_t idx_stage_offset(int rows, int cnt_words, int lg, int C, int nthr)
 {
-    return (4 * (((size_t)rows << lg) + (size_t)cnt_words + (size_t)2 * C * nthr) + 15) / 16 * 16;
+    return (4 * (((size_t)rows << lg) + (size_t)cnt_words + (size_t)queue_draws(C) * C * nthr) + 15) / 16 * 16;
 }
 
 // Clocks, counts and targets of a tile of PT = 2^lg outer paths in one block.
@@ -72,7 +77,7 @@ __host__ __device__ constexpr size_t idx_stage_offset(int rows, int cnt_words, i
 // What bounds it: instruction issue while the clocks are drawn, HBM while thresholds and
 // exposures are read. Most clocks outlive the horizon (w > T(n)): a lane compares each
 // with its path's T(n), as an integer bound on the draw's 23 bits, and only queues the
-// ones that default (two draws' at most, in its own column of the queue), so that the
+// ones that default (a few draws' at most, in its own column of the queue), so that the
 // lower bounds run over queues a few entries long. The blocks of a multiprocessor are in
 // different phases, which overlaps the two bounds.
 // Paper shape, 2^17 paths, 64 draws, 100 dates: 0.40 ms; as two kernels with the counts in
@@ -94,7 +99,8 @@ __global__ void __launch_bounds__(512) inner_kernel(InnerArgs a)
     float *T = reinterpret_cast<float *>(smem);                                  // [rows][PT]: thresholds, then sums
     uint32_t *cnt = reinterpret_cast<uint32_t *>(T + ((size_t)a.rows << lg));    // counts
     const int cnt_words = ((n * C + ps) >> ps) << lg;
-    uint32_t *queue = cnt + cnt_words + tid;                                     // [2 C][nthr], this thread's column
+    constexpr int D = queue_draws(C);
+    uint32_t *queue = cnt + cnt_words + tid;                                     // [D C][nthr], this thread's column
     uint8_t *stage = reinterpret_cast<uint8_t *>(smem + idx_stage_offset(a.rows, cnt_words, lg, C, nthr));   // IDX: [PT][pitch]
     const int pitch = idx_stage_pitch(lg, C, nthr);
     const uint32_t M = a.M, tile0 = blockIdx.x << lg;
@@ -148,10 +154,10 @@ __global__ void __launch_bounds__(512) inner_kernel(InnerArgs a)
     // this thread's draws of [l0, l1)
     auto draw = [&](uint32_t l0, uint32_t l1) {
         int queued = 0;
-        bool even = false;
+        uint32_t held = 0;   // draws in the queue
         for (uint32_t l = l0 + (uint32_t)(tid >> lg); l < l1; l += stride) {
-            // an entry: the draw's 23 bits, (IDX) which of the two draws, the counterparty
-            const uint32_t tag = IDX && even ? 16u : 0u;
+            // an entry: the draw's 23 bits, (IDX) which of the queue's draws, the counterparty
+            const uint32_t tag = IDX ? held << 4 : 0u;
 #pragma unroll
             for (int cb = 0; cb < (C + 3) / 4; ++cb) {
                 const uint4 x = philox4x32_10(make_uint4(k, l, a.branch, (kStreamInner << 24) | (uint32_t)cb),
@@ -167,11 +173,10 @@ __global__ void __launch_bounds__(512) inner_kernel(InnerArgs a)
                     }
                 }
             }
-            even = !even;
-            if (even && l + stride < l1) continue;   // the queue holds two draws' defaults
+            if (++held < (uint32_t)D && l + stride < l1) continue;
             // the first draw's place in the staged row
-            const uint32_t row = IDX ? (uint32_t)(p * pitch) + (l - l0 - (even ? 0u : stride)) * C : 0u;
-            even = false;
+            const uint32_t row = IDX ? (uint32_t)(p * pitch) + (l - l0 - (held - 1) * stride) * C : 0u;
+            held = 0;
             // four entries at a time: their searches interleave
             for (int t = 0; t < queued; t += 4 * nthr) {
                 float w[4];
@@ -181,7 +186,7 @@ __global__ void __launch_bounds__(512) inner_kernel(InnerArgs a)
                     const uint32_t x = t + u * nthr < queued ? queue[t + u * nthr] : 0u;
                     w[u] = uniform23(x);
                     at[u] = Tp + ((x & (IDX ? 0xfu : 0x1ffu)) << (lg + 2));
-                    if (IDX) to[u] = row + (x & 16u ? stride * C : 0u);
+                    if (IDX) to[u] = row + (x >> 4 & (uint32_t)(D - 1)) * stride * C;
                 }
                 // first j with T(j) >= w among 1..n (T(n) >= w): the halving of a range of
                 // n depends on n only, so its steps are the same for every lane
