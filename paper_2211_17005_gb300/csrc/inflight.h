@@ -1,0 +1,30 @@
+// Bounded waits for the copies that one thread issues on B mbarriers in turn: copy u completes
+// phase u / B of barrier u % B. A barrier's parity tells two neighbouring phases apart and no
+// more, so at most one copy may be in flight per barrier. After a wait that gave up, the issuer
+// therefore requests nothing more, and before it goes on it waits once more, in full, for all it
+// has in flight: no copy outlives its CTA.
+//
+// Plain C++, so that the protocol can be run on the host.
+#pragma once
+#include <stdint.h>
+
+#ifdef __CUDACC__
+#define CVA_HD __host__ __device__ __forceinline__
+#else
+#define CVA_HD inline
+#endif
+
+namespace cva {
+
+// Whether copy u is complete, by wait(barrier, parity). `issued`: the copies issued so far, of
+// which the last B may be in flight; `issuer`: this thread issues them.
+template <uint32_t B, class Wait>
+CVA_HD bool await_copy(uint32_t u, uint32_t issued, bool issuer, Wait wait)
+{
+    if (wait(u % B, (u / B) & 1u)) return true;
+    if (issuer)
+        for (uint32_t v = issued > B ? issued - B : 0u; v < issued; ++v) (void)wait(v % B, (v / B) & 1u);
+    return false;
+}
+
+}  // namespace cva

@@ -158,10 +158,10 @@ struct Net {
     using L = Layout<U>;
     unsigned char *smem;
     uint32_t tmem = 0;
-    uint64_t *mbar, *sbar;         // tensor-core completion, input staging (this slot's)
+    uint64_t *mbar, *sbar, *dbar;  // tensor-core completion, input staging, a last completion (this slot's)
     uint32_t phase = 0, sphase = 0;
     bool good = true;              // no wait of this thread has given up
-    bool pending = false;          // a staging copy was issued and not yet consumed
+    bool pending = false;          // this thread issued a staging copy that is not yet consumed
     int tid, warp, lane, slot, row;
     const float *th, *mean, *istd;
     float *stage;
@@ -175,6 +175,7 @@ struct Net {
         row = tid & 127;
         mbar = mbars + slot;
         sbar = mbars + 2 + slot;
+        dbar = mbars + 4 + slot;
         th = reinterpret_cast<const float *>(smem + L::sTh);
         mean = reinterpret_cast<const float *>(smem + L::sVec);
         istd = mean + kIn;
@@ -269,12 +270,12 @@ struct Net {
     // reading the staging area; one thread issues the copies.
     __device__ void prefetch(const CUtensorMap *tm, const float *targ, int F, uint32_t path0)
     {
-        if (row == 32) {
+        if (row == 32 && good) {   // (nothing more after a wait that gave up)
             umma::mbar_arrive_expect_tx(sbar, (uint32_t)(F + 1) * kRows * 4u);
             umma::tma_load_2d(umma::smem_u32(stage), tm, (int32_t)path0, 0, sbar);
             umma::bulk_g2s(umma::smem_u32(stage + kIn * kRows), targ + path0, kRows * 4u, sbar);
+            pending = true;
         }
-        pending = true;
     }
 
     // wait for the staged tile; standardised inputs of this thread's row into the X
@@ -282,7 +283,7 @@ struct Net {
     // 1/std); y receives the target. False if the bounded wait gave up.
     __device__ bool stage_x(float &y)
     {
-        const bool ok = umma::mbar_wait(sbar, sphase, kMbarPolls);
+        const bool ok = await_copy<1>(sphase, sphase + 1u, row == 32, [&](uint32_t, uint32_t p) { return umma::mbar_wait(sbar, p, kMbarPolls); });
         sphase ^= 1u;
         pending = false;
         const float4 *mv = reinterpret_cast<const float4 *>(mean), *iv = reinterpret_cast<const float4 *>(istd);
@@ -512,7 +513,7 @@ __device__ void net_setup(Net<U> &n, uint32_t *s_tmem, uint64_t *s_mbar, const f
         umma::tmem_relinquish();
     }
     if (n.tid == 0) {
-        for (int i = 0; i < 4; ++i) umma::mbar_init(&s_mbar[i], 1);
+        for (int i = 0; i < 6; ++i) umma::mbar_init(&s_mbar[i], 1);
         umma::fence_mbar_init();
     }
     float *th = reinterpret_cast<float *>(n.smem + L::sTh);
@@ -544,7 +545,11 @@ __device__ void net_setup(Net<U> &n, uint32_t *s_tmem, uint64_t *s_mbar, const f
 template <int U>
 __device__ void net_teardown(Net<U> &n)
 {
-    if (n.pending) (void)umma::mbar_wait(n.sbar, n.sphase, kMbarPolls);   // no copy outlives the CTA
+    if (n.pending) (void)umma::mbar_wait(n.sbar, n.sphase, kMbarPolls);   // no copy outlives the CTA,
+    if (n.row == 0 && !n.good) {   // nor, after a wait that gave up, a product this thread issued
+        umma::commit(n.dbar);
+        (void)umma::mbar_wait(n.dbar, 0u, kMbarPolls);
+    }
     umma::fence_before_sync();
     __syncthreads();
     if (n.warp == 0) umma::tmem_dealloc(n.tmem, Layout<U>::tmem_cols);
@@ -608,7 +613,7 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_train_kernel(TrainArgs a, con
     using L = Layout<U>;
     extern __shared__ __align__(1024) unsigned char smem[];
     __shared__ uint32_t s_tmem;
-    __shared__ __align__(8) uint64_t s_mbar[4];
+    __shared__ __align__(8) uint64_t s_mbar[6];
     __shared__ __align__(8) uint64_t s_xbar[2];   // exchange: partial slices received, parameter slices received
     Net<U> n(smem, s_mbar);
     const uint32_t rank = umma::cluster_rank(), CL = umma::cluster_size();
@@ -799,7 +804,7 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_sweep_kernel(SweepArgs a, con
     constexpr int Z = L::Z;
     extern __shared__ __align__(1024) unsigned char smem[];
     __shared__ uint32_t s_tmem;
-    __shared__ __align__(8) uint64_t s_mbar[4];
+    __shared__ __align__(8) uint64_t s_mbar[6];
     __shared__ double s_red[8];
     __shared__ int s_flag[2];
     Net<U> n(smem, s_mbar);

@@ -12,6 +12,7 @@
 #include <string>
 
 #include "cva_internal.h"
+#include "inflight.h"
 
 namespace cva {
 namespace {

@@ -218,7 +218,7 @@ struct WNetT {
     uint64_t *mbar, *sbar;
     uint32_t phase = 0, sphase = 0;
     bool good = true;              // no wait of this thread has given up
-    bool pending = false;
+    bool pending = false;          // this thread issued a staging copy that is not yet consumed
     int tid, warp, lane, row, half;
     float *vec, *stage;
     const float *mean, *istd;
@@ -266,6 +266,13 @@ struct WNetT {
     {
         mma(issue, [] {});
     }
+    // the products this thread issued are complete (waited for once, at the end, on a barrier
+    // of its own: the parity of the others says nothing after a wait that gave up)
+    __device__ static void drain(uint64_t *dbar)
+    {
+        umma::commit(dbar);
+        (void)umma::mbar_wait(dbar, 0u, kMbarPolls);
+    }
     __device__ bool all_good() const { return __syncthreads_and(good) != 0; }
 
     // D = A B^T: A = K columns of a row buffer (width w, from column c0, K-major),
@@ -311,19 +318,19 @@ struct WNetT {
     // staging area
     __device__ void prefetch(const CUtensorMap *tm, const float *targ, int F, uint32_t path0)
     {
-        if (tid == 32) {
+        if (tid == 32 && good) {   // (nothing more after a wait that gave up)
             umma::mbar_arrive_expect_tx(sbar, (uint32_t)(F + 1) * kRows * 4u);
             umma::tma_load_2d(umma::smem_u32(stage), tm, (int32_t)path0, 0, sbar);
             umma::bulk_g2s(umma::smem_u32(stage + kIn * kRows), targ + path0, kRows * 4u, sbar);
+            pending = true;
         }
-        pending = true;
     }
 
     // wait for the staged tile; this thread's 16 standardised inputs into the X
     // columns of B; y receives the target
     __device__ bool stage_x(float &y)
     {
-        const bool ok = umma::mbar_wait(sbar, sphase, kMbarPolls);
+        const bool ok = await_copy<1>(sphase, sphase + 1u, tid == 32, [&](uint32_t, uint32_t p) { return umma::mbar_wait(sbar, p, kMbarPolls); });
         sphase ^= 1u;
         pending = false;
         const float4 *mv = reinterpret_cast<const float4 *>(mean), *iv = reinterpret_cast<const float4 *>(istd);
@@ -515,9 +522,10 @@ __device__ void wide_finish_setup(WNetT<L> &n, uint32_t *s_tmem)
 }
 
 template <class L>
-__device__ void wide_teardown(WNetT<L> &n)
+__device__ void wide_teardown(WNetT<L> &n, uint64_t *dbar)
 {
-    if (n.pending) (void)umma::mbar_wait(n.sbar, n.sphase, kMbarPolls);
+    if (n.pending) (void)umma::mbar_wait(n.sbar, n.sphase, kMbarPolls);   // no copy outlives the CTA,
+    if (n.tid == 0 && !n.good) n.drain(dbar);   // nor, after a wait that gave up, a product
     umma::fence_before_sync();
     __syncthreads();
     if (n.warp == 0) umma::tmem_dealloc(n.tmem, L::tmem_cols);
@@ -530,7 +538,7 @@ __global__ void __launch_bounds__(kWThreads, 1) wide_train_kernel(WTrainArgs a, 
 {
     extern __shared__ __align__(1024) unsigned char smem[];
     __shared__ uint32_t s_tmem;
-    __shared__ __align__(8) uint64_t s_mbar[3];   // tensor core, input staging, parameter reload
+    __shared__ __align__(8) uint64_t s_mbar[4];   // tensor core, input staging, parameter reload, tensor core at the end
     WNet n(smem, s_mbar);
     const int G = (int)gridDim.x, cta = (int)blockIdx.x;
     // owned slice [lo, hi) of the padded parameter vector (multiples of 4 entries)
@@ -540,6 +548,7 @@ __global__ void __launch_bounds__(kWThreads, 1) wide_train_kernel(WTrainArgs a, 
     wide_setup(n, &s_tmem, s_mbar, a.stats, a.F, false);
     if (n.tid == 0) {
         umma::mbar_init(&s_mbar[2], 1);
+        umma::mbar_init(&s_mbar[3], 1);
         umma::fence_mbar_init();
     }
     wide_load_params(n, a.init);
@@ -778,7 +787,7 @@ __global__ void __launch_bounds__(kWThreads, 1) wide_train_kernel(WTrainArgs a, 
             if (a.snap) a.snap[WL::p_of(q)] = t;
         }
     if (rpending) (void)umma::mbar_wait(rbar, rphase ^ 1u, kMbarPolls);   // no copy outlives the CTA
-    wide_teardown(n);
+    wide_teardown(n, &s_mbar[3]);
 }
 
 // Full-sample passes with fixed parameters, output ReLU on: the loss (mode 0), the
@@ -790,11 +799,15 @@ __global__ void __launch_bounds__(kWThreads, MinBlocks) wide_sweep_kernel(WSweep
     constexpr int Z = L::Z;
     extern __shared__ __align__(1024) unsigned char smem[];
     __shared__ uint32_t s_tmem;
-    __shared__ __align__(8) uint64_t s_mbar[2];
+    __shared__ __align__(8) uint64_t s_mbar[3];   // tensor core, input staging, tensor core at the end
     __shared__ double s_red[8][3];
     __shared__ int s_flag[2];
     WNetT<L> n(smem, s_mbar);
     wide_setup(n, &s_tmem, s_mbar, a.stats, a.F, a.mode == 1);
+    if (n.tid == 0) {
+        umma::mbar_init(&s_mbar[2], 1);
+        umma::fence_mbar_init();
+    }
     wide_load_params(n, a.theta);
     wide_finish_setup(n, &s_tmem);
 
@@ -914,7 +927,7 @@ __global__ void __launch_bounds__(kWThreads, MinBlocks) wide_sweep_kernel(WSweep
             P[(L::U + 1) * Z + L::U + 1] = c2;
         }
     }
-    wide_teardown(n);
+    wide_teardown(n, &s_mbar[2]);
 }
 
 // Loss (mode 0) and prediction (mode 2) passes: the forward pass of the trainer's tiles.
@@ -935,7 +948,7 @@ __global__ void __launch_bounds__(kFwdThreads, 1) wide_fwd_kernel(WSweepArgs a, 
     using L = WLP;
     extern __shared__ __align__(1024) unsigned char smem[];
     __shared__ uint32_t s_tmem;
-    __shared__ __align__(8) uint64_t s_mbar[4];   // tensor-core completion of group g: [2 g]
+    __shared__ __align__(8) uint64_t s_mbar[4];   // tensor-core completion of group g: [2 g], its last: [2 g + 1]
     __shared__ __align__(8) uint64_t s_sbar[L::kStages];   // staging buffer s complete
     __shared__ double s_red[kFwdThreads / 32];
     __shared__ int s_flag[2];
@@ -945,6 +958,7 @@ __global__ void __launch_bounds__(kFwdThreads, 1) wide_fwd_kernel(WSweepArgs a, 
     wide_setup(n, &s_tmem, s_mbar, a.stats, a.F, false);
     if (n.tid == 0) {
         umma::mbar_init(&s_mbar[2], 1);
+        umma::mbar_init(&s_mbar[3], 1);
         for (int q = 0; q < L::kStages; ++q) umma::mbar_init(&s_sbar[q], 1);
         umma::fence_mbar_init();
     }
@@ -957,10 +971,15 @@ __global__ void __launch_bounds__(kFwdThreads, 1) wide_fwd_kernel(WSweepArgs a, 
     wide_finish_setup(n, &s_tmem);
     uint64_t *bar = &s_mbar[2 * grp];
     uint32_t ph = 0;
-    bool ok = true, pend = false;   // pend: a GEMM issued and not yet waited for
+    bool ok = true, copies_ok = true;   // no wait of this thread (no wait for its copies) gave up
     unsigned char *const bp = smem + (grp ? L::sB1 : L::sB);
     const int b_off = grp ? L::sB1 : L::sB;
     const uint32_t dcol = 128u * (uint32_t)grp;
+
+    // the group's tiles: first, first + stride, ...
+    const uint32_t tiles = a.M / kRows, stride = 2u * gridDim.x, first = blockIdx.x + (uint32_t)grp * gridDim.x;
+    const uint32_t K = first < tiles ? (tiles - 1 - first) / stride + 1 : 0;
+    auto path_of = [&](uint32_t i) { return (first + i * stride) * kRows; };
 
     auto group_sync = [&] { asm volatile("bar.sync %0, 256;" ::"r"(1 + grp) : "memory"); };
     // tensor-core issue by the group's thread 0 once every thread's operands are written
@@ -973,19 +992,17 @@ __global__ void __launch_bounds__(kFwdThreads, 1) wide_fwd_kernel(WSweepArgs a, 
             f();
             umma::commit(bar);
         }
-        pend = true;
     };
     // (a wait that gave up is not repeated: every later one would run out too)
     auto wait = [&] {
         if (ok) ok = umma::mbar_wait(bar, ph, kMbarPolls);
         ph ^= 1u;
-        pend = !ok;
         umma::fence_after_sync();
     };
     // the inputs of the group's tile i (paths path0 ...) into its staging buffer i % 2
     // (one thread issues; called once no thread of the group reads that buffer any more)
     auto request = [&](uint32_t i, uint32_t path0) {
-        if (gt == 32 && ok) {
+        if (gt == 32 && copies_ok) {
             const int q = 2 * grp + (int)(i & 1u);
             const uint32_t dst = n.saddr(L::sStage + q * L::stage_bytes);
             umma::mbar_arrive_expect_tx(&s_sbar[q], (uint32_t)(a.F + 1) * kRows * 4u);
@@ -997,7 +1014,11 @@ __global__ void __launch_bounds__(kFwdThreads, 1) wide_fwd_kernel(WSweepArgs a, 
     // y receives the target
     auto stage_into = [&](uint32_t i, float &y) {
         const int q = 2 * grp + (int)(i & 1u);
-        if (ok) ok = umma::mbar_wait(&s_sbar[q], (i >> 1) & 1u, kMbarPolls);
+        if (copies_ok)   // (tiles i and i + 1 are requested by now)
+            copies_ok = await_copy<2>(i, min(K, i + 2u), gt == 32, [&](uint32_t b, uint32_t p) {
+                return umma::mbar_wait(&s_sbar[2 * grp + (int)b], p, kMbarPolls);
+            });
+        ok = ok && copies_ok;
         const float *stg = reinterpret_cast<const float *>(smem + L::sStage + q * L::stage_bytes);
         const float4 *mv = reinterpret_cast<const float4 *>(n.mean), *iv = reinterpret_cast<const float4 *>(n.istd);
         float x[16];
@@ -1035,10 +1056,6 @@ __global__ void __launch_bounds__(kFwdThreads, 1) wide_fwd_kernel(WSweepArgs a, 
         return (x.x + x.y) + (y.x + y.y);
     };
 
-    // the group's tiles: first, first + stride, ...
-    const uint32_t tiles = a.M / kRows, stride = 2u * gridDim.x, first = blockIdx.x + (uint32_t)grp * gridDim.x;
-    const uint32_t K = first < tiles ? (tiles - 1 - first) / stride + 1 : 0;
-    auto path_of = [&](uint32_t i) { return (first + i * stride) * kRows; };
     double acc = 0.0;
     float y = 0.f, y_next = 0.f;
     float *so = reinterpret_cast<float *>(smem + L::sOut) + grp * 2 * kRows;
@@ -1066,13 +1083,8 @@ __global__ void __launch_bounds__(kFwdThreads, 1) wide_fwd_kernel(WSweepArgs a, 
             }
         }
     }
-    // after a wait that gave up: no tensor-core work and no input copy outlives the CTA
-    // (bounded)
-    if (pend) (void)umma::mbar_wait(bar, ph ^ 1u, kMbarPolls);
-    if (!ok)
-        for (int q = 2 * grp; q < 2 * grp + 2; ++q)
-            for (uint32_t par = 0; par < 2; ++par) (void)umma::mbar_wait(&s_sbar[q], par, kMbarPolls >> 6);
-    if (!ok && gt == 0) atomicExch(a.err, 2);
+    if (gt == 0 && !ok) n.drain(&s_mbar[1 + 2 * grp]);   // no product outlives the CTA
+    if (!ok) atomicExch(a.err, 2);
     umma::fence_before_sync();
     __syncthreads();
     umma::fence_after_sync();
@@ -1107,7 +1119,7 @@ __global__ void __launch_bounds__(kFwdThreads, 1) wide_fwd_kernel(WSweepArgs a, 
                 for (int p = n.tid; p < L::NP; p += kFwdThreads) a.best[p] = __ldg(a.theta + p);
         }
     }
-    wide_teardown(n);
+    wide_teardown(n, &s_mbar[1]);
 }
 
 // ---- host side ----

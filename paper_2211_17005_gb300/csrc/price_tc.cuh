@@ -110,7 +110,7 @@ __global__ void __launch_bounds__(128 * kPriceSlots, 1) price_tc_kernel(OuterArg
     constexpr int F = 2 * E - 1 + CS, R = NPF * C;
     extern __shared__ __align__(1024) unsigned char tsm[];
     __shared__ uint32_t s_tmem;
-    __shared__ __align__(8) uint64_t s_mbar[2 * kPriceSlots];
+    __shared__ __align__(8) uint64_t s_mbar[3 * kPriceSlots];   // [slot][X buffer], then each slot's last
     const int tid = threadIdx.x, warp = tid >> 5, slot = tid >> 7, row = tid & 127;
     const size_t M = a.M;
     const int n = c_sim.n, ppp = c_sim.ppp;
@@ -143,7 +143,7 @@ __global__ void __launch_bounds__(128 * kPriceSlots, 1) price_tc_kernel(OuterArg
                 umma::tmem_relinquish();
             }
             if (tid == 0) {
-                for (int q = 0; q < 2 * kPriceSlots; ++q) umma::mbar_init(&s_mbar[q], 1);
+                for (int q = 0; q < 3 * kPriceSlots; ++q) umma::mbar_init(&s_mbar[q], 1);
                 umma::fence_mbar_init();
             }
             // the weights as TF32 head and tail: row r = pf C + c, column e GK + g: wA (g < LV),
@@ -292,10 +292,13 @@ __global__ void __launch_bounds__(128 * kPriceSlots, 1) price_tc_kernel(OuterArg
                     umma::fence_before_sync();
                 }
             }
-            // after a wait that gave up, the slot's MMAs still in flight complete (bounded)
-            // before the accumulators are freed
-            if (!ok && uses > 0)
-                (void)umma::mbar_wait(&s_mbar[2 * slot + (int)((uses - 1) % BUFS)], ((uses - 1) / BUFS) & 1u, kPriceMbarPolls);
+            // after a wait that gave up, the slot's MMAs still in flight complete (bounded) before
+            // the accumulators are freed: on a barrier of its own, as the parity of the buffers'
+            // says nothing once a phase was not waited for
+            if (!ok && row == 0) {
+                umma::commit(&s_mbar[2 * kPriceSlots + slot]);
+                (void)umma::mbar_wait(&s_mbar[2 * kPriceSlots + slot], 0u, kPriceMbarPolls);
+            }
             umma::fence_before_sync();
             __syncthreads();
             if (warp == 0) umma::tmem_dealloc(s_tmem, P::tmem_cols);
