@@ -345,6 +345,125 @@ __global__ void __launch_bounds__(32 * NW, NW == 8 ? 3 : 5) sim_kernel(OuterArgs
     }
 }
 
+// sim_kernel for one economy: a thread per path, with the noise of a step (one Philox block) in its
+// registers. There are no factors to split over warps, and where the paths fill the chip the
+// barriers and idle warps of sim_kernel only cost. Same operations in the same order, so
+// the same bits. Two counterparties of constant intensity, 50 dates, four warps per 32 paths / a
+// thread per path: 2^14 paths 27 / 28 us, 2^15 36 / 31, 2^17 97 / 63, 2^20 669 / 382 us.
+template <int C, int CS, SimMode MODE>
+__global__ void __launch_bounds__(128, 8) sim_thread_kernel(OuterArgs a)
+{
+    constexpr int F = 1 + CS, NB = (F + 3) / 4;
+    constexpr bool ADJ = MODE == SimMode::adjoint, CKPT = MODE == SimMode::restart;
+    const uint32_t kl = blockIdx.x * 128u + threadIdx.x;
+    if (kl >= a.M) return;
+    const uint32_t k = a.k0 + kl;
+    const size_t M = a.M;
+    const int n = c_sim.n, S = c_sim.S;
+    const float ds = c_sim.ds;
+    const double ds_d = c_sim.ds_d;
+    float r = c_sim.r0[0], gam[C], lam[C], lamc[C];
+    double I0 = 0.0;
+#pragma unroll
+    for (int c = 0; c < C; ++c) {
+        gam[c] = c_sim.gamma0[c];
+        lam[c] = lamc[c] = 0.f;
+    }
+    const int start = CKPT ? a.start : 0;
+    float *fe = a.features + kl, *th = a.thr + kl, *di = a.disc + kl;
+    auto write_date = [&](int j) {
+        fe[0] = r;
+        *di = (float)I0;
+#pragma unroll
+        for (int c = 0; c < C; ++c) {
+            if (c < CS) fe[(size_t)(1 + c) * M] = gam[c];
+            th[(size_t)c * M] = ADJ ? expf(-lam[c]) : -expm1f(-lam[c]);   // survival factor or threshold
+            if (CKPT && j == a.save_date) {
+                a.ckpt[(size_t)c * M + kl] = lam[c];
+                a.ckpt[(size_t)(C + c) * M + kl] = lamc[c];
+            }
+        }
+        if (CKPT && j == a.save_date) a.ckpt_I0[kl] = I0;
+        fe += (size_t)F * M;
+        th += (size_t)C * M;
+        di += M;
+    };
+    if (start > 0) {   // the dates up to the start are in place
+        fe += (size_t)start * F * M;
+        r = fe[0];
+#pragma unroll
+        for (int c = 0; c < C; ++c) {
+            if (c < CS) gam[c] = fe[(size_t)(1 + c) * M];
+            lam[c] = a.ckpt[(size_t)c * M + kl];
+            lamc[c] = a.ckpt[(size_t)(C + c) * M + kl];
+        }
+        I0 = a.ckpt_I0[kl];
+        fe += (size_t)F * M;
+        th += (size_t)(start + 1) * C * M;
+        di += (size_t)(start + 1) * M;
+    } else {
+        write_date(0);
+    }
+    for (int j = start + 1; j <= n; ++j) {
+        for (int q = (j - 1) * S; q < j * S; ++q) {
+            float W[F];
+#pragma unroll
+            for (int i = 0; i < F; ++i) W[i] = 0.f;
+#pragma unroll
+            for (int b = 0; b < NB; ++b) {
+                const uint4 x = philox4x32_10(make_uint4(k, (uint32_t)q, q >= a.branch_step ? a.branch : 0u,
+                                                         (kStreamOuter << 24) | (uint32_t)b),
+                                              a.seed_lo, a.seed_hi);
+                float z[4];
+                box_muller(x.x, x.y, z[0], z[1]);
+                box_muller(x.z, x.w, z[2], z[3]);
+#pragma unroll
+                for (int t = 0; t < 4; ++t)
+#pragma unroll
+                    for (int i = 4 * b + t; i < F; ++i) W[i] = fmaf(c_sim.L[i * (i + 1) / 2 + 4 * b + t], z[t], W[i]);
+            }
+            I0 = fma((double)r, ds_d, I0);
+#pragma unroll
+            for (int i = 0; i < F; ++i)
+                if (ADJ) a.inc[((size_t)q * F + i) * M + kl] = W[i];
+#pragma unroll
+            for (int c = 0; c < C; ++c) {
+                if (ADJ) a.gpre[((size_t)q * C + c) * M + kl] = gam[c];
+                const float gp = fmaxf(gam[c], 0.f);
+                const float y = fmaf(gp, ds, -lamc[c]);
+                const float t = lam[c] + y;
+                lamc[c] = (t - lam[c]) - y;
+                lam[c] = fmaxf(t, lam[c]);
+                if (c < CS)
+                    gam[c] += c_sim.cir_ktds[c] - c_sim.cir_kds[c] * gp + c_sim.cir_nu_sqds[c] * sqrtf(gp) * W[c < CS ? 1 + c : 0];
+            }
+            r += (__ldg(a.drift + q) - c_sim.hw_a_ds[0] * r) + c_sim.hw_sig_sqds[0] * W[0];
+        }
+        write_date(j);
+    }
+}
+
+// The path simulation in the form for its shape and path count. warps: 4 or 8 per 32 paths, 0 by
+// the number of paths.
+//  - 4 warps have the fewest instructions (more factors a warp) unless such blocks leave the
+//    chip short of warps: at the paper shape 8 warps take 91 us against 115 us for 2^10 paths,
+//    215 against 184 for 2^14 and 1265 against 1111 for 2^17;
+//  - one economy takes a thread per path from six blocks of 32 paths a multiprocessor on
+//    (sim_thread_kernel).
+template <int E, int C, int CS, SimMode MODE>
+void launch_sim(const OuterArgs &a, int warps, int sms, cudaStream_t st)
+{
+    const unsigned blocks = (a.M + 31u) / 32u;
+    if constexpr (E == 1) {
+        if (warps == 0 && blocks >= 6u * (unsigned)sms) {
+            sim_thread_kernel<C, CS, MODE><<<(a.M + 127u) / 128u, 128, 0, st>>>(a);
+            return;
+        }
+    }
+    if (warps ? warps == 8 : blocks < 2u * (unsigned)sms) sim_kernel<E, C, CS, 8, MODE><<<blocks, 256, 0, st>>>(a);
+    else sim_kernel<E, C, CS, 4, MODE><<<blocks, 128, 0, st>>>(a);
+}
+
 // Pricing on the FMA pipe: two paths per thread in packed FP32 pairs, the dates of one
 // period (p delta, (p+1) delta] per block, NPB portfolios per block (blockIdx.z picks the
 // group).
@@ -642,18 +761,11 @@ cva_status outer_launch(Sim &s, uint64_t seed, uint64_t k0, cudaStream_t st)
         }
     }
     const unsigned pb = (unsigned)(s.tune_price_block > 0 && s.tune_price_block <= 256 ? s.tune_price_block : 256);
-    // 4 warps per 32 paths (fewest instructions: more factors a warp) unless such blocks
-    // leave the chip short of warps: at the paper shape 8 warps take 91 us against 115 us
-    // for 2^10 paths, 215 against 184 for 2^14 and 1265 against 1111 for 2^17
     int sms = 0;
     CVA_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    const unsigned sgrid = (args.M + 31u) / 32u;
-    const bool wide = s.tune_sim_block ? s.tune_sim_block == 128 : sgrid < 2u * (unsigned)sms;
-    const bool restart = s.start_date > 0 || s.save_date >= 0;
-    if (restart && wide) sim_kernel<E, C, CS, 8, SimMode::restart><<<sgrid, 256, 0, st>>>(args);
-    else if (restart) sim_kernel<E, C, CS, 4, SimMode::restart><<<sgrid, 128, 0, st>>>(args);
-    else if (wide) sim_kernel<E, C, CS, 8, SimMode::plain><<<sgrid, 256, 0, st>>>(args);
-    else sim_kernel<E, C, CS, 4, SimMode::plain><<<sgrid, 128, 0, st>>>(args);
+    const int warps = s.tune_sim_block ? (s.tune_sim_block == 128 ? 8 : 4) : 0;
+    if (s.start_date > 0 || s.save_date >= 0) launch_sim<E, C, CS, SimMode::restart>(args, warps, sms, st);
+    else launch_sim<E, C, CS, SimMode::plain>(args, warps, sms, st);
     CVA_CUDA_TRY(cudaGetLastError());
     if (s.ev[1]) CVA_CUDA_TRY(cudaEventRecord(s.ev[1], st));
     if (s.tune_price_pf == 4) {   // every portfolio per 128-path tile on the tensor cores
@@ -774,8 +886,7 @@ cva_status adjoint_launch(Sim &s, AdjBuffers &b, uint64_t seed, uint64_t k0, uin
         CVA_CUDA_TRY(upload_consts(s, st));
         t_owner[dev] = &s;
     }
-    if (rblocks < 2u * (unsigned)sms) sim_kernel<E, C, CS, 8, SimMode::adjoint><<<rblocks, 256, 0, st>>>(o);
-    else sim_kernel<E, C, CS, 4, SimMode::adjoint><<<rblocks, 128, 0, st>>>(o);
+    launch_sim<E, C, CS, SimMode::adjoint>(o, 0, sms, st);
     CVA_CUDA_TRY(cudaGetLastError());
     const dim3 pgrid(tiles, periods * (unsigned)ps.splits);
     // weights, fixing adjoints, coupons, tables, parameter adjoints

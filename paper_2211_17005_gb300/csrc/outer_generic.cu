@@ -18,13 +18,15 @@
 namespace cva {
 namespace {
 
-constexpr int kGenWarps = 8;            // warps (and fine steps at a time) of the simulation
+constexpr int kGenSteps = 8;            // fine steps at a time of the simulation
 constexpr int kGenPriceThreads = 128;
+static_assert(kMaxE <= 16 && kMaxC <= 16, "eight warps hold two factors each");
 
-
-__global__ void __launch_bounds__(32 * kGenWarps) sim_generic_kernel(OuterArgs a)
+// NW warps per 32 paths, at most two economies and two counterparties a warp.
+template <int NW>
+__global__ void __launch_bounds__(32 * NW) sim_generic_kernel(OuterArgs a)
 {
-    constexpr int NW = kGenWarps, NS = NW, ME = (kMaxE + NW - 1) / NW, MC = (kMaxC + NW - 1) / NW;
+    constexpr int NS = kGenSteps, ME = 2, MC = 2;
     extern __shared__ __align__(16) unsigned char smem[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const uint32_t kl = blockIdx.x * 32u + (uint32_t)lane;
@@ -77,9 +79,9 @@ __global__ void __launch_bounds__(32 * kGenWarps) sim_generic_kernel(OuterArgs a
     const int steps = n * S;
     int j = 0, s = 0, jd = 0, sd = 0;
     for (int q0 = 0; q0 < steps; q0 += NS) {
-        const int q = q0 + warp;
-        if (q < steps) {   // warp w: the increments W = L z of step q0 + w, in place of the normals
-            float *w = Ws + warp * FR * 32 + lane;
+        for (int v = warp; v < NS && q0 + v < steps; v += NW) {   // the increments W = L z of a step, in place of the normals
+            const int q = q0 + v;
+            float *w = Ws + v * FR * 32 + lane;
             for (int b = 0; b < NB; ++b) {
                 const uint4 x = philox4x32_10(make_uint4(k, (uint32_t)q, q >= a.branch_step ? a.branch : 0u,
                                                          (kStreamOuter << 24) | (uint32_t)b),
@@ -682,14 +684,23 @@ cva_status outer_generic_launch(Sim &s, uint64_t seed, uint64_t k0, cudaStream_t
     }
     static std::atomic<bool> attr[64];
     if (!attr[dev].load(std::memory_order_acquire)) {
-        CVA_CUDA_TRY(cudaFuncSetAttribute(sim_generic_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * 1024));
+        for (auto kern : {sim_generic_kernel<1>, sim_generic_kernel<4>, sim_generic_kernel<8>})
+            CVA_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * 1024));
         CVA_CUDA_TRY(cudaFuncSetAttribute(price_generic_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
         attr[dev].store(true, std::memory_order_release);
     }
     int sms = 0;
     CVA_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    const size_t ssmem = (size_t)kGenWarps * (((size_t)s.F + 3) / 4 * 4 + 1) * 32 * sizeof(float);
-    sim_generic_kernel<<<(args.M + 31u) / 32u, 32 * kGenWarps, ssmem, st>>>(args);
+    // eight warps per 32 paths while such blocks do not fill the chip twice (and for shapes that
+    // need them), then four, and one where it can hold the factors and the blocks fill the chip
+    // six times. Two economies and counterparties, 50 dates, eight / four / one warp: 2^11 paths
+    // 42 / 48 / 89 us, 2^14 64 / 58 / 91, 2^16 181 / 149 / 130, 2^18 642 / 503 / 386 us
+    const size_t ssmem = (size_t)kGenSteps * (((size_t)s.F + 3) / 4 * 4 + 1) * 32 * sizeof(float);
+    const unsigned sblocks = (args.M + 31u) / 32u;
+    const int most = std::max(s.E, s.C);
+    if (sblocks < 2u * (unsigned)sms || most > 8) sim_generic_kernel<8><<<sblocks, 256, ssmem, st>>>(args);
+    else if (sblocks < 6u * (unsigned)sms || most > 2) sim_generic_kernel<4><<<sblocks, 128, ssmem, st>>>(args);
+    else sim_generic_kernel<1><<<sblocks, 32, ssmem, st>>>(args);
     CVA_CUDA_TRY(cudaGetLastError());
     if (s.ev[1]) CVA_CUDA_TRY(cudaEventRecord(s.ev[1], st));
     // portfolios per block: bond prices are computed once for them; up to 32 sums a thread

@@ -1,6 +1,8 @@
 """Edges of the kernels' tiles: path counts around a tile and a warp, step counts that leave
 a partial chunk, draw counts around the staging and counter widths, every width of the
 normal equations. References are computed here in FP64 or are the same paths of a larger run."""
+import dataclasses
+
 import numpy as np
 import pytest
 import torch
@@ -199,3 +201,31 @@ def test_kept_default_steps_at_the_edges_of_the_staged_draws(api, C, M, N):
             ref = np.stack([1 + np.searchsorted(thr[1:, c, k], w[k, :, c], side="left") for k in range(M)])
             np.testing.assert_array_equal(idx[:, :, c], ref)
     sim.close()
+
+
+@pytest.mark.parametrize("E,C,CS,M", [(1, 2, 0, 29184), (1, 2, 0, 29185), (1, 1, 1, 30001), (2, 2, 1, 29217),
+                                      (3, 5, 3, 9745), (3, 5, 3, 30001)])
+@pytest.mark.parametrize("S", [1, 3])
+def test_paths_do_not_depend_on_the_number_of_paths(api, E, C, CS, M, S):
+    """The forms taken at large path counts (a thread per path, one and four warps per 32 paths) give
+    the paths that 64 paths at a time give, branches and restarts included."""
+    model = W.small_model() if (E, C, CS) == (1, 2, 0) else W.paper_model(np.random.default_rng(E), E=E, C=C)
+    if CS < C and E > 1:   # the last ones of constant intensity
+        nu = np.array(model.cir_nu)
+        nu[CS:] = 0.0
+        model = dataclasses.replace(model, cir_nu=nu, corr=model.corr[:2 * E - 1 + CS, :2 * E - 1 + CS])
+    pf = W._swaps(np.random.default_rng(1), 12, E, C, 1.0, 5.0)
+    grid = W.Grid(5.0, 10, S)
+    big = api.Simulation(model, [pf], grid, M, 2)
+    few = api.Simulation(model, [pf], grid, 64, 2)
+    what = ("features", "discount_integral", "thresholds")
+    for k0 in (0, M - 64):
+        runs = [lambda s, k: s.run(5, k0=k), lambda s, k: s.run_twin(5, 4, 2, k0=k),
+                lambda s, k: s.nested_reference(5, 4, 2, k0=k)]
+        for run in runs:
+            run(big, 0)
+            run(few, k0)
+            for w in what:
+                assert torch.equal(getattr(few, w)(), getattr(big, w)()[..., k0:k0 + 64]), w
+    big.close()
+    few.close()
