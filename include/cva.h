@@ -336,8 +336,8 @@ CVA_API cva_status cva_regress_portfolios(cva_sim *sim, int basis, float *pred_d
 CVA_API cva_status cva_regress_alive(cva_sim *sim, int pf, float *pred_dev, double *coef_host, int *dropped_host,
                                      void *stream);
 
-/* Tile shapes of a simulation chosen by measurement (the values of cva_set_tiles): warps
- * per 32 paths of the path-simulation kernel, threads per block of the pricing kernel,
+/* Tile shapes of a simulation chosen by measurement (the values of cva_set_tiles): form
+ * of the path-simulation kernel, threads per block of the pricing kernel,
  * the tile of the inner-default kernel, the number of blocks of the grouped regression
  * (basis `basis`) and the pricing form. Each candidate runs on the simulation's own shapes (CUDA-event
  * timings, best of two after a warm-up); the choice is kept in the simulation and
@@ -347,8 +347,8 @@ CVA_API cva_status cva_autotune(cva_sim *sim, uint64_t seed, int basis, char *re
                                 void *stream);
 
 /* Sets the tile shapes of a simulation directly (e.g. a choice cva_autotune made
- * in an earlier process): sim_block in {64, 128} (4 and 8
- * warps per 32 paths), price_block in {128, 256},
+ * in an earlier process): sim_block in {64, 128} (64: four warps per 32 paths; 128, the
+ * default: the form for the number of paths), price_block in {128, 256},
  * inner_paths_per_block in {0 (automatic), 2, 4, 8 (tiles of 8, 16 and 32 paths, as
  * far as they fit shared memory)}, lsq_chunk_target in
  * [152, 2^20], and the pricing form portfolios_per_price_block: 1, 2 or 3 dividing

@@ -87,8 +87,8 @@ struct Sim {
     // device image of consts + weights (constant uploads are device-to-device, so
     // they can be captured in a CUDA graph)
     unsigned char *d_const_img = nullptr;
-    // tile shapes, set by cva_autotune (sim_block 0: by the number of paths)
-    int tune_sim_block = 0, tune_price_block = 256, tune_inner_P = 0, tune_lsq_chunks = 2432;
+    // tile shapes, set by cva_autotune
+    int tune_sim_block = 128, tune_price_block = 256, tune_inner_P = 0, tune_lsq_chunks = 2432;
     int tune_price_pf = 0;         // portfolios per pricing block (1, 2 or 3, dividing n_pf; 0: the largest of them; 4: tensor cores)
     // scratch of the portfolio-grouped regression, owned by the simulation
     double *d_lsq = nullptr;

@@ -443,24 +443,24 @@ __global__ void __launch_bounds__(128, 8) sim_thread_kernel(OuterArgs a)
     }
 }
 
-// The path simulation in the form for its shape and path count. warps: 4 or 8 per 32 paths, 0 by
-// the number of paths.
+// The path simulation in the form for its shape and path count (four: four warps per 32 paths
+// whatever the count).
 //  - 4 warps have the fewest instructions (more factors a warp) unless such blocks leave the
 //    chip short of warps: at the paper shape 8 warps take 91 us against 115 us for 2^10 paths,
 //    215 against 184 for 2^14 and 1265 against 1111 for 2^17;
 //  - one economy takes a thread per path from six blocks of 32 paths a multiprocessor on
 //    (sim_thread_kernel).
 template <int E, int C, int CS, SimMode MODE>
-void launch_sim(const OuterArgs &a, int warps, int sms, cudaStream_t st)
+void launch_sim(const OuterArgs &a, bool four, int sms, cudaStream_t st)
 {
     const unsigned blocks = (a.M + 31u) / 32u;
     if constexpr (E == 1) {
-        if (warps == 0 && blocks >= 6u * (unsigned)sms) {
+        if (!four && blocks >= 6u * (unsigned)sms) {
             sim_thread_kernel<C, CS, MODE><<<(a.M + 127u) / 128u, 128, 0, st>>>(a);
             return;
         }
     }
-    if (warps ? warps == 8 : blocks < 2u * (unsigned)sms) sim_kernel<E, C, CS, 8, MODE><<<blocks, 256, 0, st>>>(a);
+    if (!four && blocks < 2u * (unsigned)sms) sim_kernel<E, C, CS, 8, MODE><<<blocks, 256, 0, st>>>(a);
     else sim_kernel<E, C, CS, 4, MODE><<<blocks, 128, 0, st>>>(a);
 }
 
@@ -763,9 +763,9 @@ cva_status outer_launch(Sim &s, uint64_t seed, uint64_t k0, cudaStream_t st)
     const unsigned pb = (unsigned)(s.tune_price_block > 0 && s.tune_price_block <= 256 ? s.tune_price_block : 256);
     int sms = 0;
     CVA_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    const int warps = s.tune_sim_block ? (s.tune_sim_block == 128 ? 8 : 4) : 0;
-    if (s.start_date > 0 || s.save_date >= 0) launch_sim<E, C, CS, SimMode::restart>(args, warps, sms, st);
-    else launch_sim<E, C, CS, SimMode::plain>(args, warps, sms, st);
+    const bool four = s.tune_sim_block == 64;
+    if (s.start_date > 0 || s.save_date >= 0) launch_sim<E, C, CS, SimMode::restart>(args, four, sms, st);
+    else launch_sim<E, C, CS, SimMode::plain>(args, four, sms, st);
     CVA_CUDA_TRY(cudaGetLastError());
     if (s.ev[1]) CVA_CUDA_TRY(cudaEventRecord(s.ev[1], st));
     if (s.tune_price_pf == 4) {   // every portfolio per 128-path tile on the tensor cores
@@ -886,7 +886,7 @@ cva_status adjoint_launch(Sim &s, AdjBuffers &b, uint64_t seed, uint64_t k0, uin
         CVA_CUDA_TRY(upload_consts(s, st));
         t_owner[dev] = &s;
     }
-    launch_sim<E, C, CS, SimMode::adjoint>(o, 0, sms, st);
+    launch_sim<E, C, CS, SimMode::adjoint>(o, false, sms, st);
     CVA_CUDA_TRY(cudaGetLastError());
     const dim3 pgrid(tiles, periods * (unsigned)ps.splits);
     // weights, fixing adjoints, coupons, tables, parameter adjoints

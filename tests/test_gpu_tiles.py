@@ -229,3 +229,24 @@ def test_paths_do_not_depend_on_the_number_of_paths(api, E, C, CS, M, S):
                 assert torch.equal(getattr(few, w)(), getattr(big, w)()[..., k0:k0 + 64]), w
     big.close()
     few.close()
+
+
+def test_the_default_tiles_can_be_set(api):
+    """Setting the values a simulation starts with leaves it in the forms it starts in (results never
+    change, so by the time of the path simulation, where a wrong form takes over twice as long)."""
+    wl = W.make("small", M=1 << 19, N=1)
+    sim = api.Simulation(wl.model, wl.portfolios, wl.grid, wl.M, 1, profile=True)
+
+    def ms():
+        t = []
+        for _ in range(7):
+            sim.run(1)
+            torch.cuda.synchronize()
+            t.append(sim.kernel_ms()[0])
+        return float(np.median(t))
+
+    ms()
+    fresh = ms()
+    sim.set_tiles(128, 256, 0, 2432, 0)
+    assert ms() < 1.5 * fresh
+    sim.close()
