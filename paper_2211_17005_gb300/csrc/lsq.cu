@@ -224,11 +224,16 @@ static LsqPlan lsq_plan(int F, int basis, int nt, uint64_t M, int groups, int ta
     p.stride = (size_t)tri_index(p.m + nt, p.rows - 1, p.m + nt - 1) + 1;
     // 1024 rows a block at least, 512 where that would leave multiprocessors without work; the
     // quadratic basis takes a quarter of the blocks, whose reduction otherwise outweighs the
-    // few products of their rows (49 dates of 2^14 paths: 17 us with 784 blocks)
+    // few products of their rows (49 dates of 2^14 paths: 17 us with 784 blocks), and fewer the
+    // more targets a block reduces (six targets, 119 dates, the whole regression, with the
+    // blocks of one target / so: 2^11 paths 59 / 39 us, 2^13 79 / 54, 30001 paths 132 / 106)
     target = target > 0 ? target : 2432;
-    if (basis == CVA_BASIS_POLY2) target = std::max(target / 4, 1);
-    gram_chunks(M, groups, target, (uint64_t)groups * ((M + 1023) / 1024) < 304 ? 512 : 1024,
-                &p.rows_per_chunk, &p.chunks);
+    uint64_t min_rows = (uint64_t)groups * ((M + 1023) / 1024) < 304 ? 512 : 1024;
+    if (basis == CVA_BASIS_POLY2) {
+        target = std::max(target / 4 / (1 + nt / 3), 1);
+        if (nt >= 3) min_rows = 2048;
+    }
+    gram_chunks(M, groups, target, min_rows, &p.rows_per_chunk, &p.chunks);
     p.reduce = p.chunks > 48;
     p.doubles = (size_t)groups * (p.chunks + p.reduce) * p.stride + 2 * (size_t)groups * nt * p.m + (size_t)groups;
     return p;
