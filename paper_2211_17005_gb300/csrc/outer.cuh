@@ -88,7 +88,7 @@ __device__ __forceinline__ float expm1_small(float x)
     return p * x;
 }
 
-enum class SimMode { plain, adjoint, restart };
+enum class SimMode { plain, adjoint, forward, restart };
 
 struct OuterArgs {
     uint32_t M, k0, seed_lo, seed_hi;
@@ -106,7 +106,7 @@ struct OuterArgs {
     int start, save_date;
     float *ckpt;
     double *ckpt_I0;
-    float *inc, *gpre;                 // the adjoint's: [n*S][F][M] increments, [n*S][C][M] intensities before a fine step
+    float *inc, *gpre;                 // the adjoint's only: [n*S][F][M] increments, [n*S][C][M] intensities before a fine step
 };
 
 // Block: 32 outer paths (lane = path), NW warps. The normals of a fine step depend on no
@@ -120,8 +120,8 @@ struct OuterArgs {
 // as a single FMA): 352 instructions a step at 27 factors against 728 with one constant
 // load and one FMA per entry.
 //
-// Modes: adjoint, its forward sweep, which keeps e^{-Lambda} in the place of the thresholds,
-// and the increments and intensities of every fine step; restart, a run that starts at a
+// Modes: forward, for the smooth CVA_0, which keeps e^{-Lambda} in the place of the thresholds;
+// adjoint, which also keeps the increments and intensities of every fine step; restart, a run that starts at a
 // pricing date or saves what such a run needs (separate instances: their pointers would
 // spill the plain one's registers).
 //
@@ -136,7 +136,7 @@ __global__ void __launch_bounds__(32 * NW, NW == 8 ? 3 : 5) sim_kernel(OuterArgs
     constexpr int F = 2 * E - 1 + CS;
     constexpr int NB = (F + 3) / 4, FP = (F + 1) / 2 * 2;
     constexpr int ME = (E + NW - 1) / NW, MC = (C + NW - 1) / NW;   // factors of a warp
-    constexpr bool ADJ = MODE == SimMode::adjoint, CKPT = MODE == SimMode::restart;
+    constexpr bool ADJ = MODE == SimMode::adjoint, SURV = ADJ || MODE == SimMode::forward, CKPT = MODE == SimMode::restart;
     constexpr int NS = F <= 8 ? 32 : 8;                             // fine steps at a time
     __shared__ float Ws[NS][F][32], R0[NS][32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -213,7 +213,7 @@ __global__ void __launch_bounds__(32 * NW, NW == 8 ? 3 : 5) sim_kernel(OuterArgs
                 if (has_c(i)) {
                     if (is_cir(i)) pg[(size_t)(NW * i) * M] = gam[i];
                     // threshold (0 at date 0) or survival factor
-                    pt[(size_t)(NW * i) * M] = ADJ ? expf(-lam[i]) : -expm1f(-lam[i]);
+                    pt[(size_t)(NW * i) * M] = SURV ? expf(-lam[i]) : -expm1f(-lam[i]);
                 }
         }
         pr += (size_t)F * M;
@@ -354,7 +354,7 @@ template <int C, int CS, SimMode MODE>
 __global__ void __launch_bounds__(128, 8) sim_thread_kernel(OuterArgs a)
 {
     constexpr int F = 1 + CS, NB = (F + 3) / 4;
-    constexpr bool ADJ = MODE == SimMode::adjoint, CKPT = MODE == SimMode::restart;
+    constexpr bool ADJ = MODE == SimMode::adjoint, SURV = ADJ || MODE == SimMode::forward, CKPT = MODE == SimMode::restart;
     const uint32_t kl = blockIdx.x * 128u + threadIdx.x;
     if (kl >= a.M) return;
     const uint32_t k = a.k0 + kl;
@@ -377,7 +377,7 @@ __global__ void __launch_bounds__(128, 8) sim_thread_kernel(OuterArgs a)
 #pragma unroll
         for (int c = 0; c < C; ++c) {
             if (c < CS) fe[(size_t)(1 + c) * M] = gam[c];
-            th[(size_t)c * M] = ADJ ? expf(-lam[c]) : -expm1f(-lam[c]);   // survival factor or threshold
+            th[(size_t)c * M] = SURV ? expf(-lam[c]) : -expm1f(-lam[c]);   // survival factor or threshold
             if (CKPT && j == a.save_date) {
                 a.ckpt[(size_t)c * M + kl] = lam[c];
                 a.ckpt[(size_t)(C + c) * M + kl] = lamc[c];
@@ -837,17 +837,18 @@ cva_status adjoint_launch(Sim &s, AdjBuffers &b, uint64_t seed, uint64_t k0, uin
     };
     AdjSplitArgs a = {};
     a.part_p = reinterpret_cast<double *>(take(pblocks * (2 * E + 1) * 8));
-    a.part_r = reinterpret_cast<double *>(take((size_t)rblocks * NPAR * 8));
+    auto take_rev = [&](size_t bytes) { return b.forward_only ? nullptr : take(bytes); };   // the reverse sweep's
+    a.part_r = reinterpret_cast<double *>(take_rev((size_t)rblocks * NPAR * 8));
     float *features = reinterpret_cast<float *>(take((n + 1) * F * Mz * 4));
     float *disc = reinterpret_cast<float *>(take((n + 1) * Mz * 4));
     float *surv = reinterpret_cast<float *>(take((n + 1) * C * Mz * 4));
-    float *inc = reinterpret_cast<float *>(take(q * F * Mz * 4));
-    float *gpre = reinterpret_cast<float *>(take(q * C * Mz * 4));
-    a.V = reinterpret_cast<float *>(take((n + 1) * C * Mz * 4));
-    a.rbin = reinterpret_cast<float *>(take(n * E * Mz * 4));
-    a.lbin = reinterpret_cast<float *>(take(n * E * Mz * 4));
-    a.ibin = reinterpret_cast<float *>(take(n * Mz * 4));
-    a.fixin = reinterpret_cast<float *>(take((size_t)periods * ps.splits * E * Mz * 4));
+    float *inc = reinterpret_cast<float *>(take_rev(q * F * Mz * 4));
+    float *gpre = reinterpret_cast<float *>(take_rev(q * C * Mz * 4));
+    a.V = reinterpret_cast<float *>(take_rev((n + 1) * C * Mz * 4));
+    a.rbin = reinterpret_cast<float *>(take_rev(n * E * Mz * 4));
+    a.lbin = reinterpret_cast<float *>(take_rev(n * E * Mz * 4));
+    a.ibin = reinterpret_cast<float *>(take_rev(n * Mz * 4));
+    a.fixin = reinterpret_cast<float *>(take_rev((size_t)periods * ps.splits * E * Mz * 4));
     if (!b.scratch) {
         b.scratch_bytes = off;
         return CVA_OK;
@@ -886,7 +887,8 @@ cva_status adjoint_launch(Sim &s, AdjBuffers &b, uint64_t seed, uint64_t k0, uin
         CVA_CUDA_TRY(upload_consts(s, st));
         t_owner[dev] = &s;
     }
-    launch_sim<E, C, CS, SimMode::adjoint>(o, false, sms, st);
+    if (b.forward_only) launch_sim<E, C, CS, SimMode::forward>(o, false, sms, st);
+    else launch_sim<E, C, CS, SimMode::adjoint>(o, false, sms, st);
     CVA_CUDA_TRY(cudaGetLastError());
     const dim3 pgrid(tiles, periods * (unsigned)ps.splits);
     // weights, fixing adjoints, coupons, tables, parameter adjoints

@@ -250,3 +250,16 @@ def test_the_default_tiles_can_be_set(api):
     sim.set_tiles(128, 256, 0, 2432, 0)
     assert ms() < 1.5 * fresh
     sim.close()
+
+
+@pytest.mark.parametrize("name,M,n,S", [("adjoint", 1, 10, 1), ("adjoint", 9800, 20, 3), ("small", 33, 25, 1),
+                                        ("small", 30001, 25, 4), ("adjoint", 70001, 100, 1)])
+def test_forward_alone_gives_the_gradients_value(api, name, M, n, S):
+    """The forward keeps fewer arrays than the gradient and may take other path ranges: the same
+    FP64 terms in another order."""
+    wl = W.make(name, M=M, n_steps=n, substeps=S)
+    pf = api.frozen(wl.model, wl.portfolios[0])
+    c, g = api.grad_cva0(wl.model, pf, wl.grid, M, wl.seed)
+    f, none = api.grad_cva0(wl.model, pf, wl.grid, M, wl.seed, forward_only=True)
+    assert none is None and np.all(np.isfinite(g))
+    assert f == pytest.approx(c, rel=1e-13)
