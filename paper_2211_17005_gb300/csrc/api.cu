@@ -13,6 +13,7 @@
 #include <vector>
 
 #include "cva_internal.h"
+#include "ranges.h"
 
 namespace cva {
 
@@ -978,35 +979,10 @@ cva_status cva_grad_cva0(const cva_model_desc *model, const cva_portfolio_desc *
     const size_t Mz = M;
     const unsigned blocks = (unsigned)((M + 127) / 128);
     cudaStream_t cs = reinterpret_cast<cudaStream_t>(stream);
-    // the compiled shapes take the paths in equal ranges whose arrays fit a limit; the
-    // run-time shapes take them at once, with checkpoints
-    uint64_t ranges = 1, Mr = M;
     const size_t nsum = s.generic ? (size_t)NPAR + 1 : (size_t)(2 * E + 1 + NPAR);
-    auto plan = [&](size_t limit) -> cva_status {
-        for (ranges = 1;;) {
-            Mr = (M + ranges - 1) / ranges;
-            const cva_status r = launch_adjoint(s, b, seed, k0, (uint32_t)Mr, cs);   // without scratch: its size
-            if (r != CVA_OK) return r;
-            if (b.scratch_bytes <= limit || Mr <= 256) break;
-            ranges = std::max(ranges + 1, ranges * (b.scratch_bytes / limit));
-        }
-        Mr = (Mr + 255) / 256 * 256;   // whole blocks
-        ranges = (M + Mr - 1) / Mr;
-        size_t most = 0;   // the full ranges and the last one
-        for (uint64_t m : {std::min<uint64_t>(Mr, M), M - (ranges - 1) * Mr}) {
-            const cva_status r = launch_adjoint(s, b, seed, k0, (uint32_t)m, cs);
-            if (r != CVA_OK) return r;
-            most = std::max(most, b.scratch_bytes);
-        }
-        b.scratch_bytes = most;
-        return CVA_OK;
-    };
+    unsigned char *tables = nullptr;
     auto cleanup = [&]() {
-        cudaFree(b.dzc);
-        cudaFree(b.dfix);
-        cudaFree(b.ddrift);
-        cudaFree(b.rho);
-        cudaFree(b.sig);
+        cudaFree(tables);
         cudaFree(b.ckpt);
         cudaFree(b.ckpt_I0);
         cudaFree(b.fixr);
@@ -1015,38 +991,69 @@ cva_status cva_grad_cva0(const cva_model_desc *model, const cva_portfolio_desc *
         cudaFree(b.scratch);
         cva_sim_destroy(hs);
     };
-    // less memory free than the arrays of the widest ranges: narrower ones
-    for (size_t limit = kAdjScratch; !s.generic && !b.scratch; limit /= 2) {
-        st = plan(limit);
-        if (st == CVA_OK && dev_alloc(&b.scratch, b.scratch_bytes) != CVA_OK) {
-            cudaGetLastError();   // (the failed allocation's)
-            if (Mr <= 256 || limit < 2) st = CVA_ENOMEM;
-        }
-        if (st != CVA_OK) {
-            cleanup();
-            return st;
-        }
+    // the tables in one block, before the arrays whose size has a choice
+    std::vector<unsigned char> img;
+    auto put = [&](const void *v, size_t bytes) {
+        const size_t at = img.size();
+        img.resize(at + (bytes + 255) / 256 * 256);
+        memcpy(img.data() + at, v, bytes);
+        return at;
+    };
+    const size_t o_dzc = put(dzc.data(), dzc.size() * sizeof(float4)), o_dfix = put(dfix.data(), dfix.size() * sizeof(float2)),
+                 o_ddrift = put(ddrift.data(), ddrift.size() * sizeof(float2)),
+                 o_rho = put(rho.data(), rho.size() * sizeof(float)), o_sig = put(sig.data(), sig.size() * sizeof(float));
+    st = dev_alloc(&tables, img.size());
+    if (st == CVA_OK) {
+        const cudaError_t e = cudaMemcpyAsync(tables, img.data(), img.size(), cudaMemcpyHostToDevice, cs);
+        if (e != cudaSuccess) st = cuda_fail(e, "grad: table upload");
     }
-    if (dev_alloc(&b.dzc, dzc.size()) != CVA_OK || dev_alloc(&b.dfix, dfix.size()) != CVA_OK ||
-        dev_alloc(&b.ddrift, ddrift.size()) != CVA_OK || dev_alloc(&b.rho, rho.size()) != CVA_OK ||
-        dev_alloc(&b.sig, sig.size()) != CVA_OK || dev_alloc(&b.sum, nsum * ranges) != CVA_OK ||
-        (s.generic && (dev_alloc(&b.ckpt, (size_t)b.nseg * NV * Mz) != CVA_OK ||
-                       dev_alloc(&b.ckpt_I0, (size_t)b.nseg * Mz) != CVA_OK ||
-                       dev_alloc(&b.fixr, (size_t)(periods + 1) * E * Mz) != CVA_OK ||
-                       dev_alloc(&b.part, (size_t)blocks * (NPAR + 1)) != CVA_OK))) {
+    if (st != CVA_OK) {
         cleanup();
-        return CVA_ENOMEM;
+        return st;
     }
-    cudaError_t e1 = cudaMemcpyAsync(b.dzc, dzc.data(), dzc.size() * sizeof(float4), cudaMemcpyHostToDevice, cs);
-    cudaError_t e2 = cudaMemcpyAsync(b.dfix, dfix.data(), dfix.size() * sizeof(float2), cudaMemcpyHostToDevice, cs);
-    cudaError_t e3 = cudaMemcpyAsync(b.ddrift, ddrift.data(), ddrift.size() * sizeof(float2), cudaMemcpyHostToDevice, cs);
-    cudaError_t e4 = cudaMemcpyAsync(b.rho, rho.data(), rho.size() * sizeof(float), cudaMemcpyHostToDevice, cs);
-    cudaError_t e5 = cudaMemcpyAsync(b.sig, sig.data(), sig.size() * sizeof(float), cudaMemcpyHostToDevice, cs);
-    for (cudaError_t e : {e1, e2, e3, e4, e5})
-        if (e != cudaSuccess) {
-            cleanup();
-            return cuda_fail(e, "grad: table upload");
+    b.dzc = reinterpret_cast<float4 *>(tables + o_dzc);
+    b.dfix = reinterpret_cast<float2 *>(tables + o_dfix);
+    b.ddrift = reinterpret_cast<float2 *>(tables + o_ddrift);
+    b.rho = reinterpret_cast<float *>(tables + o_rho);
+    b.sig = reinterpret_cast<float *>(tables + o_sig);
+    // the compiled shapes take the paths in equal ranges whose arrays fit a limit and half of
+    // the memory that is free, in narrower ones where that cannot be had; the run-time shapes
+    // take them at once, with checkpoints
+    RangePlan plan;
+    plan.per = M;
+    plan.ranges = 1;
+    if (s.generic) {
+        if (dev_alloc(&b.sum, nsum) != CVA_OK || dev_alloc(&b.ckpt, (size_t)b.nseg * NV * Mz) != CVA_OK ||
+            dev_alloc(&b.ckpt_I0, (size_t)b.nseg * Mz) != CVA_OK ||
+            dev_alloc(&b.fixr, (size_t)(periods + 1) * E * Mz) != CVA_OK ||
+            dev_alloc(&b.part, (size_t)blocks * (NPAR + 1)) != CVA_OK)
+            st = CVA_ENOMEM;
+    } else {
+        st = launch_adjoint(s, b, seed, k0, (uint32_t)M, cs);   // without scratch: its size
+        size_t room = 0, all = 0;
+        if (st == CVA_OK) {
+            const cudaError_t e = cudaMemGetInfo(&room, &all);
+            if (e != cudaSuccess) st = cuda_fail(e, "grad: free memory");
         }
+        auto bytes = [&](uint64_t paths) {
+            (void)launch_adjoint(s, b, seed, k0, (uint32_t)paths, cs);
+            return b.scratch_bytes;
+        };
+        auto allocate = [&](const RangePlan &p) {
+            if (dev_alloc(&b.sum, nsum * p.ranges) == CVA_OK && dev_alloc(&b.scratch, p.bytes) == CVA_OK) return true;
+            cudaGetLastError();   // (the failed allocation's)
+            cudaFree(b.sum);
+            b.sum = nullptr;
+            return false;
+        };
+        if (st == CVA_OK && !fit_ranges(M, std::min(kAdjScratch, room / 2), bytes, allocate, &plan)) st = CVA_ENOMEM;
+        b.scratch_bytes = plan.bytes;
+    }
+    if (st != CVA_OK) {
+        cleanup();
+        return st;
+    }
+    const uint64_t ranges = plan.ranges, Mr = plan.per;
     if (s.generic) {
         st = launch_adjoint(s, b, seed, k0, (uint32_t)M, cs);
         if (st == CVA_OK) st = sum_columns_fp64(b.part, (int)blocks, NPAR + 1, b.sum, cs);
