@@ -892,8 +892,10 @@ cva_status adjoint_launch(Sim &s, AdjBuffers &b, uint64_t seed, uint64_t k0, uin
     CVA_CUDA_TRY(cudaGetLastError());
     const dim3 pgrid(tiles, periods * (unsigned)ps.splits);
     // weights, fixing adjoints, coupons, tables, parameter adjoints
-    constexpr size_t psmem = (size_t)E * C * 2 * G * 8 + (size_t)E * 128 * (8 + 8 + 8) + 2 * (size_t)E * G * 16;
-    static_assert(psmem <= 47 * 1024, "adjoint pricing: default shared-memory limit");
+    constexpr size_t psmem = (size_t)E * C * 2 * G * 8 + (size_t)E * 128 * (8 + 8 + 16) + 2 * (size_t)E * G * 16;
+    static_assert(3 * (psmem + 2048) <= 227 * 1024, "adjoint pricing: three blocks a multiprocessor");
+    for (auto kern : {adj_price_kernel<E, C, CS, G, false>, adj_price_kernel<E, C, CS, G, true>})
+        CVA_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)psmem));
     if (b.forward_only) {
         adj_price_kernel<E, C, CS, G, false><<<pgrid, 128, psmem, st>>>(a, ps);
         CVA_CUDA_TRY(cudaGetLastError());

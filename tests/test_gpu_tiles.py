@@ -263,3 +263,17 @@ def test_forward_alone_gives_the_gradients_value(api, name, M, n, S):
     f, none = api.grad_cva0(wl.model, pf, wl.grid, M, wl.seed, forward_only=True)
     assert none is None and np.all(np.isfinite(g))
     assert f == pytest.approx(c, rel=1e-13)
+
+
+@pytest.mark.parametrize("name,n", [("adjoint", 10), ("small", 25)])
+def test_adjoints_of_paths_are_added_in_fp64(api, name, n):
+    """A path's adjoints do not depend on the other paths of its thread and block, so the sums of two
+    calls are those of one to FP64 rounding (paths 0 and 128 share a thread)."""
+    wl = W.make(name, M=129, n_steps=n)
+    pf = api.frozen(wl.model, wl.portfolios[0])
+    c, g = api.grad_cva0(wl.model, pf, wl.grid, 129, wl.seed)
+    c1, g1 = api.grad_cva0(wl.model, pf, wl.grid, 128, wl.seed)
+    c2, g2 = api.grad_cva0(wl.model, pf, wl.grid, 1, wl.seed, k0=128)
+    assert c * 129 == pytest.approx(c1 * 128 + c2, rel=1e-12)
+    ref = g1 * 128 + g2
+    np.testing.assert_allclose(g * 129, ref, rtol=1e-12, atol=1e-12 * np.abs(ref).max())
