@@ -329,8 +329,8 @@ CVA_API cva_status cva_regress_portfolios(cva_sim *sim, int basis, float *pred_d
  * (every counterparty alive). coef_host: double [n][1+F+C] (nullable; date 0
  * untouched) receives w_i in the raw basis [1, Y_i, X_i]. dropped_host: int [n]
  * (nullable) receives the number of dropped columns per date (0 at date 0). The
- * scratch (n C M floats of per-path default counts, the pair and loss sums of each
- * tile of at most 32 paths, and the Gram partials) belongs to the simulation: the first
+ * scratch (n C M floats of per-path default counts, the pair sums of each tile of at most
+ * 32 paths, the loss sums of each 8, and the Gram partials) belongs to the simulation: the first
  * call allocates it, so make one call before capturing this one in a CUDA graph. Synchronises `stream` only when coef_host or dropped_host is
  * given. */
 CVA_API cva_status cva_regress_alive(cva_sim *sim, int pf, float *pred_dev, double *coef_host, int *dropped_host,

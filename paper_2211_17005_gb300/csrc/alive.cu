@@ -14,9 +14,9 @@
 // and N xi_bar^k for the right-hand side of Y. P_cd and q_c enter only through their
 // sums over the paths, d_c also through its products with Y.
 //
-// alive_stats_kernel turns a tile of paths' default steps into d_c per path and the
-// tile's sums of P_cd and q_c at every date. gram.cuh accumulates sum_k [1, Y - Y^0]^T
-// [1, Y - Y^0, d, xi_bar]. alive_pq_kernel adds the tiles' P_cd and q_c.
+// alive_stats_kernel turns a tile of paths' default steps into d_c per path, the tile's
+// sums of P_cd and the sums of q_c over at most eight paths at every date. gram.cuh accumulates sum_k [1, Y - Y^0]^T
+// [1, Y - Y^0, d, xi_bar]. alive_pq_kernel adds the P_cd and q_c.
 // alive_solve_kernel adds the Gram chunks, assembles the (1 + F + C)-square system and
 // solves it by a Jacobi-scaled Cholesky factorisation in FP64, dropping a column whose
 // pivot vanishes (a counterparty with no default by t_i anywhere in the sample).
@@ -41,9 +41,10 @@ struct AliveArgs {
     const float *disc;        // [n+1][M]
     const float *feat;        // [n+1][F][M]
     float *dstat;             // [n][C][M] d_c per path
-    float *qsum;              // [n][NQ][nblk] P_cd, q_c summed over a tile's paths
+    float *psum;              // [n][NP][nblk] P_cd summed over a tile's paths
+    float *qsum;              // [n][C][nblk << (lg - lq)] q_c summed over at most eight of them
     uint32_t nblk;            // tiles of the statistics kernel
-    int lg;                   // log2 of its paths per tile
+    int lg, lq;               // log2 of its paths per tile, of the paths q_c is summed over in FP32
     int chunks;
     size_t stride;            // doubles of a Gram partial
     double *part;             // [n-1][chunks][stride]
@@ -93,7 +94,7 @@ __host__ __device__ inline StatShape stat_shape(int lg, int C, int n)
 template <int C>
 __global__ void __launch_bounds__(256) alive_stats_kernel(AliveArgs a)
 {
-    constexpr int NP = C * (C - 1) / 2, NQ = NP + C;
+    constexpr int NP = C * (C - 1) / 2;
     extern __shared__ __align__(16) unsigned char smem[];
     const int n = a.n, lg = a.lg, PT = 1 << lg, tid = threadIdx.x, nthr = blockDim.x;
     const StatShape sh = stat_shape(lg, C, n);
@@ -187,20 +188,22 @@ __global__ void __launch_bounds__(256) alive_stats_kernel(AliveArgs a)
         if (live) a.dstat[((size_t)i * C + c) * M + kl] = (float)defaults;
     }
     __syncthreads();
-    // q_c over the tile's paths: a thread per (date, c), which starts at a path of its own so
-    // that a warp's reads spread over the banks
-    for (int t = tid; t < (n - 1) * C; t += nthr) {
-        const int i = 1 + t / C, d = t % C;
-        const float *src = reinterpret_cast<const float *>(smem + sh.dq) + i * nthr + (d << lg);
+    // q_c over eight of the tile's paths at a time (the sums go on in FP64 from there): a thread
+    // per (date, c, eight paths), which starts at a path of its own so that a warp's reads
+    // spread over the banks
+    const int lr = lg - a.lq, QT = 1 << a.lq;
+    for (int t = tid; t < ((n - 1) * C) << lr; t += nthr) {
+        const int e = t & ((1 << lr) - 1), i = 1 + (t >> lr) / C, d = (t >> lr) % C;
+        const float *src = reinterpret_cast<const float *>(smem + sh.dq) + i * nthr + (d << lg) + (e << a.lq);
         float s = 0.f;
-        for (int u = 0; u < PT; ++u) s += src[(u + tid) & (PT - 1)];
-        a.qsum[((size_t)i * NQ + NP + d) * a.nblk + blockIdx.x] = s;
+        for (int u = 0; u < QT; ++u) s += src[(u + (tid >> 2)) & (QT - 1)];
+        a.qsum[(((size_t)i * C + d) * a.nblk + blockIdx.x << lr) + e] = s;
     }
     for (int t = tid; t < NP; t += nthr) {
         int s = 0;
         for (int i = 1; i < n; ++i) {
             s += pair[i * NP + t];
-            a.qsum[((size_t)i * NQ + t) * a.nblk + blockIdx.x] = (float)s;
+            a.psum[((size_t)i * NP + t) * a.nblk + blockIdx.x] = (float)s;
         }
     }
 }
@@ -211,7 +214,9 @@ __global__ void __launch_bounds__(256) alive_pq_kernel(AliveArgs a)
 {
     __shared__ double sh[256];
     const int q = blockIdx.x, i = blockIdx.y + 1, tid = threadIdx.x, NP = a.NQ - a.C;
-    const float *src = a.qsum + ((size_t)i * a.NQ + q) * a.nblk;
+    const int lr = a.lg - a.lq;
+    const float *src = q < NP ? a.psum + ((size_t)i * NP + q) * a.nblk
+                              : a.qsum + (((size_t)i * a.C + (q - NP)) * a.nblk << lr);
     double s = 0.0;
     if (q < NP) {
         long long t = 0;
@@ -220,7 +225,7 @@ __global__ void __launch_bounds__(256) alive_pq_kernel(AliveArgs a)
         s = (double)t;
     } else {
 #pragma unroll 8
-        for (uint32_t b = tid; b < a.nblk; b += 256) s += (double)__ldg(src + b);
+        for (uint32_t b = tid; b < a.nblk << lr; b += 256) s += (double)__ldg(src + b);
     }
     sh[tid] = s;
     __syncthreads();
@@ -319,7 +324,8 @@ cva_status alive_regress(Sim &s, int pf, float *pred_dev, double *coef_host, int
     gram_chunks(M, groups, s.tune_lsq_chunks > 0 ? s.tune_lsq_chunks : 2432, 1024, &rows_per_chunk, &chunks);
     const size_t stride = (size_t)tri_index(cols, mY - 1, cols - 1) + 1;
     const size_t need = (size_t)groups * (chunks * stride + NQ + 2 * (size_t)m + 1);
-    const size_t need_stats = (size_t)s.n * C * M + (size_t)s.n * NQ * nblk;
+    const int lq = lg < 3 ? lg : 3;
+    const size_t need_stats = (size_t)s.n * C * M + (size_t)s.n * ((size_t)(NQ - C) * nblk + ((size_t)C * nblk << (lg - lq)));
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     CVA_CUDA_TRY(cudaStreamIsCapturing(st, &cap));
     if (s.alive_cap < need || s.alive_stats_cap < need_stats) {
@@ -356,9 +362,11 @@ cva_status alive_regress(Sim &s, int pf, float *pred_dev, double *coef_host, int
     a.disc = s.d_disc;
     a.feat = s.d_features;
     a.dstat = s.d_alive_stats;
-    a.qsum = s.d_alive_stats + (size_t)s.n * C * M;
+    a.psum = s.d_alive_stats + (size_t)s.n * C * M;
+    a.qsum = a.psum + (size_t)s.n * (NQ - C) * nblk;
     a.nblk = nblk;
     a.lg = lg;
+    a.lq = lq;
     a.chunks = (int)chunks;
     a.stride = stride;
     a.part = s.d_alive;

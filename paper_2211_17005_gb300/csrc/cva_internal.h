@@ -94,7 +94,7 @@ struct Sim {
     double *d_lsq = nullptr;
     size_t lsq_cap = 0;
     // scratch of the regression on (default indicators, state), owned by the simulation
-    float *d_alive_stats = nullptr;   // [n][C][M] per-path default counts, [n][C(C-1)/2 + C][tiles] pair and loss sums
+    float *d_alive_stats = nullptr;   // [n][C][M] per-path default counts, [n][C(C-1)/2][tiles] pair sums, [n][C][..] loss sums
     size_t alive_stats_cap = 0;
     double *d_alive = nullptr;        // Gram partials, coefficients, status
     size_t alive_cap = 0;

@@ -277,3 +277,33 @@ def test_adjoints_of_paths_are_added_in_fp64(api, name, n):
     assert c * 129 == pytest.approx(c1 * 128 + c2, rel=1e-12)
     ref = g1 * 128 + g2
     np.testing.assert_allclose(g * 129, ref, rtol=1e-12, atol=1e-12 * np.abs(ref).max())
+
+
+@pytest.mark.parametrize("C", [2, 8])
+def test_alive_losses_are_added_in_fp64_beyond_eight_paths(api, C):
+    """Losses whose sums over eight paths are exact in FP32 and whose sum over a tile is not: the
+    buffers of a simulation are overwritten with them, one counterparty defaulting at step 1 in
+    every other draw and the next one, with the loss, at step 3."""
+    M, N, n, j = 32, 2, 5, 2
+    model = W.single_swap_model(tuple(0.02 + 0.01 * c for c in range(C)))
+    pf = W._swaps(np.random.default_rng(2), 10, 1, C, 1.0, 5.0)
+    sim = api.Simulation(model, [pf], W.Grid(5.0, n), M, N, keep_defaults=True)
+    sim.run(1)
+    loss = np.repeat([2.0 ** 30, 1.0, -2.0 ** 30, 1.0], 8)
+    y = np.arange(M) % 4 + np.arange(M) // 16
+    sim.defaults().fill_(n + 1)
+    sim.defaults()[:, 0, 0] = 1
+    sim.defaults()[:, 0, 1] = 3
+    sim.exposures().zero_()
+    sim.exposures()[0, 3, 1] = torch.from_numpy(loss.astype(np.float32)).cuda()
+    sim.discount_integral().zero_()
+    sim.targets().zero_()
+    sim.features()[:, 0] = torch.from_numpy(y.astype(np.float32)).cuda()
+    _, coef, dropped = sim.regress_alive(0)
+    # unknowns: constant, state, the first counterparty; M N rows, of which M with its default
+    A = np.array([[N * M, N * y.sum(), M], [N * y.sum(), N * (y * y).sum(), y.sum()], [M, y.sum(), M]], dtype=np.float64)
+    w = np.linalg.solve(A, [0.0, 0.0, loss.sum()])
+    assert dropped[j] == C - 1
+    rows = np.stack([np.ones(2 * M), np.tile(y, 2), np.repeat([0.0, 1.0], M)], axis=1)   # no loss before, one after
+    np.testing.assert_allclose(rows @ coef[j][:3], rows @ w, rtol=1e-9)
+    sim.close()
