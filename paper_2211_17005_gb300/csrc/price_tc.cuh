@@ -27,7 +27,9 @@
 // tiles 4 b + s, 4 b + s + 4 gridDim.x, ... and for each the part's dates, whose fixing it
 // shares. Each slot has two X buffers (one where K = 24 leaves no room), so that an
 // economy's row is written while the tensor core works on the last one, and two
-// accumulators, so that a date's MtM is read while the next date's is accumulated.
+// accumulators, so that a date's MtM is read while the next date's is accumulated. With one
+// economy a row has no last one to hide behind: one buffer, and two blocks a multiprocessor
+// (50001 paths, 50 dates: 120 us with two buffers, 70 so).
 //
 // Shared memory: W hi | W lo ([NN][KT] each, K-major core matrices), the X buffers
 // (Xhi | Xlo, [128][GK] each) of every slot, the coupons at the fixing [E][512], the bond
@@ -54,7 +56,7 @@ struct PriceTc {
     static constexpr int sX = 2 * NN * KT * 4;            // buffer b of slot s at sX + (s bufs + b) xbuf
     static constexpr int xbuf = 2 * 128 * GK * 4;         // Xhi, then Xlo at + 128 GK 4
     static constexpr int sFixBytes = E * 128 * kPriceSlots * 4, sTabBytes = kPriceTcDates * E * LV * 16;
-    static constexpr int bufs = sX + 2 * kPriceSlots * xbuf + sFixBytes + sTabBytes <= 224 * 1024 ? 2 : 1;
+    static constexpr int bufs = E > 1 && sX + 2 * kPriceSlots * xbuf + sFixBytes + sTabBytes <= 224 * 1024 ? 2 : 1;
     static constexpr int sTab = sX + bufs * kPriceSlots * xbuf;
     static constexpr int sFix = sTab + sTabBytes;
     static constexpr int bytes = sFix + sFixBytes;
@@ -105,7 +107,7 @@ __device__ __forceinline__ void price_row(float (&x)[GK], const float4 *tab, flo
 }
 
 template <int E, int C, int CS, int G, int NPF>
-__global__ void __launch_bounds__(128 * kPriceSlots, 1) price_tc_kernel(OuterArgs a, uint32_t tiles, PriceShape ps)
+__global__ void __launch_bounds__(128 * kPriceSlots, E > 1 ? 1 : 2) price_tc_kernel(OuterArgs a, uint32_t tiles, PriceShape ps)
 {
     constexpr int F = 2 * E - 1 + CS, R = NPF * C;
     extern __shared__ __align__(1024) unsigned char tsm[];
