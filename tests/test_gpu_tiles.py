@@ -307,3 +307,56 @@ def test_alive_losses_are_added_in_fp64_beyond_eight_paths(api, C):
     rows = np.stack([np.ones(2 * M), np.tile(y, 2), np.repeat([0.0, 1.0], M)], axis=1)   # no loss before, one after
     np.testing.assert_allclose(rows @ coef[j][:3], rows @ w, rtol=1e-9)
     sim.close()
+
+
+@pytest.mark.parametrize("name,M,n,S,tiles", [
+    ("paper", 130, 20, 2, (64, 256, 0, 2432, 0)), ("paper", 700, 100, 1, (64, 128, 0, 2432, 4)),
+    ("batched", 130, 20, 1, (64, 256, 0, 2432, 0)), ("batched", 300, 20, 1, (128, 256, 0, 2432, 1)),
+    ("batched", 300, 120, 1, (128, 256, 0, 2432, 4)), ("small", 257, 50, 1, (64, 256, 0, 2432, 4)),
+    ("small", 30001, 50, 1, (128, 256, 0, 2432, 0)), ("mixed", 70, 40, 1, (128, 256, 0, 2432, 0))])
+def test_nested_restart_in_every_form(api, name, M, n, S, tiles):
+    """Copies that start at the branch date leave what whole copies leave: every simulation form,
+    pricing form and portfolio count, branches at a reset date and inside a period."""
+    wl = W.make(name, M=M, N=4, n_steps=n, substeps=S)
+    sim = api.Simulation(wl.model, wl.portfolios, wl.grid, M, 4)
+    sim.set_tiles(*tiles)
+    what = ("features", "discount_integral", "thresholds", "exposures", "targets")
+    for date in (n // 5, n // 2 + 1, n - 1):
+        sim.nested_reference(wl.seed, date, 2)
+        left = {w: getattr(sim, w)().clone() for w in what}
+        for w in what:
+            getattr(sim, w)().fill_(float("nan"))
+        sim.run_twin(wl.seed, date, 2)
+        for w in what:
+            assert torch.equal(getattr(sim, w)(), left[w]), (w, date)
+    sim.close()
+
+
+@pytest.mark.parametrize("name,basis,M", [("paper", "linear", 70000), ("paper", "linear", 70001), ("small", "linear", 140003),
+                                          ("batched", "poly2", 9001)])
+def test_fit_of_long_chunks(api, name, basis, M):
+    """Chunks of more rows than a lane's FP32 run (256), and several chunks of six targets."""
+    wl = W.make(name, M=M, N=2, n_steps=20)
+    sim = api.Simulation(wl.model, wl.portfolios, wl.grid, M, 2)
+    sim.set_tiles(128, 256, 0, 152 if basis == "linear" else 2432, 0)
+    sim.run(wl.seed)
+    pred, _ = sim.regress_portfolios(basis)
+    j = 7
+    Y = sim.features()[j].cpu().numpy().astype(np.float64)
+    xi = sim.targets()[:, j].cpu().numpy().astype(np.float64)
+    d = Y[0] - Y[0].mean()
+    ref = _fit64(np.stack([d, d ** 2]) if basis == "poly2" else Y, xi)
+    gap = np.sqrt(np.mean((pred[:, j].cpu().numpy() - ref) ** 2, axis=1))
+    assert np.all(gap <= 261 * 2.0 ** -24 * 30 * np.sqrt(np.mean(xi ** 2, axis=1))), gap   # correlated factors
+    sim.close()
+
+
+@pytest.mark.parametrize("K", [1, 3, 16])
+def test_checkpoints_of_the_run_time_shapes(api, K):
+    """Only these recompute from checkpoints: the interval changes no operation of a path."""
+    wl = W.make("mixed", M=300, n_steps=20)
+    pf = api.frozen(wl.model, wl.portfolios[1])
+    c, g = api.grad_cva0(wl.model, pf, wl.grid, 300, wl.seed, ckpt_every=10)
+    ck, gk = api.grad_cva0(wl.model, pf, wl.grid, 300, wl.seed, ckpt_every=K)
+    assert ck == pytest.approx(c, rel=1e-12)
+    np.testing.assert_allclose(gk, g, rtol=1e-12, atol=1e-12 * np.abs(g).max())
