@@ -980,19 +980,16 @@ cva_status cva_grad_cva0(const cva_model_desc *model, const cva_portfolio_desc *
     const unsigned blocks = (unsigned)((M + 127) / 128);
     cudaStream_t cs = reinterpret_cast<cudaStream_t>(stream);
     const size_t nsum = s.generic ? (size_t)NPAR + 1 : (size_t)(2 * E + 1 + NPAR);
-    unsigned char *tables = nullptr;
+    unsigned char *block = nullptr;   // tables, sums and (compiled shapes) arrays
     auto cleanup = [&]() {
-        cudaFree(tables);
+        cudaFree(block);
         cudaFree(b.ckpt);
         cudaFree(b.ckpt_I0);
         cudaFree(b.fixr);
         cudaFree(b.part);
-        cudaFree(b.sum);
-        cudaFree(b.scratch);
         cva_sim_destroy(hs);
     };
-    // the tables in one block, before the arrays whose size has a choice
-    std::vector<unsigned char> img;
+    std::vector<unsigned char> img;   // the tables
     auto put = [&](const void *v, size_t bytes) {
         const size_t at = img.size();
         img.resize(at + (bytes + 255) / 256 * 256);
@@ -1002,20 +999,6 @@ cva_status cva_grad_cva0(const cva_model_desc *model, const cva_portfolio_desc *
     const size_t o_dzc = put(dzc.data(), dzc.size() * sizeof(float4)), o_dfix = put(dfix.data(), dfix.size() * sizeof(float2)),
                  o_ddrift = put(ddrift.data(), ddrift.size() * sizeof(float2)),
                  o_rho = put(rho.data(), rho.size() * sizeof(float)), o_sig = put(sig.data(), sig.size() * sizeof(float));
-    st = dev_alloc(&tables, img.size());
-    if (st == CVA_OK) {
-        const cudaError_t e = cudaMemcpyAsync(tables, img.data(), img.size(), cudaMemcpyHostToDevice, cs);
-        if (e != cudaSuccess) st = cuda_fail(e, "grad: table upload");
-    }
-    if (st != CVA_OK) {
-        cleanup();
-        return st;
-    }
-    b.dzc = reinterpret_cast<float4 *>(tables + o_dzc);
-    b.dfix = reinterpret_cast<float2 *>(tables + o_dfix);
-    b.ddrift = reinterpret_cast<float2 *>(tables + o_ddrift);
-    b.rho = reinterpret_cast<float *>(tables + o_rho);
-    b.sig = reinterpret_cast<float *>(tables + o_sig);
     // the compiled shapes take the paths in equal ranges whose arrays fit a limit and half of
     // the memory that is free, in narrower ones where that cannot be had; the run-time shapes
     // take them at once, with checkpoints
@@ -1023,7 +1006,7 @@ cva_status cva_grad_cva0(const cva_model_desc *model, const cva_portfolio_desc *
     plan.per = M;
     plan.ranges = 1;
     if (s.generic) {
-        if (dev_alloc(&b.sum, nsum) != CVA_OK || dev_alloc(&b.ckpt, (size_t)b.nseg * NV * Mz) != CVA_OK ||
+        if (dev_alloc(&block, img.size() + nsum * sizeof(double)) != CVA_OK || dev_alloc(&b.ckpt, (size_t)b.nseg * NV * Mz) != CVA_OK ||
             dev_alloc(&b.ckpt_I0, (size_t)b.nseg * Mz) != CVA_OK ||
             dev_alloc(&b.fixr, (size_t)(periods + 1) * E * Mz) != CVA_OK ||
             dev_alloc(&b.part, (size_t)blocks * (NPAR + 1)) != CVA_OK)
@@ -1039,15 +1022,25 @@ cva_status cva_grad_cva0(const cva_model_desc *model, const cva_portfolio_desc *
             (void)launch_adjoint(s, b, seed, k0, (uint32_t)paths, cs);
             return b.scratch_bytes;
         };
+        auto sum_bytes = [&](const RangePlan &p) { return (nsum * p.ranges * sizeof(double) + 255) / 256 * 256; };
         auto allocate = [&](const RangePlan &p) {
-            if (dev_alloc(&b.sum, nsum * p.ranges) == CVA_OK && dev_alloc(&b.scratch, p.bytes) == CVA_OK) return true;
+            if (dev_alloc(&block, img.size() + sum_bytes(p) + p.bytes) == CVA_OK) return true;
             cudaGetLastError();   // (the failed allocation's)
-            cudaFree(b.sum);
-            b.sum = nullptr;
             return false;
         };
         if (st == CVA_OK && !fit_ranges(M, std::min(kAdjScratch, room / 2), bytes, allocate, &plan)) st = CVA_ENOMEM;
+        if (st == CVA_OK) b.scratch = block + img.size() + sum_bytes(plan);
         b.scratch_bytes = plan.bytes;
+    }
+    if (st == CVA_OK) {
+        b.dzc = reinterpret_cast<float4 *>(block + o_dzc);
+        b.dfix = reinterpret_cast<float2 *>(block + o_dfix);
+        b.ddrift = reinterpret_cast<float2 *>(block + o_ddrift);
+        b.rho = reinterpret_cast<float *>(block + o_rho);
+        b.sig = reinterpret_cast<float *>(block + o_sig);
+        b.sum = reinterpret_cast<double *>(block + img.size());
+        const cudaError_t e = cudaMemcpyAsync(block, img.data(), img.size(), cudaMemcpyHostToDevice, cs);
+        if (e != cudaSuccess) st = cuda_fail(e, "grad: table upload");
     }
     if (st != CVA_OK) {
         cleanup();
