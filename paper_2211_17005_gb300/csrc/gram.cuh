@@ -9,6 +9,7 @@
 #include <atomic>
 
 #include "cva_internal.h"
+#include "sum_pair.cuh"
 
 namespace cva {
 namespace {
@@ -221,17 +222,7 @@ __global__ void __launch_bounds__(MAXT, MINB) gram_kernel(GramArgs a)
 
 // The sums of the quadratic basis [1, d, d^2], d = y - y^0 of factor 0, and NT targets.
 // The normal equations of d and d^2 are sensitive to rounding, so every FP32 product is
-// added to a pair (sum, its rounding errors): as exact as FP64 sums, without the FP64 pipe.
-struct SumPair {
-    float hi, lo;
-    __device__ void add(float p, float e = 0.f)
-    {
-        const float s = hi + p, b = s - hi;
-        lo += ((hi - (s - b)) + (p - b)) + e;
-        hi = s;
-    }
-};
-
+// added to a SumPair.
 // Bound by latency: 49 dates of 2^14 paths take 16 us (49 us as a case of the general kernel,
 // with its FP64 runs).
 template <int NT>

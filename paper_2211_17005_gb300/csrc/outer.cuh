@@ -26,13 +26,16 @@
 
 #include "cva_internal.h"
 #include "rng.cuh"
+#include "sum_pair.cuh"
 #include "umma.cuh"
 
 namespace cva {
 namespace {
 
 static __constant__ SimConsts c_sim;
+#ifdef CVA_CONST_WEIGHTS   // the run-time-shape adjoint's; every other kernel reads them from global memory
 static __constant__ SimWeights c_w;
+#endif
 
 // two FP32 values in one register pair, operated on together
 using f32x2 = unsigned long long;
@@ -61,17 +64,6 @@ __device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b)
     return r;
 }
 
-// a sum of FP32 terms and the rounding errors made in it: as exact as an FP64 sum
-struct SumPair {
-    float hi, lo;
-    __device__ void add(float p, float e = 0.f)   // p + e, e the error of p
-    {
-        const float s = hi + p, b = s - hi;
-        lo += ((hi - (s - b)) + (p - b)) + e;
-        hi = s;
-    }
-};
-
 // expm1(x) by its Taylor series to degree 8 for |x| <= 1/4 (relative error below
 // 2e-10 there, so the rounding of the FMAs dominates), library expm1f elsewhere.
 __device__ __forceinline__ float expm1_small(float x)
@@ -96,7 +88,6 @@ struct OuterArgs {
     uint32_t branch;
     const float4 *__restrict__ zc;     // [n+1][E][G] (lnA, B, dlnA, dB)
     const float2 *__restrict__ fix;    // [periods+1][E] (lnA, B)
-    const int *__restrict__ date_p;    // [n+1]
     const float *__restrict__ drift;   // [n*S][E]
     float *features, *disc, *thr, *expo, *mtm;
     const float *w_glob;               // device copy of the date-bucketed weights: wA [kMaxW], then wK [kMaxW]
@@ -693,9 +684,12 @@ static cudaEvent_t t_last[64] = {};
 static cudaError_t upload_consts(const Sim &s, cudaStream_t st)
 {
     cudaError_t e = cudaMemcpyToSymbolAsync(c_sim, s.d_const_img, sizeof(SimConsts), 0, cudaMemcpyDeviceToDevice, st);
-    if (e != cudaSuccess) return e;
-    return cudaMemcpyToSymbolAsync(c_w, s.d_const_img + sizeof(SimConsts), sizeof(SimWeights), 0,
-                                   cudaMemcpyDeviceToDevice, st);
+#ifdef CVA_CONST_WEIGHTS
+    if (e == cudaSuccess)
+        e = cudaMemcpyToSymbolAsync(c_w, s.d_const_img + sizeof(SimConsts), sizeof(SimWeights), 0,
+                                    cudaMemcpyDeviceToDevice, st);
+#endif
+    return e;
 }
 
 static void outer_forget(const Sim *s)
@@ -736,7 +730,6 @@ cva_status outer_launch(Sim &s, uint64_t seed, uint64_t k0, cudaStream_t st)
     args.seed_hi = (uint32_t)(seed >> 32);
     args.zc = s.d_zc;
     args.fix = s.d_fix;
-    args.date_p = s.d_date_p;
     args.drift = s.d_drift;
     args.features = s.d_features;
     args.disc = s.d_disc;

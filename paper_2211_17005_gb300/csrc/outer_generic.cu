@@ -13,6 +13,7 @@
 // 80 us.
 #include <atomic>
 
+#define CVA_CONST_WEIGHTS
 #include "outer.cuh"
 
 namespace cva {
@@ -659,7 +660,6 @@ cva_status outer_generic_launch(Sim &s, uint64_t seed, uint64_t k0, cudaStream_t
     args.branch = s.branch;
     args.zc = s.d_zc;
     args.fix = s.d_fix;
-    args.date_p = s.d_date_p;
     args.drift = s.d_drift;
     args.features = s.d_features;
     args.disc = s.d_disc;
