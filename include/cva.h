@@ -144,9 +144,13 @@ CVA_API cva_status cva_simulate_twin(cva_sim *sim, uint64_t seed, uint64_t k0, i
  * receives, for every outer path, the mean over twin copies b = 1..copies
  * (cva_simulate_twin, branched at `date`) of the averaged target of portfolio pf
  * at that date, an estimate of E[xi_bar_date | state at t_date] whose error falls
- * as 1/sqrt(copies). Runs `copies` full simulations on `stream` and leaves the
- * last copy in the simulation's buffers. CVA_EINVAL for date outside [0, n),
- * copies outside [1, 2^24) or a bad portfolio index. */
+ * as 1/sqrt(copies). Runs the copies on `stream`, the compiled shapes' from the second
+ * on from the branch date, and leaves the last one in the simulation's buffers, whole. The
+ * first call of a compiled shape with a date above 0 and two copies or more allocates (8 C + 8) M
+ * bytes, which the simulation keeps for its life: make one before capturing this one in
+ * a CUDA graph (without the memory, or captured first, every copy runs from date 0, with the
+ * same results). CVA_EINVAL for date outside [0, n), copies outside [1, 2^24) or a
+ * bad portfolio index. */
 CVA_API cva_status cva_nested_reference(cva_sim *sim, uint64_t seed, uint64_t k0, int pf, int date, int copies,
                                         float *out_dev, void *stream);
 
@@ -245,7 +249,7 @@ CVA_API cva_status cva_cva0(const float *xi0_dev, uint64_t M, double *out2_host,
  * basis: CVA_BASIS_LINEAR  phi = [1, Y_1, ..., Y_F]        (m = F + 1)
  *        CVA_BASIS_POLY2   phi = [1, y, y^2] of factor 0     (m = 3)
  * The normal equations are accumulated in FP64 on the centred, scaled basis and
- * solved by Cholesky in FP64. pred_dev (float [M], nullable) receives
+ * solved by L D L^T in FP64. pred_dev (float [M], nullable) receives
  * phi(Y_k)^T w; coef_host (double [m], nullable) receives w in the raw basis
  * (w_0 + w_1 y + ... ). Synchronises `stream` when coef_host is not NULL.
  * CVA_ENUMERIC if the normal matrix is singular. */
@@ -301,7 +305,7 @@ CVA_API cva_status cva_regress_all(const cva_sim *sim, int pf, int basis, float 
 /* Least squares of eq. (e:forw) for every date 1..n-1 and every portfolio of a
  * simulation in one grouped launch: the portfolios share each date's features,
  * so every date's normal matrix is accumulated once (FP64) with one target column
- * per portfolio and solved once (Cholesky, FP64) for all of them. pred_dev: float
+ * per portfolio and solved once (L D L^T, FP64) for all of them. pred_dev: float
  * [n_pf][n][M] (date 0 untouched), nullable; coef_host: double [n_pf][n][m]
  * (date 0 untouched), nullable. The scratch belongs to the simulation: the first
  * call allocates it, so make one call before capturing this one in a CUDA graph.
@@ -321,7 +325,7 @@ CVA_API cva_status cva_regress_portfolios(cva_sim *sim, int basis, float *pred_d
  * The M N rows are not formed: per path, exact integer counts over the N draws
  * (defaults of c, joint defaults of c and d) and the sums of the target over the
  * draws where c has defaulted give the normal equations (FP64 accumulation), solved
- * by a Jacobi-scaled Cholesky factorisation in FP64; a column whose pivot vanishes
+ * by a Jacobi-scaled factorisation L D L^T in FP64; a column whose pivot vanishes
  * (no default of c by t_i in the whole sample) is dropped, with coefficient 0.
  * Needs a simulation created with CVA_KEEP_DEFAULTS after cva_simulate; C <= 8,
  * 1 + F + C <= 40 and N (5C + 6) <= 160 KB (N <= 3400 at C = 8; else CVA_ENOTSUP).
@@ -377,8 +381,8 @@ CVA_API cva_status cva_set_tiles(cva_sim *sim, int sim_block, int price_block, i
  * FP64. The fast-path shapes of cva_sim_create with one portfolio, (E, C) = (1, 2
  * constant) and (10, 8 CIR), have compiled adjoint kernels: simulate, price with the
  * pricing's derivatives, and sweep the Euler steps back, over ranges of paths whose
- * arrays (every pricing date's state and derivatives) take up to 1.4 GB, less where that
- * is not free. Every other shape within the limits of cva_sim_create runs the
+ * arrays (every pricing date's state and derivatives) take up to 1.4 GB and half of the
+ * free memory at most, less where that cannot be had. Every other shape within the limits of cva_sim_create runs the
  * run-time-shape adjoint, slower (its per-path arrays live in local memory): its forward
  * sweep keeps the state every ckpt_every pricing dates, and the reverse sweep recomputes
  * each segment from its checkpoint. ckpt_every <= 16 and sub-steps <= 4 for both. A constant intensity's kappa_c,
@@ -476,7 +480,7 @@ CVA_API cva_status cva_mlp_regress_all(const cva_sim *sim, int pf, int hidden, i
  * device-wide synchronisation of cudaMalloc/cudaFree.
  *
  * It fits `groups` independent least-squares problems exactly like cva_regress
- * (same bases, same FP64 normal equations and Cholesky solve), group g reading
+ * (same bases, same FP64 normal equations and solve), group g reading
  * targets_dev + g*M (float [M]) and features_dev + g*F*M (float [F][M]) and
  * writing pred_dev + g*M (float [M], nullable) and coef_host + g*m (double,
  * nullable; m = F+1 linear, 3 poly2).

@@ -18,7 +18,7 @@
 // sums of P_cd and the sums of q_c over at most eight paths at every date. gram.cuh accumulates sum_k [1, Y - Y^0]^T
 // [1, Y - Y^0, d, xi_bar]. alive_pq_kernel adds the P_cd and q_c.
 // alive_solve_kernel adds the Gram chunks, assembles the (1 + F + C)-square system and
-// solves it by a Jacobi-scaled Cholesky factorisation in FP64, dropping a column whose
+// solves it by a Jacobi-scaled factorisation L D L^T in FP64, dropping a column whose
 // pivot vanishes (a counterparty with no default by t_i anywhere in the sample).
 #include <math.h>
 
@@ -310,7 +310,8 @@ cva_status alive_regress(Sim &s, int pf, float *pred_dev, double *coef_host, int
     if (s.M > 0x7fffffffull) return fail(CVA_EINVAL, "regress_alive: M too large");
     const int C = s.C, NQ = C * (C - 1) / 2 + C, mY = s.F + 1, m = mY + C;
     if (m > kMaxUnknowns) return fail(CVA_ENOTSUP, "regress_alive: 1 + F + C must be <= 40");
-    // the number of draws this call takes
+    // the number of draws this call takes: N (5C + 6) within 160 KB (the kernel stages 64 at a time
+    // and could take more: up to 65535, which its 16-bit counters hold)
     const size_t draw_floats = ((size_t)s.N * (C + 1) * 4 + 15) / 16 * 16;
     if ((draw_floats + (size_t)s.N * (C + 2) + 15) / 16 * 16 + 64 * (size_t)(2 * C + C * (C - 1) / 2) > (size_t)160 * 1024)
         return fail(CVA_ENOTSUP, "regress_alive: N * C too large for the per-path draw tables");

@@ -3,7 +3,7 @@
 // The augmented Gram matrix [phi, xi]^T [phi, xi] of the basis centred on path 0's
 // state is accumulated by gram.cuh (FP32 products in short FP32 runs, then FP64 in a
 // fixed order; every byte of the features and targets is read once) and solved by a
-// Jacobi-scaled Cholesky factorisation in FP64. A second pass over the features makes
+// Jacobi-scaled factorisation L D L^T in FP64. A second pass over the features makes
 // the predictions, from the last group back, whose features are still in L2.
 #include <cuda.h>
 #include <cudaTypedefs.h>

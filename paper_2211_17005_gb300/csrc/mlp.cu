@@ -74,7 +74,7 @@ __host__ __device__ constexpr uint32_t row_off(uint32_t r, uint32_t c)
 
 template <int U>
 struct Layout {
-    static_assert(U == 64, "the operand rows [dH2 | dH1] and [H1 | 1 | X | 1] are 128 wide for U = 64");
+    static_assert(U == 64, "the operand rows [dH2 | dH1] and [H1 | 1 | X] fit 128 columns for U = 64");
     static constexpr int NP = 35 * U + U * U + 2;     // parameters
     static constexpr int NPpad = (NP + 63) / 64 * 64;
     static constexpr int oW1 = 0, ob1 = kIn * U, oW2 = ob1 + U, ob2 = oW2 + U * U, ow3 = ob2 + U,
@@ -555,10 +555,6 @@ __device__ void net_teardown(Net<U> &n)
     if (n.warp == 0) umma::tmem_dealloc(n.tmem, Layout<U>::tmem_cols);
 }
 
-// One epoch (or its first n_steps batches) of Adam on one cluster of CL >= 4 CTAs.
-// Batch b covers paths [b * P, (b + 1) * P), P = tiles_per_batch * 128; in each
-// step the cluster's 2 CL slots take the batch's tiles round-robin.
-//
 // W consecutive words (aligned to them) in one access
 template <int W>
 __device__ __forceinline__ void load_words(const float *p, float *v)
@@ -593,6 +589,10 @@ __device__ __forceinline__ void store_words_cg(float *p, const float *v)
     for (int i = 0; i < W; i += 2) __stcg(reinterpret_cast<float2 *>(p + i), make_float2(v[i], v[i + 1]));
 }
 
+// One epoch (or its first n_steps batches) of Adam on one cluster of CL >= 4 CTAs.
+// Batch b covers paths [b * P, (b + 1) * P), P = tiles_per_batch * 128; in each
+// step the cluster's 2 CL slots take the batch's tiles round-robin.
+//
 // The exchange of one Adam step moves data only by bulk copies between the CTAs'
 // shared memories, each completing on the receiver's mbarrier (no cluster-wide
 // barrier inside the step loop):

@@ -112,9 +112,11 @@ struct OuterArgs {
 // load and one FMA per entry.
 //
 // Modes: forward, for the smooth CVA_0, which keeps e^{-Lambda} in the place of the thresholds;
-// adjoint, which also keeps the increments and intensities of every fine step; restart, a run that starts at a
-// pricing date or saves what such a run needs (separate instances: their pointers would
-// spill the plain one's registers).
+// adjoint, which also keeps the increments and intensities of every fine step; restart, a
+// run that starts at a pricing date or saves what such a run needs. Separate instances, as
+// their pointers would cost the plain one's four-warp form its registers; the eight-warp
+// forms, which small path counts take, hold 80 for three blocks a multiprocessor and spill
+// some of them.
 //
 // Bound by instruction issue (Philox, logarithm, square root and sine-cosine of 14
 // Box-Muller pairs, the correlation): 2650 instructions a (path, step) at 27 factors and

@@ -243,10 +243,10 @@ __global__ void __launch_bounds__(kGenPriceThreads, 4) price_generic_kernel(Oute
 }
 
 // ---- adjoint of the smooth CVA_0 for run-time shapes ----
-// adjoint_kernel (adjoint.cuh) with the model's sizes as run-time values: the same
-// forward sweep with checkpoints every K dates, the same segment recompute and
-// reverse of the pricing and of the Euler sub-steps, in the same order, so a shape
-// with a compiled adjoint gives its bits. The stochastic intensity of counterparty c
+// One thread per path: a forward sweep with checkpoints every K dates, then segment by segment
+// from the last a recompute and the reverse of the pricing and of the Euler sub-steps. The
+// functional and its derivatives are those of adjoint.cuh, whose kernels add in another
+// order. The stochastic intensity of counterparty c
 // is state factor c_sim.gpos[c] (-1: constant, whose kappa, theta, nu receive
 // nothing). Per-thread arrays are sized at the library's limits (local memory); the
 // parameter adjoints live in dynamic shared memory, NPAR x 128 floats.
