@@ -94,14 +94,26 @@ def sim_instr_per_path_step(wl):
     return S * sub + 12 * C
 
 
-def price_instr_per_path_date(wl):
-    """Algorithmic lane-instructions of the pricing kernel per (path, pricing date):
-    20 per economy for the first live bond and the running fixing, 12 per (economy,
-    reset date) for the chained bond prices and their differences (degree-8 series),
-    (2G+1) per (portfolio, counterparty, economy) for the date-bucketed MtM, 3 per
-    (portfolio, counterparty) for the exposure and 6 for the discount factor."""
+def price_instr_per_path_date(wl, live=None):
+    """Algorithmic lane-instructions of the pricing kernel per (path, pricing date) with
+    `live` reset dates still to come (default: all G, a date of the first period): 20 per
+    economy for the first live bond and the running fixing, 12 per (economy, live reset
+    date) for the chained bond prices and their differences (degree-8 series), 2 live + 1
+    per (portfolio, counterparty, economy) for the date-bucketed MtM, 3 per (portfolio,
+    counterparty) for the exposure and 6 for the discount factor."""
     E, C, CS, F, G, NPF, S = _shape(wl)
-    return 20 * E + 12 * E * G + NPF * C * E * (2 * G + 1) + 3 * NPF * C + 6
+    live = G if live is None else live
+    return 20 * E + 12 * E * live + NPF * C * E * (2 * live + 1) + 3 * NPF * C + 6
+
+
+def price_instr_mean(wl):
+    """price_instr_per_path_date averaged over the dates 1..n: date j lies in period
+    p = (j - 1) // (dates per period), whose live reset dates are the G - p later ones (none:
+    the exposures are zero and nothing is computed)."""
+    G, n = _shape(wl)[4], wl.grid.n_steps
+    per = round(wl.portfolios[0].delta * n / wl.grid.horizon)
+    live = [max(G - (j - 1) // per, 0) for j in range(1, n + 1)]
+    return sum(price_instr_per_path_date(wl, v) for v in live if v) / n
 
 
 # DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) per unit of work from one
@@ -555,7 +567,7 @@ def main():
     peak_alu = alu_peak_lane_instr_per_s(sm_mhz, n_sms)
     pipes = api.pipe_peaks() if rank == 0 else None
     kern = {"sim_kernel": (sim_instr_per_path_step(wl), s_avg, "path-step"),
-            "price_kernel": (price_instr_per_path_date(wl), p_avg, "path-date")}
+            "price_kernel": (price_instr_mean(wl), p_avg, "path-date")}
     alu = {}
     for name, (per_unit, ms, unit) in kern.items():
         ach = per_unit * wl.M * n / (ms / 1e3)
