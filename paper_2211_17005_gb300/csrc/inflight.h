@@ -16,14 +16,20 @@
 
 namespace cva {
 
-// Whether copy u is complete, by wait(barrier, parity). `issued`: the copies issued so far, of
-// which the last B may be in flight; `issuer`: this thread issues them.
+// The second wait, by wait(barrier, parity): of the copies issued so far the last B may be in
+// flight.
+template <uint32_t B, class Wait>
+CVA_HD void settle_copies(uint32_t issued, Wait wait)
+{
+    for (uint32_t v = issued > B ? issued - B : 0u; v < issued; ++v) (void)wait(v % B, (v / B) & 1u);
+}
+
+// Whether copy u is complete; `issuer`: this thread issues them.
 template <uint32_t B, class Wait>
 CVA_HD bool await_copy(uint32_t u, uint32_t issued, bool issuer, Wait wait)
 {
     if (wait(u % B, (u / B) & 1u)) return true;
-    if (issuer)
-        for (uint32_t v = issued > B ? issued - B : 0u; v < issued; ++v) (void)wait(v % B, (v / B) & 1u);
+    if (issuer) settle_copies<B>(issued, wait);
     return false;
 }
 

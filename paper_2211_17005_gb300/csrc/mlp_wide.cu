@@ -930,6 +930,13 @@ __global__ void __launch_bounds__(kWThreads, MinBlocks) wide_sweep_kernel(WSweep
     wide_teardown(n, &s_mbar[2]);
 }
 
+// await_copy's second wait for the two staging buffers at sbar; out of line, as inlined where it
+// is never reached it costs the pass 3%
+__device__ __noinline__ void fwd_settle(uint64_t *sbar, uint32_t issued)
+{
+    settle_copies<2>(issued, [&](uint32_t b, uint32_t p) { return umma::mbar_wait(sbar + b, p, kMbarPolls); });
+}
+
 // Loss (mode 0) and prediction (mode 2) passes: the forward pass of the trainer's tiles.
 // Two groups of 256 threads (two threads per row, 64 hidden columns each) take the CTA's
 // tiles alternately, each with its own B buffer, accumulator and two staging buffers, so
@@ -1014,11 +1021,10 @@ __global__ void __launch_bounds__(kFwdThreads, 1) wide_fwd_kernel(WSweepArgs a, 
     // y receives the target
     auto stage_into = [&](uint32_t i, float &y) {
         const int q = 2 * grp + (int)(i & 1u);
-        if (copies_ok)   // (tiles i and i + 1 are requested by now)
-            copies_ok = await_copy<2>(i, min(K, i + 2u), gt == 32, [&](uint32_t b, uint32_t p) {
-                return umma::mbar_wait(&s_sbar[2 * grp + (int)b], p, kMbarPolls);
-            });
-        ok = ok && copies_ok;
+        if (copies_ok && !umma::mbar_wait(&s_sbar[q], (i >> 1) & 1u, kMbarPolls)) {
+            ok = copies_ok = false;
+            if (gt == 32) fwd_settle(&s_sbar[2 * grp], min(K, i + 2u));   // (tiles up to i + 1 are requested)
+        }
         const float *stg = reinterpret_cast<const float *>(smem + L::sStage + q * L::stage_bytes);
         const float4 *mv = reinterpret_cast<const float4 *>(n.mean), *iv = reinterpret_cast<const float4 *>(n.istd);
         float x[16];

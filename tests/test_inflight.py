@@ -65,7 +65,10 @@ int main()
             Bars<2> bars;
             bool good = true;
             auto stage = [&](unsigned i) {
-                if (good) good = cva::await_copy<2>(i, K < i + 2 ? K : i + 2, true, bars.bounded());
+                if (good && !bars.wait(i & 1u, (i >> 1) & 1u)) {
+                    good = false;
+                    cva::settle_copies<2>(K < i + 2 ? K : i + 2, bars.bounded());
+                }
             };
             for (unsigned i = 0; i < K && i < 2; ++i) bars.issue(i & 1u);
             stage(0);
