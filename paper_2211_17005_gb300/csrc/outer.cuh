@@ -813,6 +813,7 @@ cva_status outer_launch(Sim &s, uint64_t seed, uint64_t k0, cudaStream_t st)
 template <int E, int C, int CS, int G>
 cva_status adjoint_launch(Sim &s, AdjBuffers &b, uint64_t seed, uint64_t k0, uint32_t M, cudaStream_t st)
 {
+    // (the run-time shapes' limits, kept here so that what a call takes does not depend on the shape)
     constexpr int KMAX = 16, SMAX = 4, F = 2 * E - 1 + CS, NPAR = 3 * E - 1 + 3 * C;
     if (b.K < 1 || b.K > KMAX || s.S > SMAX) return fail(CVA_ENOTSUP, "adjoint: checkpoint interval <= 16, sub-steps <= 4");
     int dev = 0, sms = 0;
