@@ -1,7 +1,7 @@
 // Bounded waits for the copies that one thread issues on B mbarriers in turn: copy u completes
 // phase u / B of barrier u % B. A barrier's parity tells two neighbouring phases apart and no
 // more, so at most one copy may be in flight per barrier. After a wait that gave up, the issuer
-// therefore requests nothing more, and before it goes on it waits once more, in full, for all it
+// therefore requests nothing more, and before it leaves it waits once more, in full, for all it
 // has in flight: no copy outlives its CTA.
 //
 // Plain C++, so that the protocol can be run on the host.
@@ -22,15 +22,6 @@ template <uint32_t B, class Wait>
 CVA_HD void settle_copies(uint32_t issued, Wait wait)
 {
     for (uint32_t v = issued > B ? issued - B : 0u; v < issued; ++v) (void)wait(v % B, (v / B) & 1u);
-}
-
-// Whether copy u is complete; `issuer`: this thread issues them.
-template <uint32_t B, class Wait>
-CVA_HD bool await_copy(uint32_t u, uint32_t issued, bool issuer, Wait wait)
-{
-    if (wait(u % B, (u / B) & 1u)) return true;
-    if (issuer) settle_copies<B>(issued, wait);
-    return false;
 }
 
 }  // namespace cva

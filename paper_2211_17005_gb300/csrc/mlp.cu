@@ -283,9 +283,9 @@ struct Net {
     // 1/std); y receives the target. False if the bounded wait gave up.
     __device__ bool stage_x(float &y)
     {
-        const bool ok = await_copy<1>(sphase, sphase + 1u, row == 32, [&](uint32_t, uint32_t p) { return umma::mbar_wait(sbar, p, kMbarPolls); });
-        sphase ^= 1u;
-        pending = false;
+        const bool ok = umma::mbar_wait(sbar, sphase, kMbarPolls);
+        sphase ^= ok ? 1u : 0u;   // (after a wait that gave up the teardown waits again)
+        pending = pending && !ok;
         const float4 *mv = reinterpret_cast<const float4 *>(mean), *iv = reinterpret_cast<const float4 *>(istd);
         float x[kIn];
 #pragma unroll

@@ -330,9 +330,9 @@ struct WNetT {
     // columns of B; y receives the target
     __device__ bool stage_x(float &y)
     {
-        const bool ok = await_copy<1>(sphase, sphase + 1u, tid == 32, [&](uint32_t, uint32_t p) { return umma::mbar_wait(sbar, p, kMbarPolls); });
-        sphase ^= 1u;
-        pending = false;
+        const bool ok = umma::mbar_wait(sbar, sphase, kMbarPolls);
+        sphase ^= ok ? 1u : 0u;   // (after a wait that gave up the teardown waits again)
+        pending = pending && !ok;
         const float4 *mv = reinterpret_cast<const float4 *>(mean), *iv = reinterpret_cast<const float4 *>(istd);
         float x[16];
 #pragma unroll
@@ -930,8 +930,8 @@ __global__ void __launch_bounds__(kWThreads, MinBlocks) wide_sweep_kernel(WSweep
     wide_teardown(n, &s_mbar[2]);
 }
 
-// await_copy's second wait for the two staging buffers at sbar; out of line, as inlined where it
-// is never reached it costs the pass 3%
+// settle_copies for the two staging buffers at sbar; out of line, as inlined where it is never
+// reached it costs the pass 3%
 __device__ __noinline__ void fwd_settle(uint64_t *sbar, uint32_t issued)
 {
     settle_copies<2>(issued, [&](uint32_t b, uint32_t p) { return umma::mbar_wait(sbar + b, p, kMbarPolls); });

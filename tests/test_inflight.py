@@ -49,14 +49,14 @@ int main()
         std::srand(trial);
         {   // a tile's copy requested while the last one is worked on
             Bars<1> bars;
-            unsigned phase = 0;
+            unsigned issued = 1;
             bool good = true;
             bars.issue(0);
-            for (int tile = 0; tile < 6 && good; ++tile) {
-                good = cva::await_copy<1>(phase, phase + 1, true, bars.bounded());
-                phase ^= 1u;
-                if (good && tile + 1 < 6) bars.issue(0);
+            for (unsigned tile = 0; tile < 6 && good; ++tile) {
+                good = bars.wait(0, tile & 1u);
+                if (good && tile + 1 < 6) { bars.issue(0); ++issued; }
             }
+            if (!good) cva::settle_copies<1>(issued, bars.bounded());
             must(good == !bars.gave_up, "status");
             must(bars.done == bars.left.size(), "a copy in flight at the end");
         }
