@@ -87,7 +87,7 @@ __host__ __device__ constexpr size_t idx_stage_offset(int rows, int cnt_words, i
 // some of a thread's draws at a time (idx_draws), and leave as whole runs of a path's row.
 // Stored from where they are found, a byte of another path's row per lane, they took longer
 // than the clocks: four counterparties, 65536 paths, 512 draws, 50 dates, the whole simulation
-// 1259 us, so 566 us (519 without the steps); the paper's shape with 256 draws and 20 dates
+// 1259 us, so 535 us (486 without the steps); the paper's shape with 256 draws and 20 dates
 // 1295 and 580 us.
 template <int C, bool IDX>
 __global__ void __launch_bounds__(512) inner_kernel(InnerArgs a)
